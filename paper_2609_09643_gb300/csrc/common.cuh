@@ -66,6 +66,7 @@ struct unison_trace {
   uint64_t n_turns = 0;
   uint64_t n_events = 0;
   uint32_t min_out_tok = 0;
+  uint64_t sum_last_out = 0;  // every session's largest KV size, summed
 
   // One page-locked host block holding every array below, copied to the
   // device with a single cudaMemcpyAsync.

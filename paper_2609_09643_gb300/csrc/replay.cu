@@ -12,11 +12,18 @@
 //                       the event loop re-ranks from these values instead of
 //                       re-dividing every live score at every event; the
 //                       decisions are identical.
-//   replay_kernel       Algorithm 1: one warp per replay; the unpinned
-//                       residents of each tier kept sorted by packed 64-bit
-//                       key in shared memory (the most evictable last), so
-//                       the argmax of a decision is a pop and an update is a
-//                       warp-parallel lower bound plus a block shift.
+//   rank_keys_kernel    the rank of every completion's key in its stream
+//                       (replay_slots.cuh): one block per stream.
+//   slot_kernel         Algorithm 1: one warp per replay; residents in
+//                       unordered slots, each decision one pass over their
+//                       ranks (replay_slots.cuh).
+//   replay_kernel       Algorithm 1 where the slot form does not apply (online
+//                       hazard table, stale snapshots, traces too large for
+//                       its words or lists too large for its slots): one warp
+//                       per replay; the unpinned residents of each tier kept
+//                       sorted by packed 64-bit key (the most evictable last),
+//                       so the argmax of a decision is a pop and an update is
+//                       a warp-parallel lower bound plus a block shift.
 //   ttft_median_kernel  Sec. V-A TTFT p50: radix select of the lower median
 //                       over each replay's per-request TTFT values.
 #include <algorithm>
@@ -28,6 +35,7 @@
 
 #include "common.cuh"
 #include "profile.cuh"
+#include "replay_slots.cuh"
 
 using namespace unison;
 
@@ -49,9 +57,10 @@ struct ComboDesc {
   uint64_t penalty_q;
   uint16_t *sigma;  // [51]
   uint64_t *t2;     // [51]
-  uint64_t *pkey;   // [E] key after the event
+  uint64_t *pkey;   // [E] key after the event, or null
   uint32_t *gq;     // [E] gap average after the event
-  uint64_t *pkb;    // [E] key before the event (arrivals of turn >= 1)
+  uint64_t *pkb;    // [E] key before the event (arrivals of turn >= 1); null with pkey
+  unison_slots::RankDesc rk;  // rank of the key after each completion (rk.rank null: not asked for)
 };
 
 struct ReplayDesc {
@@ -78,6 +87,7 @@ struct ReplayDesc {
   uint64_t penalty;  // P_Z in quantised units (online hazard replays)
   const uint64_t *t2;  // eq. (t2) per turn index of the offline table (stale-snapshot replays)
   uint32_t stale_sync, stale_m;  // UNISON_SYNC_* and arrivals per sync
+  unison_slots::SlotDesc slot;   // replays of the slot form
 };
 
 // --------------------------------------------------------------------------
@@ -179,13 +189,28 @@ __global__ void key_stream_kernel(const ComboDesc *combos) {
     const uint64_t key = __umul64hi((no_gap ? 0 : g) * kLambda, mg[t]) + t2[t];
     const uint64_t pk = pack_key(key, s);
     const uint32_t ea = c.turn_ev[2 * ti], ec = c.turn_ev[2 * ti + 1];
-    c.pkey[ea] = pk;
     c.gq[ea] = (uint32_t)g;
-    c.pkb[ea] = prev_pk;  // the key the session carried into this arrival
-    prev_pk = (k + 1 == ts) ? pack_key(kKeyMax40, s) : pk;
-    c.pkey[ec] = prev_pk;
     c.gq[ec] = (uint32_t)g;
+    if (c.pkey) {
+      c.pkey[ea] = pk;
+      c.pkb[ea] = prev_pk;  // the key the session carried into this arrival
+      prev_pk = (k + 1 == ts) ? pack_key(kKeyMax40, s) : pk;
+      c.pkey[ec] = prev_pk;
+    }
+    if (c.rk.rank) {
+      // live completions in order of descending session; the final ones, all
+      // of the maximal key, rank above them by descending session
+      if (k + 1 < ts) c.rk.a[c.rk.n - (b + ts - (s + 1)) + k] = (key << 24) | ti;
+      else c.rk.rank[ec] = c.rk.n + (c.n_sessions - 1 - s);
+    }
   }
+}
+
+// Ranks of each combination's completion keys (replay_slots.cuh).
+__global__ void __launch_bounds__(unison_slots::kSortThreads) rank_keys_kernel(const ComboDesc *combos) {
+  __shared__ uint32_t cnt[unison_slots::kSortWarps][256];
+  __shared__ unison_slots::SortShared sh;
+  if (combos[blockIdx.x].rk.rank) unison_slots::rank_keys_body(combos[blockIdx.x].rk, cnt, sh);
 }
 
 // --------------------------------------------------------------------------
@@ -237,7 +262,7 @@ __device__ __forceinline__ uint32_t lower_bound(const Sorted &T, uint64_t k, int
 
 // Move e[lo, hi) by delta places (delta > 0 toward the end), warp-parallel.
 // Out of line on purpose: inlined at every call site, the shifts' register
-// demand crowds the event loop (measured: the sweep runs about 8% faster).
+// demand crowds the event loop.
 __device__ __noinline__ void shift_block(uint4 *e, uint32_t lo, uint32_t hi, int32_t delta, int lane) {
   if (lo >= hi || delta == 0) return;
   if (delta > 0) {  // top chunk first
@@ -281,146 +306,6 @@ __device__ __noinline__ void shift_block(uint4 *e, uint32_t lo, uint32_t hi, int
   }
 }
 
-// The fast tier in registers (kRegS launches, every replay's fast tier at
-// most 32 entries): lane i holds entry i of the sorted array, so a search is
-// one ballot and an insert, an erase or a pop is a few shuffles, with no
-// shared-memory round trip.
-struct RegTier {
-  uint4 v;  // this lane's entry
-  uint32_t n;
-};
-__device__ __forceinline__ uint32_t reg_lower_bound(const RegTier &R, uint64_t k, int lane) {
-  return __popc(__ballot_sync(kFull, (uint32_t)lane < R.n && ekey(R.v) < k));
-}
-__device__ __forceinline__ uint4 reg_at(const RegTier &R, uint32_t i) {
-  return make_uint4(__shfl_sync(kFull, R.v.x, i), __shfl_sync(kFull, R.v.y, i), __shfl_sync(kFull, R.v.z, i),
-                    __shfl_sync(kFull, R.v.w, i));
-}
-__device__ __forceinline__ void reg_insert_at(RegTier &R, uint32_t p, uint4 e, int lane) {
-  const uint4 u = make_uint4(__shfl_up_sync(kFull, R.v.x, 1), __shfl_up_sync(kFull, R.v.y, 1),
-                             __shfl_up_sync(kFull, R.v.z, 1), __shfl_up_sync(kFull, R.v.w, 1));
-  if ((uint32_t)lane > p) R.v = u;
-  if ((uint32_t)lane == p) R.v = e;
-  R.n++;
-}
-__device__ __forceinline__ void reg_erase_at(RegTier &R, uint32_t p, int lane) {
-  const uint4 u = make_uint4(__shfl_down_sync(kFull, R.v.x, 1), __shfl_down_sync(kFull, R.v.y, 1),
-                             __shfl_down_sync(kFull, R.v.z, 1), __shfl_down_sync(kFull, R.v.w, 1));
-  if ((uint32_t)lane >= p) R.v = u;
-  R.n--;
-}
-
-// The HBM tier in registers (kHK > 0 slots a lane): lane l holds entries l,
-// 32 + l, 64 + l, ... of the sorted array, three words each (key and size; an
-// entry's fourth word, its completion time, is read only by the timeout
-// policy, which these launches never run).  A search is kHK ballots; an
-// insert, an erase or a drop of the first entries one shuffle per word and
-// slot.  A replay whose HBM tier would pass 32 kHK entries stops (kRegFull)
-// and is replayed from its start with the tier in shared memory: a replay is
-// deterministic, so its results are the same, and the register body needs no
-// test of where the tier is (measured: the sweep runs 6% faster than with a
-// one-way move of the tier to shared memory tested at every operation).
-// The restart is kept for the rare replay: while warps of one SM run
-// different bodies the launch slows down far beyond the repeated work
-// (measured: independent-gap sweep, 128 GiB replays restarting with 6
-// slots: 121 ms, against 70 ms with 6 slots from the start).  Five slots hold
-// both sweeps' HBM tiers (at most about 125 entries with per-session gap
-// recurrence, about 140 with independent gaps); four run the recurrent-gap
-// sweep 7% faster but send the other's 128 GiB replays to shared memory.
-constexpr int kHSlots = 5;
-constexpr int kRegFull = -1000;  // internal status: never reported
-struct RegTierH {
-  // key low, key high, size (and the promoted bit)
-  uint32_t x[kHSlots], y[kHSlots], z[kHSlots];
-};
-__device__ __forceinline__ uint64_t hkey(const RegTierH &G, int j) { return ((uint64_t)G.y[j] << 32) | G.x[j]; }
-// Entry i (warp-uniform, below 32 K; a larger i reads a slot-0 entry).
-template <int K>
-__device__ __forceinline__ uint4 hreg_at(const RegTierH &G, uint32_t i) {
-  const uint32_t sl = i >> 5, ln = i & 31;
-  uint32_t a = G.x[0], b = G.y[0], c = G.z[0];
-#pragma unroll
-  for (int j = 1; j < K; j++)
-    if (sl == (uint32_t)j) {
-      a = G.x[j];
-      b = G.y[j];
-      c = G.z[j];
-    }
-  return make_uint4(__shfl_sync(kFull, a, ln), __shfl_sync(kFull, b, ln), __shfl_sync(kFull, c, ln), 0u);
-}
-// Entries with key < k among the first n.
-template <int K>
-__device__ __forceinline__ uint32_t hreg_lower_bound(const RegTierH &G, uint32_t n, uint64_t k, int lane) {
-  uint32_t cnt = 0;
-#pragma unroll
-  for (int j = 0; j < K; j++) cnt += __popc(__ballot_sync(kFull, 32u * j + lane < n && hkey(G, j) < k));
-  return cnt;
-}
-// Insert e at position p (fewer than 32 K entries): entries p.. move up one
-// place.  Lane l of a slot takes lane l - 1's entry, lane 0 the slot below's
-// lane 31: the providing lane picks the slot, so a word moves in one shuffle
-// (slots from the top down, each reading the slot below before it changes).
-// Here and below every slot moves whatever the count and position: entries
-// past the count may hold anything, and the shuffles cost less than branches
-// that would skip the unchanged slots (measured: the sweep runs 8% faster).
-template <int K>
-__device__ __forceinline__ void hreg_insert_at(RegTierH &G, uint32_t p, uint4 e, int lane) {
-  const uint32_t from = (lane - 1) & 31;
-#pragma unroll
-  for (int j = K - 1; j >= 0; j--) {
-    const bool low = j > 0 && lane == 31;  // lane 31 provides the slot below's entry
-    const uint32_t ux = __shfl_sync(kFull, low ? G.x[j > 0 ? j - 1 : 0] : G.x[j], from),
-                   uy = __shfl_sync(kFull, low ? G.y[j > 0 ? j - 1 : 0] : G.y[j], from),
-                   uz = __shfl_sync(kFull, low ? G.z[j > 0 ? j - 1 : 0] : G.z[j], from);
-    const uint32_t idx = 32u * j + lane;
-    if (idx > p) {
-      G.x[j] = ux;
-      G.y[j] = uy;
-      G.z[j] = uz;
-    } else if (idx == p) {
-      G.x[j] = e.x;
-      G.y[j] = e.y;
-      G.z[j] = e.z;
-    }
-  }
-}
-// Erase position p: entries p + 1.. move down one place.  Lane l
-// takes lane l + 1's entry, lane 31 the slot above's lane 0 (slots from the
-// bottom up, each reading the slot above before it changes).
-template <int K>
-__device__ __forceinline__ void hreg_erase_at(RegTierH &G, uint32_t p, int lane) {
-  const uint32_t from = (lane + 1) & 31;
-#pragma unroll
-  for (int j = 0; j < K; j++) {
-    constexpr int kTop = K - 1;
-    const bool high = j < kTop && lane == 0;  // lane 0 provides the slot above's entry
-    const uint32_t dx = __shfl_sync(kFull, high ? G.x[j < kTop ? j + 1 : kTop] : G.x[j], from),
-                   dy = __shfl_sync(kFull, high ? G.y[j < kTop ? j + 1 : kTop] : G.y[j], from),
-                   dz = __shfl_sync(kFull, high ? G.z[j < kTop ? j + 1 : kTop] : G.z[j], from);
-    if (32u * j + lane >= p) {
-      G.x[j] = dx;
-      G.y[j] = dy;
-      G.z[j] = dz;
-    }
-  }
-}
-// Drop the first m (1..32) entries: entry i takes entry i + m, from
-// lane (l + m) mod 32 of the same slot, or of the next one where l + m >= 32;
-// the providing lanes below m give the next slot's entry.
-template <int K>
-__device__ __forceinline__ void hreg_drop_front(RegTierH &G, uint32_t m, int lane) {
-  const uint32_t from = (lane + m) & 31;
-  const bool next = (uint32_t)lane < m;
-#pragma unroll
-  for (int j = 0; j < K; j++) {
-    constexpr int kTop = K - 1;
-    const bool up = j < kTop && next;
-    G.x[j] = __shfl_sync(kFull, up ? G.x[j < kTop ? j + 1 : kTop] : G.x[j], from);
-    G.y[j] = __shfl_sync(kFull, up ? G.y[j < kTop ? j + 1 : kTop] : G.y[j], from);
-    G.z[j] = __shfl_sync(kFull, up ? G.z[j < kTop ? j + 1 : kTop] : G.z[j], from);
-  }
-}
-
 // Descriptor fields the placement and fill read on every event, held in
 // registers (the descriptor itself sits in shared memory).
 struct Hot {
@@ -431,8 +316,6 @@ struct Hot {
 
 struct ReplayState {
   Sorted S, H;      // unpinned residents per tier
-  RegTier R;        // the fast tier's residents instead of S, in kRegS launches
-  RegTierH G;       // the HBM tier's residents instead of H.e, in kHK > 0 bodies; the count is H.n
   uint4 *pin;       // pinned residents
   uint32_t npin, pin_cap;
   uint4 *tmp;       // TIDE staging: [0, cap_s) promoted, [cap_s, 2 cap_s) demoted
@@ -458,13 +341,10 @@ struct ReplayState {
 
 constexpr uint16_t kNoSlot = 0xFFFF;
 
-// kLean (here and below): the replay keeps no decision log, has the tier map
-// and pin slots, and no slot limit -- known at compile time.
-template <bool kLean>
 __device__ __forceinline__ void log_dec(ReplayState &st, uint32_t kind, uint32_t s, int lane) {
   const uint64_t w = ((uint64_t)st.e << 32) | ((uint64_t)kind << 24) | s;
   st.hash = (st.hash ^ w) * kFnvPrime;
-  if (!kLean && st.log) {
+  if (st.log) {
     if (st.log_len < st.log_cap) {
       if (lane == 0) {
         unison_decision d;
@@ -481,12 +361,10 @@ __device__ __forceinline__ void log_dec(ReplayState &st, uint32_t kind, uint32_t
 
 // Tier-map update: every lane stores the same byte, so each lane's later
 // reads see it without a warp barrier.
-template <bool kLean>
 __device__ __forceinline__ void set_tier(ReplayState &st, uint32_t id, uint32_t tier) {
-  if (kLean || st.tmap) st.tmap[id] = (uint8_t)tier;
+  if (st.tmap) st.tmap[id] = (uint8_t)tier;
 }
 
-template <bool kLean>
 __device__ __forceinline__ bool sorted_insert(ReplayState &st, Sorted &T, uint4 v, int lane, uint32_t tier) {
   if (T.n >= T.cap) {
     st.status = UNISON_ERR_CAPACITY;
@@ -500,7 +378,7 @@ __device__ __forceinline__ bool sorted_insert(ReplayState &st, Sorted &T, uint4 
   if (lane == 0) T.e[p] = v;
   __syncwarp();
   T.n++;
-  set_tier<kLean>(st, packed_id(ekey(v)), tier);
+  set_tier(st, packed_id(ekey(v)), tier);
   return true;
 }
 
@@ -509,79 +387,18 @@ __device__ __forceinline__ void sorted_erase(Sorted &T, uint32_t p, int lane) {
   T.n--;
 }
 
-template <bool kLean>
+// Drop the first m entries.
+__device__ __forceinline__ void drop_front(Sorted &T, uint32_t m, int lane) {
+  shift_block(T.e, m, T.n, -(int32_t)m, lane);
+  T.n -= m;
+}
+
 __device__ __forceinline__ uint4 sorted_pop_back(ReplayState &st, Sorted &T) {
   const uint4 v = T.e[T.n - 1];
   __syncwarp();
   T.n--;
-  set_tier<kLean>(st, packed_id(ekey(v)), kTierNone);
+  set_tier(st, packed_id(ekey(v)), kTierNone);
   return v;
-}
-
-template <bool kLean>
-__device__ __forceinline__ bool reg_sorted_insert(ReplayState &st, uint4 v, int lane) {
-  if (st.R.n >= st.S.cap) {
-    st.status = UNISON_ERR_CAPACITY;
-    return false;
-  }
-  reg_insert_at(st.R, reg_lower_bound(st.R, ekey(v), lane), v, lane);
-  set_tier<kLean>(st, packed_id(ekey(v)), kTierS);
-  return true;
-}
-template <bool kLean>
-__device__ __forceinline__ uint4 reg_pop_back(ReplayState &st) {
-  const uint4 v = reg_at(st.R, st.R.n - 1);
-  st.R.n--;
-  set_tier<kLean>(st, packed_id(ekey(v)), kTierNone);
-  return v;
-}
-
-// HBM-tier operations on kHK register slots a lane, or on the array (kHK 0).
-template <int kHK>
-__device__ __forceinline__ uint4 h_at(const ReplayState &st, uint32_t i) {
-  if constexpr (kHK > 0) return hreg_at<kHK>(st.G, i);
-  return st.H.e[i];
-}
-template <int kHK>
-__device__ __forceinline__ void h_erase_at(ReplayState &st, uint32_t p, int lane) {
-  if constexpr (kHK > 0) {
-    hreg_erase_at<kHK>(st.G, p, lane);
-    st.H.n--;
-  } else {
-    sorted_erase(st.H, p, lane);
-  }
-}
-template <bool kLean, int kHK>
-__device__ __forceinline__ uint4 h_pop_back(ReplayState &st) {
-  if constexpr (kHK > 0) {
-    const uint4 v = hreg_at<kHK>(st.G, st.H.n - 1);
-    st.H.n--;
-    set_tier<kLean>(st, packed_id(ekey(v)), kTierNone);
-    return v;
-  }
-  return sorted_pop_back<kLean>(st, st.H);
-}
-// Drop the first m entries (m <= 32 in register bodies).
-template <int kHK>
-__device__ __forceinline__ void h_drop_front(ReplayState &st, uint32_t m, int lane) {
-  if constexpr (kHK > 0) hreg_drop_front<kHK>(st.G, m, lane);
-  else shift_block(st.H.e, m, st.H.n, -(int32_t)m, lane);
-  st.H.n -= m;
-}
-template <bool kLean, int kHK>
-__device__ __forceinline__ bool h_insert(ReplayState &st, uint4 v, int lane) {
-  if constexpr (kHK > 0) {
-    if (st.H.n >= st.H.cap || st.H.n >= 32u * kHK) {
-      // the list bound, or the registers' 32 kHK entries (the replay starts over)
-      st.status = st.H.n >= st.H.cap ? UNISON_ERR_CAPACITY : kRegFull;
-      return false;
-    }
-    hreg_insert_at<kHK>(st.G, hreg_lower_bound<kHK>(st.G, st.H.n, ekey(v), lane), v, lane);
-    st.H.n++;
-    set_tier<kLean>(st, packed_id(ekey(v)), kTierH);
-    return true;
-  }
-  return sorted_insert<kLean>(st, st.H, v, lane, kTierH);
 }
 
 __device__ __forceinline__ uint32_t esize(uint4 v) { return v.z & kSizeMask; }
@@ -624,13 +441,12 @@ __device__ __forceinline__ void count_promotion(ReplayState &st, uint32_t chosen
 // A session demoted out of the fast tier enters HBM, displacing the most
 // evictable unpinned HBM sessions, or is dropped when it is itself the most
 // evictable of (unpinned HBM) + {itself}.
-template <bool kStale, bool kLean, int kHK = 0>
+template <bool kStale>
 __device__ __forceinline__ bool admit_demoted(ReplayState &st, const Hot &D, uint4 d, int lane) {
-  static_assert(!(kHK > 0 && kStale), "the register HBM tier serves live-key replays only");
   const uint32_t id = packed_id(ekey(d));
   const uint32_t size = esize(d);
   if (st.pinned_h > D.cap_h || size > D.cap_h - st.pinned_h) {
-    log_dec<kLean>(st, UNISON_KIND_EVICT, id, lane);
+    log_dec(st, UNISON_KIND_EVICT, id, lane);
     CNT(st, n_evict, 1);
     return true;
   }
@@ -640,19 +456,19 @@ __device__ __forceinline__ bool admit_demoted(ReplayState &st, const Hot &D, uin
       count_victim(st, drop ? id : packed_id(ekey(st.H.e[st.H.n - 1])),
                    max(live_max(st, st.H, 0, st.H.n, lane), st.live[id]));
     }
-    if (st.H.n == 0 || ekey(d) > ekey(h_at<kHK>(st, st.H.n - 1))) {
-      log_dec<kLean>(st, UNISON_KIND_EVICT, id, lane);
+    if (st.H.n == 0 || ekey(d) > ekey(st.H.e[st.H.n - 1])) {
+      log_dec(st, UNISON_KIND_EVICT, id, lane);
       CNT(st, n_evict, 1);
       return true;
     }
-    const uint4 v = h_pop_back<kLean, kHK>(st);
+    const uint4 v = sorted_pop_back(st, st.H);
     st.used_h -= esize(v);
-    log_dec<kLean>(st, UNISON_KIND_EVICT, packed_id(ekey(v)), lane);
+    log_dec(st, UNISON_KIND_EVICT, packed_id(ekey(v)), lane);
     CNT(st, n_evict, 1);
   }
-  if (!h_insert<kLean, kHK>(st, d, lane)) return false;
+  if (!sorted_insert(st, st.H, d, lane, kTierH)) return false;
   st.used_h += size;
-  log_dec<kLean>(st, UNISON_KIND_DEMOTE, id, lane);
+  log_dec(st, UNISON_KIND_DEMOTE, id, lane);
   CNT(st, n_demote, 1);
   return true;
 }
@@ -671,30 +487,30 @@ __device__ __forceinline__ bool pin_append(ReplayState &st, uint64_t pk, uint32_
 }
 
 // Placement of the arriving (pinned) session s with n tokens.
-template <bool kStale, bool kLean, bool kRegS = false, int kHK = 0>
+template <bool kStale>
 __device__ __forceinline__ bool place(ReplayState &st, const Hot &D, uint32_t s, uint64_t pk, uint32_t n,
                                       int lane) {
-  if (!kLean && D.max_sessions && st.npin >= D.max_sessions) {
-    log_dec<kLean>(st, UNISON_KIND_BYPASS, s, lane);
+  if (D.max_sessions && st.npin >= D.max_sessions) {
+    log_dec(st, UNISON_KIND_BYPASS, s, lane);
     CNT(st, n_bypass, 1);
     return true;
   }
   if (st.pinned_s <= D.cap_s && n <= D.cap_s - st.pinned_s) {
     while (st.used_s + n > D.cap_s) {
-      if ((kRegS ? st.R.n : st.S.n) == 0) {
+      if (st.S.n == 0) {
         st.status = UNISON_ERR_CAPACITY;
         return false;
       }
       if (kStale) count_victim(st, packed_id(ekey(st.S.e[st.S.n - 1])), live_max(st, st.S, 0, st.S.n, lane));
       // most evictable unpinned fast-tier session
-      const uint4 d = kRegS ? reg_pop_back<kLean>(st) : sorted_pop_back<kLean>(st, st.S);
+      const uint4 d = sorted_pop_back(st, st.S);
       st.used_s -= esize(d);
-      if (!admit_demoted<kStale, kLean, kHK>(st, D, d, lane)) return false;
+      if (!admit_demoted<kStale>(st, D, d, lane)) return false;
     }
     if (!pin_append(st, pk, n, s, kTierS, lane)) return false;
     st.used_s += n;
     st.pinned_s += n;
-    log_dec<kLean>(st, UNISON_KIND_PLACE_S, s, lane);
+    log_dec(st, UNISON_KIND_PLACE_S, s, lane);
     CNT(st, n_place_s, 1);
   } else if (st.pinned_h <= D.cap_h && n <= D.cap_h - st.pinned_h) {
     while (st.used_h + n > D.cap_h) {
@@ -703,22 +519,22 @@ __device__ __forceinline__ bool place(ReplayState &st, const Hot &D, uint32_t s,
         return false;
       }
       if (kStale) count_victim(st, packed_id(ekey(st.H.e[st.H.n - 1])), live_max(st, st.H, 0, st.H.n, lane));
-      const uint4 v = h_pop_back<kLean, kHK>(st);
+      const uint4 v = sorted_pop_back(st, st.H);
       st.used_h -= esize(v);
-      log_dec<kLean>(st, UNISON_KIND_EVICT, packed_id(ekey(v)), lane);
+      log_dec(st, UNISON_KIND_EVICT, packed_id(ekey(v)), lane);
       CNT(st, n_evict, 1);
     }
     if (!pin_append(st, pk, n, s, kTierH, lane)) return false;
     st.used_h += n;
     st.pinned_h += n;
-    log_dec<kLean>(st, UNISON_KIND_PLACE_H, s, lane);
+    log_dec(st, UNISON_KIND_PLACE_H, s, lane);
     CNT(st, n_place_h, 1);
   } else {
-    log_dec<kLean>(st, UNISON_KIND_BYPASS, s, lane);
+    log_dec(st, UNISON_KIND_BYPASS, s, lane);
     CNT(st, n_bypass, 1);
     return true;
   }
-  if (!kLean && D.max_sessions) {
+  if (D.max_sessions) {
     while (st.S.n + st.H.n + st.npin > D.max_sessions) {
       if (st.S.n == 0 && st.H.n == 0) {
         st.status = UNISON_ERR_CAPACITY;
@@ -729,12 +545,12 @@ __device__ __forceinline__ bool place(ReplayState &st, const Hot &D, uint32_t s,
       if (kStale)
         count_victim(st, packed_id(ekey(from_s ? st.S.e[st.S.n - 1] : st.H.e[st.H.n - 1])),
                      max(live_max(st, st.S, 0, st.S.n, lane), live_max(st, st.H, 0, st.H.n, lane)));
-      const uint4 v = sorted_pop_back<kLean>(st, from_s ? st.S : st.H);
+      const uint4 v = sorted_pop_back(st, from_s ? st.S : st.H);
       if (from_s)
         st.used_s -= esize(v);
       else
         st.used_h -= esize(v);
-      log_dec<kLean>(st, UNISON_KIND_EVICT, packed_id(ekey(v)), lane);
+      log_dec(st, UNISON_KIND_EVICT, packed_id(ekey(v)), lane);
       CNT(st, n_evict, 1);
     }
   }
@@ -746,15 +562,15 @@ __device__ __forceinline__ bool place(ReplayState &st, const Hot &D, uint32_t s,
 // free fast-tier space; phase 2: pair the next least evictable HBM session
 // with the most evictable fast-tier one), which makes the same moves as the
 // pair loop of Algorithm 1, and are then applied in bulk.
-template <bool kStale, bool kLean, bool kRegS = false, int kHK = 0>
+template <bool kStale>
 __device__ __forceinline__ uint64_t tide(ReplayState &st, const Hot &D, uint64_t budget, uint32_t rcap_s,
                                          int lane) {
-  const uint32_t sn = kRegS ? st.R.n : st.S.n;  // fast-tier entries; the fast tier changes only at the end
+  const uint32_t sn = st.S.n;  // fast-tier entries; the fast tier changes only at the end
   uint64_t rem = budget;
   const uint64_t kvb = D.kvb;
   uint32_t n1 = 0;
   while (n1 < st.H.n) {
-    const uint4 p = h_at<kHK>(st, n1);
+    const uint4 p = st.H.e[n1];
     const uint64_t sz = esize(p), by = sz * kvb;
     if (by > rem || st.used_s + sz > D.cap_s) break;
     // (the loop form's candidates: HBM less the sessions promoted so far)
@@ -762,17 +578,17 @@ __device__ __forceinline__ uint64_t tide(ReplayState &st, const Hot &D, uint64_t
     rem -= by;
     st.used_s += sz;
     st.used_h -= sz;
-    log_dec<kLean>(st, UNISON_KIND_PROMOTE, packed_id(ekey(p)), lane);
+    log_dec(st, UNISON_KIND_PROMOTE, packed_id(ekey(p)), lane);
     n1++;
   }
   uint32_t pairs = 0;
   for (;;) {
     if (n1 + pairs >= st.H.n || pairs >= sn) break;
-    const uint4 p = h_at<kHK>(st, n1 + pairs);
-    const uint4 d = kRegS ? reg_at(st.R, sn - 1 - pairs) : st.S.e[st.S.n - 1 - pairs];
+    const uint4 p = st.H.e[n1 + pairs];
+    const uint4 d = st.S.e[sn - 1 - pairs];
     // the next most evictable of (fast tier + promoted) is a promoted session
     // when the largest promoted key beats d: then it cannot beat p, stop
-    if (n1 > 0 && ekey(h_at<kHK>(st, n1 - 1)) > ekey(d)) break;
+    if (n1 > 0 && ekey(st.H.e[n1 - 1]) > ekey(d)) break;
     if (!(ekey(d) > ekey(p))) break;
     const uint64_t sp = esize(p), sd = esize(d), by = (sp + sd) * kvb;
     if (by > rem) break;
@@ -790,8 +606,8 @@ __device__ __forceinline__ uint64_t tide(ReplayState &st, const Hot &D, uint64_t
     rem -= by;
     st.used_s = st.used_s - sd + sp;
     st.used_h = st.used_h - sp + sd;
-    log_dec<kLean>(st, UNISON_KIND_PROMOTE, packed_id(ekey(p)), lane);
-    log_dec<kLean>(st, UNISON_KIND_TIDE_DEMOTE, packed_id(ekey(d)), lane);
+    log_dec(st, UNISON_KIND_PROMOTE, packed_id(ekey(p)), lane);
+    log_dec(st, UNISON_KIND_TIDE_DEMOTE, packed_id(ekey(d)), lane);
     pairs++;
   }
   const uint32_t m = n1 + pairs;
@@ -803,63 +619,45 @@ __device__ __forceinline__ uint64_t tide(ReplayState &st, const Hot &D, uint64_t
     return budget - rem;
   }
   if (m == 1 && pairs == 0) {  // one promotion (the common case): move it directly
-    uint4 v = h_at<kHK>(st, 0);
+    uint4 v = st.H.e[0];
     v.z |= kPromotedBit;
     __syncwarp();
-    h_drop_front<kHK>(st, 1, lane);
-    if (kRegS) reg_sorted_insert<kLean>(st, v, lane);
-    else sorted_insert<kLean>(st, st.S, v, lane, kTierS);
+    drop_front(st.H, 1, lane);
+    sorted_insert(st, st.S, v, lane, kTierS);
     return budget - rem;
   }
   if (m == 1 && pairs == 1) {  // one pair (the next most common): swap it directly
-    uint4 v = h_at<kHK>(st, 0);
+    uint4 v = st.H.e[0];
     v.z |= kPromotedBit;
-    const uint4 d = kRegS ? reg_at(st.R, sn - 1) : st.S.e[st.S.n - 1];
+    const uint4 d = st.S.e[st.S.n - 1];
     __syncwarp();
-    h_drop_front<kHK>(st, 1, lane);
-    if (kRegS) {
-      st.R.n -= 1;
-      if (!reg_sorted_insert<kLean>(st, v, lane)) return budget - rem;
-    } else {
-      st.S.n -= 1;
-      if (!sorted_insert<kLean>(st, st.S, v, lane, kTierS)) return budget - rem;
-    }
-    h_insert<kLean, kHK>(st, d, lane);
+    drop_front(st.H, 1, lane);
+    st.S.n -= 1;
+    if (!sorted_insert(st, st.S, v, lane, kTierS)) return budget - rem;
+    sorted_insert(st, st.H, d, lane, kTierH);
     return budget - rem;
   }
   // stage the moved entries, then fix both arrays
   uint4 *pro = st.tmp, *dem = st.tmp + rcap_s;
-  if constexpr (kHK > 0) {  // m <= 32: the first m entries are slot 0's
-    if ((uint32_t)lane < m) pro[lane] = make_uint4(st.G.x[0], st.G.y[0], st.G.z[0] | kPromotedBit, 0u);
-  } else {
-    for (uint32_t i = lane; i < m; i += 32) {
-      uint4 v = st.H.e[i];
-      v.z |= kPromotedBit;
-      pro[i] = v;
-    }
+  for (uint32_t i = lane; i < m; i += 32) {
+    uint4 v = st.H.e[i];
+    v.z |= kPromotedBit;
+    pro[i] = v;
   }
-  if (kRegS) {  // pairs <= fast-tier entries <= 32: one entry a lane
-    const uint4 dv = reg_at(st.R, min(sn - pairs + (uint32_t)lane, 31u));
-    if ((uint32_t)lane < pairs) dem[lane] = dv;
-  } else {
-    for (uint32_t i = lane; i < pairs; i += 32) dem[i] = st.S.e[st.S.n - pairs + i];
-  }
+  for (uint32_t i = lane; i < pairs; i += 32) dem[i] = st.S.e[st.S.n - pairs + i];
   __syncwarp();
-  h_drop_front<kHK>(st, m, lane);
-  if (kRegS) st.R.n -= pairs;
-  else st.S.n -= pairs;
+  drop_front(st.H, m, lane);
+  st.S.n -= pairs;
   for (uint32_t i = 0; i < m; i++)
-    if (kRegS ? !reg_sorted_insert<kLean>(st, pro[i], lane) : !sorted_insert<kLean>(st, st.S, pro[i], lane, kTierS))
-      return budget - rem;
+    if (!sorted_insert(st, st.S, pro[i], lane, kTierS)) return budget - rem;
   for (uint32_t i = 0; i < pairs; i++)
-    if (!h_insert<kLean, kHK>(st, dem[i], lane)) return budget - rem;
+    if (!sorted_insert(st, st.H, dem[i], lane, kTierH)) return budget - rem;
   return budget - rem;
 }
 
 // Timeout: expire unpinned residents idle >= ttl, smallest session id first.
 // Under recency keys the last return time falls as the key grows, so the
 // expired sessions of a tier are a top suffix of its array.
-template <bool kLean>
 __device__ __forceinline__ void expire_idle(ReplayState &st, uint32_t now, uint32_t ttl, int lane) {
   for (;;) {
     // expired suffix lengths
@@ -890,8 +688,8 @@ __device__ __forceinline__ void expire_idle(ReplayState &st, uint32_t now, uint3
     else
       st.used_h -= sz;
     sorted_erase(T, pos, lane);
-    set_tier<kLean>(st, mid, kTierNone);
-    log_dec<kLean>(st, UNISON_KIND_EXPIRE, mid, lane);
+    set_tier(st, mid, kTierNone);
+    log_dec(st, UNISON_KIND_EXPIRE, mid, lane);
     CNT(st, n_expire, 1);
   }
 }
@@ -1051,16 +849,9 @@ struct EventBufs {
 // One replay: Algorithm 1 over the trace's events.  kPol is the replay's
 // policy when the body is specialised for it (its policy tests then fold
 // away), or -1 for the body that reads the policy from the descriptor.
-// False when a register body (kHK > 0) stopped at its HBM tier's register
-// bound (no result written): the caller replays it again with more slots or
-// none.
-template <bool kGlobalLists, int kKeys, int kPol, bool kLean, bool kRegS = false, int kHK = 0>
-__device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs, unsigned char *smem, int lane) {
+template <bool kGlobalLists, int kKeys, int kPol>
+__device__ __forceinline__ void replay_body(const ReplayDesc &D, EventBufs &bufs, unsigned char *smem, int lane) {
   constexpr bool kOnline = kKeys == kKeyOnline, kStale = kKeys == kKeyStale;
-  // the register HBM tier drops the entries' completion times (timeout only)
-  // and drop_front's m <= 32 rests on the fast tier's 32-entry bound
-  static_assert(kHK == 0 || (kHK <= kHSlots && kRegS && kLean && kPol == UNISON_SPEAR_TIDE && !kOnline && !kStale),
-                "register HBM tier: lean SPEAR+TIDE launches with the register fast tier");
   const Hot hot{D.cap_s, D.cap_h, D.kvb, D.dma, D.max_sessions};
 
   ReplayState st;
@@ -1097,7 +888,7 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
       st.tmap = reinterpret_cast<uint8_t *>(p);
       uint32_t *m32 = reinterpret_cast<uint32_t *>(p);
       for (uint32_t i = lane; i < (D.n_sessions + 3) / 4; i += 32) m32[i] = 0u;
-      if (kLean || D.tmap == kMapSlots) {
+      if (D.tmap == kMapSlots) {
         st.pslot = reinterpret_cast<uint16_t *>(reinterpret_cast<unsigned char *>(p) + ((D.n_sessions + 15) & ~15u));
         uint32_t *s32 = reinterpret_cast<uint32_t *>(st.pslot);
         for (uint32_t i = lane; i < (D.n_sessions + 1) / 2; i += 32) s32[i] = 0xFFFFFFFFu;
@@ -1147,10 +938,6 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
     st.live = stale_live;
     st.vict_n = st.vict_diff = st.prom_n = st.prom_diff = 0;
     st.S.n = st.H.n = 0;
-    st.R.n = 0;
-    st.R.v = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-    for (int j = 0; j < kHK; j++) st.G.x[j] = st.G.y[j] = st.G.z[j] = 0u;
     st.S.cap = D.rcap_s;
     st.H.cap = D.rcap_h;
     st.npin = 0;
@@ -1210,7 +997,7 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
   if (E) prev_now = sev[0][0].x;
 
   int bi = 0;
-  for (uint32_t b = 0; b < E && st.status != UNISON_ERR_CAPACITY && st.status != kRegFull; b += 32, bi ^= 1) {
+  for (uint32_t b = 0; b < E && st.status != UNISON_ERR_CAPACITY; b += 32, bi ^= 1) {
     if (b + 32 < E) {
       fetch(b + 32, bi ^ 1);
       cp_async_wait_one();  // this batch's copies have landed
@@ -1231,7 +1018,7 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
       n_ev++;
       rel_us += (uint32_t)(now - prev_now);
       prev_now = now;
-      if (timeout) expire_idle<kLean>(st, now, D.ttl, lane);
+      if (timeout) expire_idle(st, now, D.ttl, lane);
       // the DMA is free again from start + ceil(bytes / rate) us on, i.e. once
       // the elapsed us times the rate cover the bytes (no division; the high
       // word of the product catches a product past 2^64)
@@ -1262,42 +1049,12 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
             pkb = pack_key(0xFFFFFFFFull - spev[bi][j], s);
           // with the tier map only the session's own tier is searched (and
           // nothing for a session that is not resident)
-          if constexpr (kHK > 0) {
-            // both tiers in registers: one equality ballot per slot finds the
-            // key (unique: it carries the session id) without the tier map
-            const unsigned fs = __ballot_sync(kFull, (uint32_t)lane < st.R.n && ekey(st.R.v) == pkb);
-            unsigned fh[kHK];
-#pragma unroll
-            for (int j = 0; j < kHK; j++)
-              fh[j] = __ballot_sync(kFull, 32u * j + lane < st.H.n && hkey(st.G, j) == pkb);
-            uint32_t ph = 0;
-            unsigned inh = 0;
-#pragma unroll
-            for (int j = kHK - 1; j >= 0; j--) {
-              if (fh[j]) ph = 32u * j + __ffs(fh[j]) - 1;
-              inh |= fh[j];
-            }
-            const uint32_t ps = fs ? __ffs(fs) - 1 : 0u;
-            const uint4 es = reg_at(st.R, ps), eh = hreg_at<kHK>(st.G, ph);
-            tier = fs ? kTierS : (inh ? kTierH : kTierNone);
-            pos = fs ? ps : ph;
-            ent = fs ? es : eh;
-          }
-          const uint32_t mt = kHK > 0 ? 0u : ((kLean || st.tmap) ? st.tmap[s] : (kTierS | kTierH));
+          const uint32_t mt = st.tmap ? st.tmap[s] : (kTierS | kTierH);
           if (mt & kTierS) {
-            if (kRegS) {
-              pos = reg_lower_bound(st.R, pkb, lane);
-              const uint4 cand = reg_at(st.R, min(pos, 31u));
-              if (pos < st.R.n && ekey(cand) == pkb) {
-                tier = kTierS;
-                ent = cand;
-              }
-            } else {
-              pos = lower_bound(st.S, pkb, lane);
-              if (pos < st.S.n && ekey(st.S.e[pos]) == pkb) {
-                tier = kTierS;
-                ent = st.S.e[pos];
-              }
+            pos = lower_bound(st.S, pkb, lane);
+            if (pos < st.S.n && ekey(st.S.e[pos]) == pkb) {
+              tier = kTierS;
+              ent = st.S.e[pos];
             }
           }
           if (tier == kTierNone && (mt & kTierH)) {
@@ -1311,25 +1068,25 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
         }
         uint64_t prefill;
         if (edge) {
-          log_dec<kLean>(st, UNISON_KIND_COLD, s, lane);
+          log_dec(st, UNISON_KIND_COLD, s, lane);
           CNT(st, n_cold, 1);
           prefill = in;
         } else {
           CNT(st, n_warm, 1);
           CNT(st, tok_needed, in);
           if (tier == kTierS) {
-            log_dec<kLean>(st, UNISON_KIND_HIT_S, s, lane);
+            log_dec(st, UNISON_KIND_HIT_S, s, lane);
             CNT(st, n_hit_s, 1);
             CNT(st, tok_hit_s, prev);
             prefill = in - prev;
             if (ent.z & kPromotedBit) CNT(st, n_pth, 1);
           } else if (tier == kTierH) {
-            log_dec<kLean>(st, UNISON_KIND_HIT_H, s, lane);
+            log_dec(st, UNISON_KIND_HIT_H, s, lane);
             CNT(st, n_hit_h, 1);
             CNT(st, tok_hit_h, prev);
             prefill = in - prev;
           } else {
-            log_dec<kLean>(st, UNISON_KIND_MISS, s, lane);
+            log_dec(st, UNISON_KIND_MISS, s, lane);
             CNT(st, n_miss, 1);
             CNT(st, tok_miss, prev);
             prefill = in;
@@ -1349,13 +1106,12 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
         }
         if (tier == kTierS) {
           st.used_s -= esize(ent);
-          if (kRegS) reg_erase_at(st.R, pos, lane);
-          else sorted_erase(st.S, pos, lane);
-          set_tier<kLean>(st, s, kTierNone);
+          sorted_erase(st.S, pos, lane);
+          set_tier(st, s, kTierNone);
         } else if (tier == kTierH) {
           st.used_h -= esize(ent);
-          h_erase_at<kHK>(st, pos, lane);
-          set_tier<kLean>(st, s, kTierNone);
+          sorted_erase(st.H, pos, lane);
+          set_tier(st, s, kTierNone);
         }
         uint64_t pk;
         if (kOnline) {
@@ -1380,7 +1136,7 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
           pk = pack_key(nr == kNoRef ? kKeyMax40 : (uint64_t)nr, s);
         } else
           pk = pack_key(0xFFFFFFFFull - e, s);
-        if (!place<kStale, kLean, kRegS, kHK>(st, hot, s, pk, out, lane)) break;
+        if (!place<kStale>(st, hot, s, pk, out, lane)) break;
       } else {
         // completion: unpin (if resident) and rank the session with its new key
         if (kStale) {
@@ -1388,7 +1144,7 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
           mark_dirty(s);
         }
         uint32_t pi = kNoSlot;
-        if (kLean || st.pslot) {
+        if (st.pslot) {
           pi = st.pslot[s];
         } else {
           int mine = -1;
@@ -1402,7 +1158,7 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
           const uint4 last = st.pin[st.npin - 1];
           __syncwarp();
           if (lane == 0) st.pin[pi] = last;
-          if (kLean || st.pslot) {  // the last entry moves into the freed slot
+          if (st.pslot) {  // the last entry moves into the freed slot
             st.pslot[last.w & kIdMask] = (uint16_t)pi;
             st.pslot[s] = kNoSlot;
           }
@@ -1422,10 +1178,10 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
           const uint4 v = make_uint4((uint32_t)pk, (uint32_t)(pk >> 32), sz, now);
           if (tier == kTierS) {
             st.pinned_s -= sz;
-            if (kRegS ? !reg_sorted_insert<kLean>(st, v, lane) : !sorted_insert<kLean>(st, st.S, v, lane, kTierS)) break;
+            if (!sorted_insert(st, st.S, v, lane, kTierS)) break;
           } else {
             st.pinned_h -= sz;
-            if (!h_insert<kLean, kHK>(st, v, lane)) break;
+            if (!sorted_insert(st, st.H, v, lane, kTierH)) break;
           }
         }
         if (kOnline && edge) {
@@ -1440,14 +1196,14 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
           const uint64_t g = sgq[bi][j];
           const uint64_t budget = g * D.dma;
           CNT(st, n_tide_calls, 1);
-          const uint64_t moved = tide<kStale, kLean, kRegS, kHK>(st, hot, budget, D.rcap_s, lane);
+          const uint64_t moved = tide<kStale>(st, hot, budget, D.rcap_s, lane);
           CNT(st, dma_bytes, moved);
           if (moved > 0 && D.dma > 0) {
             dma_busy = true;
             busy_from = rel_us;
             busy_bytes = moved;
           }
-          if (st.status == UNISON_ERR_CAPACITY || st.status == kRegFull) break;
+          if (st.status == UNISON_ERR_CAPACITY) break;
         }
       }
       if (kStale) {
@@ -1472,7 +1228,7 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
               v.x = (uint32_t)nk;
               v.y = (uint32_t)(nk >> 32);
               sorted_erase(T, pos, lane);
-              sorted_insert<kLean>(st, T, v, lane, t);
+              sorted_insert(st, T, v, lane, t);
             }
           }
           __syncwarp();
@@ -1490,11 +1246,6 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
         }
       }
     }
-  }
-  if (kHK > 0 && st.status == kRegFull) {
-    cp_async_wait_all();  // the next batch's copies land before the replay starts over
-    __syncwarp();
-    return false;
   }
   if (lane == 0) {
     unison_replay_result r = {};
@@ -1533,15 +1284,10 @@ __device__ __forceinline__ bool replay_body(const ReplayDesc &D, EventBufs &bufs
     r.status = st.status;
     *D.result = r;
   }
-  return true;
 }
 
-// One warp per replay.  SPEAR+TIDE replays (the sweep's policy) run a body
-// specialised for it: a smaller, branch-free event loop.  kOnly >= 0: every
-// replay of the launch has that policy, and the kernel holds only its body
-// (and is sized for it alone); kLean: every replay of the launch is lean
-// (see log_dec).
-template <bool kGlobalLists, int kKeys, int kOnly, bool kLean, bool kRegS = false, int kHK = 0>
+// One warp per replay.  SPEAR+TIDE replays run a body with the policy folded in.
+template <bool kGlobalLists, int kKeys>
 __global__ void __launch_bounds__(32) replay_kernel(const ReplayDesc *descs, const uint32_t *order) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ReplayDesc Dsh;
@@ -1549,19 +1295,30 @@ __global__ void __launch_bounds__(32) replay_kernel(const ReplayDesc *descs, con
   const int lane = threadIdx.x & 31;
   if (lane == 0) Dsh = descs[order[blockIdx.x]];
   __syncwarp();
-  if (kOnly >= 0) {
-    if constexpr (kHK > 0) {
-      // a replay whose HBM tier outgrows kHK slots starts over with the tier
-      // in shared memory
-      if (!replay_body<kGlobalLists, kKeys, kOnly, kLean, kRegS, kHK>(Dsh, bufs, smem, lane))
-        replay_body<kGlobalLists, kKeys, kOnly, kLean, kRegS, 0>(Dsh, bufs, smem, lane);
-    } else {
-      replay_body<kGlobalLists, kKeys, kOnly, kLean, kRegS, 0>(Dsh, bufs, smem, lane);
-    }
-  } else if (kKeys == kKeyStream && Dsh.policy == UNISON_SPEAR_TIDE)
-    replay_body<kGlobalLists, kKeys, UNISON_SPEAR_TIDE, false>(Dsh, bufs, smem, lane);
+  if (kKeys == kKeyStream && Dsh.policy == UNISON_SPEAR_TIDE)
+    replay_body<kGlobalLists, kKeys, UNISON_SPEAR_TIDE>(Dsh, bufs, smem, lane);
   else
-    replay_body<kGlobalLists, kKeys, -1, false>(Dsh, bufs, smem, lane);
+    replay_body<kGlobalLists, kKeys, -1>(Dsh, bufs, smem, lane);
+}
+
+// Replays of the slot form.  kOnly >= 0: every replay of the launch is a lean
+// one of that policy (no log, no slot limit); else each takes its own body.
+template <int kOnly>
+__global__ void __launch_bounds__(32) slot_kernel(const ReplayDesc *descs, const uint32_t *order) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ ReplayDesc Dsh;
+  __shared__ __align__(16) unison_slots::SlotBufs bufs;
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) Dsh = descs[order[blockIdx.x]];
+  __syncwarp();
+  if constexpr (kOnly >= 0) {
+    unison_slots::slot_replay<kOnly, true>(Dsh, Dsh.slot, bufs, smem, lane);
+  } else {
+    if (Dsh.policy == UNISON_SPEAR_TIDE)
+      unison_slots::slot_replay<UNISON_SPEAR_TIDE, false>(Dsh, Dsh.slot, bufs, smem, lane);
+    else
+      unison_slots::slot_replay<-1, false>(Dsh, Dsh.slot, bufs, smem, lane);
+  }
 }
 
 // Lower median (element floor((n-1)/2) in sorted order) by MSB-first radix select.
@@ -1696,14 +1453,15 @@ struct ReplayPlan {
   std::vector<int> replay_combo;
   size_t off_desc = 0, off_order = 0, off_combo = 0, bytes = 0;
   std::vector<size_t> off_lut, off_stream, off_ttft, off_glist;
-  // Replay groups, one kernel launch each: lists in shared memory (SPEAR+TIDE,
-  // other policies), in global memory (the same split), online hazard table,
-  // stale snapshot.  The launches are independent and run concurrently.
-  std::vector<uint32_t> in_st, in_mix, in_gst, in_gmix, in_online, in_stale;
+  std::vector<char> need_keys, need_rank;  // per combination: packed keys (sorted lists), ranks (slot form)
+  // Replay groups, one kernel launch each: the slot form (lean SPEAR+TIDE
+  // replays, the others), sorted lists in shared memory, in global memory,
+  // online hazard table, stale snapshot.  The launches are independent and
+  // run concurrently.
+  std::vector<uint32_t> in_slot_st, in_slot_mix, in_list, in_glist, in_online, in_stale;
   std::vector<uint32_t> rcap_s, rcap_h, tmap;
-  size_t max_smem_st = 0, max_smem_mix = 0, max_smem_online = 0, max_smem_stale = 0;
-  bool st_lean = true;  // every shared-memory SPEAR+TIDE replay has the map with pin slots and no slot limit
-  bool st_reg = true;   // and a fast tier of at most 32 entries (held in the warp's registers)
+  std::vector<unison_slots::SlotDesc> slot;  // nslots 0: not of the slot form
+  size_t smem_slot_st = 0, smem_slot_mix = 0, max_smem_list = 0, max_smem_online = 0, max_smem_stale = 0;
 };
 
 // Resident-list capacity of a tier: at most one entry per session and no more
@@ -1741,14 +1499,6 @@ size_t online_bytes(uint32_t cs, uint32_t ch, uint32_t n_sessions) {
 
 using ReplayKernel = void (*)(const ReplayDesc *, const uint32_t *);
 
-// The kernel of the shared-memory SPEAR+TIDE group, for a log or not.
-ReplayKernel st_kernel(const ReplayPlan &P, bool logged) {
-  if (P.st_lean && !logged)
-    return P.st_reg ? replay_kernel<false, kKeyStream, UNISON_SPEAR_TIDE, true, true, kHSlots>
-                    : replay_kernel<false, kKeyStream, UNISON_SPEAR_TIDE, true>;
-  return replay_kernel<false, kKeyStream, UNISON_SPEAR_TIDE, false>;
-}
-
 // Waves of CTAs a group of n replays needs with `dyn` bytes per CTA.
 uint64_t smem_waves(ReplayKernel k, size_t n, size_t dyn) {
   int dev = 0, sms = 0, nb = 0;
@@ -1784,8 +1534,56 @@ void add_tier_maps(const unison_trace *const *traces, const unison_replay_params
   max_smem = with;
 }
 
+// Whether a replay can take the slot form, and its sizes.  A word holds the
+// tier bit, the rank and the slot; sums of tokens stay below 2^31 because a
+// capacity above every session's largest size together is never reached; the
+// sort's values hold a 24-bit turn.
+bool slot_plan(const unison_replay_params &p, const unison_trace *tr, uint32_t rcap_s, uint32_t rcap_h,
+               unison_slots::SlotDesc &q) {
+  if (tr->sum_last_out >= (1ull << 31) || tr->n_turns >= (1ull << 24)) return false;
+  const uint64_t n = std::min<uint64_t>(tr->n_sessions, (uint64_t)(rcap_s - 1) + (rcap_h - 1)) + 1;
+  if (n > unison_slots::kMostSlots) return false;
+  // ranks run from 1 to the completions, under Belady to the events and sessions
+  uint64_t most = p.policy == UNISON_BELADY ? tr->n_events + tr->n_sessions : tr->n_turns;
+  uint32_t sb = 1, rb = 1;
+  while ((1ull << sb) < n) sb++;
+  while ((1ull << rb) <= most) rb++;
+  if (sb + rb > 31) return false;
+  q.cap_s = (uint32_t)std::min<uint64_t>(p.cap_fast_bytes / p.kv_bytes_per_token, tr->sum_last_out);
+  q.cap_h = (uint32_t)std::min<uint64_t>(p.cap_hbm_bytes / p.kv_bytes_per_token, tr->sum_last_out);
+  q.nslots = (uint32_t)n;
+  q.sbits = sb;
+  return true;
+}
+
+ReplayKernel slot_kernel_of(bool lean_st) { return lean_st ? slot_kernel<UNISON_SPEAR_TIDE> : slot_kernel<-1>; }
+
+// The session maps of a slot group: two bytes a session name the slot
+// directly; one byte (its low eight bits, the slot told apart by the session
+// it holds) when two would not fit or would need more waves of CTAs.
+void slot_maps(const unison_trace *const *traces, const unison_replay_params *params, size_t smem_limit,
+               std::vector<uint32_t> &group, bool lean_st, size_t &smem, ReplayPlan &P) {
+  size_t most16 = 0, most8 = 0;
+  for (uint32_t r : group) {
+    const uint32_t S = traces[params[r].trace_idx]->n_sessions, n = P.slot[r].nslots;
+    const bool wide = params[r].policy != UNISON_SPEAR_TIDE;
+    most16 = std::max(most16, unison_slots::slot_bytes(n, S, wide, false));
+    most8 = std::max(most8, unison_slots::slot_bytes(n, S, wide, true));
+  }
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const ReplayKernel k = slot_kernel_of(lean_st);
+  const bool narrow = most16 > smem_limit || (group.size() > (size_t)sms && smem_waves(k, group.size(), most16) >
+                                                                                 smem_waves(k, group.size(), most8));
+  for (uint32_t r : group) P.slot[r].map8 = narrow ? 1u : 0u;
+  smem = narrow ? most8 : most16;
+}
+
+// slots: whether replays may take the slot form (false: the layout of the
+// sorted lists alone); logged: the call keeps decision logs.
 int plan_replays(const unison_trace *const *traces, const unison_replay_params *params, int n_replays,
-                 size_t smem_limit, bool results_in_scratch, ReplayPlan &P, size_t &off_res) {
+                 size_t smem_limit, bool results_in_scratch, bool slots, bool logged, ReplayPlan &P, size_t &off_res) {
   std::map<std::tuple<uint32_t, uint32_t, uint32_t, uint32_t, uint64_t, uint32_t>, int> combo_of;
   P.replay_combo.assign(n_replays, -1);
   for (int r = 0; r < n_replays; r++) {
@@ -1807,20 +1605,18 @@ int plan_replays(const unison_trace *const *traces, const unison_replay_params *
   off = align_up(off + sizeof(uint32_t) * 2 * n_replays, 256);
   P.off_combo = off;
   off = align_up(off + sizeof(ComboDesc) * P.combos.size() + 1, 256);
-  P.off_lut.resize(P.combos.size());
-  P.off_stream.resize(P.combos.size());
-  for (size_t c = 0; c < P.combos.size(); c++) {
-    P.off_lut[c] = off;
-    off = align_up(off + 128 + 51 * 8, 256);
-    const uint64_t E = traces[std::get<0>(P.combos[c])]->n_events;
-    P.off_stream[c] = off;
-    off = align_up(off + align_up(12 * E, 8) + 8 * E, 256);
-  }
   P.off_ttft.assign(n_replays, 0);
   P.off_glist.assign(n_replays, 0);
   P.rcap_s.resize(n_replays);
   P.rcap_h.resize(n_replays);
   P.tmap.assign(n_replays, 0);
+  P.slot.assign(n_replays, unison_slots::SlotDesc{});
+  P.off_lut.resize(P.combos.size());
+  P.off_stream.resize(P.combos.size());
+  P.need_keys.assign(P.combos.size(), 0);
+  P.need_rank.assign(P.combos.size(), 0);
+  // the slot kernels' static shared memory (event batches, descriptor) stays below 4 KB
+  const size_t slot_limit = smem_limit > 4096 ? smem_limit - 4096 : 0;
   for (int r = 0; r < n_replays; r++) {
     const unison_replay_params &p = params[r];
     const unison_trace *tr = traces[p.trace_idx];
@@ -1844,25 +1640,47 @@ int plan_replays(const unison_trace *const *traces, const unison_replay_params *
       P.tmap[r] = kMapSlots;
       P.in_stale.push_back((uint32_t)r);
       P.max_smem_stale = std::max(P.max_smem_stale, sb);
+    } else if (slots && slot_plan(p, tr, P.rcap_s[r], P.rcap_h[r], P.slot[r]) &&
+               unison_slots::slot_bytes(P.slot[r].nslots, tr->n_sessions, p.policy != UNISON_SPEAR_TIDE, true) <=
+                   slot_limit) {
+      const bool lean_st = p.policy == UNISON_SPEAR_TIDE && p.max_sessions == 0 && !logged;
+      (lean_st ? P.in_slot_st : P.in_slot_mix).push_back((uint32_t)r);
     } else if (lists <= smem_limit) {
-      const bool st = p.policy == UNISON_SPEAR_TIDE;
-      (st ? P.in_st : P.in_mix).push_back((uint32_t)r);
-      size_t &m = st ? P.max_smem_st : P.max_smem_mix;
-      m = std::max<size_t>(m, lists + (P.tmap[r] == kMapSlots ? map : 0));
+      P.slot[r].nslots = 0;
+      P.in_list.push_back((uint32_t)r);
+      P.max_smem_list = std::max<size_t>(P.max_smem_list, lists + (P.tmap[r] == kMapSlots ? map : 0));
     } else {
+      P.slot[r].nslots = 0;
       P.tmap[r] = kMapNone;
-      (p.policy == UNISON_SPEAR_TIDE ? P.in_gst : P.in_gmix).push_back((uint32_t)r);
+      P.in_glist.push_back((uint32_t)r);
       P.off_glist[r] = off;
       off = align_up(off + lists, 256);
     }
     P.off_ttft[r] = off;
     off = align_up(off + 8 * (tr->n_turns + 1), 256);
+    const int c = P.replay_combo[r];
+    if (c >= 0 && p.policy != UNISON_LRU_TIDE) {
+      if (P.slot[r].nslots) P.need_rank[c] = 1;
+      else P.need_keys[c] = 1;
+    }
   }
-  add_tier_maps(traces, params, smem_limit, P.in_st, st_kernel(P, true), P.max_smem_st, P);
-  add_tier_maps(traces, params, smem_limit, P.in_mix, replay_kernel<false, kKeyStream, -1, false>, P.max_smem_mix,
-                P);
-  for (uint32_t r : P.in_st) P.st_lean &= P.tmap[r] == kMapSlots && params[r].max_sessions == 0;
-  for (uint32_t r : P.in_st) P.st_reg &= P.rcap_s[r] <= 32;
+  if (!slots) P.need_keys.assign(P.combos.size(), 1);
+  for (size_t c = 0; c < P.combos.size(); c++) {
+    P.off_lut[c] = off;
+    off = align_up(off + 128 + 51 * 8, 256);
+    const unison_trace *tr = traces[std::get<0>(P.combos[c])];
+    const uint64_t E = tr->n_events;
+    P.off_stream[c] = off;
+    // gap averages; keys after and before each event; ranks and the sort's two buffers
+    if (P.need_keys[c]) off += align_up(12 * E, 8) + 8 * E;
+    else off += align_up(4 * E, 8);
+    if (P.need_rank[c]) off += align_up(4 * E, 8) + 16 * (tr->n_turns - tr->n_sessions);
+    off = align_up(off, 256);
+  }
+  if (!P.in_list.empty())
+    add_tier_maps(traces, params, smem_limit, P.in_list, replay_kernel<false, kKeyStream>, P.max_smem_list, P);
+  if (!P.in_slot_st.empty()) slot_maps(traces, params, slot_limit, P.in_slot_st, true, P.smem_slot_st, P);
+  if (!P.in_slot_mix.empty()) slot_maps(traces, params, slot_limit, P.in_slot_mix, false, P.smem_slot_mix, P);
   off_res = 0;
   if (results_in_scratch) {
     off_res = off;
@@ -1894,9 +1712,27 @@ void fill_descs(const unison_trace *const *traces, const unison_replay_params *p
     d.penalty_q = std::get<4>(P.combos[c]);
     d.sigma = reinterpret_cast<uint16_t *>(scratch + P.off_lut[c]);
     d.t2 = reinterpret_cast<uint64_t *>(scratch + P.off_lut[c] + 128);
-    d.pkey = reinterpret_cast<uint64_t *>(scratch + P.off_stream[c]);
-    d.gq = reinterpret_cast<uint32_t *>(scratch + P.off_stream[c] + 8 * tr->n_events);
-    d.pkb = reinterpret_cast<uint64_t *>(scratch + P.off_stream[c] + align_up(12 * tr->n_events, 8));
+    const uint64_t E = tr->n_events;
+    char *q = scratch + P.off_stream[c];
+    d.pkey = d.pkb = nullptr;
+    if (P.need_keys[c]) {
+      d.pkey = reinterpret_cast<uint64_t *>(q);
+      d.gq = reinterpret_cast<uint32_t *>(q + 8 * E);
+      d.pkb = reinterpret_cast<uint64_t *>(q + align_up(12 * E, 8));
+      q += align_up(12 * E, 8) + 8 * E;
+    } else {
+      d.gq = reinterpret_cast<uint32_t *>(q);
+      q += align_up(4 * E, 8);
+    }
+    d.rk = unison_slots::RankDesc{};
+    if (P.need_rank[c]) {
+      d.rk.rank = reinterpret_cast<uint32_t *>(q);
+      q += align_up(4 * E, 8);
+      d.rk.n = (uint32_t)(tr->n_turns - tr->n_sessions);
+      d.rk.a = reinterpret_cast<unsigned long long *>(q);
+      d.rk.b = d.rk.a + d.rk.n;
+      d.rk.turn_ev = d.turn_ev;
+    }
   }
   hd.resize(n_replays);
   for (int r = 0; r < n_replays; r++) {
@@ -1935,9 +1771,11 @@ void fill_descs(const unison_trace *const *traces, const unison_replay_params *p
     d.t2 = P.replay_combo[r] >= 0 ? hc[P.replay_combo[r]].t2 : nullptr;
     d.stale_sync = p.stale_sync;
     d.stale_m = p.stale_m;
+    d.slot = P.slot[r];
+    d.slot.rank = P.replay_combo[r] >= 0 ? hc[P.replay_combo[r]].rk.rank : nullptr;
   }
   order.clear();
-  for (const auto *g : {&P.in_st, &P.in_mix, &P.in_gst, &P.in_gmix, &P.in_online, &P.in_stale})
+  for (const auto *g : {&P.in_slot_st, &P.in_slot_mix, &P.in_list, &P.in_glist, &P.in_online, &P.in_stale})
     order.insert(order.end(), g->begin(), g->end());
   // A launch lasts as long as its slowest replay, and CTAs start in index
   // order: the SPEAR+TIDE launch takes its replays by predicted cost,
@@ -1945,7 +1783,7 @@ void fill_descs(const unison_trace *const *traces, const unison_replay_params *p
   // The predictor is the product of the tiers' capacities (the larger both
   // tiers, the more tier moves a replay makes); decisions do not depend on
   // the order.
-  std::stable_sort(order.begin(), order.begin() + P.in_st.size(), [&](uint32_t a, uint32_t b) {
+  std::stable_sort(order.begin(), order.begin() + P.in_slot_st.size(), [&](uint32_t a, uint32_t b) {
     return (double)hd[a].cap_s * (double)hd[a].cap_h > (double)hd[b].cap_s * (double)hd[b].cap_h;
   });
 }
@@ -1989,7 +1827,7 @@ SideStreams *side_streams(std::unique_lock<std::mutex> &hold) {
 // Queue the kernels of a planned batch on `stream`.
 int launch_replays(const ReplayPlan &P, char *scratch, const std::vector<ComboDesc> &hc,
                    const std::vector<ReplayDesc> &hd, const std::vector<uint32_t> &order, int n_replays,
-                   cudaStream_t stream, bool profile, bool logged) {
+                   cudaStream_t stream, bool profile) {
   int rc = UNISON_OK;
   auto ck = [&](cudaError_t e) {
     if (e != cudaSuccess && rc == UNISON_OK) rc = UNISON_ERR_CUDA;
@@ -2014,6 +1852,12 @@ int launch_replays(const ReplayPlan &P, char *scratch, const std::vector<ComboDe
         key_stream_kernel<<<dim3((max_s + 127) / 128, rows), 128, 0, stream>>>(d_combo + c0);
         count_launches(1);
       }
+      bool ranks = false;
+      for (char f : P.need_rank) ranks |= f != 0;
+      if (ranks) {
+        rank_keys_kernel<<<(unsigned)P.combos.size(), unison_slots::kSortThreads, 0, stream>>>(d_combo);
+        count_launches(1);
+      }
     }
     ck(cudaGetLastError());
   }
@@ -2025,12 +1869,12 @@ int launch_replays(const ReplayPlan &P, char *scratch, const std::vector<ComboDe
       size_t n, smem;
     };
     const Launch all[] = {
-        {st_kernel(P, logged), P.in_st.size(), P.max_smem_st},
-        {replay_kernel<false, kKeyStream, -1, false>, P.in_mix.size(), P.max_smem_mix},
-        {replay_kernel<true, kKeyStream, UNISON_SPEAR_TIDE, false>, P.in_gst.size(), 0},
-        {replay_kernel<true, kKeyStream, -1, false>, P.in_gmix.size(), 0},
-        {replay_kernel<false, kKeyOnline, -1, false>, P.in_online.size(), P.max_smem_online},
-        {replay_kernel<false, kKeyStale, -1, false>, P.in_stale.size(), P.max_smem_stale}};
+        {slot_kernel_of(true), P.in_slot_st.size(), P.smem_slot_st},
+        {slot_kernel_of(false), P.in_slot_mix.size(), P.smem_slot_mix},
+        {replay_kernel<false, kKeyStream>, P.in_list.size(), P.max_smem_list},
+        {replay_kernel<true, kKeyStream>, P.in_glist.size(), 0},
+        {replay_kernel<false, kKeyOnline>, P.in_online.size(), P.max_smem_online},
+        {replay_kernel<false, kKeyStale>, P.in_stale.size(), P.max_smem_stale}};
     std::vector<Launch> ls;
     std::vector<size_t> first;
     size_t off = 0;
@@ -2103,7 +1947,7 @@ extern "C" int unison_replay_batch(const unison_trace *const *traces, int n_trac
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   ReplayPlan P;
   size_t off_res = 0;
-  rc = plan_replays(traces, params, n_replays, smem_limit, results_dev == nullptr, P, off_res);
+  rc = plan_replays(traces, params, n_replays, smem_limit, results_dev == nullptr, true, log_dev != nullptr, P, off_res);
   if (rc != UNISON_OK) return rc;
   char *scratch = nullptr;
   if (unison_fault_alloc() || cudaMallocAsync(reinterpret_cast<void **>(&scratch), P.bytes, stream) != cudaSuccess) {
@@ -2115,7 +1959,7 @@ extern "C" int unison_replay_batch(const unison_trace *const *traces, int n_trac
   std::vector<ReplayDesc> hd;
   std::vector<uint32_t> order;
   fill_descs(traces, params, n_replays, P, scratch, res, log_dev, log_capacity_per_replay, hc, hd, order);
-  rc = launch_replays(P, scratch, hc, hd, order, n_replays, stream, true, log_dev != nullptr);
+  rc = launch_replays(P, scratch, hc, hd, order, n_replays, stream, true);
   if (results_host &&
       cudaMemcpyAsync(results_host, res, sizeof(unison_replay_result) * n_replays, cudaMemcpyDeviceToHost, stream) !=
           cudaSuccess &&
@@ -2291,9 +2135,17 @@ extern "C" int unison_replay_batch_noalloc(const unison_trace *const *traces, in
   if (rc != UNISON_OK) return rc;
   ReplayPlan P;
   size_t off_res = 0;
-  rc = plan_replays(traces, params, n_replays, smem_limit, false, P, off_res);
-  if (rc != UNISON_OK) return rc;
-  if (P.bytes > UNISON_NOALLOC_SCRATCH_BYTES) return UNISON_ERR_RANGE;  // batch too large for the fixed scratch
+  // What fits is decided by the layout of the sorted lists, as documented; the
+  // slot form's layout is taken where it fits as well.
+  {
+    ReplayPlan lists;
+    rc = plan_replays(traces, params, n_replays, smem_limit, false, false, log_dev != nullptr, lists, off_res);
+    if (rc != UNISON_OK) return rc;
+    if (lists.bytes > UNISON_NOALLOC_SCRATCH_BYTES) return UNISON_ERR_RANGE;  // batch too large for the fixed scratch
+    rc = plan_replays(traces, params, n_replays, smem_limit, false, true, log_dev != nullptr, P, off_res);
+    if (rc != UNISON_OK) return rc;
+    if (P.bytes > UNISON_NOALLOC_SCRATCH_BYTES) P = std::move(lists);
+  }
   // Every scratch region is written before it is read within one call (the
   // descriptors by the copies in launch_replays, the tables and streams by
   // their kernels, TTFT values and lists by the event loop), so nothing left
@@ -2302,7 +2154,7 @@ extern "C" int unison_replay_batch_noalloc(const unison_trace *const *traces, in
   std::vector<ReplayDesc> hd;
   std::vector<uint32_t> order;
   fill_descs(traces, params, n_replays, P, scratch, results_dev, log_dev, log_capacity_per_replay, hc, hd, order);
-  rc = launch_replays(P, scratch, hc, hd, order, n_replays, stream, false, log_dev != nullptr);
+  rc = launch_replays(P, scratch, hc, hd, order, n_replays, stream, false);
   if (results_host) {
     if (cudaMemcpyAsync(results_host, results_dev, sizeof(unison_replay_result) * n_replays, cudaMemcpyDeviceToHost,
                         stream) != cudaSuccess &&

@@ -150,6 +150,7 @@ extern "C" int unison_trace_create(const unison_turns *turns, unison_trace **out
     min_out = std::min(min_out, turns->out_tok[i]);
   }
   tr->min_out_tok = T ? min_out : 1;
+  for (uint64_t s = 0; s < S; s++) tr->sum_last_out += turns->out_tok[turns->turn_off[s + 1] - 1];  // sizes only grow
   for (uint64_t e = 0; e < E; e++) {
     const HostEvent &x = ev[e];
     const uint64_t ti = turns->turn_off[x.session] + x.turn;

@@ -337,6 +337,31 @@ def test_many_sessions_paths(B, n_sessions):
         assert_same(res[i], oracle.replay(tr, to_oracle(p)), p["policy"])
 
 
+@pytest.mark.parametrize("n_sessions", [127, 128, 129, 256, 2047, 2048])
+def test_slot_form_edges(B, n_sessions):
+    """Every session resident at once (unbounded tiers), and the same trace
+    with both tiers tight: residents at and beside one and two passes of 128
+    slots, and at the most slots the slot form takes (2,048) with one session
+    more, which runs on the sorted lists.  Every policy, and a slot limit."""
+    tr = synth.make_trace(31, np.full(n_sessions, 3), 0.01, synth.GAP_MIX_CODING)
+    reps = [(0, base(pol, cs, ch, 28672, **kw)) for cs, ch in ((1 << 60, 1 << 60), (256 * MIB, 1 << 60), (1 * GIB, 4 * GIB))
+            for pol, kw in [(q, {}) for q in POLS] + [("spear_tide", {"max_sessions": 100})]]
+    res, _, _ = run_gpu(B, [tr], reps)
+    for i, (_, p) in enumerate(reps):
+        assert_same(res[i], oracle.replay(tr, to_oracle(p)), (p["policy"], p["cap_s"], p["max_sessions"]))
+
+
+def test_slot_form_one_byte_map(B):
+    """130,000 sessions: two bytes of session map do not fit in shared memory,
+    so a one-byte entry names several of the replay's slots (about 900) and
+    the session is told apart by what they hold."""
+    tr = synth.make_trace(32, np.full(130_000, 2), 0.005, synth.GAP_MIX_GENERAL)
+    reps = [(0, base(pol, 2 * GIB, 28 * GIB, 16384)) for pol in ("spear_tide", "lru", "spear")]
+    res, _, _ = run_gpu(B, [tr], reps)
+    for i, (_, p) in enumerate(reps):
+        assert_same(res[i], oracle.replay(tr, to_oracle(p)), p["policy"])
+
+
 def test_degenerate_traces(B):
     """One session with one turn; one session with the most turns a session
     may have (65,535, spanning 40 hours of 32-bit wrapping microseconds);

@@ -67,6 +67,8 @@ struct unison_trace {
   uint64_t n_events = 0;
   uint32_t min_out_tok = 0;
   uint64_t sum_last_out = 0;  // every session's largest KV size, summed
+  uint64_t sum_in = 0;        // every turn's l^in, summed
+  uint64_t span_us = 0;       // first event to last
 
   // One page-locked host block holding every array below, copied to the
   // device with a single cudaMemcpyAsync.

@@ -1303,7 +1303,8 @@ __global__ void __launch_bounds__(32) replay_kernel(const ReplayDesc *descs, con
 
 // Replays of the slot form.  kOnly >= 0: every replay of the launch is a lean
 // one of that policy (no log, no slot limit); else each takes its own body.
-template <int kOnly>
+// kMap8: the launch's session maps hold one byte a session, else two.
+template <int kOnly, bool kMap8>
 __global__ void __launch_bounds__(32) slot_kernel(const ReplayDesc *descs, const uint32_t *order) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ReplayDesc Dsh;
@@ -1312,23 +1313,38 @@ __global__ void __launch_bounds__(32) slot_kernel(const ReplayDesc *descs, const
   if (lane == 0) Dsh = descs[order[blockIdx.x]];
   __syncwarp();
   if constexpr (kOnly >= 0) {
-    unison_slots::slot_replay<kOnly, true>(Dsh, Dsh.slot, bufs, smem, lane);
+    unison_slots::slot_replay<kOnly, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
   } else {
+    using unison_slots::slot_replay;
     if (Dsh.policy == UNISON_SPEAR_TIDE)
-      unison_slots::slot_replay<UNISON_SPEAR_TIDE, false>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<UNISON_SPEAR_TIDE, false, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+    else if (Dsh.log || Dsh.max_sessions)
+      slot_replay<-1, false, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+    else if (Dsh.policy == UNISON_SPEAR)
+      slot_replay<UNISON_SPEAR, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+    else if (Dsh.policy == UNISON_LRU)
+      slot_replay<UNISON_LRU, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+    else if (Dsh.policy == UNISON_BELADY)
+      slot_replay<UNISON_BELADY, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+    else if (Dsh.policy == UNISON_TIMEOUT)
+      slot_replay<UNISON_TIMEOUT, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
     else
-      unison_slots::slot_replay<-1, false>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<UNISON_LRU_TIDE, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
   }
 }
 
 // Lower median (element floor((n-1)/2) in sorted order) by MSB-first radix select.
-__global__ void __launch_bounds__(256) ttft_median_kernel(const ReplayDesc *descs, uint32_t n_replays) {
+__global__ void __launch_bounds__(256, 3) ttft_median_kernel(const ReplayDesc *descs, uint32_t n_replays) {
   const ReplayDesc &D = descs[blockIdx.x];
   __shared__ unsigned int hist[256];
   __shared__ unsigned long long red[8];
   __shared__ unsigned int sel_digit, sel_count;
   __shared__ unsigned long long sel_target;
   const uint64_t n = min((uint64_t)D.result->ttft_n, (uint64_t)D.n_turns);
+  if (D.slot.nslots) {
+    __shared__ unison_slots::AccShared acc;
+    unison_slots::account_arrivals(D, acc);
+  }
   if (n == 0) {
     if (threadIdx.x == 0) D.result->ttft_p50_ns = 0;
     return;
@@ -1553,10 +1569,16 @@ bool slot_plan(const unison_replay_params &p, const unison_trace *tr, uint32_t r
   q.cap_h = (uint32_t)std::min<uint64_t>(p.cap_hbm_bytes / p.kv_bytes_per_token, tr->sum_last_out);
   q.nslots = (uint32_t)n;
   q.sbits = sb;
+  const unsigned __int128 most_ns =
+      (unsigned __int128)tr->sum_in * (p.t_p_ps_per_tok / 1000) + (unsigned __int128)tr->span_us * 1000;
+  q.serial = most_ns >> 63 ? 1u : 0u;
   return true;
 }
 
-ReplayKernel slot_kernel_of(bool lean_st) { return lean_st ? slot_kernel<UNISON_SPEAR_TIDE> : slot_kernel<-1>; }
+ReplayKernel slot_kernel_of(bool lean_st, bool map8) {
+  if (lean_st) return map8 ? slot_kernel<UNISON_SPEAR_TIDE, true> : slot_kernel<UNISON_SPEAR_TIDE, false>;
+  return map8 ? slot_kernel<-1, true> : slot_kernel<-1, false>;
+}
 
 // The session maps of a slot group: two bytes a session name the slot
 // directly; one byte (its low eight bits, the slot told apart by the session
@@ -1573,9 +1595,10 @@ void slot_maps(const unison_trace *const *traces, const unison_replay_params *pa
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const ReplayKernel k = slot_kernel_of(lean_st);
-  const bool narrow = most16 > smem_limit || (group.size() > (size_t)sms && smem_waves(k, group.size(), most16) >
-                                                                                 smem_waves(k, group.size(), most8));
+  const bool narrow =
+      most16 > smem_limit ||
+      (group.size() > (size_t)sms && smem_waves(slot_kernel_of(lean_st, false), group.size(), most16) >
+                                         smem_waves(slot_kernel_of(lean_st, true), group.size(), most8));
   for (uint32_t r : group) P.slot[r].map8 = narrow ? 1u : 0u;
   smem = narrow ? most8 : most16;
 }
@@ -1868,9 +1891,10 @@ int launch_replays(const ReplayPlan &P, char *scratch, const std::vector<ComboDe
       ReplayKernel k;
       size_t n, smem;
     };
+    auto map8 = [&](const std::vector<uint32_t> &g) { return !g.empty() && P.slot[g[0]].map8; };
     const Launch all[] = {
-        {slot_kernel_of(true), P.in_slot_st.size(), P.smem_slot_st},
-        {slot_kernel_of(false), P.in_slot_mix.size(), P.smem_slot_mix},
+        {slot_kernel_of(true, map8(P.in_slot_st)), P.in_slot_st.size(), P.smem_slot_st},
+        {slot_kernel_of(false, map8(P.in_slot_mix)), P.in_slot_mix.size(), P.smem_slot_mix},
         {replay_kernel<false, kKeyStream>, P.in_list.size(), P.max_smem_list},
         {replay_kernel<true, kKeyStream>, P.in_glist.size(), 0},
         {replay_kernel<false, kKeyOnline>, P.in_online.size(), P.max_smem_online},

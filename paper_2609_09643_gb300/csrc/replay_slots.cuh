@@ -16,12 +16,15 @@
 //
 // What bounds it: the dependence chain of one warp.  The chain of a choice is
 // a 16-byte shared load a lane for up to 128 slots, three maxima, one REDUX
-// and the load of the winner's size: 188 warp instructions and 1,010 cycles an
-// event for the slowest of 152 sweep replays.  Sorted lists of 64-bit keys in
-// the warp's registers, which this replaced, took 375 and 1,513 (49.2 -> 32.8 ms).
-// One GB300, before and after: 1,024-replay sweep 65.0 -> 45.4 ms, 30 mixed
-// paper-scale replays 76.3 -> 38.1 ms, 40,000-session pool 1,359 -> 760 ms, four
-// tiny replays 1.68 -> 1.04 ms.
+// and the load of the winner's size.  158 warp instructions an event, and 842
+// cycles for the slowest of 152 sweep replays (27.3 ms): an instruction costs
+// about 2.7 cycles to issue and wait for, so what follows from an arrival's
+// class is left to account_arrivals and branches are kept few (188
+// instructions, 1,010 cycles, 32.8 ms with the accounting in the loop).
+// Sorted lists of 64-bit keys in the warp's registers, which this replaced,
+// took 375 and 1,513 (49.2 ms).  Tried and not kept: the words' extremes found
+// at the top of every event, beside the session's lookup (185 instructions,
+// sweep 32.5 -> 34.3 ms); 256 words loaded at once (34.0 ms).
 #pragma once
 
 #include "common.cuh"
@@ -34,11 +37,10 @@ constexpr uint32_t kAll = 0xFFFFFFFFu;
 constexpr uint32_t kFastBit = 0x80000000u;   // of a slot word
 constexpr uint32_t kPromoted = 0x80000000u;  // of a payload's size word
 constexpr uint32_t kSizeBits = 0x7FFFFFFFu;
-constexpr uint32_t kInFast = 1, kInHbm = 2;
 constexpr uint32_t kMostSlots = 2048;  // 16 words a lane
 
 // A resident's payload: size (and whether TIDE promoted it), session and tier
-// (bits 30-31).  Policies other than SPEAR+TIDE also keep the rank a Belady
+// (bit 31: fast).  Policies other than SPEAR+TIDE also keep the rank a Belady
 // session will have once unpinned, and the time it was unpinned (Timeout).
 template <bool kWide>
 struct Payload;
@@ -51,12 +53,15 @@ struct Payload<true> {
   uint4 v;
 };
 
+// Events reach the warp through a ring of shared memory, 32 at a time, with
+// the next batch landed and the one after it on its way.
 struct SlotEvent {
   uint4 ev;   // time32, session | flags, in_tok, out_tok
-  uint4 aux;  // previous turn's size (arrivals); rank and gap average (completions); next reference
+  uint4 aux;  // rank, gap average (completions); next reference (arrivals)
 };
+constexpr uint32_t kRing = 128;
 struct SlotBufs {
-  SlotEvent e[2][32];
+  SlotEvent e[kRing];
 };
 
 // What one replay of the slot form reads besides its ReplayDesc.
@@ -66,7 +71,15 @@ struct SlotDesc {
   uint32_t nslots;        // slots the replay can need
   uint32_t sbits;         // slot bits of a word
   uint32_t map8;          // 1: the session map holds the slot's low byte only
+  uint32_t serial;        // 1: the prefill queue's times may pass 2^63 ns (account_arrivals)
 };
+
+// What the event loop notes of each arrival, one byte in arrival order: the
+// request class, whether TIDE had promoted the session, and where it was
+// placed.  The bytes lie in the last eighth of the replay's TTFT area: arrival
+// i's at byte 7 n_turns + i.
+constexpr uint32_t kClassCold = 0, kClassFast = 1, kClassHbm = 2, kClassMiss = 3;  // the decision kinds
+constexpr uint32_t kNotePromoted = 4, kNotePlaceShift = 3;  // bits 3-4: 0 fast tier, 1 HBM, 2 bypassed
 
 // Bytes of shared memory of one replay: words, payloads, free slots, map.
 __host__ __device__ inline size_t slot_words(uint32_t nslots) { return ((size_t)nslots + 127) / 128 * 128; }
@@ -76,29 +89,33 @@ __host__ inline size_t slot_bytes(uint32_t nslots, uint32_t n_sessions, bool wid
   return slot_words(nslots) * 4 + (pay + 15) / 16 * 16 + fr + map;
 }
 
-template <bool kWide>
+// The replay's state.  kLean: no decision log and no slot limit.
+template <bool kLean, bool kWide>
 struct Slots {
   uint32_t *W;
   Payload<kWide> *P;
-  uint16_t *F;       // freed slots, a stack
+  uint16_t *F;            // freed slots, a stack
   uint32_t nfree, fresh;  // entries of F; slots handed out at least once
-  uint32_t nslots, sbits, smask;
-  uint32_t used_s, used_h, pinned_s, pinned_h, cap_s, cap_h;  // tokens
+  uint32_t sbits, smask;
+  // tokens: a tier's space beside all its residents, and beside its pinned ones
+  uint32_t free_s, free_h, room_s, room_h;
   int status;
-  // decision stream
-  uint32_t e;
-  uint64_t hash, log_len, log_cap;
+  // decision stream: event, hash (two halves), log
+  uint32_t e, h_lo, h_hi;
+  uint64_t log_len, log_cap;
   unison_decision *log;
-  // counters (warp-uniform registers)
-  uint32_t n_cold, n_hit_s, n_hit_h, n_miss, n_bypass, n_place_s, n_place_h;
-  uint32_t n_evict, n_demote, n_promote, n_tide_demote, n_expire, n_tide_calls, n_pth, n_res;
+  // counters (warp-uniform registers); those of arrivals come from the notes
+  uint32_t n_evict, n_demote, n_promote, n_tide_demote, n_expire, n_tide_calls, n_res;
 };
 
-// kLean: no decision log and no slot limit.
-template <bool kLean, class St>
-__device__ __forceinline__ void decide(St &st, uint32_t kind, uint32_t s, int lane) {
-  const uint64_t w = ((uint64_t)st.e << 32) | (kind << 24 | s);
-  st.hash = (st.hash ^ w) * kFnvPrime;
+// h = (h ^ (event << 32 | kind << 24 | session)) * 0x100000001B3 mod 2^64.
+template <bool kLean, bool kWide>
+__device__ __forceinline__ void decide(Slots<kLean, kWide> &st, uint32_t kind, uint32_t s, int lane) {
+  static_assert(kFnvPrime == (1ull << 40 | 0x1B3u), "the multiplication below");
+  const uint32_t lo = st.h_lo ^ (s | kind << 24), hi = st.h_hi ^ st.e;
+  const uint64_t m = (uint64_t)lo * 0x1B3u;
+  st.h_lo = (uint32_t)m;
+  st.h_hi = (uint32_t)(m >> 32) + hi * 0x1B3u + (lo << 8);
   if constexpr (!kLean) {
     if (st.log) {
       if (st.log_len < st.log_cap) {
@@ -134,9 +151,11 @@ __device__ __forceinline__ uint32_t max_word(const St &st, int lane) {
 template <class St>
 __device__ __forceinline__ uint32_t max_hbm(const St &st, int lane) {
   const uint4 *w4 = reinterpret_cast<const uint4 *>(st.W) + lane;
-  uint32_t m = 0;
-  for (uint32_t q = 0; q == 0 || q < st.fresh; q += 128, w4 += 32) {
-    const uint4 v = *w4;
+  uint4 v = w4[0];
+  uint32_t m = max(max(v.x ^ kFastBit, v.y ^ kFastBit), max(v.z ^ kFastBit, v.w ^ kFastBit));
+  for (uint32_t q = 128; q < st.fresh; q += 128) {
+    w4 += 32;
+    v = *w4;
     m = max(max(m, max(v.x ^ kFastBit, v.y ^ kFastBit)), max(v.z ^ kFastBit, v.w ^ kFastBit));
   }
   return __reduce_max_sync(kAll, m);
@@ -168,49 +187,31 @@ __device__ __forceinline__ void release_slot(St &st, uint32_t slot) {
   st.P[slot].v.y = kIdMask;  // no session has this id
   st.F[st.nfree] = (uint16_t)slot;
   st.nfree++;
-}
-
-template <bool kLean, class St>
-__device__ __forceinline__ void evict_slot(St &st, uint32_t slot, uint32_t id, int lane) {
-  decide<kLean>(st, UNISON_KIND_EVICT, id, lane);
-  st.n_evict++;
   st.n_res--;
-  release_slot(st, slot);
+}
+template <class St>
+__device__ __forceinline__ uint2 payload(const St &st, uint32_t slot) {
+  const uint2 p = *reinterpret_cast<const uint2 *>(&st.P[slot]);
+  __syncwarp();
+  return p;
 }
 
 // Room in HBM for `size` tokens against its unpinned residents: evicts the
 // most evictable ones, only those above `floor_word` (a word without the tier
 // bit; 0 accepts every one).  False when the next one is not above it.
-template <bool kLean, class St>
+template <class St>
 __device__ __forceinline__ bool make_hbm_room(St &st, uint32_t size, uint32_t floor_word, int lane) {
-  while (st.used_h + size > st.cap_h) {
+  while (size > st.free_h) {
     const uint32_t m = max_hbm(st, lane);
-    const uint32_t w = m ^ kFastBit;
-    if (m <= kFastBit || w < floor_word) return false;
-    const uint32_t slot = w & st.smask;
-    const uint2 p = make_uint2(st.P[slot].v.x, st.P[slot].v.y);
-    __syncwarp();
-    st.used_h -= p.x & kSizeBits;
-    evict_slot<kLean>(st, slot, p.y & kIdMask, lane);
+    if (m <= max(kFastBit, floor_word | kFastBit)) return false;
+    const uint32_t slot = m & st.smask;
+    const uint2 p = payload(st, slot);
+    st.free_h += p.x & kSizeBits;
+    decide(st, UNISON_KIND_EVICT, p.y & kIdMask, lane);
+    st.n_evict++;
+    release_slot(st, slot);
   }
   return true;
-}
-
-// A session demoted out of the fast tier (its word w, payload p): into HBM,
-// displacing more evictable sessions there, or dropped.
-template <bool kLean, class St>
-__device__ __forceinline__ void demote_slot(St &st, uint32_t w, uint32_t slot, uint32_t px, uint32_t py, int lane) {
-  const uint32_t size = px & kSizeBits, id = py & kIdMask;
-  const uint32_t hw = w & ~kFastBit;
-  if (size > st.cap_h - st.pinned_h || !make_hbm_room<kLean>(st, size, hw, lane)) {
-    evict_slot<kLean>(st, slot, id, lane);
-    return;
-  }
-  st.W[slot] = hw;
-  st.P[slot].v.y = id | (kInHbm << 30);
-  st.used_h += size;
-  decide<kLean>(st, UNISON_KIND_DEMOTE, id, lane);
-  st.n_demote++;
 }
 
 __device__ __forceinline__ void async16(void *dst, const void *src) {
@@ -253,13 +254,12 @@ __device__ __forceinline__ void expire_slots(St &st, uint32_t now, uint32_t ttl,
       return;
     }
     const uint32_t slot = __shfl_sync(kAll, at, __ffs(__ballot_sync(kAll, id == first)) - 1);
-    const uint32_t w = st.W[slot], size = st.P[slot].v.x & kSizeBits;
-    __syncwarp();
-    if (w & kFastBit) st.used_s -= size;
-    else st.used_h -= size;
-    decide<false>(st, UNISON_KIND_EXPIRE, first, lane);
+    const uint32_t w = st.W[slot];
+    const uint32_t size = payload(st, slot).x & kSizeBits;
+    st.free_s += w & kFastBit ? size : 0u;
+    st.free_h += w & kFastBit ? 0u : size;
+    decide(st, UNISON_KIND_EXPIRE, first, lane);
     st.n_expire++;
-    st.n_res--;
     release_slot(st, slot);
     __syncwarp();
   }
@@ -269,7 +269,7 @@ __device__ __forceinline__ void expire_slots(St &st, uint32_t now, uint32_t ttl,
 // of Algorithm 1 has it: phase 1 promotes the least evictable HBM sessions
 // into free fast-tier space, phase 2 swaps the least evictable HBM session
 // with the most evictable fast-tier one.  Returns the bytes moved.
-template <bool kLean, class St>
+template <class St>
 __device__ __forceinline__ uint64_t tide_slots(St &st, uint64_t budget, uint32_t kvb, int lane) {
   uint64_t rem = budget;
   bool fill = true;  // phase 1
@@ -279,48 +279,44 @@ __device__ __forceinline__ uint64_t tide_slots(St &st, uint64_t budget, uint32_t
     if (mn >= kFastBit - 1u) break;  // HBM holds no unpinned session
     const uint32_t pw = mn + 1u, pslot = pw & st.smask;
     const uint32_t dslot = mx & st.smask;  // a valid slot even when mx names none
-    const uint2 p = make_uint2(st.P[pslot].v.x, st.P[pslot].v.y);
-    const uint2 d = make_uint2(st.P[dslot].v.x, st.P[dslot].v.y);
+    const uint2 p = *reinterpret_cast<const uint2 *>(&st.P[pslot]);
+    const uint2 d = payload(st, dslot);
     const uint32_t sp = p.x & kSizeBits, pid = p.y & kIdMask;
-    __syncwarp();
-    if (fill) {
-      const uint64_t by = (uint64_t)sp * kvb;
-      if (by <= rem && st.used_s + sp <= st.cap_s) {
-        rem -= by;
-        st.used_s += sp;
-        st.used_h -= sp;
-        st.W[pslot] = pw | kFastBit;
-        st.P[pslot].v.x = p.x | kPromoted;
-        st.P[pslot].v.y = pid | (kInFast << 30);
-        decide<kLean>(st, UNISON_KIND_PROMOTE, pid, lane);
-        st.n_promote++;
-        continue;
-      }
-      fill = false;
+    uint64_t by = (uint64_t)sp * kvb;
+    fill = fill && by <= rem && sp <= st.free_s;
+    if (!fill) {
+      // phase 2: the swap is legal and the demoted session the more evictable
+      const uint32_t sd = d.x & kSizeBits, did = d.y & kIdMask;
+      by += (uint64_t)sd * kvb;
+      const bool swap = (mx & kFastBit) != 0 && (mx & ~kFastBit) > pw && by <= rem && sp <= st.free_s + sd &&
+                        sd <= st.free_h + sp;
+      if (!swap) break;
+      st.W[dslot] = mx & ~kFastBit;
+      st.P[dslot].v.y = did;
+      st.free_s += sd;
+      st.free_h -= sd;
+      st.n_tide_demote++;
+      decide(st, UNISON_KIND_PROMOTE, pid, lane);
+      decide(st, UNISON_KIND_TIDE_DEMOTE, did, lane);
+    } else {
+      decide(st, UNISON_KIND_PROMOTE, pid, lane);
     }
-    if (mx < kFastBit || (mx & ~kFastBit) <= pw) break;  // no fast-tier session, or none more evictable
-    const uint32_t sd = d.x & kSizeBits, did = d.y & kIdMask;
-    const uint64_t by = (uint64_t)(sp + sd) * kvb;
-    if (by > rem || st.used_s - sd + sp > st.cap_s || st.used_h - sp + sd > st.cap_h) break;
     rem -= by;
-    st.used_s = st.used_s - sd + sp;
-    st.used_h = st.used_h - sp + sd;
+    st.free_s -= sp;
+    st.free_h += sp;
     st.W[pslot] = pw | kFastBit;
-    st.P[pslot].v.x = p.x | kPromoted;
-    st.P[pslot].v.y = pid | (kInFast << 30);
-    st.W[dslot] = mx & ~kFastBit;
-    st.P[dslot].v.y = did | (kInHbm << 30);
-    decide<kLean>(st, UNISON_KIND_PROMOTE, pid, lane);
-    decide<kLean>(st, UNISON_KIND_TIDE_DEMOTE, did, lane);
+    *reinterpret_cast<uint2 *>(&st.P[pslot]) = make_uint2(p.x | kPromoted, pid | kFastBit);
     st.n_promote++;
-    st.n_tide_demote++;
   }
   return budget - rem;
 }
 
 // One replay.  kPol: its policy when the body is specialised for it, or -1
-// for the body that reads the policy from the descriptor.
-template <int kPol, bool kLean, class Desc>
+// for the body that reads the policy from the descriptor.  Branches are kept
+// few (each costs an issue slot and a fetch, and one warp hides neither):
+// classes and tiers are selected, and the loops that make room and migrate are
+// the only ones an ordinary event passes.
+template <int kPol, bool kLean, bool kMap8, class Desc>
 __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, SlotBufs &bufs, unsigned char *smem,
                                             int lane) {
   constexpr bool kWide = kPol != UNISON_SPEAR_TIDE;
@@ -330,8 +326,8 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
   const bool belady = policy == UNISON_BELADY;
   const bool timeout = policy == UNISON_TIMEOUT && D.ttl != 0xFFFFFFFFu;
 
-  Slots<kWide> st;
-  st.nslots = Q.nslots;
+  Slots<kLean, kWide> st;
+  const uint32_t nslots = Q.nslots;
   st.sbits = Q.sbits;
   st.smask = (1u << Q.sbits) - 1u;
   unsigned char *p = smem;
@@ -341,212 +337,180 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
   p += ((size_t)Q.nslots * sizeof(Payload<kWide>) + 15) / 16 * 16;
   st.F = reinterpret_cast<uint16_t *>(p);
   p += ((size_t)Q.nslots * 2 + 15) / 16 * 16;
-  uint8_t *const map8 = Q.map8 ? p : nullptr;
+  uint8_t *const map8 = p;
   uint16_t *const map16 = reinterpret_cast<uint16_t *>(p);
   {
     uint4 *w4 = reinterpret_cast<uint4 *>(st.W);
     for (uint32_t i = lane; i < slot_words(Q.nslots) / 4; i += 32) w4[i] = make_uint4(0u, 0u, 0u, 0u);
     uint4 *m4 = reinterpret_cast<uint4 *>(p);
-    const uint32_t mq = (D.n_sessions * (Q.map8 ? 1u : 2u) + 15) / 16;
+    const uint32_t mq = (D.n_sessions * (kMap8 ? 1u : 2u) + 15) / 16;
     for (uint32_t i = lane; i < mq; i += 32) m4[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (lane == 0) st.P[0].v.y = kIdMask;  // a zero map entry finds no session
+    // the ring past the last event names session 0
+    for (uint32_t i = lane; i < kRing; i += 32) bufs.e[i].ev = make_uint4(0u, 0u, 0u, 0u);
+    if (lane == 0) {
+      st.P[0].v.y = kIdMask;  // a zero map entry finds no session
+      st.F[0] = 0;
+    }
     __syncwarp();
   }
   st.nfree = st.fresh = 0;
-  st.used_s = st.used_h = st.pinned_s = st.pinned_h = 0;
-  st.cap_s = Q.cap_s;
-  st.cap_h = Q.cap_h;
+  st.free_s = st.room_s = Q.cap_s;
+  st.free_h = st.room_h = Q.cap_h;
   st.status = UNISON_OK;
-  st.hash = kFnvOffset;
+  st.h_lo = (uint32_t)kFnvOffset;
+  st.h_hi = (uint32_t)(kFnvOffset >> 32);
   st.log = D.log;
   st.log_cap = D.log_cap;
   st.log_len = 0;
-  st.n_cold = st.n_hit_s = st.n_hit_h = st.n_miss = st.n_bypass = st.n_place_s = st.n_place_h = 0;
-  st.n_evict = st.n_demote = st.n_promote = st.n_tide_demote = st.n_expire = st.n_tide_calls = st.n_pth = 0;
+  st.n_evict = st.n_demote = st.n_promote = st.n_tide_demote = st.n_expire = st.n_tide_calls = 0;
   st.n_res = 0;
-  uint64_t tok_hit_s = 0, tok_hit_h = 0, tok_miss = 0, tok_needed = 0, dma_bytes = 0;
-
-  // TTFT queue (Sec. V-A): arrivals compressed by the load factor.
-  uint64_t rel_us = 0, q_free = 0;
-  uint32_t n_arr = 0, n_ev = 0, n_done = 0;
-  const uint32_t load = D.load;
-  const uint64_t prefill_ns = D.prefill_ns;
+  uint64_t dma_bytes = 0;
+  uint32_t n_done = 0;
   const uint32_t n_turns = D.n_turns;
-  uint64_t *const ttft_out = D.ttft;
-  const uint64_t ns_per_us = (1000u % load == 0) ? 1000u / load : 0u;  // 0: divide exactly
-  unsigned long long s_lo = 0, s_hi = 0;
-  bool dma_busy = false;
-  uint64_t busy_from = 0, busy_bytes = 0;  // the DMA's last batch: start (rel_us) and bytes
-  uint32_t oldest = 0;                     // Timeout: see expire_slots
-  const uint32_t kvb = D.kvb, max_sessions = D.max_sessions;
-  const uint64_t dma = D.dma;
+  uint8_t *note_out = reinterpret_cast<uint8_t *>(D.ttft) + 7ull * n_turns;
+  // the DMA's last batch: its bytes (0: none in flight) and the time since it
+  // began, advanced from completion to completion, which are less than 2^32
+  // us apart (the next event, and a turn, take less than 2^31)
+  uint64_t busy_bytes = 0, busy_us = 0;
+  uint32_t oldest = 0;  // Timeout: see expire_slots
+  const uint32_t kvb = D.kvb, max_sessions = D.max_sessions, dma = (uint32_t)D.dma;
 
   const uint32_t E = D.n_events;
-  auto fetch = [&](uint32_t b, int bi) {
+  auto fetch = [&](uint32_t b) {
     const uint32_t i = b + lane;
     if (i < E) {
-      SlotEvent &d = bufs.e[bi][lane];
+      SlotEvent &d = bufs.e[i & (kRing - 1)];
       async16(&d.ev, &D.ev[i]);
-      async4(&d.aux.x, &D.prev_out[i]);
-      if (spear) async4(&d.aux.y, &Q.rank[i]);
-      if (tide_on) async4(&d.aux.z, &D.gq[i]);
-      if (belady) async4(&d.aux.w, &D.nref[i]);
+      if (spear) async4(&d.aux.x, &Q.rank[i]);
+      if (tide_on) async4(&d.aux.y, &D.gq[i]);
+      if (belady) async4(&d.aux.z, &D.nref[i]);
     }
     async_commit();
   };
-  auto map_of = [&](uint32_t s) -> uint32_t { return map8 ? map8[s] : map16[s]; };
-  fetch(0, 0);
-  async_wait<0>();
+  auto map_of = [&](uint32_t s) -> uint32_t { return kMap8 ? map8[s] : map16[s]; };
+  fetch(0);
+  fetch(32);
+  async_wait<1>();
   __syncwarp();
-  uint32_t prev_now = E ? bufs.e[0][0].ev.x : 0u;
-  oldest = prev_now;
+  uint32_t last_done = bufs.e[0].ev.x;
+  oldest = last_done;
+  // the next event's session word and map entry are loaded while an event is
+  // processed; a map entry changes only when its session is placed
+  uint32_t nw = bufs.e[0].ev.y, nmap = map_of(nw & kIdMask), e = 0;
 
-  int bi = 0;
-  for (uint32_t b = 0; b < E && st.status != UNISON_ERR_CAPACITY; b += 32, bi ^= 1) {
-    if (b + 32 < E) {
-      fetch(b + 32, bi ^ 1);
-      async_wait<1>();  // this batch's copies have landed
-    } else {
-      async_wait<0>();
-    }
+  while (e < E && st.status != UNISON_ERR_CAPACITY) {
+    fetch(e + 64);
+    async_wait<1>();  // the batch after this one has landed
     __syncwarp();
-    const uint32_t cnt = min(32u, E - b);
-    // the next event's record and map entry are loaded while this one is
-    // processed; a map entry changes only when its session is placed
-    uint4 nev = bufs.e[bi][0].ev, naux = bufs.e[bi][0].aux;
-    uint32_t nmap = map_of(nev.y & kIdMask);
-    for (uint32_t j = 0; j < cnt; j++) {
-      const uint4 ev = nev, aux = naux;
+    const uint32_t end = min(E, e + 32);
+    for (; e < end; e++) {
+      const SlotEvent &rec = bufs.e[e & (kRing - 1)];
+      const uint32_t w1 = nw, s = w1 & kIdMask;
       uint32_t slot = nmap;
-      const uint32_t jn = min(j + 1, cnt - 1);
-      nev = bufs.e[bi][jn].ev;
-      naux = bufs.e[bi][jn].aux;
-      const uint32_t now = ev.x, s = ev.y & kIdMask;
-      const bool arrival = (ev.y & kEvArrival) != 0, edge = (ev.y & kEvEdge) != 0;
-      st.e = b + j;
-      n_ev++;
-      rel_us += (uint32_t)(now - prev_now);
-      prev_now = now;
-      if (kPol < 0 && timeout) {
-        if constexpr (kWide) expire_slots(st, now, D.ttl, oldest, lane);
+      nw = bufs.e[(e + 1) & (kRing - 1)].ev.y;
+      const uint32_t ns = nw & kIdMask;
+      st.e = e;
+      if (timeout) {
+        if constexpr (kWide) expire_slots(st, rec.ev.x, D.ttl, oldest, lane);
       }
       // the session's slot: the one its map entry names, if that slot is still
       // the session's own (an 8-bit entry names up to eight slots)
-      bool found;
-      if (map8) {
+      if (kMap8) {
         const uint32_t c = slot + 256u * lane;
         const unsigned hit = __ballot_sync(kAll, c < st.fresh && (st.P[c].v.y & kIdMask) == s);
-        found = hit != 0;
-        slot += found ? 256u * (__ffs(hit) - 1) : 0u;
+        slot += hit ? 256u * (__ffs(hit) - 1) : 0u;
       }
-      const uint2 pl = make_uint2(st.P[slot].v.x, st.P[slot].v.y);
-      if (!map8) found = (pl.y & kIdMask) == s;
-      nmap = map_of(nev.y & kIdMask);
+      const uint2 pl = *reinterpret_cast<const uint2 *>(&st.P[slot]);
+      nmap = map_of(ns);
       __syncwarp();
+      const bool found = (pl.y & kIdMask) == s, fast = (pl.y & kFastBit) != 0;
+      const uint32_t size = pl.x & kSizeBits;
 
-      if (arrival) {
-        const uint32_t in = ev.z, n = ev.w, prev = aux.x;
-        uint64_t prefill = in;
-        if (edge) {
-          decide<kLean>(st, UNISON_KIND_COLD, s, lane);
-          st.n_cold++;
-        } else {
-          tok_needed += in;
-          if (found) {
-            const uint32_t size = pl.x & kSizeBits;
-            prefill = in - prev;
-            st.W[slot] = 0u;
-            if (pl.y >> 30 == kInFast) {
-              decide<kLean>(st, UNISON_KIND_HIT_S, s, lane);
-              st.n_hit_s++;
-              tok_hit_s += prev;
-              if (pl.x & kPromoted) st.n_pth++;
-              st.used_s -= size;
-            } else {
-              decide<kLean>(st, UNISON_KIND_HIT_H, s, lane);
-              st.n_hit_h++;
-              tok_hit_h += prev;
-              st.used_h -= size;
-            }
-          } else {
-            decide<kLean>(st, UNISON_KIND_MISS, s, lane);
-            st.n_miss++;
-            tok_miss += prev;
-          }
-        }
-        {
-          const uint64_t arr = ns_per_us ? rel_us * ns_per_us : rel_us * 1000ull / load;
-          if (q_free < arr) q_free = arr;
-          q_free += prefill * prefill_ns;
-          const uint64_t v = q_free - arr;
-          if (lane == 0 && n_arr < n_turns) ttft_out[n_arr] = v;
-          n_arr++;
-          const unsigned long long lo2 = s_lo + v;
-          s_hi += (lo2 < s_lo);
-          s_lo = lo2;
+      if (w1 & kEvArrival) {
+        const uint32_t n = rec.ev.w;
+        const uint32_t cls = found ? (fast ? kClassFast : kClassHbm) : (w1 & kEvEdge ? kClassCold : kClassMiss);
+        decide(st, cls, s, lane);
+        uint32_t note = cls | (pl.x >> 31) * kNotePromoted;  // (the bit counts for fast-tier hits only)
+        if (found) {
+          st.W[slot] = 0u;
+          st.free_s += fast ? size : 0u;
+          st.free_h += fast ? 0u : size;
         }
         // placement; a session that was resident keeps its slot
-        uint32_t tier = 0;
+        uint32_t tier = 0;  // 0 fast, 1 HBM, 2 bypassed
         if (!kLean && max_sessions && st.n_res - (found ? 1u : 0u) >= max_sessions && [&] {
               // as many pinned sessions as the limit allows: bypass
               uint32_t un = 0;
               for (uint32_t i = lane; i < st.fresh; i += 32) un += st.W[i] != 0u;
               return st.n_res - (found ? 1u : 0u) - __reduce_add_sync(kAll, un) >= max_sessions;
             }()) {
-        } else if (n <= st.cap_s - st.pinned_s) {
-          tier = kInFast;
-          while (st.used_s + n > st.cap_s) {
+          tier = 2;
+        } else if (n <= st.room_s) {
+          while (n > st.free_s) {
             const uint32_t w = max_word(st, lane);  // the most evictable unpinned fast-tier session
             if (w < kFastBit) {
               st.status = UNISON_ERR_CAPACITY;
               break;
             }
-            const uint32_t ds = w & st.smask;
-            const uint2 d = make_uint2(st.P[ds].v.x, st.P[ds].v.y);
-            __syncwarp();
-            st.used_s -= d.x & kSizeBits;
-            demote_slot<kLean>(st, w, ds, d.x, d.y, lane);
+            // it is demoted into HBM, displacing more evictable sessions
+            // there, or dropped
+            const uint32_t ds = w & st.smask, hw = w & ~kFastBit;
+            const uint2 d = payload(st, ds);
+            const uint32_t sd = d.x & kSizeBits, did = d.y & kIdMask;
+            st.free_s += sd;
+            const bool keep = sd <= st.room_h && make_hbm_room(st, sd, hw, lane);
+            decide(st, keep ? (uint32_t)UNISON_KIND_DEMOTE : (uint32_t)UNISON_KIND_EVICT, did, lane);
+            if (keep) {
+              st.W[ds] = hw;
+              st.P[ds].v.y = did;
+              st.free_h -= sd;
+              st.n_demote++;
+            } else {
+              st.n_evict++;
+              release_slot(st, ds);
+            }
           }
-        } else if (n <= st.cap_h - st.pinned_h) {
-          tier = kInHbm;
-          if (!make_hbm_room<kLean>(st, n, 0u, lane)) st.status = UNISON_ERR_CAPACITY;
+          st.free_s -= n;
+          st.room_s -= n;
+        } else if (n <= st.room_h) {
+          tier = 1;
+          if (!make_hbm_room(st, n, 0u, lane)) st.status = UNISON_ERR_CAPACITY;
+          st.free_h -= n;
+          st.room_h -= n;
+        } else {
+          tier = 2;
         }
         if (st.status == UNISON_ERR_CAPACITY) break;
-        if (tier) {
+        static_assert(UNISON_KIND_PLACE_H == UNISON_KIND_PLACE_S + 1 && UNISON_KIND_BYPASS == UNISON_KIND_PLACE_S + 2,
+                      "placement kinds");
+        decide(st, UNISON_KIND_PLACE_S + tier, s, lane);
+        if (tier < 2) {
           if (!found) {
-            if (st.nfree) {
-              slot = st.F[--st.nfree];
-            } else {
-              slot = st.fresh++;
-              if (slot >= st.nslots) {
-                st.status = UNISON_ERR_CAPACITY;
-                break;
-              }
-            }
+            // the last slot freed, else a new one
+            const bool reuse = st.nfree != 0;
+            const uint32_t f = st.F[reuse ? st.nfree - 1 : 0];
+            slot = reuse ? f : st.fresh;
+            st.nfree -= reuse ? 1u : 0u;
+            st.fresh += reuse ? 0u : 1u;
             st.n_res++;
+            if (slot >= nslots) {
+              st.status = UNISON_ERR_CAPACITY;
+              break;
+            }
             __syncwarp();
-            if (map8) map8[s] = (uint8_t)slot;
+            if (kMap8) map8[s] = (uint8_t)slot;
             else map16[s] = (uint16_t)slot;
           }
-          st.P[slot].v.x = n;
-          st.P[slot].v.y = s | (tier << 30);
+          if (ns == s) nmap = kMap8 ? (slot & 255u) : slot;  // read before it was set
+          *reinterpret_cast<uint2 *>(&st.P[slot]) = make_uint2(n, s | (tier ? 0u : kFastBit));
           if constexpr (kWide) {
             // a session with no next arrival ranks above every event index,
             // the smaller id higher
-            if (belady) st.P[slot].v.z = aux.w == kNoRef ? E + D.n_sessions - s : aux.w + 1u;
+            if (belady) {
+              const uint32_t nr = rec.aux.z;
+              st.P[slot].v.z = nr == kNoRef ? E + D.n_sessions - s : nr + 1u;
+            }
           }
-          if (tier == kInFast) {
-            st.used_s += n;
-            st.pinned_s += n;
-            decide<kLean>(st, UNISON_KIND_PLACE_S, s, lane);
-            st.n_place_s++;
-          } else {
-            st.used_h += n;
-            st.pinned_h += n;
-            decide<kLean>(st, UNISON_KIND_PLACE_H, s, lane);
-            st.n_place_h++;
-          }
-          if ((nev.y & kIdMask) == s) nmap = map8 ? (slot & 255u) : slot;  // read before it was set
           if (!kLean && max_sessions) {
             while (st.n_res > max_sessions) {
               // the most evictable of both tiers
@@ -558,59 +522,49 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
                 break;
               }
               const uint32_t vs = m & st.smask, vw = st.W[vs];
-              const uint2 v = make_uint2(st.P[vs].v.x, st.P[vs].v.y);
-              __syncwarp();
-              if (vw & kFastBit) st.used_s -= v.x & kSizeBits;
-              else st.used_h -= v.x & kSizeBits;
-              evict_slot<kLean>(st, vs, v.y & kIdMask, lane);
+              const uint2 v = payload(st, vs);
+              const uint32_t sv = v.x & kSizeBits;
+              st.free_s += vw & kFastBit ? sv : 0u;
+              st.free_h += vw & kFastBit ? 0u : sv;
+              decide(st, UNISON_KIND_EVICT, v.y & kIdMask, lane);
+              st.n_evict++;
+              release_slot(st, vs);
               __syncwarp();
             }
             if (st.status == UNISON_ERR_CAPACITY) break;
           }
-        } else {
-          decide<kLean>(st, UNISON_KIND_BYPASS, s, lane);
-          st.n_bypass++;
-          if (found) {
-            st.n_res--;
-            release_slot(st, slot);
-          }
+        } else if (found) {
+          release_slot(st, slot);
         }
+        *note_out++ = (uint8_t)(note | tier << kNotePlaceShift);  // (every lane the same byte)
       } else {
         // completion: the session is unpinned (if resident) with its new rank
         n_done++;
+        const uint32_t now = rec.ev.x;
+        busy_us += (uint32_t)(now - last_done);
+        last_done = now;
         if (found) {
           uint32_t rk;
-          if (spear) rk = aux.y + 1u;
+          if (spear) rk = rec.aux.x + 1u;
           else rk = n_turns - n_done + 1u;  // the later the touch, the less evictable
           if constexpr (kWide) {
             if (belady) rk = st.P[slot].v.z;
-            st.P[slot].v.w = now;
+            if (timeout) st.P[slot].v.w = now;
           }
-          const uint32_t size = pl.x & kSizeBits;
-          const bool fast = pl.y >> 30 == kInFast;
-          st.W[slot] = rk << st.sbits | slot | (fast ? kFastBit : 0u);
-          if (fast) st.pinned_s -= size;
-          else st.pinned_h -= size;
+          st.W[slot] = rk << st.sbits | slot | (pl.y & kFastBit);
+          st.room_s += fast ? size : 0u;
+          st.room_h += fast ? 0u : size;
         }
-        if (!edge && tide_on) {
+        if (tide_on && !(w1 & kEvEdge)) {
           // the DMA is free again from start + ceil(bytes / rate) us on, i.e.
-          // once the elapsed us times the rate cover the bytes (the high word
-          // of the product catches one past 2^64)
-          if (dma_busy) {
-            const uint64_t el = rel_us - busy_from;
-            if (__umul64hi(el, dma) != 0 || el * dma >= busy_bytes) dma_busy = false;
-          }
-          if (!dma_busy) {
+          // once the elapsed us times the rate cover the bytes.  A batch's
+          // bytes are at most 2^31 us of the rate.
+          const bool busy = busy_us >> 31 == 0 && (uint64_t)(uint32_t)busy_us * dma < busy_bytes;
+          if (!busy) {
             st.n_tide_calls++;
-            const uint64_t moved = tide_slots<kLean>(st, aux.z * dma, kvb, lane);
-            if (moved) {
-              dma_bytes += moved;
-              if (dma) {
-                dma_busy = true;
-                busy_from = rel_us;
-                busy_bytes = moved;
-              }
-            }
+            busy_bytes = tide_slots(st, (uint64_t)rec.aux.y * dma, kvb, lane);  // (0 at rate 0: no budget)
+            dma_bytes += busy_bytes;
+            busy_us = 0;
           }
         }
       }
@@ -618,41 +572,224 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
   }
   async_wait<0>();
   if (lane == 0) {
-    const uint32_t warm = st.n_hit_s + st.n_hit_h + st.n_miss;
+    // the counters that follow from the arrivals' notes are account_arrivals'
     unison_replay_result r = {};
-    r.events = n_ev;
-    r.req_warm = warm;
-    r.cold = st.n_cold;
-    r.hit_s = st.n_hit_s;
-    r.hit_h = st.n_hit_h;
-    r.miss = st.n_miss;
-    r.bypass = st.n_bypass;
-    r.place_s = st.n_place_s;
-    r.place_h = st.n_place_h;
+    r.events = min(e + (e < E ? 1u : 0u), E);
     r.evict = st.n_evict;
     r.demote = st.n_demote;
     r.promote = st.n_promote;
     r.tide_demote = st.n_tide_demote;
     r.expire = st.n_expire;
-    r.tok_hit_s = tok_hit_s;
-    r.tok_hit_h = tok_hit_h;
-    r.tok_miss = tok_miss;
-    r.tok_computed = tok_needed - tok_hit_s - tok_hit_h;  // a hit computes in - prev
-    r.tok_needed = tok_needed;
     r.dma_bytes = dma_bytes;
     r.tide_calls = st.n_tide_calls;
-    r.promoted_then_hit_s = st.n_pth;
-    r.ttft_sum_lo = s_lo;
-    r.ttft_sum_hi = s_hi;
-    r.ttft_p50_ns = 0;
-    r.ttft_n = n_arr;
-    r.decision_hash = st.hash;
-    // every decision has its counter
-    r.log_len = (uint64_t)st.n_cold + warm + st.n_bypass + st.n_place_s + st.n_place_h + st.n_evict + st.n_demote +
-                st.n_promote + st.n_tide_demote + st.n_expire;
+    r.ttft_n = (uint64_t)(note_out - (reinterpret_cast<uint8_t *>(D.ttft) + 7ull * n_turns));
+    r.decision_hash = (uint64_t)st.h_hi << 32 | st.h_lo;
     r.status = st.status;
     *D.result = r;
   }
+}
+
+// --------------------------------------------------------------------------
+// Accounting of a replay's arrivals (Sec. V-A), from the event loop's notes:
+// request and placement counters, token sums, and the TTFT of every request.
+// The prefill queue is q' = max(q, a) + p with arrival a and prefill p; a run
+// of requests is q' = max(q + P, M), and two runs compose to P1 + P2 and
+// max(M1 + P2, M2), so the block scans 1,024 events at a time.  The event loop
+// is a serial chain and the queue took about 22 of an arrival's instructions
+// in it; here it costs 0.2-0.4 ms for the 1,024-replay sweep.  Times that
+// could pass 2^63 ns (D.slot.serial) wrap as the recurrence does when one
+// thread walks it.
+// Values overwrite the notes in place: the 8-byte values of arrivals up to i
+// end at or before the notes of arrivals past i (8 (i + 1) <= 7 n + i + 1), and
+// a chunk's notes are read before its values are stored.
+// --------------------------------------------------------------------------
+constexpr int kAccThreads = 256, kAccItems = 4, kAccChunk = kAccThreads * kAccItems;
+
+struct AccShared {
+  unsigned long long us[8], p[8], m[8];
+  uint32_t n[8];
+  uint32_t cnt[8];
+  unsigned long long tok[4], sum[2];
+};
+
+template <class Desc>
+__device__ void account_arrivals(const Desc &D, AccShared &sh) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t E = D.n_events, load = D.load;
+  const uint64_t n_arr = D.result->ttft_n;
+  const uint64_t prefill_ns = D.prefill_ns;
+  const uint64_t ns_per_us = (1000u % load == 0) ? 1000u / load : 0u;  // 0: divide exactly
+  const uint8_t *const notes = reinterpret_cast<const uint8_t *>(D.ttft) + 7ull * D.n_turns;
+  uint32_t cnt[8] = {};            // cold, fast, HBM, miss; promoted; placed fast, HBM, bypassed
+  unsigned long long tok[4] = {};  // fast, HBM, miss; needed
+  unsigned long long s_lo = 0, s_hi = 0;
+  auto arrival_ns = [&](uint64_t us) { return ns_per_us ? us * ns_per_us : us * 1000ull / load; };
+  auto note = [&](uint32_t c, uint32_t in, uint32_t prev) -> uint64_t {  // counts it; its prefill tokens
+    const uint32_t cls = c & 3u;
+#pragma unroll
+    for (uint32_t k = 0; k < 4; k++) cnt[k] += cls == k;
+    cnt[4] += (c & (kNotePromoted | 3u)) == (kNotePromoted | kClassFast);
+#pragma unroll
+    for (uint32_t k = 0; k < 3; k++) cnt[5 + k] += c >> kNotePlaceShift == k;
+#pragma unroll
+    for (uint32_t k = 0; k < 3; k++) tok[k] += cls == k + 1 ? prev : 0u;
+    tok[3] += cls != kClassCold ? in : 0u;
+    return cls == kClassFast || cls == kClassHbm ? in - prev : in;
+  };
+  auto add = [&](uint64_t v) {
+    const unsigned long long lo = s_lo + v;
+    s_hi += lo < s_lo;
+    s_lo = lo;
+  };
+  if (tid < 8) sh.cnt[tid] = 0;
+  if (tid < 4) sh.tok[tid] = 0;
+  if (tid < 2) sh.sum[tid] = 0;
+  __syncthreads();
+  if (D.slot.serial) {
+    if (tid == 0) {
+      uint64_t us = 0, q = 0, i = 0;
+      for (uint32_t e = 0; e < E && i < n_arr; e++) {
+        const uint4 ev = D.ev[e];
+        if (e) us += (uint32_t)(ev.x - D.ev[e - 1].x);
+        if (!(ev.y & kEvArrival)) continue;
+        const uint64_t p = note(notes[i], ev.z, D.prev_out[e]), a = arrival_ns(us);
+        if (q < a) q = a;
+        q += p * prefill_ns;
+        D.ttft[i++] = q - a;
+        add(q - a);
+      }
+    }
+  } else {
+    unsigned long long us0 = 0, q0 = 0;  // before the chunk
+    uint64_t i0 = 0;
+    for (uint32_t base = 0; base < E && i0 < n_arr; base += kAccChunk) {
+      const uint32_t e0 = base + kAccItems * tid;
+      uint4 ev[kAccItems];
+      uint32_t prev[kAccItems];
+      uint32_t t = e0 > 0 && e0 < E ? D.ev[e0 - 1].x : 0u;
+#pragma unroll
+      for (int k = 0; k < kAccItems; k++) {
+        const bool in = e0 + k < E;
+        ev[k] = in ? D.ev[e0 + k] : make_uint4(0u, 0u, 0u, 0u);
+        prev[k] = in ? D.prev_out[e0 + k] : 0u;
+      }
+      // time and arrivals up to each thread's first event
+      if (e0 == 0) t = ev[0].x;
+      unsigned long long us = 0, rel[kAccItems];
+      uint32_t n = 0;
+#pragma unroll
+      for (int k = 0; k < kAccItems; k++) {
+        if (e0 + k < E) us += (uint32_t)(ev[k].x - t);
+        t = ev[k].x;
+        rel[k] = us;
+        n += ev[k].y >> 31;
+      }
+      static_assert(kEvArrival == 1u << 31, "arrival flag");
+      unsigned long long us_in = us;
+      uint32_t n_in = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(kAll, us_in, o);
+        const uint32_t z = __shfl_up_sync(kAll, n_in, o);
+        if ((int)lane >= o) {
+          us_in += y;
+          n_in += z;
+        }
+      }
+      if (lane == 31) {
+        sh.us[warp] = us_in;
+        sh.n[warp] = n_in;
+      }
+      __syncthreads();
+      unsigned long long us_b = us0 + us_in - us;
+      uint64_t i = i0 + n_in - n;
+      uint32_t n_all = 0;
+#pragma unroll
+      for (uint32_t w = 0; w < 8; w++) {
+        if (w < warp) {
+          us_b += sh.us[w];
+          i += sh.n[w];
+        }
+        us0 += sh.us[w];
+        n_all += sh.n[w];
+      }
+      // each arrival's time and prefill, the thread's run of the queue
+      unsigned long long P = 0, M = 0, a[kAccItems], p[kAccItems];
+      uint64_t at = i;
+#pragma unroll
+      for (int k = 0; k < kAccItems; k++) {
+        a[k] = p[k] = 0;
+        if ((ev[k].y & kEvArrival) && at < n_arr) {
+          p[k] = note(notes[at], ev[k].z, prev[k]) * prefill_ns;
+          a[k] = arrival_ns(us_b + rel[k]);
+          at++;
+          M = max(M, a[k]) + p[k];  // max(M + p, a + p)
+          P += p[k];
+        }
+      }
+      unsigned long long Pi = P, Mi = M;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(kAll, Pi, o), z = __shfl_up_sync(kAll, Mi, o);
+        if ((int)lane >= o) {
+          Mi = max(z + Pi, Mi);
+          Pi += y;
+        }
+      }
+      if (lane == 31) {
+        sh.p[warp] = Pi;
+        sh.m[warp] = Mi;
+      }
+      __syncthreads();  // and every note of the chunk has been read
+      const unsigned long long Pe = __shfl_up_sync(kAll, Pi, 1), Me = __shfl_up_sync(kAll, Mi, 1);
+      unsigned long long q = q0;
+#pragma unroll
+      for (uint32_t w = 0; w < 8; w++) {
+        if (w < warp) q = max(q + sh.p[w], sh.m[w]);
+        q0 = max(q0 + sh.p[w], sh.m[w]);
+      }
+      if (lane) q = max(q + Pe, Me);
+#pragma unroll
+      for (int k = 0; k < kAccItems; k++) {
+        if ((ev[k].y & kEvArrival) && i < n_arr) {
+          q = max(q, a[k]) + p[k];
+          D.ttft[i++] = q - a[k];
+          add(q - a[k]);
+        }
+      }
+      i0 += n_all;
+      __syncthreads();  // the next chunk rewrites the shared totals
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 8; k++) atomicAdd(&sh.cnt[k], cnt[k]);
+#pragma unroll
+  for (int k = 0; k < 4; k++) atomicAdd(&sh.tok[k], tok[k]);
+  const unsigned long long before = atomicAdd(&sh.sum[0], s_lo);
+  atomicAdd(&sh.sum[1], s_hi + (before + s_lo < before ? 1ull : 0ull));
+  __syncthreads();
+  if (tid == 0) {
+    unison_replay_result &r = *D.result;
+    r.cold = sh.cnt[0];
+    r.hit_s = sh.cnt[1];
+    r.hit_h = sh.cnt[2];
+    r.miss = sh.cnt[3];
+    r.req_warm = sh.cnt[1] + sh.cnt[2] + sh.cnt[3];
+    r.promoted_then_hit_s = sh.cnt[4];
+    r.place_s = sh.cnt[5];
+    r.place_h = sh.cnt[6];
+    r.bypass = sh.cnt[7];
+    r.tok_hit_s = sh.tok[0];
+    r.tok_hit_h = sh.tok[1];
+    r.tok_miss = sh.tok[2];
+    r.tok_needed = sh.tok[3];
+    r.tok_computed = sh.tok[3] - sh.tok[0] - sh.tok[1];  // a hit computes in - prev
+    r.ttft_sum_lo = sh.sum[0];
+    r.ttft_sum_hi = sh.sum[1];
+    // every decision has its counter
+    r.log_len = n_arr * 2 + r.evict + r.demote + r.promote + r.tide_demote + r.expire;
+  }
+  __syncthreads();
 }
 
 // --------------------------------------------------------------------------

@@ -148,8 +148,10 @@ extern "C" int unison_trace_create(const unison_turns *turns, unison_trace **out
     turn_t[2 * i] = (uint32_t)turns->arrival_us[i];
     turn_t[2 * i + 1] = (uint32_t)turns->completion_us[i];
     min_out = std::min(min_out, turns->out_tok[i]);
+    tr->sum_in += turns->in_tok[i];
   }
   tr->min_out_tok = T ? min_out : 1;
+  tr->span_us = E ? ev[E - 1].time - ev[0].time : 0;
   for (uint64_t s = 0; s < S; s++) tr->sum_last_out += turns->out_tok[turns->turn_off[s + 1] - 1];  // sizes only grow
   for (uint64_t e = 0; e < E; e++) {
     const HostEvent &x = ev[e];

@@ -17,13 +17,15 @@
 //   slot_kernel         Algorithm 1: one warp per replay; residents in
 //                       unordered slots, each decision one pass over their
 //                       ranks (replay_slots.cuh).
-//   replay_kernel       Algorithm 1 where the slot form does not apply (online
-//                       hazard table, stale snapshots, traces too large for
-//                       its words or lists too large for its slots): one warp
-//                       per replay; the unpinned residents of each tier kept
-//                       sorted by packed 64-bit key (the most evictable last),
-//                       so the argmax of a decision is a pop and an update is
-//                       a warp-parallel lower bound plus a block shift.
+//                       slot_variant_kernel: the same under the online hazard
+//                       table and with stale snapshots.
+//   replay_kernel       Algorithm 1 where the slot form does not apply (traces
+//                       too large for its words, tiers for its slots): one
+//                       warp per replay; the unpinned residents of each tier
+//                       kept sorted by packed 64-bit key (the most evictable
+//                       last), so the argmax of a decision is a pop and an
+//                       update is a warp-parallel lower bound plus a block
+//                       shift.
 //   ttft_median_kernel  Sec. V-A TTFT p50: radix select of the lower median
 //                       over each replay's per-request TTFT values.
 #include <algorithm>
@@ -198,10 +200,18 @@ __global__ void key_stream_kernel(const ComboDesc *combos) {
       c.pkey[ec] = prev_pk;
     }
     if (c.rk.rank) {
-      // live completions in order of descending session; the final ones, all
-      // of the maximal key, rank above them by descending session
-      if (k + 1 < ts) c.rk.a[c.rk.n - (b + ts - (s + 1)) + k] = (key << 24) | ti;
-      else c.rk.rank[ec] = c.rk.n + (c.n_sessions - 1 - s);
+      // live keys in order of descending session; the final completions', all
+      // maximal, rank above them by descending session
+      if (c.rk.all) {
+        // per session: the zero register row, every arrival, every live completion
+        unsigned long long *a = c.rk.a + c.rk.n - 2ull * (b + ts);
+        if (k == 0) a[0] = t2[0] << 24 | (c.n_events + s);
+        a[1 + 2 * k] = key << 24 | ea;
+        if (k + 1 < ts) a[2 + 2 * k] = key << 24 | ec;
+      } else if (k + 1 < ts) {
+        c.rk.a[c.rk.n - (b + ts - (s + 1)) + k] = key << 24 | ec;
+      }
+      if (k + 1 == ts) c.rk.rank[ec] = c.rk.n + (c.n_sessions - 1 - s);
     }
   }
 }
@@ -720,61 +730,10 @@ __device__ __forceinline__ bool has_tide(uint32_t policy) {
 // (hazard), (hq), (survq), (t2); bucket pooling).  Lives in shared memory
 // after the per-session state of an online replay.
 // --------------------------------------------------------------------------
-struct OnlineTable {
-  uint32_t n[kLutN], d[kLutN], sig[kLutN];
-  unsigned long long t2[kLutN];
-  unsigned long long mg[kLutN];  // magic_for(sig): eq. (t1)'s division by a multiply-high
-};
-
-// g < 2^31 (gaps are clamped below 2^31 us), so g * Lambda < 2^43.
+using unison_slots::online_add;
+using unison_slots::OnlineTable;
 __device__ __forceinline__ uint64_t online_key(const OnlineTable &ot, uint32_t g, uint32_t t, uint32_t s) {
-  const uint32_t tt = t < kTMax ? t : kTMax;
-  return pack_key(__umul64hi((uint64_t)g * kLambda, ot.mg[tt]) + ot.t2[tt], s);
-}
-
-// A session of `turns` turns has completed: add it to the counts and rebuild
-// sigma and T2 for every turn index.
-__device__ bool online_add(OnlineTable &ot, uint32_t turns, uint32_t bucket, uint64_t penalty, int lane) {
-  for (uint32_t t = lane; t < kLutN; t += 32) {
-    ot.n[t] += turns >= t + 1 ? 1u : 0u;
-    ot.d[t] += turns == t + 1 ? 1u : 0u;
-  }
-  __syncwarp();
-  uint32_t sg[2];
-  unsigned long long t2[2];
-#pragma unroll
-  for (int q = 0; q < 2; q++) {
-    const uint32_t t = lane + 32 * q;
-    sg[q] = kLambda;
-    t2[q] = 0;
-    if (t < kLutN) {
-      uint64_t nn = 0, dd = 0;
-      for (uint32_t u = (t / bucket) * bucket; u < kLutN && u / bucket == t / bucket; u++) {
-        nn += ot.n[u];
-        dd += ot.d[u];
-      }
-      uint64_t hq = nn ? (2 * dd * kLambda + nn) / (2 * nn) : 0;
-      if (hq > kLambda) hq = kLambda;
-      const uint32_t sq = (uint32_t)(kLambda - hq) < kEpsQ ? kEpsQ : (uint32_t)(kLambda - hq);
-      sg[q] = sq;
-      t2[q] = ((unsigned long long)(kLambda - sq) * penalty) / kLambda;
-    }
-  }
-  bool changed = false;
-#pragma unroll
-  for (int q = 0; q < 2; q++) changed |= (lane + 32 * q < kLutN) && ot.sig[lane + 32 * q] != sg[q];
-  __syncwarp();
-#pragma unroll
-  for (int q = 0; q < 2; q++) {
-    const uint32_t t = lane + 32 * q;
-    if (t < kLutN) {
-      if (ot.sig[t] != sg[q]) ot.mg[t] = magic_for(sg[q]);
-      ot.sig[t] = sg[q];
-      ot.t2[t] = t2[q];
-    }
-  }
-  __syncwarp();
-  return __any_sync(kFull, changed);  // T2 is a function of sigma
+  return pack_key(unison_slots::online_score(ot, g, t), s);
 }
 
 // Every resident takes a new key (new_key maps an entry's key to it), then the
@@ -909,12 +868,7 @@ __device__ __forceinline__ void replay_body(const ReplayDesc &D, EventBufs &bufs
         online_gs[i] = 0u;
         online_ks[i] = 0;
       }
-      for (uint32_t t = lane; t < kLutN; t += 32) {
-        online_tab->n[t] = online_tab->d[t] = 0u;
-        online_tab->sig[t] = kLambda;  // no session completed: zero hazard
-        online_tab->t2[t] = 0ull;
-        online_tab->mg[t] = magic_for(kLambda);
-      }
+      unison_slots::online_init(*online_tab, lane);
       __syncwarp();
     }
     if (kStale) {
@@ -1313,24 +1267,40 @@ __global__ void __launch_bounds__(32) slot_kernel(const ReplayDesc *descs, const
   if (lane == 0) Dsh = descs[order[blockIdx.x]];
   __syncwarp();
   if constexpr (kOnly >= 0) {
-    unison_slots::slot_replay<kOnly, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+    unison_slots::slot_replay<unison_slots::kRanked, kOnly, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
   } else {
+    using unison_slots::kRanked;
     using unison_slots::slot_replay;
     if (Dsh.policy == UNISON_SPEAR_TIDE)
-      slot_replay<UNISON_SPEAR_TIDE, false, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_SPEAR_TIDE, false, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
     else if (Dsh.log || Dsh.max_sessions)
-      slot_replay<-1, false, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, -1, false, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
     else if (Dsh.policy == UNISON_SPEAR)
-      slot_replay<UNISON_SPEAR, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_SPEAR, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
     else if (Dsh.policy == UNISON_LRU)
-      slot_replay<UNISON_LRU, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_LRU, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
     else if (Dsh.policy == UNISON_BELADY)
-      slot_replay<UNISON_BELADY, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_BELADY, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
     else if (Dsh.policy == UNISON_TIMEOUT)
-      slot_replay<UNISON_TIMEOUT, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_TIMEOUT, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
     else
-      slot_replay<UNISON_LRU_TIDE, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_LRU_TIDE, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
   }
+}
+
+// The slot form's variants: online hazard table, stale snapshots.
+template <int kMode>
+__global__ void __launch_bounds__(32) slot_variant_kernel(const ReplayDesc *descs, const uint32_t *order) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ ReplayDesc Dsh;
+  __shared__ __align__(16) unison_slots::SlotBufs bufs;
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) Dsh = descs[order[blockIdx.x]];
+  __syncwarp();
+  if (Dsh.log || Dsh.max_sessions)
+    unison_slots::slot_replay<kMode, -1, false, false>(Dsh, Dsh.slot, bufs, smem, lane);
+  else
+    unison_slots::slot_replay<kMode, -1, true, false>(Dsh, Dsh.slot, bufs, smem, lane);
 }
 
 // Lower median (element floor((n-1)/2) in sorted order) by MSB-first radix select.
@@ -1465,19 +1435,21 @@ namespace {
 
 // Scratch layout and launch plan of one batch (shared by both entry points).
 struct ReplayPlan {
-  std::vector<std::tuple<uint32_t, uint32_t, uint32_t, uint32_t, uint64_t, uint32_t>> combos;
+  // key streams: trace, EMA weight, bucket, P_Z, signals, and whether for the
+  // slot form of stale replays
+  std::vector<std::tuple<uint32_t, uint32_t, uint32_t, uint32_t, uint64_t, uint32_t, bool>> combos;
   std::vector<int> replay_combo;
   size_t off_desc = 0, off_order = 0, off_combo = 0, bytes = 0;
   std::vector<size_t> off_lut, off_stream, off_ttft, off_glist;
   std::vector<char> need_keys, need_rank;  // per combination: packed keys (sorted lists), ranks (slot form)
   // Replay groups, one kernel launch each: the slot form (lean SPEAR+TIDE
-  // replays, the others), sorted lists in shared memory, in global memory,
+  // replays, the other policies, online hazard table, stale snapshot), sorted lists in shared memory, in global memory,
   // online hazard table, stale snapshot.  The launches are independent and
   // run concurrently.
-  std::vector<uint32_t> in_slot_st, in_slot_mix, in_list, in_glist, in_online, in_stale;
+  std::vector<uint32_t> in_slot_st, in_slot_mix, in_slot_online, in_slot_stale, in_list, in_glist, in_online, in_stale;
   std::vector<uint32_t> rcap_s, rcap_h, tmap;
   std::vector<unison_slots::SlotDesc> slot;  // nslots 0: not of the slot form
-  size_t smem_slot_st = 0, smem_slot_mix = 0, max_smem_list = 0, max_smem_online = 0, max_smem_stale = 0;
+  size_t smem_slot_st = 0, smem_slot_mix = 0, smem_slot_online = 0, smem_slot_stale = 0, max_smem_list = 0, max_smem_online = 0, max_smem_stale = 0;
 };
 
 // Resident-list capacity of a tier: at most one entry per session and no more
@@ -1553,18 +1525,21 @@ void add_tier_maps(const unison_trace *const *traces, const unison_replay_params
 // Whether a replay can take the slot form, and its sizes.  A word holds the
 // tier bit, the rank and the slot; sums of tokens stay below 2^31 because a
 // capacity above every session's largest size together is never reached; the
-// sort's values hold a 24-bit turn.
+// sort's values hold a 24-bit entry.
 bool slot_plan(const unison_replay_params &p, const unison_trace *tr, uint32_t rcap_s, uint32_t rcap_h,
                unison_slots::SlotDesc &q) {
-  if (tr->sum_last_out >= (1ull << 31) || tr->n_turns >= (1ull << 24)) return false;
+  if (tr->sum_last_out >= (1ull << 31) || tr->n_events + tr->n_sessions >= (1ull << 24)) return false;
   const uint64_t n = std::min<uint64_t>(tr->n_sessions, (uint64_t)(rcap_s - 1) + (rcap_h - 1)) + 1;
   if (n > unison_slots::kMostSlots) return false;
-  // ranks run from 1 to the completions, under Belady to the events and sessions
-  uint64_t most = p.policy == UNISON_BELADY ? tr->n_events + tr->n_sessions : tr->n_turns;
+  // ranks run from 1 to the completions; under Belady and with a snapshot, to
+  // the events and sessions (an online replay's words hold no ranks)
+  const bool online = (p.flags & UNISON_HAZARD_ONLINE) != 0, stale = p.stale_sync != UNISON_SYNC_LIVE;
+  if (online && tr->n_sessions > kTierMapMax) return false;
+  uint64_t most = p.policy == UNISON_BELADY || stale ? tr->n_events + tr->n_sessions : tr->n_turns;
   uint32_t sb = 1, rb = 1;
   while ((1ull << sb) < n) sb++;
   while ((1ull << rb) <= most) rb++;
-  if (sb + rb > 31) return false;
+  if (sb + rb > 31 && !online) return false;
   q.cap_s = (uint32_t)std::min<uint64_t>(p.cap_fast_bytes / p.kv_bytes_per_token, tr->sum_last_out);
   q.cap_h = (uint32_t)std::min<uint64_t>(p.cap_hbm_bytes / p.kv_bytes_per_token, tr->sum_last_out);
   q.nslots = (uint32_t)n;
@@ -1573,6 +1548,28 @@ bool slot_plan(const unison_replay_params &p, const unison_trace *tr, uint32_t r
       (unsigned __int128)tr->sum_in * (p.t_p_ps_per_tok / 1000) + (unsigned __int128)tr->span_us * 1000;
   q.serial = most_ns >> 63 ? 1u : 0u;
   return true;
+}
+
+// Shared memory of one replay of the slot form (map8: with the smaller session
+// map, which the variants do not have).
+size_t slot_smem(const unison_replay_params &p, const unison_trace *tr, const unison_slots::SlotDesc &q, bool map8) {
+  using namespace unison_slots;
+  const bool online = (p.flags & UNISON_HAZARD_ONLINE) != 0, stale = p.stale_sync != UNISON_SYNC_LIVE;
+  const size_t S = tr->n_sessions;
+  size_t b = slot_bytes(q.nslots, tr->n_sessions, online || stale || p.policy != UNISON_SPEAR_TIDE,
+                        map8 && !online && !stale);
+  if (online || stale) b += slot_words(q.nslots) * 4;
+  if (stale) b += round16(8 * S + 4 * kDirtySlots);
+  if (online) b += round16(sizeof(OnlineTable)) + round16(2 * S);
+  return b;
+}
+
+// Ranks a key stream holds, and the values its sort takes.
+uint64_t rank_entries(const ReplayPlan &P, size_t c, const unison_trace *tr) {
+  return tr->n_events + (std::get<6>(P.combos[c]) ? tr->n_sessions : 0);
+}
+uint64_t rank_values(const ReplayPlan &P, size_t c, const unison_trace *tr) {
+  return std::get<6>(P.combos[c]) ? tr->n_events : tr->n_turns - tr->n_sessions;
 }
 
 ReplayKernel slot_kernel_of(bool lean_st, bool map8) {
@@ -1607,13 +1604,28 @@ void slot_maps(const unison_trace *const *traces, const unison_replay_params *pa
 // sorted lists alone); logged: the call keeps decision logs.
 int plan_replays(const unison_trace *const *traces, const unison_replay_params *params, int n_replays,
                  size_t smem_limit, bool results_in_scratch, bool slots, bool logged, ReplayPlan &P, size_t &off_res) {
-  std::map<std::tuple<uint32_t, uint32_t, uint32_t, uint32_t, uint64_t, uint32_t>, int> combo_of;
+  // the slot kernels' static shared memory (event ring, descriptor) stays below 5 KB
+  const size_t slot_limit = smem_limit > 4096 ? smem_limit - 4096 : 0;
+  P.rcap_s.resize(n_replays);
+  P.rcap_h.resize(n_replays);
+  P.slot.assign(n_replays, unison_slots::SlotDesc{});
+  for (int r = 0; r < n_replays; r++) {
+    const unison_replay_params &p = params[r];
+    const unison_trace *tr = traces[p.trace_idx];
+    P.rcap_s[r] = list_cap(p.cap_fast_bytes / p.kv_bytes_per_token, tr);
+    P.rcap_h[r] = list_cap(p.cap_hbm_bytes / p.kv_bytes_per_token, tr);
+    if (!slots || !slot_plan(p, tr, P.rcap_s[r], P.rcap_h[r], P.slot[r]) ||
+        slot_smem(p, tr, P.slot[r], true) > slot_limit)
+      P.slot[r].nslots = 0;
+  }
+  std::map<std::tuple<uint32_t, uint32_t, uint32_t, uint32_t, uint64_t, uint32_t, bool>, int> combo_of;
   P.replay_combo.assign(n_replays, -1);
   for (int r = 0; r < n_replays; r++) {
     const unison_replay_params &p = params[r];
     if (!needs_stream(p.policy)) continue;
     auto key = std::make_tuple(p.trace_idx, p.ema_num, p.ema_den, p.hazard_bucket, p.penalty_q,
-                               p.flags & (UNISON_SIGNAL_NO_GAP | UNISON_SIGNAL_NO_HAZARD));
+                               p.flags & (UNISON_SIGNAL_NO_GAP | UNISON_SIGNAL_NO_HAZARD),
+                               P.slot[r].nslots != 0 && p.stale_sync != UNISON_SYNC_LIVE);
     auto it = combo_of.find(key);
     if (it == combo_of.end()) {
       it = combo_of.emplace(key, (int)P.combos.size()).first;
@@ -1630,21 +1642,14 @@ int plan_replays(const unison_trace *const *traces, const unison_replay_params *
   off = align_up(off + sizeof(ComboDesc) * P.combos.size() + 1, 256);
   P.off_ttft.assign(n_replays, 0);
   P.off_glist.assign(n_replays, 0);
-  P.rcap_s.resize(n_replays);
-  P.rcap_h.resize(n_replays);
   P.tmap.assign(n_replays, 0);
-  P.slot.assign(n_replays, unison_slots::SlotDesc{});
   P.off_lut.resize(P.combos.size());
   P.off_stream.resize(P.combos.size());
   P.need_keys.assign(P.combos.size(), 0);
   P.need_rank.assign(P.combos.size(), 0);
-  // the slot kernels' static shared memory (event batches, descriptor) stays below 4 KB
-  const size_t slot_limit = smem_limit > 4096 ? smem_limit - 4096 : 0;
   for (int r = 0; r < n_replays; r++) {
     const unison_replay_params &p = params[r];
     const unison_trace *tr = traces[p.trace_idx];
-    P.rcap_s[r] = list_cap(p.cap_fast_bytes / p.kv_bytes_per_token, tr);
-    P.rcap_h[r] = list_cap(p.cap_hbm_bytes / p.kv_bytes_per_token, tr);
     const size_t lists = list_bytes(P.rcap_s[r], P.rcap_h[r]);
     // the tier map and pin slots (3 bytes per session) when they fit beside the lists
     const size_t map = align_up(tr->n_sessions, 16) + 2 * align_up(tr->n_sessions, 8);
@@ -1654,26 +1659,32 @@ int plan_replays(const unison_trace *const *traces, const unison_replay_params *
       const size_t ob = online_bytes(P.rcap_s[r], P.rcap_h[r], tr->n_sessions);
       if (tr->n_sessions > kTierMapMax || ob > smem_limit) return UNISON_ERR_RANGE;
       P.tmap[r] = kMapSlots;
-      P.in_online.push_back((uint32_t)r);
-      P.max_smem_online = std::max(P.max_smem_online, ob);
+      if (P.slot[r].nslots) {
+        P.in_slot_online.push_back((uint32_t)r);
+        P.smem_slot_online = std::max(P.smem_slot_online, slot_smem(p, tr, P.slot[r], false));
+      } else {
+        P.in_online.push_back((uint32_t)r);
+        P.max_smem_online = std::max(P.max_smem_online, ob);
+      }
     } else if (p.stale_sync != UNISON_SYNC_LIVE) {
       // stale-snapshot replays too
       const size_t sb = stale_bytes(P.rcap_s[r], P.rcap_h[r], tr->n_sessions);
       if (tr->n_sessions > kTierMapMax || sb > smem_limit) return UNISON_ERR_RANGE;
       P.tmap[r] = kMapSlots;
-      P.in_stale.push_back((uint32_t)r);
-      P.max_smem_stale = std::max(P.max_smem_stale, sb);
-    } else if (slots && slot_plan(p, tr, P.rcap_s[r], P.rcap_h[r], P.slot[r]) &&
-               unison_slots::slot_bytes(P.slot[r].nslots, tr->n_sessions, p.policy != UNISON_SPEAR_TIDE, true) <=
-                   slot_limit) {
+      if (P.slot[r].nslots) {
+        P.in_slot_stale.push_back((uint32_t)r);
+        P.smem_slot_stale = std::max(P.smem_slot_stale, slot_smem(p, tr, P.slot[r], false));
+      } else {
+        P.in_stale.push_back((uint32_t)r);
+        P.max_smem_stale = std::max(P.max_smem_stale, sb);
+      }
+    } else if (P.slot[r].nslots) {
       const bool lean_st = p.policy == UNISON_SPEAR_TIDE && p.max_sessions == 0 && !logged;
       (lean_st ? P.in_slot_st : P.in_slot_mix).push_back((uint32_t)r);
     } else if (lists <= smem_limit) {
-      P.slot[r].nslots = 0;
       P.in_list.push_back((uint32_t)r);
       P.max_smem_list = std::max<size_t>(P.max_smem_list, lists + (P.tmap[r] == kMapSlots ? map : 0));
     } else {
-      P.slot[r].nslots = 0;
       P.tmap[r] = kMapNone;
       P.in_glist.push_back((uint32_t)r);
       P.off_glist[r] = off;
@@ -1682,7 +1693,7 @@ int plan_replays(const unison_trace *const *traces, const unison_replay_params *
     P.off_ttft[r] = off;
     off = align_up(off + 8 * (tr->n_turns + 1), 256);
     const int c = P.replay_combo[r];
-    if (c >= 0 && p.policy != UNISON_LRU_TIDE) {
+    if (c >= 0 && p.policy != UNISON_LRU_TIDE && !(P.slot[r].nslots && (p.flags & UNISON_HAZARD_ONLINE))) {
       if (P.slot[r].nslots) P.need_rank[c] = 1;
       else P.need_keys[c] = 1;
     }
@@ -1697,7 +1708,7 @@ int plan_replays(const unison_trace *const *traces, const unison_replay_params *
     // gap averages; keys after and before each event; ranks and the sort's two buffers
     if (P.need_keys[c]) off += align_up(12 * E, 8) + 8 * E;
     else off += align_up(4 * E, 8);
-    if (P.need_rank[c]) off += align_up(4 * E, 8) + 16 * (tr->n_turns - tr->n_sessions);
+    if (P.need_rank[c]) off += align_up(4 * rank_entries(P, c, tr), 8) + 16 * rank_values(P, c, tr);
     off = align_up(off, 256);
   }
   if (!P.in_list.empty())
@@ -1750,11 +1761,11 @@ void fill_descs(const unison_trace *const *traces, const unison_replay_params *p
     d.rk = unison_slots::RankDesc{};
     if (P.need_rank[c]) {
       d.rk.rank = reinterpret_cast<uint32_t *>(q);
-      q += align_up(4 * E, 8);
-      d.rk.n = (uint32_t)(tr->n_turns - tr->n_sessions);
+      q += align_up(4 * rank_entries(P, c, tr), 8);
+      d.rk.n = (uint32_t)rank_values(P, c, tr);
+      d.rk.all = std::get<6>(P.combos[c]) ? 1u : 0u;
       d.rk.a = reinterpret_cast<unsigned long long *>(q);
       d.rk.b = d.rk.a + d.rk.n;
-      d.rk.turn_ev = d.turn_ev;
     }
   }
   hd.resize(n_replays);
@@ -1798,7 +1809,7 @@ void fill_descs(const unison_trace *const *traces, const unison_replay_params *p
     d.slot.rank = P.replay_combo[r] >= 0 ? hc[P.replay_combo[r]].rk.rank : nullptr;
   }
   order.clear();
-  for (const auto *g : {&P.in_slot_st, &P.in_slot_mix, &P.in_list, &P.in_glist, &P.in_online, &P.in_stale})
+  for (const auto *g : {&P.in_slot_st, &P.in_slot_mix, &P.in_slot_online, &P.in_slot_stale, &P.in_list, &P.in_glist, &P.in_online, &P.in_stale})
     order.insert(order.end(), g->begin(), g->end());
   // A launch lasts as long as its slowest replay, and CTAs start in index
   // order: the SPEAR+TIDE launch takes its replays by predicted cost,
@@ -1814,7 +1825,7 @@ void fill_descs(const unison_trace *const *traces, const unison_replay_params *p
 // Side streams for the replay groups of one call, one set per device, made
 // on first use.  The caller holds the lock while it forks and joins, so two
 // host threads never interleave their events.
-constexpr int kSideStreams = 5;
+constexpr int kSideStreams = 7;
 struct SideStreams {
   cudaStream_t s[kSideStreams] = {};
   cudaEvent_t fork = nullptr, join[kSideStreams] = {};
@@ -1895,6 +1906,8 @@ int launch_replays(const ReplayPlan &P, char *scratch, const std::vector<ComboDe
     const Launch all[] = {
         {slot_kernel_of(true, map8(P.in_slot_st)), P.in_slot_st.size(), P.smem_slot_st},
         {slot_kernel_of(false, map8(P.in_slot_mix)), P.in_slot_mix.size(), P.smem_slot_mix},
+        {slot_variant_kernel<unison_slots::kOnline>, P.in_slot_online.size(), P.smem_slot_online},
+        {slot_variant_kernel<unison_slots::kStale>, P.in_slot_stale.size(), P.smem_slot_stale},
         {replay_kernel<false, kKeyStream>, P.in_list.size(), P.max_smem_list},
         {replay_kernel<true, kKeyStream>, P.in_glist.size(), 0},
         {replay_kernel<false, kKeyOnline>, P.in_online.size(), P.max_smem_online},

@@ -25,6 +25,15 @@
 // took 375 and 1,513 (49.2 ms).  Tried and not kept: the words' extremes found
 // at the top of every event, beside the session's lookup (185 instructions,
 // sweep 32.5 -> 34.3 ms); 256 words loaded at once (34.0 ms).
+//
+// Two variants keep a second array of words.  A stale-snapshot replay ranks by
+// the snapshot's ranks and keeps the live ones beside them, so a choice is
+// compared with the live one by a second pass and a sync rewrites the words of
+// the sessions that changed, a lane each (16 replays over the four sync modes
+// 151 -> 55 ms).  Under the online hazard table keys change while sessions are
+// resident, so a word is the key itself in 64 bits, and a rebuilt table rewrites
+// every word in place where sorted lists had to be sorted again (6 online, 6
+// offline and 6 LRU replays with logs 116 -> 51 ms).
 #pragma once
 
 #include "common.cuh"
@@ -88,11 +97,22 @@ __host__ inline size_t slot_bytes(uint32_t nslots, uint32_t n_sessions, bool wid
   const size_t map = ((size_t)n_sessions * (map8 ? 1 : 2) + 15) / 16 * 16;
   return slot_words(nslots) * 4 + (pay + 15) / 16 * 16 + fr + map;
 }
+// Beside those: a second array of words; a stale replay's live and snapshot
+// ranks of every session and the sessions changed since the last sync; an
+// online replay's arrivals of every session and its table.
+constexpr uint32_t kDirtySlots = 64;
+__host__ __device__ inline size_t round16(size_t b) { return (b + 15) / 16 * 16; }
+
+// Where a replay's ranking comes from.
+constexpr int kRanked = 0;  // ranks of the key stream, or recency
+constexpr int kStale = 1;   // ranks of a register-file snapshot (eq. stale)
+constexpr int kOnline = 2;  // keys under the online hazard table (Sec. V-F)
 
 // The replay's state.  kLean: no decision log and no slot limit.
-template <bool kLean, bool kWide>
+template <int kMode, bool kLean, bool kWide>
 struct Slots {
   uint32_t *W;
+  uint32_t *L;            // kStale: the words by live ranks; kOnline: the words' low halves
   Payload<kWide> *P;
   uint16_t *F;            // freed slots, a stack
   uint32_t nfree, fresh;  // entries of F; slots handed out at least once
@@ -102,58 +122,49 @@ struct Slots {
   int status;
   // decision stream: event, hash (two halves), log
   uint32_t e, h_lo, h_hi;
-  uint64_t log_len, log_cap;
-  unison_decision *log;
+  uint2 *log;         // the next entry
+  uint64_t log_left;  // entries left (0 without a log)
   // counters (warp-uniform registers); those of arrivals come from the notes
   uint32_t n_evict, n_demote, n_promote, n_tide_demote, n_expire, n_tide_calls, n_res;
+  uint32_t vict_n, vict_diff, prom_n, prom_diff;  // kStale: choices, and those unlike the live one
 };
 
 // h = (h ^ (event << 32 | kind << 24 | session)) * 0x100000001B3 mod 2^64.
-template <bool kLean, bool kWide>
-__device__ __forceinline__ void decide(Slots<kLean, kWide> &st, uint32_t kind, uint32_t s, int lane) {
+template <int kMode, bool kLean, bool kWide>
+__device__ __forceinline__ void decide(Slots<kMode, kLean, kWide> &st, uint32_t kind, uint32_t s, int lane) {
   static_assert(kFnvPrime == (1ull << 40 | 0x1B3u), "the multiplication below");
   const uint32_t lo = st.h_lo ^ (s | kind << 24), hi = st.h_hi ^ st.e;
   const uint64_t m = (uint64_t)lo * 0x1B3u;
   st.h_lo = (uint32_t)m;
   st.h_hi = (uint32_t)(m >> 32) + hi * 0x1B3u + (lo << 8);
   if constexpr (!kLean) {
-    if (st.log) {
-      if (st.log_len < st.log_cap) {
-        if (lane == 0) {
-          unison_decision d;
-          d.event = st.e;
-          d.kind_session = (kind << 24) | s;
-          st.log[st.log_len] = d;
-        }
-      } else if (st.status == UNISON_OK) {
-        st.status = UNISON_ERR_LOG_FULL;
-      }
+    static_assert(sizeof(unison_decision) == sizeof(uint2), "a log entry: event, kind << 24 | session");
+    if (st.log_left) {
+      *st.log++ = make_uint2(st.e, kind << 24 | s);  // (every lane the same)
+      st.log_left--;
     }
-    st.log_len++;
   }
 }
 
 // Extremes over the words of every slot handed out so far (a multiple of 128
 // words; the words past them are 0).
-template <class St>
-__device__ __forceinline__ uint32_t max_word(const St &st, int lane) {
-  const uint4 *w4 = reinterpret_cast<const uint4 *>(st.W) + lane;
+__device__ __forceinline__ uint32_t max_of(const uint32_t *W, uint32_t fresh, int lane) {
+  const uint4 *w4 = reinterpret_cast<const uint4 *>(W) + lane;
   uint4 v = w4[0];
   uint32_t m = max(max(v.x, v.y), max(v.z, v.w));
-  for (uint32_t q = 128; q < st.fresh; q += 128) {
+  for (uint32_t q = 128; q < fresh; q += 128) {
     w4 += 32;
     v = *w4;
     m = max(max(m, max(v.x, v.y)), max(v.z, v.w));
   }
   return __reduce_max_sync(kAll, m);
 }
-// The largest HBM word with its tier bit flipped: > kFastBit if there is one.
-template <class St>
-__device__ __forceinline__ uint32_t max_hbm(const St &st, int lane) {
-  const uint4 *w4 = reinterpret_cast<const uint4 *>(st.W) + lane;
+// The largest word with the tier bit flipped: > kFastBit if there is an HBM word.
+__device__ __forceinline__ uint32_t max_hbm_of(const uint32_t *W, uint32_t fresh, int lane) {
+  const uint4 *w4 = reinterpret_cast<const uint4 *>(W) + lane;
   uint4 v = w4[0];
   uint32_t m = max(max(v.x ^ kFastBit, v.y ^ kFastBit), max(v.z ^ kFastBit, v.w ^ kFastBit));
-  for (uint32_t q = 128; q < st.fresh; q += 128) {
+  for (uint32_t q = 128; q < fresh; q += 128) {
     w4 += 32;
     v = *w4;
     m = max(max(m, max(v.x ^ kFastBit, v.y ^ kFastBit)), max(v.z ^ kFastBit, v.w ^ kFastBit));
@@ -162,13 +173,12 @@ __device__ __forceinline__ uint32_t max_hbm(const St &st, int lane) {
 }
 // The largest word, and the smallest word above 0 less 1 (below
 // kFastBit - 1 if there is an HBM word).
-template <class St>
-__device__ __forceinline__ void extremes(const St &st, uint32_t &mx, uint32_t &mn, int lane) {
-  const uint4 *w4 = reinterpret_cast<const uint4 *>(st.W) + lane;
+__device__ __forceinline__ void extremes_of(const uint32_t *W, uint32_t fresh, uint32_t &mx, uint32_t &mn, int lane) {
+  const uint4 *w4 = reinterpret_cast<const uint4 *>(W) + lane;
   uint4 v = w4[0];
   uint32_t a = max(max(v.x, v.y), max(v.z, v.w));
   uint32_t b = min(min(v.x - 1u, v.y - 1u), min(v.z - 1u, v.w - 1u));
-  for (uint32_t q = 128; q < st.fresh; q += 128) {
+  for (uint32_t q = 128; q < fresh; q += 128) {
     w4 += 32;
     v = *w4;
     a = max(max(a, max(v.x, v.y)), max(v.z, v.w));
@@ -178,12 +188,176 @@ __device__ __forceinline__ void extremes(const St &st, uint32_t &mx, uint32_t &m
   mn = __reduce_min_sync(kAll, b);
 }
 
+// The online table's keys change while sessions are resident, so a word holds
+// the key itself: W a tier bit, a 1 and the key's upper 23 bits, L its lower
+// 17 bits and the inverted session (15 bits, larger key and smaller id first).
+// A completed session's maximal key is 2^39 here; live keys are below it.
+constexpr uint32_t kOnlineLive = 0x40000000u;
+constexpr uint32_t kOnlineIds = 0x7FFFu;
+__device__ __forceinline__ uint64_t online_word(uint64_t key, uint32_t s) {
+  return ((uint64_t)(kOnlineLive | (uint32_t)(key >> 17)) << 32) | ((uint32_t)key << 15) | (kOnlineIds - s);
+}
+// The most evictable word once W ^ flip (the wanted tier's words then have the
+// top bit), as W ^ flip and L.  The least evictable HBM word comes as W ^
+// kOnlineLive and L (the first below kOnlineLive if there is one).
+__device__ __forceinline__ uint64_t online_max(const uint32_t *W, const uint32_t *L, uint32_t fresh, uint32_t flip,
+                                               int lane) {
+  uint64_t m = 0;
+  for (uint32_t i = 4 * lane, q = 0; q == 0 || q < fresh; q += 128, i += 128) {
+    const uint4 w = *reinterpret_cast<const uint4 *>(W + i), l = *reinterpret_cast<const uint4 *>(L + i);
+    const uint64_t a = max((uint64_t)(w.x ^ flip) << 32 | l.x, (uint64_t)(w.y ^ flip) << 32 | l.y);
+    const uint64_t b = max((uint64_t)(w.z ^ flip) << 32 | l.z, (uint64_t)(w.w ^ flip) << 32 | l.w);
+    m = max(m, max(a, b));
+  }
+  const uint32_t hi = __reduce_max_sync(kAll, (uint32_t)(m >> 32));
+  return (uint64_t)hi << 32 | __reduce_max_sync(kAll, (uint32_t)(m >> 32) == hi ? (uint32_t)m : 0u);
+}
+// Both at once: the most evictable fast-tier word and the least evictable HBM one.
+__device__ __forceinline__ void online_ends(const uint32_t *W, const uint32_t *L, uint32_t fresh, uint64_t &top,
+                                            uint64_t &low, int lane) {
+  uint64_t m = 0, n = ~0ull;
+  for (uint32_t i = 4 * lane, q = 0; q == 0 || q < fresh; q += 128, i += 128) {
+    const uint4 w = *reinterpret_cast<const uint4 *>(W + i), l = *reinterpret_cast<const uint4 *>(L + i);
+    constexpr uint32_t x = kOnlineLive;
+    m = max(m, max(max((uint64_t)w.x << 32 | l.x, (uint64_t)w.y << 32 | l.y),
+                   max((uint64_t)w.z << 32 | l.z, (uint64_t)w.w << 32 | l.w)));
+    n = min(n, min(min((uint64_t)(w.x ^ x) << 32 | l.x, (uint64_t)(w.y ^ x) << 32 | l.y),
+                   min((uint64_t)(w.z ^ x) << 32 | l.z, (uint64_t)(w.w ^ x) << 32 | l.w)));
+  }
+  const uint32_t hi = __reduce_max_sync(kAll, (uint32_t)(m >> 32)), lo = __reduce_min_sync(kAll, (uint32_t)(n >> 32));
+  top = (uint64_t)hi << 32 | __reduce_max_sync(kAll, (uint32_t)(m >> 32) == hi ? (uint32_t)m : 0u);
+  low = (uint64_t)lo << 32 | __reduce_min_sync(kAll, (uint32_t)(n >> 32) == lo ? (uint32_t)n : kAll);
+}
+
+// The table of the sessions completed so far (eqs. (hazard), (hq), (survq),
+// (t2) with bucket pooling), in shared memory.
+struct OnlineTable {
+  uint32_t n[kLutN], d[kLutN], sig[kLutN];
+  unsigned long long t2[kLutN];
+  unsigned long long mg[kLutN];  // magic_for(sig): eq. (t1)'s division by a multiply-high
+};
+__device__ __forceinline__ void online_init(OnlineTable &ot, int lane) {
+  for (uint32_t t = lane; t < kLutN; t += 32) {
+    ot.n[t] = ot.d[t] = 0u;
+    ot.sig[t] = kLambda;  // no session completed: zero hazard
+    ot.t2[t] = 0ull;
+    ot.mg[t] = magic_for(kLambda);
+  }
+}
+// A score under the table; g < 2^31 (gaps are clamped below 2^31 us), so g *
+// Lambda < 2^43.
+__device__ __forceinline__ uint64_t online_score(const OnlineTable &ot, uint32_t g, uint32_t t) {
+  const uint32_t tt = t < kTMax ? t : kTMax;
+  return __umul64hi((uint64_t)g * kLambda, ot.mg[tt]) + ot.t2[tt];
+}
+// A session of `turns` turns has completed: add it to the counts and rebuild
+// sigma and T2 for every turn index.  With at most 32,768 sessions the pooled
+// counts are below 2^15 (d) and 2^21 (n), so the quotient's terms fit 32 bits.
+// True if an entry changed.
+__device__ __noinline__ bool online_add(OnlineTable &ot, uint32_t turns, uint32_t bucket, uint64_t penalty, int lane) {
+  for (uint32_t t = lane; t < kLutN; t += 32) {
+    ot.n[t] += turns >= t + 1 ? 1u : 0u;
+    ot.d[t] += turns == t + 1 ? 1u : 0u;
+  }
+  __syncwarp();
+  bucket = min(bucket, kLutN);
+  bool changed = false;
+  uint32_t sg[2];
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    const uint32_t t = lane + 32 * q;
+    sg[q] = kLambda;
+    if (t < kLutN) {
+      const uint32_t u0 = t - t % bucket, u1 = min(u0 + bucket, kLutN);
+      uint32_t nn = 0, dd = 0;
+      for (uint32_t u = u0; u < u1; u++) {
+        nn += ot.n[u];
+        dd += ot.d[u];
+      }
+      const uint32_t hq = nn ? min((2u * dd * kLambda + nn) / (2u * nn), kLambda) : 0u;
+      sg[q] = max(kLambda - hq, kEpsQ);
+      changed |= ot.sig[t] != sg[q];
+    }
+  }
+  changed = __any_sync(kAll, changed);  // T2 and the divisors follow from sigma
+  if (!changed) return false;
+#pragma unroll
+  for (int q = 0; q < 2; q++) {
+    const uint32_t t = lane + 32 * q;
+    if (t < kLutN && ot.sig[t] != sg[q]) {
+      ot.sig[t] = sg[q];
+      ot.t2[t] = ((unsigned long long)(kLambda - sg[q]) * penalty) / kLambda;
+      ot.mg[t] = magic_for(sg[q]);
+    }
+  }
+  __syncwarp();
+  return true;
+}
+
+// A choice among the residents: whether there is one, its slot, and a value
+// that orders choices of either tier (larger: more evictable).
+struct Choice {
+  bool any;
+  uint32_t slot;
+  uint64_t order;
+};
+template <int kMode, bool kLean, bool kWide>
+__device__ __forceinline__ Choice most_evictable_fast(const Slots<kMode, kLean, kWide> &st, const uint16_t *map,
+                                                      int lane) {
+  if constexpr (kMode == kOnline) {
+    const uint64_t m = online_max(st.W, st.L, st.fresh, 0u, lane);
+    const bool any = m >> 63 != 0;
+    return {any, any ? map[kOnlineIds - ((uint32_t)m & kOnlineIds)] : 0u, m & ~(1ull << 63)};
+  } else {
+    const uint32_t w = max_of(st.W, st.fresh, lane);
+    return {(w & kFastBit) != 0, w & st.smask, w & ~kFastBit};
+  }
+}
+template <int kMode, bool kLean, bool kWide>
+__device__ __forceinline__ Choice most_evictable_hbm(const Slots<kMode, kLean, kWide> &st, const uint16_t *map,
+                                                     int lane) {
+  if constexpr (kMode == kOnline) {
+    const uint64_t m = online_max(st.W, st.L, st.fresh, kFastBit, lane);  // (an empty slot: kFastBit, 0)
+    const bool any = m > (1ull << 63);
+    return {any, any ? map[kOnlineIds - ((uint32_t)m & kOnlineIds)] : 0u, m & ~(1ull << 63)};
+  } else {
+    const uint32_t m = max_hbm_of(st.W, st.fresh, lane);
+    return {m > kFastBit, m & st.smask, m & ~kFastBit};
+  }
+}
+// The words of a choice in the other tier, or none.
+template <int kMode, bool kLean, bool kWide>
+__device__ __forceinline__ void set_word(Slots<kMode, kLean, kWide> &st, uint32_t slot, bool fast, uint64_t order) {
+  const uint32_t bit = fast ? kFastBit : 0u;
+  if constexpr (kMode == kOnline) {
+    st.W[slot] = (uint32_t)(order >> 32) | bit;
+    st.L[slot] = (uint32_t)order;
+  } else {
+    st.W[slot] = (uint32_t)order | bit;
+    if constexpr (kMode == kStale) st.L[slot] = (st.L[slot] & ~kFastBit) | bit;
+  }
+}
+template <int kMode, bool kLean, bool kWide>
+__device__ __forceinline__ void clear_word(Slots<kMode, kLean, kWide> &st, uint32_t slot) {
+  st.W[slot] = 0u;
+  if constexpr (kMode != kRanked) st.L[slot] = 0u;
+}
+
+// kStale: a choice (slot) against the live ranks' over the same sessions.
+template <int kMode, bool kLean, bool kWide>
+__device__ __forceinline__ void count_victim(Slots<kMode, kLean, kWide> &st, uint32_t slot, uint32_t live_word) {
+  if constexpr (kMode == kStale) {
+    st.vict_n++;
+    st.vict_diff += (live_word & st.smask) != slot;
+  }
+}
+
 // Slot stores: every lane stores the same value to the same place, so each
 // lane's later loads see it without a warp barrier; a __syncwarp separates a
 // store from the loads of the old value before it.
 template <class St>
 __device__ __forceinline__ void release_slot(St &st, uint32_t slot) {
-  st.W[slot] = 0u;
+  clear_word(st, slot);
   st.P[slot].v.y = kIdMask;  // no session has this id
   st.F[st.nfree] = (uint16_t)slot;
   st.nfree++;
@@ -197,19 +371,27 @@ __device__ __forceinline__ uint2 payload(const St &st, uint32_t slot) {
 }
 
 // Room in HBM for `size` tokens against its unpinned residents: evicts the
-// most evictable ones, only those above `floor_word` (a word without the tier
-// bit; 0 accepts every one).  False when the next one is not above it.
-template <class St>
-__device__ __forceinline__ bool make_hbm_room(St &st, uint32_t size, uint32_t floor_word, int lane) {
+// most evictable ones, only those above `d` (a session demoted out of the fast
+// tier; without one every resident is above).  False when the next one is not.
+template <int kMode, bool kLean, bool kWide>
+__device__ __forceinline__ bool make_hbm_room(Slots<kMode, kLean, kWide> &st, const uint16_t *map, uint32_t size,
+                                              const Choice &d, int lane) {
   while (size > st.free_h) {
-    const uint32_t m = max_hbm(st, lane);
-    if (m <= max(kFastBit, floor_word | kFastBit)) return false;
-    const uint32_t slot = m & st.smask;
-    const uint2 p = payload(st, slot);
+    const Choice v = most_evictable_hbm(st, map, lane);
+    const bool drop = !v.any || (d.any && d.order > v.order);
+    if constexpr (kMode == kStale) {
+      // the live choice: among HBM's sessions and the demoted one
+      uint32_t live = max_hbm_of(st.L, st.fresh, lane);
+      live = live > kFastBit ? live & ~kFastBit : 0u;
+      if (d.any) live = max(live, st.L[d.slot] & ~kFastBit);
+      count_victim(st, drop ? d.slot : v.slot, live);
+    }
+    if (drop) return false;
+    const uint2 p = payload(st, v.slot);
     st.free_h += p.x & kSizeBits;
     decide(st, UNISON_KIND_EVICT, p.y & kIdMask, lane);
     st.n_evict++;
-    release_slot(st, slot);
+    release_slot(st, v.slot);
   }
   return true;
 }
@@ -269,18 +451,28 @@ __device__ __forceinline__ void expire_slots(St &st, uint32_t now, uint32_t ttl,
 // of Algorithm 1 has it: phase 1 promotes the least evictable HBM sessions
 // into free fast-tier space, phase 2 swaps the least evictable HBM session
 // with the most evictable fast-tier one.  Returns the bytes moved.
-template <class St>
-__device__ __forceinline__ uint64_t tide_slots(St &st, uint64_t budget, uint32_t kvb, int lane) {
+template <int kMode, bool kLean, bool kWide>
+__device__ __forceinline__ uint64_t tide_slots(Slots<kMode, kLean, kWide> &st, const uint16_t *map, uint64_t budget,
+                                               uint32_t kvb, int lane) {
   uint64_t rem = budget;
   bool fill = true;  // phase 1
   for (;;) {
-    uint32_t mx, mn;
-    extremes(st, mx, mn, lane);
-    if (mn >= kFastBit - 1u) break;  // HBM holds no unpinned session
-    const uint32_t pw = mn + 1u, pslot = pw & st.smask;
-    const uint32_t dslot = mx & st.smask;  // a valid slot even when mx names none
-    const uint2 p = *reinterpret_cast<const uint2 *>(&st.P[pslot]);
-    const uint2 d = payload(st, dslot);
+    Choice pc, dc;  // the least evictable HBM session, the most evictable fast-tier one
+    if constexpr (kMode == kOnline) {
+      uint64_t top, low;
+      online_ends(st.W, st.L, st.fresh, top, low, lane);
+      const bool any = low >> 32 < kOnlineLive, fast = top >> 63 != 0;
+      pc = {any, any ? map[kOnlineIds - ((uint32_t)low & kOnlineIds)] : 0u, low | (uint64_t)kOnlineLive << 32};
+      dc = {fast, fast ? map[kOnlineIds - ((uint32_t)top & kOnlineIds)] : 0u, top & ~(1ull << 63)};
+    } else {
+      uint32_t mx, mn;
+      extremes_of(st.W, st.fresh, mx, mn, lane);
+      pc = {mn < kFastBit - 1u, (mn + 1u) & st.smask, mn + 1u};
+      dc = {(mx & kFastBit) != 0, mx & st.smask, mx & ~kFastBit};  // (a valid slot even when mx names none)
+    }
+    if (!pc.any) break;
+    const uint2 p = *reinterpret_cast<const uint2 *>(&st.P[pc.slot]);
+    const uint2 d = payload(st, dc.slot);
     const uint32_t sp = p.x & kSizeBits, pid = p.y & kIdMask;
     uint64_t by = (uint64_t)sp * kvb;
     fill = fill && by <= rem && sp <= st.free_s;
@@ -288,24 +480,36 @@ __device__ __forceinline__ uint64_t tide_slots(St &st, uint64_t budget, uint32_t
       // phase 2: the swap is legal and the demoted session the more evictable
       const uint32_t sd = d.x & kSizeBits, did = d.y & kIdMask;
       by += (uint64_t)sd * kvb;
-      const bool swap = (mx & kFastBit) != 0 && (mx & ~kFastBit) > pw && by <= rem && sp <= st.free_s + sd &&
-                        sd <= st.free_h + sp;
+      const bool swap = dc.any && dc.order > pc.order && by <= rem && sp <= st.free_s + sd && sd <= st.free_h + sp;
       if (!swap) break;
-      st.W[dslot] = mx & ~kFastBit;
-      st.P[dslot].v.y = did;
+      if constexpr (kMode == kStale) {
+        uint32_t mx, mn;
+        extremes_of(st.L, st.fresh, mx, mn, lane);
+        st.prom_n++;
+        st.prom_diff += ((mn + 1u) & st.smask) != pc.slot;
+        count_victim(st, dc.slot, mx);
+      }
+      set_word(st, dc.slot, false, dc.order);
+      st.P[dc.slot].v.y = did;
       st.free_s += sd;
       st.free_h -= sd;
       st.n_tide_demote++;
       decide(st, UNISON_KIND_PROMOTE, pid, lane);
       decide(st, UNISON_KIND_TIDE_DEMOTE, did, lane);
     } else {
+      if constexpr (kMode == kStale) {
+        uint32_t mx, mn;
+        extremes_of(st.L, st.fresh, mx, mn, lane);
+        st.prom_n++;
+        st.prom_diff += ((mn + 1u) & st.smask) != pc.slot;
+      }
       decide(st, UNISON_KIND_PROMOTE, pid, lane);
     }
     rem -= by;
     st.free_s -= sp;
     st.free_h += sp;
-    st.W[pslot] = pw | kFastBit;
-    *reinterpret_cast<uint2 *>(&st.P[pslot]) = make_uint2(p.x | kPromoted, pid | kFastBit);
+    set_word(st, pc.slot, true, pc.order);
+    *reinterpret_cast<uint2 *>(&st.P[pc.slot]) = make_uint2(p.x | kPromoted, pid | kFastBit);
     st.n_promote++;
   }
   return budget - rem;
@@ -316,17 +520,17 @@ __device__ __forceinline__ uint64_t tide_slots(St &st, uint64_t budget, uint32_t
 // few (each costs an issue slot and a fetch, and one warp hides neither):
 // classes and tiers are selected, and the loops that make room and migrate are
 // the only ones an ordinary event passes.
-template <int kPol, bool kLean, bool kMap8, class Desc>
+template <int kMode, int kPol, bool kLean, bool kMap8, class Desc>
 __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, SlotBufs &bufs, unsigned char *smem,
                                             int lane) {
   constexpr bool kWide = kPol != UNISON_SPEAR_TIDE;
   const uint32_t policy = kPol >= 0 ? (uint32_t)kPol : D.policy;
-  const bool spear = policy == UNISON_SPEAR || policy == UNISON_SPEAR_TIDE;
+  const bool spear = kMode != kRanked || policy == UNISON_SPEAR || policy == UNISON_SPEAR_TIDE;
   const bool tide_on = policy == UNISON_SPEAR_TIDE || policy == UNISON_LRU_TIDE;
-  const bool belady = policy == UNISON_BELADY;
-  const bool timeout = policy == UNISON_TIMEOUT && D.ttl != 0xFFFFFFFFu;
+  const bool belady = kMode == kRanked && policy == UNISON_BELADY;
+  const bool timeout = kMode == kRanked && policy == UNISON_TIMEOUT && D.ttl != 0xFFFFFFFFu;
 
-  Slots<kLean, kWide> st;
+  Slots<kMode, kLean, kWide> st;
   const uint32_t nslots = Q.nslots;
   st.sbits = Q.sbits;
   st.smask = (1u << Q.sbits) - 1u;
@@ -339,6 +543,31 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
   p += ((size_t)Q.nslots * 2 + 15) / 16 * 16;
   uint8_t *const map8 = p;
   uint16_t *const map16 = reinterpret_cast<uint16_t *>(p);
+  static_assert(kMode == kRanked || (!kMap8 && kPol < 0), "stale and online replays: SPEAR or SPEAR+TIDE, two-byte maps");
+  // kStale: every session's live and snapshot rank, sessions changed since the
+  // last sync; kOnline: every session's arrivals so far (saturating far above
+  // the table's last row), the table
+  uint32_t *live = nullptr, *snap = nullptr, *dirty = nullptr, n_dirty = 0, sync_arrivals = 0;
+  uint16_t *turns = nullptr;
+  OnlineTable *table = nullptr;
+  if constexpr (kMode != kRanked) {
+    unsigned char *q = p + round16((size_t)D.n_sessions * 2);
+    st.L = reinterpret_cast<uint32_t *>(q);
+    for (uint32_t i = lane; i < slot_words(Q.nslots); i += 32) st.L[i] = 0u;
+    q += slot_words(Q.nslots) * 4;
+    if constexpr (kMode == kStale) {
+      live = reinterpret_cast<uint32_t *>(q);
+      snap = live + D.n_sessions;
+      dirty = snap + D.n_sessions;
+      // a zero register row (gap average 0, turn 0, not done)
+      for (uint32_t i = lane; i < D.n_sessions; i += 32) live[i] = snap[i] = Q.rank[D.n_events + i] + 1u;
+    } else {
+      table = reinterpret_cast<OnlineTable *>(q);
+      turns = reinterpret_cast<uint16_t *>(q + round16(sizeof(OnlineTable)));
+      for (uint32_t i = lane; i < D.n_sessions; i += 32) turns[i] = 0;
+      online_init(*table, lane);
+    }
+  }
   {
     uint4 *w4 = reinterpret_cast<uint4 *>(st.W);
     for (uint32_t i = lane; i < slot_words(Q.nslots) / 4; i += 32) w4[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -359,11 +588,11 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
   st.status = UNISON_OK;
   st.h_lo = (uint32_t)kFnvOffset;
   st.h_hi = (uint32_t)(kFnvOffset >> 32);
-  st.log = D.log;
-  st.log_cap = D.log_cap;
-  st.log_len = 0;
+  st.log = reinterpret_cast<uint2 *>(D.log);
+  st.log_left = D.log ? D.log_cap : 0;
   st.n_evict = st.n_demote = st.n_promote = st.n_tide_demote = st.n_expire = st.n_tide_calls = 0;
   st.n_res = 0;
+  st.vict_n = st.vict_diff = st.prom_n = st.prom_diff = 0;
   uint64_t dma_bytes = 0;
   uint32_t n_done = 0;
   const uint32_t n_turns = D.n_turns;
@@ -381,8 +610,8 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
     if (i < E) {
       SlotEvent &d = bufs.e[i & (kRing - 1)];
       async16(&d.ev, &D.ev[i]);
-      if (spear) async4(&d.aux.x, &Q.rank[i]);
-      if (tide_on) async4(&d.aux.y, &D.gq[i]);
+      if (spear && kMode != kOnline) async4(&d.aux.x, &Q.rank[i]);
+      if (tide_on || kMode == kOnline) async4(&d.aux.y, &D.gq[i]);
       if (belady) async4(&d.aux.z, &D.nref[i]);
     }
     async_commit();
@@ -432,7 +661,7 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
         decide(st, cls, s, lane);
         uint32_t note = cls | (pl.x >> 31) * kNotePromoted;  // (the bit counts for fast-tier hits only)
         if (found) {
-          st.W[slot] = 0u;
+          clear_word(st, slot);
           st.free_s += fast ? size : 0u;
           st.free_h += fast ? 0u : size;
         }
@@ -447,34 +676,34 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
           tier = 2;
         } else if (n <= st.room_s) {
           while (n > st.free_s) {
-            const uint32_t w = max_word(st, lane);  // the most evictable unpinned fast-tier session
-            if (w < kFastBit) {
+            const Choice c = most_evictable_fast(st, map16, lane);
+            if (!c.any) {
               st.status = UNISON_ERR_CAPACITY;
               break;
             }
+            if constexpr (kMode == kStale) count_victim(st, c.slot, max_of(st.L, st.fresh, lane));
             // it is demoted into HBM, displacing more evictable sessions
             // there, or dropped
-            const uint32_t ds = w & st.smask, hw = w & ~kFastBit;
-            const uint2 d = payload(st, ds);
+            const uint2 d = payload(st, c.slot);
             const uint32_t sd = d.x & kSizeBits, did = d.y & kIdMask;
             st.free_s += sd;
-            const bool keep = sd <= st.room_h && make_hbm_room(st, sd, hw, lane);
+            const bool keep = sd <= st.room_h && make_hbm_room(st, map16, sd, c, lane);
             decide(st, keep ? (uint32_t)UNISON_KIND_DEMOTE : (uint32_t)UNISON_KIND_EVICT, did, lane);
             if (keep) {
-              st.W[ds] = hw;
-              st.P[ds].v.y = did;
+              set_word(st, c.slot, false, c.order);
+              st.P[c.slot].v.y = did;
               st.free_h -= sd;
               st.n_demote++;
             } else {
               st.n_evict++;
-              release_slot(st, ds);
+              release_slot(st, c.slot);
             }
           }
           st.free_s -= n;
           st.room_s -= n;
         } else if (n <= st.room_h) {
           tier = 1;
-          if (!make_hbm_room(st, n, 0u, lane)) st.status = UNISON_ERR_CAPACITY;
+          if (!make_hbm_room(st, map16, n, Choice{false, 0u, 0ull}, lane)) st.status = UNISON_ERR_CAPACITY;
           st.free_h -= n;
           st.room_h -= n;
         } else {
@@ -514,14 +743,16 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
           if (!kLean && max_sessions) {
             while (st.n_res > max_sessions) {
               // the most evictable of both tiers
-              uint32_t m = 0;
-              for (uint32_t i = lane; i < st.fresh; i += 32) m = max(m, st.W[i] & ~kFastBit);
-              m = __reduce_max_sync(kAll, m);
-              if (m == 0) {
+              const Choice f = most_evictable_fast(st, map16, lane), h = most_evictable_hbm(st, map16, lane);
+              if (!f.any && !h.any) {
                 st.status = UNISON_ERR_CAPACITY;
                 break;
               }
-              const uint32_t vs = m & st.smask, vw = st.W[vs];
+              const uint32_t vs = f.any && (!h.any || f.order > h.order) ? f.slot : h.slot, vw = st.W[vs];
+              if constexpr (kMode == kStale) {
+                const uint32_t lh = max_hbm_of(st.L, st.fresh, lane), lf = max_of(st.L, st.fresh, lane);
+                count_victim(st, vs, max(lh > kFastBit ? lh & ~kFastBit : 0u, lf & kFastBit ? lf & ~kFastBit : 0u));
+              }
               const uint2 v = payload(st, vs);
               const uint32_t sv = v.x & kSizeBits;
               st.free_s += vw & kFastBit ? sv : 0u;
@@ -537,6 +768,11 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
           release_slot(st, slot);
         }
         *note_out++ = (uint8_t)(note | tier << kNotePlaceShift);  // (every lane the same byte)
+        if constexpr (kMode == kOnline) {
+          const uint32_t k = turns[s];
+          __syncwarp();
+          turns[s] = (uint16_t)(k < 0xFFFFu ? k + 1 : k);
+        }
       } else {
         // completion: the session is unpinned (if resident) with its new rank
         n_done++;
@@ -544,16 +780,41 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
         busy_us += (uint32_t)(now - last_done);
         last_done = now;
         if (found) {
-          uint32_t rk;
-          if (spear) rk = rec.aux.x + 1u;
-          else rk = n_turns - n_done + 1u;  // the later the touch, the less evictable
-          if constexpr (kWide) {
-            if (belady) rk = st.P[slot].v.z;
-            if (timeout) st.P[slot].v.w = now;
+          if constexpr (kMode == kOnline) {
+            const bool done = (w1 & kEvEdge) != 0;
+            const uint32_t g = rec.aux.y, t = (uint32_t)turns[s] - 1u;
+            st.P[slot].v.z = g;
+            st.P[slot].v.w = done ? kAll : t;  // a completed session keeps the maximal key
+            set_word(st, slot, fast, online_word(done ? 1ull << 39 : online_score(*table, g, t), s));
+          } else {
+            uint32_t rk;
+            if (kMode == kStale) rk = snap[s];  // residents rank by their snapshot rows
+            else if (spear) rk = rec.aux.x + 1u;
+            else rk = n_turns - n_done + 1u;  // the later the touch, the less evictable
+            if constexpr (kWide) {
+              if (belady) rk = st.P[slot].v.z;
+              if (timeout) st.P[slot].v.w = now;
+            }
+            st.W[slot] = rk << st.sbits | slot | (pl.y & kFastBit);
+            if constexpr (kMode == kStale) st.L[slot] = (rec.aux.x + 1u) << st.sbits | slot | (pl.y & kFastBit);
           }
-          st.W[slot] = rk << st.sbits | slot | (pl.y & kFastBit);
           st.room_s += fast ? size : 0u;
           st.room_h += fast ? 0u : size;
+        }
+        if constexpr (kMode == kOnline) {
+          // Sec. V-F: the finished session's turn count joins the table, and
+          // every resident is ranked under the rebuilt one
+          if ((w1 & kEvEdge) && online_add(*table, turns[s], D.bucket, D.penalty, lane)) {
+            for (uint32_t i = lane; i < st.fresh; i += 32) {
+              const uint32_t w = st.W[i];
+              const uint4 v = st.P[i].v;
+              if (w == 0u || v.w == kAll) continue;
+              const uint64_t o = online_word(online_score(*table, v.z, v.w), v.y & kIdMask);
+              st.W[i] = (uint32_t)(o >> 32) | (w & kFastBit);
+              st.L[i] = (uint32_t)o;
+            }
+            __syncwarp();
+          }
         }
         if (tide_on && !(w1 & kEvEdge)) {
           // the DMA is free again from start + ceil(bytes / rate) us on, i.e.
@@ -562,10 +823,38 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
           const bool busy = busy_us >> 31 == 0 && (uint64_t)(uint32_t)busy_us * dma < busy_bytes;
           if (!busy) {
             st.n_tide_calls++;
-            busy_bytes = tide_slots(st, (uint64_t)rec.aux.y * dma, kvb, lane);  // (0 at rate 0: no budget)
+            busy_bytes = tide_slots(st, map16, (uint64_t)rec.aux.y * dma, kvb, lane);  // (0 at rate 0: no budget)
             dma_bytes += busy_bytes;
             busy_us = 0;
           }
+        }
+      }
+      if constexpr (kMode == kStale) {
+        live[s] = rec.aux.x + 1u;
+        __syncwarp();
+        if (n_dirty < kDirtySlots) dirty[n_dirty] = s;
+        n_dirty++;
+        // a sync point copies every live row into the snapshot, after the
+        // event's own decisions: the rows changed since the last one, a lane
+        // each (a session noted twice is copied twice, alike), or all of them
+        bool sync = D.stale_sync == UNISON_SYNC_EVENT;
+        if ((w1 & kEvArrival) && D.stale_sync == UNISON_SYNC_ARRIVALS) sync = ++sync_arrivals % D.stale_m == 0;
+        if (!(w1 & kEvArrival) && D.stale_sync == UNISON_SYNC_GAP_START) sync = !(w1 & kEvEdge);
+        if (sync) {
+          __syncwarp();
+          if (n_dirty <= kDirtySlots) {
+            for (uint32_t i = lane; i < n_dirty; i += 32) {
+              const uint32_t d = dirty[i], r = live[d], at = map16[d];
+              snap[d] = r;
+              const uint32_t w = st.W[at];
+              if ((st.P[at].v.y & kIdMask) == d && w != 0u) st.W[at] = r << st.sbits | at | (w & kFastBit);
+            }
+          } else {
+            for (uint32_t i = lane; i < D.n_sessions; i += 32) snap[i] = live[i];
+            for (uint32_t i = lane; i < st.fresh; i += 32) st.W[i] = st.L[i];
+          }
+          __syncwarp();
+          n_dirty = 0;
         }
       }
     }
@@ -584,6 +873,14 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
     r.tide_calls = st.n_tide_calls;
     r.ttft_n = (uint64_t)(note_out - (reinterpret_cast<uint8_t *>(D.ttft) + 7ull * n_turns));
     r.decision_hash = (uint64_t)st.h_hi << 32 | st.h_lo;
+    r.vict_n = st.vict_n;
+    r.vict_diff = st.vict_diff;
+    r.prom_n = st.prom_n;
+    r.prom_diff = st.prom_diff;
+    if constexpr (!kLean) {
+      const uint64_t made = r.ttft_n * 2 + r.evict + r.demote + r.promote + r.tide_demote + r.expire;
+      if (D.log && made > D.log_cap && st.status == UNISON_OK) st.status = UNISON_ERR_LOG_FULL;
+    }
     r.status = st.status;
     *D.result = r;
   }
@@ -808,10 +1105,10 @@ constexpr int kSortWarps = kSortThreads / 32;
 constexpr size_t kSortSmem = sizeof(uint32_t) * kSortWarps * 256;
 
 struct RankDesc {
-  unsigned long long *a, *b;  // [n] values key40 << 24 | turn, and a second buffer
-  const uint32_t *turn_ev;    // [2T]
-  uint32_t *rank;             // [E]
+  unsigned long long *a, *b;  // [n] values key40 << 24 | entry of `rank`, and a second buffer
+  uint32_t *rank;             // [E], or [E + S] with every event's rank and the zero rows'
   uint32_t n;
+  uint32_t all;  // 1: ranks of every event's key and of the zero register rows (stale replays)
 };
 
 // Scratch of rank_keys_body beside the digit counts.
@@ -908,7 +1205,7 @@ __device__ void rank_keys_body(const RankDesc &d, uint32_t (*cnt)[256], SortShar
     src = dst;
     dst = t;
   }
-  for (uint32_t i = tid; i < n; i += kSortThreads) d.rank[d.turn_ev[2 * (uint32_t)(src[i] & 0xFFFFFFull) + 1]] = i;
+  for (uint32_t i = tid; i < n; i += kSortThreads) d.rank[(uint32_t)(src[i] & 0xFFFFFFull)] = i;
 }
 
 }  // namespace unison_slots

@@ -351,6 +351,23 @@ def test_slot_form_edges(B, n_sessions):
         assert_same(res[i], oracle.replay(tr, to_oracle(p)), (p["policy"], p["cap_s"], p["max_sessions"]))
 
 
+@pytest.mark.parametrize("n_sessions", [128, 129, 1700])
+def test_slot_form_variants(B, n_sessions):
+    """The online hazard table and stale snapshots with every session resident
+    and with tight tiers, beside one pass of 128 slots and near the most
+    sessions their shared-memory limit takes unbounded: syncs so far apart that
+    more sessions change than a sync updates one by one, a pooled hazard table,
+    a slot limit, SPEAR without TIDE."""
+    tr = synth.make_trace(33, np.full(n_sessions, 4), 0.01, synth.GAP_MIX_CODING)
+    kws = [dict(online=True), dict(online=True, bucket=60), dict(online=True, max_sessions=60), dict(stale="event"),
+           dict(stale="arrivals", stale_m=100), dict(stale="gap_start", max_sessions=60), dict(stale="arrivals", stale_m=7)]
+    reps = [(0, base(pol, cs, ch, 28672, **kw)) for cs, ch in ((1 << 60, 1 << 60), (256 * MIB, 1 << 60), (1 * GIB, 4 * GIB))
+            for pol in ("spear", "spear_tide") for kw in kws]
+    res, _, _ = run_gpu(B, [tr], reps)
+    for i, (_, p) in enumerate(reps):
+        assert_same(res[i], oracle.replay(tr, to_oracle(p)), (p["policy"], p["cap_s"], p["stale"], p["online"]))
+
+
 def test_slot_form_one_byte_map(B):
     """130,000 sessions: two bytes of session map do not fit in shared memory,
     so a one-byte entry names several of the replay's slots (about 900) and

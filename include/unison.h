@@ -458,8 +458,8 @@ typedef struct {
  * is more evictable).  Results are exact: candidate thresholds come from a
  * sample, and a set whose candidates fall short is re-selected exactly on
  * the device.  sets, params, outs: host arrays [n_sets].  Asynchronous: the
- * call queues one upload of its descriptors and one cooperative kernel on
- * cuda_stream (every CTA of the grid resident at once; each set is ranked
+ * call queues one cooperative kernel on cuda_stream, after one upload of its
+ * descriptors when it has several sets (every CTA of the grid resident at once; each set is ranked
  * by a group of CTAs, or, with more sets than resident CTAs, each CTA takes
  * whole sets in turn).  Any n_sets >= 0 that fits in memory is accepted.
  * Memory: the call's device scratch (about 1.7 MB per set) is kept per

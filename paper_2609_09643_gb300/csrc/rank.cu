@@ -28,15 +28,14 @@
 //            the CTA's own region, which moves into the set's list when the
 //            CTA is done.
 //   finish   the last three CTAs of the group to finish streaming take one
-//            list each: a 256-bucket cut below the candidates' common prefix
-//            keeps the bucket holding the rank-M value and those above it,
-//            which are bucket-sorted and the first M kept; a list whose cut
-//            holds too many values falls back to a radix select, and one
-//            whose candidates overflowed or fell short is re-selected exactly
-//            by streaming the set.  The last list's CTA runs the fill, 256
+//            list each: cuts into 256 buckets below the common prefix narrow the
+//            candidates to few beyond the first M, which are sorted and the
+//            first M kept; a list whose candidates overflowed or fell short is
+//            re-selected exactly by streaming the set.  The last list's CTA runs the fill, 256
 //            items at a time, and writes the outputs.
-// The work words and sample histograms of a call are held twice: calls on a
-// stream alternate between the two, and each call zeroes the other.
+// The work words and sample histograms lie in one of two blocks: calls on a
+// stream alternate between them, and each call zeroes what the one before it
+// used.
 // Every wait on another CTA or on a copy is bounded: a wait that gives up
 // records UNISON_ERR_TIMEOUT in the set's status word and the CTA carries on
 // to the end of the kernel.  A cooperative launch keeps every CTA of the grid
@@ -44,6 +43,7 @@
 #include <algorithm>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -346,8 +346,9 @@ struct FilterScratch {
   uint16_t wbuf[kConsumers / 32][kWarpBuf];
 };
 struct SelectScratch {
+  unsigned long long split[256];  // the splitter sort's splitters
   unsigned int hist[256];
-  unsigned int off[256];  // the bucket sort's bucket starts
+  unsigned int off[256];  // the bucket sorts' bucket starts
   unsigned int pick[2];
   unsigned long long bcast[2];
   unsigned int cnt;
@@ -387,6 +388,16 @@ __device__ __forceinline__ uint32_t bin_floor(uint32_t b) {
   if (b >= 2048u) return 0x80000000u | ((b - 2048u) << 13);
   const uint32_t e = b / 64u, m = b % 64u;
   return e < 6u ? m : (64u + m) << (e - 6u);
+}
+// The same per list.  P's values fall as keys rise, and its wanted ones are the
+// smallest keys, which the octaves from the top would leave in one bin: its
+// summaries are binned by their distance from the top, i.e. by octaves of the
+// key.  (Key 0 has the flagged summaries, by index.)
+__device__ __forceinline__ uint32_t list_bin(uint32_t f, int L) {
+  return L != 2 || (f & 0x80000000u) ? bin_of(f) : 1983u - bin_of(0x7FFFFFFFu - f);
+}
+__device__ __forceinline__ uint32_t list_bin_floor(uint32_t b, int L) {
+  return L != 2 || b >= 2048u ? bin_floor(b) : 0x7FFFFFFFu - (bin_floor(1984u - b) - 1u);
 }
 
 // Value with the given rank (1 = largest) among get(0..n-1), 64-bit values,
@@ -531,114 +542,6 @@ __device__ void hist_cut3(unsigned int *hist, const uint32_t (&need)[kLists], in
   for (int L = 0; L < kLists; L++) cut[L] = scut[L];
 }
 
-// Sort, descending, of a[0..n) padded with zeros to a power of two p >= 64
-// (bitonic network in shared memory), carrying pay[] along when given.
-// Stages whose partners lie less than 64 apart run warp by warp (each warp
-// owns blocks of 64 entries), with a warp barrier; the wider stages pair
-// entries across the array and take a block barrier.
-__device__ void bitonic_sort_desc(uint64_t *a, uint32_t n, uint32_t *pay = nullptr) {
-  if (n <= 1) return;
-  uint32_t p = 64;
-  while (p < n) p <<= 1;
-  for (uint32_t i = n + threadIdx.x; i < p; i += kConsumers) {
-    a[i] = 0;
-    if (pay) pay[i] = 0;
-  }
-  consumers_sync();
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  auto cmpx = [&](uint32_t x, uint32_t y, bool desc) {
-    const uint64_t u = a[x], v = a[y];
-    if ((u < v) == desc) {
-      a[x] = v;
-      a[y] = u;
-      if (pay) {
-        const uint32_t t = pay[x];
-        pay[x] = pay[y];
-        pay[y] = t;
-      }
-    }
-  };
-  for (uint32_t k = 2; k <= p; k <<= 1) {
-    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      if (j >= 64) {
-        for (uint32_t i = threadIdx.x; i < p / 2; i += kConsumers) {
-          const uint32_t x = ((i & ~(j - 1)) << 1) | (i & (j - 1));
-          cmpx(x, x + j, (x & k) == 0);
-        }
-        consumers_sync();
-      } else {
-        // block b (64 entries) is warp b % 8's; lane l takes pair l of it
-        for (uint32_t b = warp; b < p / 64; b += kConsumers / 32) {
-          const uint32_t x = 64 * b + (((lane & ~(j - 1)) << 1) | (lane & (j - 1)));
-          cmpx(x, x + j, (x & k) == 0);
-        }
-        __syncwarp();
-      }
-    }
-    // the next level opens with a stride of k: across blocks once k >= 64
-    if (k < p && k >= 64) consumers_sync();
-  }
-  consumers_sync();
-}
-
-// Sort, descending, of a[0..n) for n <= kRegSort: the same bitonic network
-// over a fixed 2,048 entries (zeros pad the tail), held in registers, 8
-// consecutive entries per consumer thread.  Partners less than 8 apart sit in
-// one thread; less than 256 apart, in one warp (exchanged by shuffles); the
-// three widest strides go through a[] with block barriers.  a[] must hold
-// kRegSort entries.
-constexpr uint32_t kRegSort = 8 * kConsumers;
-template <uint32_t J>
-__device__ __forceinline__ void reg_stage(uint64_t (&x)[8], uint32_t e0, uint32_t k) {
-#pragma unroll
-  for (uint32_t r = 0; r < 8; r++) {
-    if (r & J) continue;
-    const bool desc = ((e0 + r) & k) == 0;  // this k-block runs descending
-    const uint64_t u = x[r], v = x[r + J];
-    if ((u < v) == desc) {
-      x[r] = v;
-      x[r + J] = u;
-    }
-  }
-}
-__device__ void reg_bitonic_desc(uint64_t *a, uint32_t n) {
-  const uint32_t tid = threadIdx.x, e0 = 8 * tid;
-  uint64_t x[8];
-#pragma unroll
-  for (uint32_t r = 0; r < 8; r++) x[r] = e0 + r < n ? a[e0 + r] : 0ull;
-  for (uint32_t k = 2; k <= kRegSort; k <<= 1) {
-    for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      if (j == 4) reg_stage<4>(x, e0, k);
-      else if (j == 2) reg_stage<2>(x, e0, k);
-      else if (j == 1) reg_stage<1>(x, e0, k);
-      else if (j < 256) {
-        const uint32_t pm = j >> 3;  // the partner thread is tid ^ pm
-        const bool lower = (e0 & j) == 0, desc = (e0 & k) == 0;
-#pragma unroll
-        for (uint32_t r = 0; r < 8; r++) {
-          const uint64_t y = __shfl_xor_sync(kFull, x[r], pm);
-          x[r] = (lower == desc) ? (x[r] > y ? x[r] : y) : (x[r] < y ? x[r] : y);
-        }
-      } else {
-#pragma unroll
-        for (uint32_t r = 0; r < 8; r++) a[e0 + r] = x[r];
-        consumers_sync();
-        const bool lower = (e0 & j) == 0, desc = (e0 & k) == 0;
-#pragma unroll
-        for (uint32_t r = 0; r < 8; r++) {
-          const uint64_t y = a[(e0 + r) ^ j];
-          x[r] = (lower == desc) ? (x[r] > y ? x[r] : y) : (x[r] < y ? x[r] : y);
-        }
-        consumers_sync();
-      }
-    }
-  }
-#pragma unroll
-  for (uint32_t r = 0; r < 8; r++)
-    if (e0 + r < n) a[e0 + r] = x[r];
-  consumers_sync();
-}
-
 // Sort, descending, of the distinct values a[0..n) by bucket: the 8 bits
 // below the values' common prefix name 256 buckets, a counting pass places
 // each value in its bucket's range (buckets in descending order, in tmp),
@@ -648,18 +551,28 @@ __device__ void reg_bitonic_desc(uint64_t *a, uint32_t n) {
 // unchanged) when that sum is large, i.e. the values crowd into few buckets.
 static_assert(kConsumers == 256, "one bucket per consumer thread");
 
-// The rank-M cut of the distinct values src[0..c), c > M: 256 buckets on
-// the 8 bits below the values' common prefix (bucket of v: (v >> sh) & 255),
-// and bcut the bucket holding the rank-M value.  Returns the count of values
-// in bcut and the buckets above it: at least M.  each(fn) calls fn(v) once
-// for every value, spread over the consumer threads in any order.
+// Values beyond the M wanted ones that a selection leaves to the sort: another
+// step of narrow() costs about what sorting twice as many does.
+__device__ __forceinline__ uint32_t slack(uint32_t M) { return max(M, 256u); }
+
+// One step towards the rank-M value of a list of distinct values.  The values
+// in [t, t + 2^sh) (all of them for sh == 64) hold it as their need-th
+// largest: 256 buckets on the 8 bits below their common prefix, and [t, t +
+// 2^sh) becomes the bucket that holds it.  Returns the values in that bucket;
+// need becomes the rank in it.  each(fn) calls fn(v) once for every value,
+// spread over the consumer threads in any order.
 template <class Each>
-__device__ uint32_t bucket_cut(Each each, uint32_t M, SelectScratch &ss, int &sh, uint32_t &bcut) {
+__device__ uint32_t narrow(Each each, uint64_t &t, int &sh, uint32_t &need, SelectScratch &ss) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint64_t lo = t;
+  const int s0 = sh;
+  auto in = [&](uint64_t v) { return s0 >= 64 || v >> s0 == lo >> s0; };
   uint64_t an = ~0ull, orv = 0ull;
   each([&](uint64_t v) {
-    an &= v;
-    orv |= v;
+    if (in(v)) {
+      an &= v;
+      orv |= v;
+    }
   });
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -677,12 +590,15 @@ __device__ uint32_t bucket_cut(Each each, uint32_t M, SelectScratch &ss, int &sh
     atomicOr(&ss.bcast[1], orv);
   }
   consumers_sync();
-  const uint64_t vary = ss.bcast[0] ^ ss.bcast[1];
+  const uint64_t vary = ss.bcast[0] ^ ss.bcast[1], common = ss.bcast[0];
   const int top = vary ? 64 - __clzll((long long)vary) : 0;
   sh = top > 8 ? top - 8 : 0;
-  each([&](uint64_t v) { atomicAdd(&ss.hist[(uint32_t)(v >> sh) & 255u], 1u); });
+  const int s1 = sh;
+  each([&](uint64_t v) {
+    if (in(v)) atomicAdd(&ss.hist[(uint32_t)(v >> s1) & 255u], 1u);
+  });
   consumers_sync();
-  // thread t owns bucket 255 - t: counts from the top
+  // thread i owns bucket 255 - i: counts from the top
   const uint32_t own = ss.hist[255 - tid];
   uint32_t incl = own;
 #pragma unroll
@@ -693,16 +609,21 @@ __device__ uint32_t bucket_cut(Each each, uint32_t M, SelectScratch &ss, int &sh
   if (lane == 31) ss.wtot[warp] = incl;
   consumers_sync();
   for (uint32_t w = 0; w < warp; w++) incl += ss.wtot[w];
-  if (incl - own < M && incl >= M) {
+  if (incl - own < need && incl >= need) {
     ss.pick[0] = 255 - tid;
-    ss.pick[1] = incl;
+    ss.pick[1] = incl - own;
+    ss.cnt = own;
   }
   consumers_sync();
-  bcut = ss.pick[0];
-  const uint32_t n = ss.pick[1];
+  // the common prefix above the 8 bits (none varies there), then the bucket
+  const uint64_t pre = s1 >= 56 ? 0ull : common >> (s1 + 8) << (s1 + 8);
+  t = pre | (uint64_t)ss.pick[0] << s1;
+  need -= ss.pick[1];
+  const uint32_t n = ss.cnt;
   consumers_sync();  // pick, hist and bcast free for the caller
   return n;
 }
+
 __device__ bool bucket_sort_desc(uint64_t *a, uint32_t n, uint64_t *tmp, SelectScratch &ss, uint32_t *pay = nullptr,
                                  uint32_t *tmp_pay = nullptr) {
   if (n <= 1) return true;
@@ -777,12 +698,97 @@ __device__ bool bucket_sort_desc(uint64_t *a, uint32_t n, uint64_t *tmp, SelectS
   return true;
 }
 
-// The bucket sort, else a sorting network by size.  tmp: room for n values
-// (and tmp_pay for n payloads when pay is given), apart from a and pay.
-__device__ __forceinline__ void sort_desc(uint64_t *a, uint32_t n, uint64_t *tmp, SelectScratch &ss) {
-  if (bucket_sort_desc(a, n, tmp, ss)) return;
-  if (n <= kRegSort) reg_bitonic_desc(a, n);
-  else bitonic_sort_desc(a, n);
+// Sort, descending, of n <= kCountSort distinct values: each value's place is
+// the count of those above it.
+constexpr uint32_t kCountSort = 2 * kConsumers;
+__device__ void count_sort_desc(uint64_t *a, uint32_t n, uint32_t *pay) {
+  const uint32_t tid = threadIdx.x, i1 = tid + kConsumers;
+  const uint64_t v0 = tid < n ? a[tid] : 0ull, v1 = i1 < n ? a[i1] : 0ull;
+  const uint32_t p0 = pay && tid < n ? pay[tid] : 0u, p1 = pay && i1 < n ? pay[i1] : 0u;
+  uint32_t r0 = 0, r1 = 0;
+#pragma unroll 8
+  for (uint32_t q = 0; q < n; q++) {
+    const uint64_t x = a[q];
+    r0 += x > v0 ? 1u : 0u;
+    r1 += x > v1 ? 1u : 0u;
+  }
+  consumers_sync();
+  if (tid < n) {
+    a[r0] = v0;
+    if (pay) pay[r0] = p0;
+  }
+  if (i1 < n) {
+    a[r1] = v1;
+    if (pay) pay[r1] = p1;
+  }
+  consumers_sync();
+}
+
+// Sort, descending, of n > 256 distinct values whose bits crowd: 256 of the
+// values, taken evenly over their (arbitrary) order and ranked by counting, split the
+// rest into buckets of about n / 256 whatever their distribution; then as the
+// bucket sort.
+__device__ void splitter_sort_desc(uint64_t *a, uint32_t n, uint64_t *tmp, SelectScratch &ss, uint32_t *pay,
+                                   uint32_t *tmp_pay) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint64_t mine = a[(uint64_t)tid * n / kConsumers];
+  tmp[tid] = mine;
+  ss.hist[tid] = 0;
+  consumers_sync();
+  uint32_t r = 0;
+#pragma unroll 8
+  for (uint32_t q = 0; q < kConsumers; q++) r += tmp[q] > mine ? 1u : 0u;
+  ss.split[r] = mine;
+  consumers_sync();
+  // the bucket of a value: the splitters above it, the last one left out
+  auto bucket = [&](uint64_t v) {
+    uint32_t lo = 0;
+#pragma unroll
+    for (uint32_t step = 128; step > 0; step >>= 1)
+      if (ss.split[lo + step - 1] > v) lo += step;
+    return lo;
+  };
+  for (uint32_t i = tid; i < n; i += kConsumers) atomicAdd(&ss.hist[bucket(a[i])], 1u);
+  consumers_sync();
+  const uint32_t c = ss.hist[tid];
+  uint32_t incl = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(kFull, incl, o);
+    if ((int)lane >= o) incl += y;
+  }
+  if (lane == 31) ss.wtot[warp] = incl;
+  consumers_sync();
+  uint32_t ex = incl - c;
+  for (uint32_t w = 0; w < warp; w++) ex += ss.wtot[w];
+  ss.off[tid] = ex;
+  ss.hist[tid] = ex;
+  consumers_sync();
+  for (uint32_t i = tid; i < n; i += kConsumers) {
+    const uint64_t v = a[i];
+    const uint32_t p = atomicAdd(&ss.hist[bucket(v)], 1u);
+    tmp[p] = v;
+    if (pay) tmp_pay[p] = pay[i];
+  }
+  consumers_sync();
+  for (uint32_t p = tid; p < n; p += kConsumers) {
+    const uint64_t v = tmp[p];
+    const uint32_t b = bucket(v), lo = ss.off[b], hi = ss.hist[b];
+    uint32_t k = 0;
+    for (uint32_t q = lo; q < hi; q++) k += tmp[q] > v ? 1u : 0u;
+    a[lo + k] = v;
+    if (pay) pay[lo + k] = tmp_pay[p];
+  }
+  consumers_sync();
+}
+
+// Sort, descending, of distinct values by the cheapest of the three.  tmp:
+// room for n values (and tmp_pay for n payloads when pay is given), apart from
+// a and pay.
+__device__ __forceinline__ void sort_desc(uint64_t *a, uint32_t n, uint64_t *tmp, SelectScratch &ss,
+                                          uint32_t *pay = nullptr, uint32_t *tmp_pay = nullptr) {
+  if (n <= kCountSort) count_sort_desc(a, n, pay);
+  else if (!bucket_sort_desc(a, n, tmp, ss, pay, tmp_pay)) splitter_sort_desc(a, n, tmp, ss, pay, tmp_pay);
 }
 
 // ------------------------------------------------------------- sample ----
@@ -807,13 +813,17 @@ __host__ __forceinline__ uint64_t list_target_of(const RankSet &S, int L, bool w
   return wide ? 6ull * M + 2048 : 2ull * M + 1024;
 }
 __host__ uint64_t sample_size_raw(const RankSet &S, bool wide) {
-  if (S.n <= kSample) return 0;
+  if (S.n <= kSmemCand) return 0;  // the finish holds every record's value in shared memory
   uint64_t tmax = 0;
   for (int L = 0; L < kLists; L++)
     if (list_active(S, L) && list_target_of(S, L, wide) > tmax) tmax = list_target_of(S, L, wide);
   if (tmax == 0) return 0;
+  if (S.n <= kSample && 2 * tmax > S.n) return 0;  // a sample would leave most records candidates
   return ((uint64_t)kSampleRank * S.n) / tmax;
 }
+
+// CTAs a set can use: one a tile, and one a list for the finish.
+__host__ __forceinline__ uint32_t most_ctas(const RankSet &S) { return std::max<uint32_t>(S.ntiles, kLists); }
 
 // The sample plan of a set whose group (cta0, nctas) is fixed.
 void plan_sample(RankSet &s) {
@@ -821,8 +831,8 @@ void plan_sample(RankSet &s) {
   const bool wide = sample_size_raw(s, false) > cap;
   uint64_t ns = umin64(sample_size_raw(s, wide), cap);
   s.sctas = ns ? (uint32_t)std::min<uint64_t>(std::min(s.nctas, kSampleCtas), (ns + kPerCtaSamples - 1) / kPerCtaSamples)
-               : 1u;
-  ns -= ns % (8ull * s.sctas);  // whole runs, evenly split over the sampling CTAs
+               : 0u;
+  if (ns) ns -= ns % (8ull * s.sctas);  // whole runs, evenly split over the sampling CTAs
   s.ns = (uint32_t)ns;
   s.nruns = s.ns / 8;
   s.sstep = s.nruns ? ((uint64_t)s.n << 16) / s.nruns : 0;
@@ -887,7 +897,7 @@ __device__ __noinline__ void sample_share(const RankSet &S, uint32_t r, const ui
     const uint32_t em = ok[q] ? elig_mask(fl[q], tr[q]) & act : 0u;
 #pragma unroll
     for (int L = 0; L < kLists; L++) {
-      const uint32_t b = ((em >> L) & 1) ? L * kBins + bin_of(summary_of(list_val(ck, L))) : 0xFFFFFFFFu;
+      const uint32_t b = ((em >> L) & 1) ? L * kBins + list_bin(summary_of(list_val(ck, L)), L) : 0xFFFFFFFFu;
       const unsigned grp = __match_any_sync(kFull, b);
       if (b != 0xFFFFFFFFu && (__ffs(grp) - 1) == (int)(tid & 31)) atomicAdd(&lh[b], (unsigned)__popc(grp));
     }
@@ -935,7 +945,7 @@ __device__ void thresholds(const RankSet &S, const uint64_t *t2s, const uint32_t
     const uint32_t need[kLists] = {S.rL[0], S.rL[1], S.rL[2]};
     hist_cut3(S.shist, need, cut);
   }
-  if (threadIdx.x < kLists) sthr[threadIdx.x] = cut[threadIdx.x] >= 0 ? summary_floor(bin_floor((uint32_t)cut[threadIdx.x])) : 0ull;
+  if (threadIdx.x < kLists) sthr[threadIdx.x] = cut[threadIdx.x] >= 0 ? summary_floor(list_bin_floor((uint32_t)cut[threadIdx.x], (int)threadIdx.x)) : 0ull;
   consumers_sync();
   const bool aV = S.act & 1, aD = (S.act >> 1) & 1, aP = (S.act >> 2) & 1;
   if (threadIdx.x < kLutN) {
@@ -1073,63 +1083,72 @@ __device__ __noinline__ bool finish_list(const RankSet &S, int L, uint64_t *fin,
           wait_phase_uniform(S, &cbar, 0);  // let the copy land before the area is reused
       }
       const uint64_t *src = in_smem ? buf : cand;
-      // every candidate, a block-wide pass (fn(v, ok): ok false past the end)
-      auto each_w = [&](auto fn) {
-        for (uint32_t base = 0; base < c; base += kConsumers) {
-          const uint32_t i = base + tid;
-          fn(i < c ? src[i] : 0ull, i < c);
+      // every value of from[0..n), a block-wide pass, eight independent loads
+      // a thread in flight (fn(v, ok): ok false past the end)
+      auto each_w = [&](const uint64_t *from, uint32_t n, auto fn) {
+        for (uint32_t base = 0; base < n; base += 8 * kConsumers) {
+          uint64_t v[8];
+#pragma unroll
+          for (uint32_t u = 0; u < 8; u++) {
+            const uint32_t i = base + u * kConsumers + tid;
+            v[u] = i < n ? from[i] : 0ull;
+          }
+#pragma unroll
+          for (uint32_t u = 0; u < 8; u++)
+            if (base + u * kConsumers < n) fn(v[u], base + u * kConsumers + tid < n);
         }
       };
-      auto each = [&](auto fn) {
-        each_w([&](uint64_t v, bool ok) {
-          if (ok) fn(v);
+      // the values of from[0..n) at or above t, in any order
+      auto keep_from = [&](const uint64_t *from, uint32_t n, uint64_t t, uint64_t *to) {
+        if (tid == 0) nsurv = 0;
+        consumers_sync();
+        each_w(from, n, [&](uint64_t v, bool ok) {
+          const bool keep = ok && v >= t;
+          const unsigned bal = __ballot_sync(kFull, keep);
+          unsigned wb = 0;
+          if (lane == 0 && bal) wb = atomicAdd(&nsurv, (unsigned)__popc(bal));
+          wb = __shfl_sync(kFull, wb, 0);
+          const uint32_t pos = wb + __popc(bal & ((1u << lane) - 1));
+          if (keep && pos < kMaxSel) to[pos] = v;
         });
+        consumers_sync();
       };
-      if (c <= M) {
-        // every candidate is kept
+      if (c <= M || (c <= M + slack(M) && c <= kMaxSel)) {
+        // every candidate is kept (and the sort drops those beyond M)
         for (uint32_t i = tid; i < c; i += kConsumers) sel[i] = src[i];
         got = c;
       } else {
-        // the values in the bucket holding the rank-M value and above it: at
-        // least M of them, and the top M among them are the top M of all
-        // candidates (every other value is in a lower bucket, hence smaller)
-        int sh = 0;
-        uint32_t bcut = 0;
-        const uint32_t ns = bucket_cut(each, M, ss, sh, bcut);
-        if (ns <= kMaxSel) {
-          if (tid == 0) nsurv = 0;
-          consumers_sync();
-          each_w([&](uint64_t v, bool ok) {
-            const bool keep = ok && ((uint32_t)(v >> sh) & 255u) >= bcut;
-            const unsigned bal = __ballot_sync(kFull, keep);
-            unsigned wb = 0;
-            if (lane == 0 && bal) wb = atomicAdd(&nsurv, (unsigned)__popc(bal));
-            wb = __shfl_sync(kFull, wb, 0);
-            const uint32_t pos = wb + __popc(bal & ((1u << lane) - 1));
-            if (keep) sel[pos] = v;
-          });
-          consumers_sync();
-          got = ns;
-        } else {
-          // the cut's bucket holds too many values: radix select of the
-          // rank-M value over every candidate
-          ss.hist[tid] = 0;
-          consumers_sync();
-          const uint64_t th = block_select_rank([&](uint32_t i) { return src[i]; }, c, M, ss);
-          if (tid == 0) ss.cnt = 0;
-          consumers_sync();
-          each_w([&](uint64_t v, bool ok) {
-            const bool keep = ok && v >= th;
-            const unsigned bal = __ballot_sync(kFull, keep);
-            unsigned wb = 0;
-            if (lane == 0 && bal) wb = atomicAdd(&ss.cnt, (unsigned)__popc(bal));
-            wb = __shfl_sync(kFull, wb, 0);
-            const uint32_t pos = wb + __popc(bal & ((1u << lane) - 1));
-            if (keep && pos < kMaxSel) sel[pos] = v;
-          });
-          consumers_sync();
-          got = min(ss.cnt, M);
+        // values at or above t hold the top M: t rises bucket by bucket until
+        // few values beyond M are left.  Values that crowd (small keys, ties)
+        // take a step more, where one cut would leave a bucket of thousands to
+        // sort.  Once they fit, the values move to shared memory.
+        const uint64_t *from = src;
+        uint32_t n = c, need = M;
+        uint64_t t = 0;
+        int sh = 64;
+        for (;;) {
+          const uint32_t in = narrow(
+              [&](auto fn) {
+                each_w(from, n, [&](uint64_t v, bool ok) {
+                  if (ok) fn(v);
+                });
+              },
+              t, sh, need, ss);
+          const uint32_t left = M - need + in;  // at or above t
+          if (left <= kMaxSel && (from != sel || left <= n / 2 || left <= M + slack(M) || sh == 0)) {
+            if (from == sel) {  // (buf is free then)
+              keep_from(sel, n, t, buf);
+              for (uint32_t i = tid; i < left; i += kConsumers) sel[i] = buf[i];
+              consumers_sync();
+            } else {
+              keep_from(from, n, t, sel);
+            }
+            from = sel;
+            n = left;
+          }
+          if (sh == 0 || (from == sel && n <= M + slack(M))) break;
         }
+        got = n;
       }
       consumers_sync();
       sort_desc(sel, got, buf, ss);
@@ -1377,13 +1396,18 @@ __device__ __noinline__ void fill(const RankSet &S, uint64_t *fin) {
 // set's counter and announces each stage's tile in stile[]; a partial last
 // tile (read directly from global memory by the consumers) and the end of
 // the set (kEndTile) are announced with a plain arrival.
-// zero_a / zero_b (n_a, n_b 16-byte words): the other parity's work words
-// and sample histograms, zeroed here for the next call on the stream.
+// zero (n_zero 16-byte words): the work words and sample histograms that the
+// stream's previous call used, zeroed here for its next one.
 // cmap (grouped launches): CTA b serves set cmap[b] & 0xFFFF, whose tables are
-// tabs[cmap[b] >> 16]; null for a sequential launch.
+// tabs[cmap[b] >> 16]; null for a sequential launch.  A call of one set brings
+// its descriptor and tables as a parameter (sets null): no upload precedes it.
+struct RankOne {
+  RankSet set;
+  RankTab tab;
+};
 __global__ void __launch_bounds__(kCtaThreads, 3)
-    rank_kernel(const RankSet *sets, int n_sets, int sequential, const uint32_t *cmap, const RankTab *tabs,
-                uint4 *zero_a, uint32_t n_a, uint4 *zero_b, uint32_t n_b) {
+    rank_kernel(const RankSet *d_sets, int n_sets, int sequential, const uint32_t *cmap, const RankTab *tabs,
+                uint4 *zero, uint32_t n_zero, const __grid_constant__ RankOne one) {
   extern __shared__ __align__(128) unsigned char dsm[];
   FilterStage *stage = reinterpret_cast<FilterStage *>(dsm);
   uint64_t *fin = reinterpret_cast<uint64_t *>(dsm);
@@ -1405,14 +1429,18 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
 
   {  // every CTA takes its share, before any returns
     const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
-    for (uint32_t w = g; w < n_a; w += gs) zero_a[w] = make_uint4(0u, 0u, 0u, 0u);
-    for (uint32_t w = g; w < n_b; w += gs) zero_b[w] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t w = g; w < n_zero; w += gs) zero[w] = make_uint4(0u, 0u, 0u, 0u);
   }
+  const RankSet *const sets = d_sets ? d_sets : &one.set;
   int s0, sstep;
   const RankTab *tab0 = nullptr;  // the first set's tables, when the map names them
   if (sequential) {
     s0 = blockIdx.x;
     sstep = gridDim.x;
+  } else if (!d_sets) {
+    s0 = 0;
+    tab0 = &one.tab;
+    sstep = 1;
   } else {
     const uint32_t e = __ldg(cmap + blockIdx.x);
     s0 = (int)(e & 0xFFFFu);
@@ -1557,7 +1585,7 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
 #ifdef UNISON_DEBUG_HOOKS
     if (s == g_hook_flag_set) wait_word(S, &S.work->dummy, 1u);  // nothing sets it: runs out
 #endif
-    wait_word(S, &S.work->sample_ticket, S.sctas);
+    if (S.sctas) wait_word(S, &S.work->sample_ticket, S.sctas);
     if (ct < kLists) ccnt_s[ct] = 0;  // published by the barriers below
     thresholds(S, t2s, sgs, vd, pp, c);
     const uint32_t s_n = S.n;
@@ -1889,9 +1917,8 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
 
 // ------------------------------------------------------------- merge ----
 // The shards' candidate lists, gathered (n_shards buffers of `stride` bytes
-// each): CTA L selects list L's global top M (a radix select when the
-// shards hold more than 4,096 entries, then a bitonic sort carrying the
-// sizes), writes it as the finish does, and the last list's CTA runs the
+// each): CTA L selects list L's global top M (narrowed and sorted as in the
+// finish, carrying the sizes), writes it as the finish does, and the last list's CTA runs the
 // fill.  One CTA per list, consumer-sized (256 threads).
 __global__ void __launch_bounds__(kConsumers) rank_merge_kernel(const RankSet *Sp, const unsigned char *gathered,
                                                                 int n_shards, uint64_t stride) {
@@ -1929,34 +1956,76 @@ __global__ void __launch_bounds__(kConsumers) rank_merge_kernel(const RankSet *S
   uint32_t *szs = reinterpret_cast<uint32_t *>(fin + kMaxSel);  // [kMaxSel]
   uint32_t got = 0;
   if (M > 0) {
-    uint32_t keepn;
-    if (c <= kMaxSel) {
-      for (uint32_t i = threadIdx.x; i < c; i += kConsumers) {
-        const CandEntry &e = entry(i);
-        val[i] = e.v;
-        szs[i] = e.kv;
+    uint64_t *tval = fin + 3 * kMaxSel / 2;  // copies of both
+    uint32_t *tszs = reinterpret_cast<uint32_t *>(fin + 5 * kMaxSel / 2);
+    // fn(entry, ok) over every entry, eight independent reads a thread in flight
+    auto each_entry = [&](auto fn) {
+      for (uint32_t base = 0; base < c; base += 8 * kConsumers) {
+        CandEntry e[8];
+#pragma unroll
+        for (uint32_t u = 0; u < 8; u++) {
+          const uint32_t i = base + u * kConsumers + threadIdx.x;
+          e[u] = i < c ? entry(i) : CandEntry{0ull, 0u, 0u};
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < 8; u++) fn(e[u], base + u * kConsumers + threadIdx.x < c);
       }
-      keepn = c;
-    } else {
-      const uint64_t th = block_select_rank([&](uint32_t i) { return entry(i).v; }, c, M, ss);
-      if (threadIdx.x == 0) ss.cnt = 0;
-      consumers_sync();
-      for (uint32_t i = threadIdx.x; i < c; i += kConsumers) {
-        const CandEntry &e = entry(i);
-        if (e.v >= th) {
-          const uint32_t pos = atomicAdd(&ss.cnt, 1u);
-          if (pos < kMaxSel) {
-            val[pos] = e.v;
-            szs[pos] = e.kv;
-          }
+    };
+    // as in finish_list: t rises until few entries beyond M are at or above it
+    uint64_t t = 0;
+    int sh = 64;
+    uint32_t need = M, left = c;
+    while (left > kMaxSel && sh > 0) {
+      const uint32_t in = narrow(
+          [&](auto fn) {
+            each_entry([&](const CandEntry &e, bool ok) {
+              if (ok) fn(e.v);
+            });
+          },
+          t, sh, need, ss);
+      left = M - need + in;
+    }
+    if (threadIdx.x == 0) ss.cnt = 0;
+    consumers_sync();
+    each_entry([&](const CandEntry &e, bool ok) {
+      if (ok && e.v >= t) {
+        const uint32_t pos = atomicAdd(&ss.cnt, 1u);
+        if (pos < kMaxSel) {
+          val[pos] = e.v;
+          szs[pos] = e.kv;
         }
       }
-      consumers_sync();
-      keepn = min(ss.cnt, kMaxSel);
-    }
+    });
     consumers_sync();
-    if (!bucket_sort_desc(val, keepn, fin + 3 * kMaxSel / 2, ss, szs, reinterpret_cast<uint32_t *>(fin + 5 * kMaxSel / 2)))
-      bitonic_sort_desc(val, keepn, szs);
+    uint32_t keepn = min(ss.cnt, kMaxSel);
+    consumers_sync();
+    left = keepn;
+    while (left > M + slack(M) && sh > 0) {
+      const uint32_t in = narrow(
+          [&](auto fn) {
+            for (uint32_t i = threadIdx.x; i < keepn; i += kConsumers) fn(val[i]);
+          },
+          t, sh, need, ss);
+      left = M - need + in;
+    }
+    if (left < keepn) {
+      if (threadIdx.x == 0) ss.cnt = 0;
+      consumers_sync();
+      for (uint32_t i = threadIdx.x; i < keepn; i += kConsumers)
+        if (val[i] >= t) {
+          const uint32_t pos = atomicAdd(&ss.cnt, 1u);
+          tval[pos] = val[i];
+          tszs[pos] = szs[i];
+        }
+      consumers_sync();
+      keepn = left;
+      for (uint32_t i = threadIdx.x; i < keepn; i += kConsumers) {
+        val[i] = tval[i];
+        szs[i] = tszs[i];
+      }
+      consumers_sync();
+    }
+    sort_desc(val, keepn, tval, ss, szs, tszs);
     got = min(keepn, M);
     for (uint32_t i = threadIdx.x; i < got; i += kConsumers) {
       S.sorted[(size_t)L * kMaxSel + i] = val[i];
@@ -1979,20 +2048,58 @@ bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) %
 
 // Device scratch of the ranking calls, kept per (device, stream) and grown
 // when a call needs more: calls on one stream run in order, so each reuses
-// the buffer after the previous one is done with it (stream order), and
+// the buffers after the previous one is done with them (stream order), and
 // calls on different streams get different buffers.  Held for the life of
 // the process.  The stream handle is the key: a stream must outlive the
 // ranking calls queued on it (a new stream that reuses a destroyed one's
 // handle would otherwise share its scratch without being ordered after it).
-// Two blocks per key: the call's working scratch, and the per-set
-// histograms, which are zeroed when allocated and left zero by every call
-// (each is zeroed by the thread that reads it).
+// Per key: the calls' working scratch, and two blocks for the state that a
+// call must find zero (work words, then the sampled sets' histograms).  Calls
+// alternate between the two; each zeroes what the one before it used, so a
+// block is all zero when its turn comes, whatever the calls' sizes, and no
+// clearing precedes a launch (a memset and the upload of a single set's
+// descriptor took about 10 of a call's 52 us at 2^20 records).
 struct Scratch {
   char *p = nullptr;
   size_t bytes = 0;
 };
-std::mutex g_scratch_mu;
-std::map<std::pair<int, cudaStream_t>, std::pair<Scratch, Scratch>> g_scratch;
+// The stream's last call of several sets: one whose arguments are byte for
+// byte the same finds its descriptors (once per block), tables and scratch
+// layout already on the device and only launches.  Any other use of the
+// working scratch drops it.
+struct RankPlan {
+  std::vector<unsigned char> key;
+  size_t desc_b = 0, cmap_off = 0, tabs_off = 0;
+  size_t zero_b = 0;  // bytes of a block that the call uses
+  uint32_t grid = 0;
+  int sequential = 0;
+};
+struct StreamState {
+  std::mutex mu;  // held from the choice of a block to the launch that uses it
+  Scratch main, zero[2];
+  size_t dirty[2] = {0, 0};  // bytes from a block's start that are not zero
+  bool planned = false;
+  RankPlan plan;
+  // the last tables built, and what they were built from
+  bool have_tab = false;
+  uint16_t tab_sigma[kLutN];
+  uint64_t tab_penalty = 0;
+  RankTab tab;
+};
+std::mutex g_state_mu;
+std::map<std::pair<int, cudaStream_t>, std::unique_ptr<StreamState>> g_state;
+
+StreamState *stream_state(cudaStream_t stream) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  std::lock_guard<std::mutex> lock(g_state_mu);
+  auto &e = g_state[std::make_pair(dev, stream)];
+  if (!e) e.reset(new StreamState());
+  return e.get();
+}
 
 int grow(Scratch &e, size_t bytes, bool zero, cudaStream_t stream) {
   if (e.bytes >= bytes) return UNISON_OK;
@@ -2014,19 +2121,15 @@ int grow(Scratch &e, size_t bytes, bool zero, cudaStream_t stream) {
   return UNISON_OK;
 }
 
-int scratch_acquire(cudaStream_t stream, size_t bytes, size_t hist_bytes, char **out, char **hist) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) {
-    cudaGetLastError();
-    return UNISON_ERR_CUDA;
+// Both zero blocks at least `bytes` long (a new block is zero).
+int grow_zero(StreamState &st, size_t bytes, cudaStream_t stream) {
+  for (int i = 0; i < 2; i++) {
+    if (st.zero[i].bytes >= bytes) continue;
+    st.dirty[i] = 0;
+    st.planned = false;  // the plan's descriptors name the old block
+    const int rc = grow(st.zero[i], bytes, true, stream);
+    if (rc != UNISON_OK) return rc;
   }
-  std::lock_guard<std::mutex> lock(g_scratch_mu);
-  auto &e = g_scratch[std::make_pair(dev, stream)];
-  int rc = grow(e.first, bytes, false, stream);
-  if (rc == UNISON_OK) rc = grow(e.second, hist_bytes, true, stream);
-  if (rc != UNISON_OK) return rc;
-  *out = e.first.p;
-  *hist = e.second.p;
   return UNISON_OK;
 }
 
@@ -2142,26 +2245,6 @@ namespace {
 // The ranking call: n_sets sets with their outputs, or (cands != null) one
 // shard of a set whose record 0 has index `off` in the whole set, with its
 // candidate lists going to cands instead of outputs.
-// The last ranking call's plan per (device, stream): a call whose arguments
-// are byte for byte those of the previous call on its stream finds its
-// descriptors, tables and scratch layout already on the device and only
-// launches.  The per-call state (work words, sample histograms) is held
-// twice; calls alternate between the two, and each launch zeroes the
-// other's for the next call.  Any other use of the stream's scratch (a
-// merge, a different call, a reallocation) replaces or drops the plan.
-struct RankPlan {
-  std::vector<unsigned char> key;
-  size_t bytes = 0, hist_bytes = 0;
-  size_t desc_b = 0, work_off = 0, work_b = 0, hist_b = 0;  // per parity: descriptors, work words, histograms
-  size_t cmap_off = 0, tabs_off = 0;
-  char *scratch = nullptr, *hists = nullptr;
-  uint32_t grid = 0;
-  int sequential = 0;
-  int parity = 0;  // the parity the next call uses (its state is zero)
-};
-std::mutex g_plan_mu;
-std::map<std::pair<int, cudaStream_t>, RankPlan> g_plan;
-
 void plan_key(std::vector<unsigned char> &k, const unison_records *sets, const unison_rank_params *params,
               const unison_rank_out *outs, int n_sets, uint32_t off, const unsigned char *cands) {
   k.clear();
@@ -2177,67 +2260,57 @@ void plan_key(std::vector<unsigned char> &k, const unison_records *sets, const u
   if (!cands) put(outs, sizeof(unison_rank_out) * n_sets);
 }
 
-void plan_drop(cudaStream_t stream) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) {
-    cudaGetLastError();
-    return;
+// Launches a call on the zero block whose turn it is (zb: the bytes of it that
+// the call uses), zeroing the other.  The caller holds st.mu and has passed
+// that block (next_block) to the descriptors.
+int next_block(const StreamState &st) { return st.dirty[0] == 0 ? 0 : 1; }
+int launch_rank_kernel(StreamState &st, uint32_t grid, const RankSet *d_sets, int n_sets, int sequential,
+                       const uint32_t *cmap, const RankTab *tabs, const RankOne &one, size_t zb, cudaStream_t stream) {
+  const int p = next_block(st);
+  cudaError_t e;
+  {
+    ProfSpan span("rank", stream);
+    cudaLaunchAttribute coop[1];
+    coop[0].id = cudaLaunchAttributeCooperative;
+    coop[0].val.cooperative = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(grid);
+    lc.blockDim = dim3(kCtaThreads);
+    lc.dynamicSmemBytes = kDynSmem;
+    lc.stream = stream;
+    lc.attrs = coop;
+    lc.numAttrs = 1;
+    e = cudaLaunchKernelEx(&lc, rank_kernel, d_sets, n_sets, sequential, cmap, tabs,
+                           reinterpret_cast<uint4 *>(st.zero[1 - p].p), (uint32_t)(st.dirty[1 - p] / 16), one);
   }
-  std::lock_guard<std::mutex> lock(g_plan_mu);
-  g_plan.erase(std::make_pair(dev, stream));
-}
-
-cudaError_t launch_rank_kernel(uint32_t grid, const RankSet *d_sets, int n_sets, int sequential, const uint32_t *cmap,
-                               const RankTab *tabs, char *zero_a, size_t bytes_a, char *zero_b, size_t bytes_b,
-                               cudaStream_t stream) {
-  ProfSpan span("rank", stream);
-  cudaLaunchAttribute coop[1];
-  coop[0].id = cudaLaunchAttributeCooperative;
-  coop[0].val.cooperative = 1;
-  cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(grid);
-  lc.blockDim = dim3(kCtaThreads);
-  lc.dynamicSmemBytes = kDynSmem;
-  lc.stream = stream;
-  lc.attrs = coop;
-  lc.numAttrs = 1;
-  return cudaLaunchKernelEx(&lc, rank_kernel, d_sets, n_sets, sequential, cmap, tabs, reinterpret_cast<uint4 *>(zero_a),
-                            (uint32_t)(bytes_a / 16), reinterpret_cast<uint4 *>(zero_b), (uint32_t)(bytes_b / 16));
+  count_launches(1);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    st.planned = false;
+    return UNISON_ERR_CUDA;  // nothing ran: the blocks are as they were
+  }
+  st.dirty[p] = zb;
+  st.dirty[1 - p] = 0;
+  return UNISON_OK;
 }
 
 int rank_launch(const unison_records *sets, const unison_rank_params *params, const unison_rank_out *outs,
                 int n_sets, uint32_t off, unsigned char *cands, cudaStream_t stream) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) {
-    cudaGetLastError();
-    return UNISON_ERR_CUDA;
-  }
+  StreamState *const state = stream_state(stream);
+  if (!state) return UNISON_ERR_CUDA;
+  StreamState &st = *state;
+  std::lock_guard<std::mutex> lock(st.mu);
+  static const RankOne none{};
   thread_local std::vector<unsigned char> key;
-  plan_key(key, sets, params, outs, n_sets, off, cands);
-  {
-    std::lock_guard<std::mutex> lock(g_plan_mu);
-    auto it = g_plan.find(std::make_pair(dev, stream));
-    if (it != g_plan.end() && it->second.key == key) {
-      RankPlan &pl = it->second;
-      char *scratch = nullptr, *hists = nullptr;
-      if (scratch_acquire(stream, pl.bytes, pl.hist_bytes, &scratch, &hists) == UNISON_OK && scratch == pl.scratch &&
-          hists == pl.hists) {
-        const int pa = pl.parity, pb = 1 - pa;
-        int rc = UNISON_OK;
-        if (launch_rank_kernel(pl.grid, reinterpret_cast<const RankSet *>(scratch + pa * pl.desc_b), n_sets,
-                               pl.sequential,
-                               pl.sequential ? nullptr : reinterpret_cast<const uint32_t *>(scratch + pl.cmap_off),
-                               reinterpret_cast<const RankTab *>(scratch + pl.tabs_off),
-                               scratch + pl.work_off + pb * pl.work_b, pl.work_b, hists + pb * pl.hist_b, pl.hist_b,
-                               stream) != cudaSuccess)
-          rc = UNISON_ERR_CUDA;
-        count_launches(1);
-        if (cudaGetLastError() != cudaSuccess) rc = UNISON_ERR_CUDA;
-        if (rc == UNISON_OK) pl.parity = pb;
-        else g_plan.erase(it);
-        return rc;
-      }
-      g_plan.erase(it);
+  if (n_sets > 1) {
+    plan_key(key, sets, params, outs, n_sets, off, cands);
+    if (st.planned && st.plan.key == key) {
+      const RankPlan &pl = st.plan;
+      return launch_rank_kernel(
+          st, pl.grid, reinterpret_cast<const RankSet *>(st.main.p + next_block(st) * pl.desc_b), n_sets, pl.sequential,
+          pl.sequential ? nullptr : reinterpret_cast<const uint32_t *>(st.main.p + pl.cmap_off),
+          reinterpret_cast<const RankTab *>(st.main.p + pl.tabs_off), none, pl.zero_b, stream);
     }
   }
   std::vector<RankSet> hs(n_sets);
@@ -2268,14 +2341,18 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
         ti = tab_keys[j].second;
     }
     if (ti < 0) {
-      RankTab tb;
-      for (int t = 0; t < (int)kLutN; t++) {
-        tb.sigma[t] = p.sigma_q[t];
-        tb.t2v[t] = ((uint64_t)(kLambda - p.sigma_q[t]) * p.penalty_q) / kLambda;  // eq. (t2)
-        tb.mgv[t] = magic_for(p.sigma_q[t]);
+      if (!st.have_tab || st.tab_penalty != p.penalty_q || std::memcmp(st.tab_sigma, p.sigma_q, sizeof st.tab_sigma)) {
+        for (int t = 0; t < (int)kLutN; t++) {
+          st.tab.sigma[t] = p.sigma_q[t];
+          st.tab.t2v[t] = ((uint64_t)(kLambda - p.sigma_q[t]) * p.penalty_q) / kLambda;  // eq. (t2)
+          st.tab.mgv[t] = magic_for(p.sigma_q[t]);
+        }
+        std::memcpy(st.tab_sigma, p.sigma_q, sizeof st.tab_sigma);
+        st.tab_penalty = p.penalty_q;
+        st.have_tab = true;
       }
       ti = (int)tabs.size();
-      tabs.push_back(tb);
+      tabs.push_back(st.tab);
       tab_keys.emplace_back(&p, ti);
     }
     tab_of[i] = ti;
@@ -2308,7 +2385,7 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
   const LaunchCfg &cfg = launch_cfg();
   if (!cfg.ok) return UNISON_ERR_CUDA;
   // Groups: each set gets CTAs in proportion to its tiles (at least 1, at
-  // most its tile count); CTAs left over go to the sets with the most tiles
+  // most one a tile, or one a list); CTAs left over go to the sets with the most tiles
   // per CTA.  With more sets than CTAs, CTA c takes sets c, c + G, ...
   const int sequential = (uint64_t)n_sets > cfg.ctas ? 1 : 0;
   uint32_t grid = cfg.ctas;
@@ -2317,13 +2394,13 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
     for (int i = 0; i < n_sets; i++) {
       RankSet &s = hs[i];
       s.nctas = (uint32_t)std::max<uint64_t>(1, (uint64_t)cfg.ctas * s.ntiles / tiles);
-      s.nctas = std::min(s.nctas, s.ntiles);
+      s.nctas = std::min(s.nctas, most_ctas(s));
       used += s.nctas;
     }
     while (used < cfg.ctas) {
       int best = -1;
       for (int i = 0; i < n_sets; i++)
-        if (hs[i].nctas < hs[i].ntiles &&
+        if (hs[i].nctas < most_ctas(hs[i]) &&
             (best < 0 || (uint64_t)hs[i].ntiles * hs[best].nctas > (uint64_t)hs[best].ntiles * hs[i].nctas))
           best = i;
       if (best < 0) break;
@@ -2361,31 +2438,25 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
               align_up(sizeof(uint64_t) * kLists * s.nctas * s.cr, 256);
     if (s.ns) hist_b += hist_set;
   }
-  const size_t desc_b = align_up(sizeof(RankSet) * n_sets, 256);
-  const size_t cmap_b = sequential ? 0 : align_up(sizeof(uint32_t) * grid, 256);
-  const size_t tab_b = align_up(sizeof(RankTab) * tabs.size(), 256);
+  const bool single = n_sets == 1;  // one descriptor goes as a launch parameter
+  const size_t desc_b = single ? 0 : align_up(sizeof(RankSet) * n_sets, 256);
+  const size_t cmap_b = sequential || single ? 0 : align_up(sizeof(uint32_t) * grid, 256);
+  const size_t tab_b = single ? 0 : align_up(sizeof(RankTab) * tabs.size(), 256);
   const size_t work_b = align_up(sizeof(RankWork) * n_sets, 256);
-  char *scratch = nullptr, *hists = nullptr;
-  {
-    plan_drop(stream);  // the scratch is rewritten below; the plan returns only if the launch succeeds
-    const int ar = scratch_acquire(stream, 2 * desc_b + cmap_b + tab_b + 2 * work_b + sets_b,
-                                   std::max<size_t>(2 * hist_b, 256), &scratch, &hists);
-    if (ar != UNISON_OK) return ar;
-  }
-  // image: descriptors of parity 0 and 1, the CTA map, tables, work words of
-  // parity 0 and 1, then the per-set areas; histograms of parity 0 then 1
+  const size_t zero_b = work_b + hist_b;
+  st.planned = false;  // the scratch is rewritten below; the plan returns only if the launch succeeds
+  int rc = grow(st.main, 2 * desc_b + cmap_b + tab_b + sets_b, false, stream);
+  if (rc == UNISON_OK) rc = grow_zero(st, zero_b, stream);
+  if (rc != UNISON_OK) return rc;
+  // image: descriptors for block 0 and 1, the CTA map, tables; then the
+  // per-set areas
   const size_t cmap_off = 2 * desc_b, tabs_off = cmap_off + cmap_b;
+  char *const scratch = st.main.p;
   RankTab *d_tabs = reinterpret_cast<RankTab *>(scratch + tabs_off);
-  const size_t work_off = tabs_off + tab_b;
-  RankWork *works = reinterpret_cast<RankWork *>(scratch + work_off);
-  char *p = scratch + work_off + 2 * work_b;
-  size_t hoff = 0;
+  char *p = scratch + tabs_off + tab_b;
   for (int i = 0; i < n_sets; i++) {
     RankSet &s = hs[i];
     s.tab = d_tabs + tab_of[i];
-    s.work = works + i;
-    s.shist = s.ns ? reinterpret_cast<unsigned int *>(hists + hoff) : nullptr;
-    if (s.ns) hoff += hist_set;
     s.sorted = reinterpret_cast<uint64_t *>(p);
     p += align_up(sizeof(uint64_t) * kLists * kMaxSel, 256);
     s.ssz = reinterpret_cast<uint32_t *>(p);
@@ -2395,25 +2466,34 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
     s.creg = reinterpret_cast<uint64_t *>(p);
     p += align_up(sizeof(uint64_t) * kLists * s.nctas * s.cr, 256);
   }
-  int rc = UNISON_OK;
-  auto ck = [&](cudaError_t e) {
-    if (e != cudaSuccess && rc == UNISON_OK) rc = UNISON_ERR_CUDA;
+  // the work words and histograms of the sets in block b
+  auto in_block = [&](int b) {
+    char *const z = st.zero[b].p;
+    size_t hoff = work_b;
+    for (int i = 0; i < n_sets; i++) {
+      RankSet &s = hs[i];
+      s.work = reinterpret_cast<RankWork *>(z) + i;
+      s.shist = s.ns ? reinterpret_cast<unsigned int *>(z + hoff) : nullptr;
+      if (s.ns) hoff += hist_set;
+    }
   };
-  RankSet *d_sets = reinterpret_cast<RankSet *>(scratch);
-  // descriptors of both parities, tables and both parities' zeroed work
-  // words: one copy from pinned staging; both parities' histograms zeroed
+  if (single) {
+    in_block(next_block(st));
+    RankOne one;
+    one.set = hs[0];
+    one.tab = tabs[0];
+    return launch_rank_kernel(st, grid, nullptr, 1, 0, nullptr, nullptr, one, zero_b, stream);
+  }
+  // one copy from pinned staging
   {
-    const size_t up = work_off + 2 * work_b;
+    const size_t up = tabs_off + tab_b;
     unsigned char *h = nullptr;
     cudaEvent_t done = nullptr;
     const int sr = staging_acquire(up, &h, &done);
     if (sr != UNISON_OK) return sr;
-    std::memcpy(h, hs.data(), sizeof(RankSet) * n_sets);
-    for (int i = 0; i < n_sets; i++) {  // parity 1: the other work words and histograms
-      RankSet s1 = hs[i];
-      s1.work = reinterpret_cast<RankWork *>(reinterpret_cast<char *>(s1.work) + work_b);
-      if (s1.shist) s1.shist = reinterpret_cast<unsigned int *>(reinterpret_cast<char *>(s1.shist) + hist_b);
-      std::memcpy(h + desc_b + sizeof(RankSet) * i, &s1, sizeof(RankSet));
+    for (int b = 0; b < 2; b++) {
+      in_block(b);
+      std::memcpy(h + b * desc_b, hs.data(), sizeof(RankSet) * n_sets);
     }
     if (!sequential) {
       uint32_t *cm = reinterpret_cast<uint32_t *>(h + cmap_off);
@@ -2421,34 +2501,27 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
         for (uint32_t b = hs[i].cta0; b < hs[i].cta0 + hs[i].nctas; b++) cm[b] = (uint32_t)i | ((uint32_t)tab_of[i] << 16);
     }
     std::memcpy(h + tabs_off, tabs.data(), sizeof(RankTab) * tabs.size());
-    std::memset(h + work_off, 0, 2 * work_b);
-    ck(cudaMemcpyAsync(d_sets, h, up, cudaMemcpyHostToDevice, stream));
-    ck(cudaEventRecord(done, stream));  // the buffer is reused after this copy
+    if (cudaMemcpyAsync(scratch, h, up, cudaMemcpyHostToDevice, stream) != cudaSuccess) rc = UNISON_ERR_CUDA;
+    if (cudaEventRecord(done, stream) != cudaSuccess) rc = UNISON_ERR_CUDA;  // the buffer is reused after this copy
     staging_release();
-    if (hist_b) ck(cudaMemsetAsync(hists, 0, 2 * hist_b, stream));
+    if (rc != UNISON_OK) {
+      cudaGetLastError();
+      return rc;
+    }
   }
-  ck(launch_rank_kernel(grid, d_sets, n_sets, sequential,
-                        sequential ? nullptr : reinterpret_cast<const uint32_t *>(scratch + cmap_off), d_tabs,
-                        scratch + work_off + work_b, work_b, hists + hist_b, hist_b, stream));
-  count_launches(1);
-  ck(cudaGetLastError());
+  rc = launch_rank_kernel(st, grid, reinterpret_cast<const RankSet *>(scratch + next_block(st) * desc_b), n_sets,
+                          sequential, sequential ? nullptr : reinterpret_cast<const uint32_t *>(scratch + cmap_off),
+                          d_tabs, none, zero_b, stream);
   if (rc == UNISON_OK) {
-    std::lock_guard<std::mutex> lock(g_plan_mu);
-    RankPlan &pl = g_plan[std::make_pair(dev, stream)];
+    RankPlan &pl = st.plan;
     pl.key = key;
-    pl.bytes = 2 * desc_b + cmap_b + tab_b + 2 * work_b + sets_b;
+    pl.desc_b = desc_b;
     pl.cmap_off = cmap_off;
     pl.tabs_off = tabs_off;
-    pl.hist_bytes = std::max<size_t>(2 * hist_b, 256);
-    pl.desc_b = desc_b;
-    pl.work_off = work_off;
-    pl.work_b = work_b;
-    pl.hist_b = hist_b;
-    pl.parity = 1;
-    pl.scratch = scratch;
-    pl.hists = hists;
+    pl.zero_b = zero_b;
     pl.grid = grid;
     pl.sequential = sequential;
+    st.planned = true;
   }
   return rc;
 }
@@ -2505,12 +2578,15 @@ extern "C" int unison_rank_merge(const void *gathered_dev, int n_shards, const u
   // scratch: descriptor and work words (one upload), sorted lists
   const size_t desc_b = align_up(sizeof(RankSet), 256), work_b = align_up(sizeof(RankWork), 256);
   const size_t lists_b = align_up(sizeof(uint64_t) * kLists * kMaxSel, 256) + align_up(sizeof(uint32_t) * kLists * kMaxSel, 256);
-  char *scratch = nullptr, *hists = nullptr;
+  StreamState *const state = stream_state(stream);
+  if (!state) return UNISON_ERR_CUDA;
+  std::lock_guard<std::mutex> lock(state->mu);
+  state->planned = false;  // the descriptor area is rewritten below
   {
-    plan_drop(stream);  // the descriptor area is rewritten below
-    const int ar = scratch_acquire(stream, desc_b + work_b + lists_b, 0, &scratch, &hists);
+    const int ar = grow(state->main, desc_b + work_b + lists_b, false, stream);
     if (ar != UNISON_OK) return ar;
   }
+  char *const scratch = state->main.p;
   s.work = reinterpret_cast<RankWork *>(scratch + desc_b);
   s.sorted = reinterpret_cast<uint64_t *>(scratch + desc_b + work_b);
   s.ssz = reinterpret_cast<uint32_t *>(scratch + desc_b + work_b + align_up(sizeof(uint64_t) * kLists * kMaxSel, 256));

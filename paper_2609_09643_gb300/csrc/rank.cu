@@ -67,6 +67,7 @@ constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr uint32_t kSampleCtas = 64;     // sampling CTAs per set, at most
 constexpr uint32_t kSampleQ = 4;         // samples per consumer thread
 constexpr uint32_t kLaunchSamples = 131072;  // samples per launch, about,
+constexpr uint32_t kSmallSample = 4096;  // the shortest lists, where this many samples give them
 constexpr uint32_t kSetSamples = 12288;      // or this many a set
 constexpr uint32_t kBins = 4096;         // histogram bins per list
 constexpr uint32_t kEndTile = 0xFFFFFFFFu;
@@ -818,11 +819,11 @@ __host__ __forceinline__ bool list_active(const RankSet &S, int L) {
   const uint32_t M = (L == 0) ? S.k : S.max_moves;
   return M > 0 && (L == 0 || S.budget > 0);
 }
-constexpr int kTargets = 4;
+constexpr int kTargets = 5;
 __host__ __forceinline__ uint64_t list_target_of(const RankSet &S, int L, int o) {
   const uint64_t M = (L == 0) ? S.k : S.max_moves;
-  const uint64_t mul[kTargets] = {2, 3, 4, 6};
-  return mul[o] * (M + 512);
+  const uint64_t mul[kTargets] = {2, 2, 3, 4, 6}, add[kTargets] = {128, 512, 512, 512, 512};
+  return mul[o] * (M + add[o]);
 }
 // The smallest rank whose chance of a shortfall is below 1e-6, for a ratio M /
 // target of at most q / 64 (q <= 32).
@@ -873,7 +874,7 @@ void plan_sample(RankSet &s, int n_sets) {
   const uint64_t cap = umin64((uint64_t)kPerCtaSamples * most, share);
   int o = 0;
   uint64_t ns = sample_size(s, 0);
-  while (ns > cap && o + 1 < kTargets) ns = sample_size(s, ++o);
+  while (ns > (o == 0 ? umin64(cap, kSmallSample) : cap) && o + 1 < kTargets) ns = sample_size(s, ++o);
   ns = umin64(ns, cap);
   // half a CTA's most a CTA where there are enough: the samples' latency is the
   // call's head
@@ -1444,15 +1445,25 @@ __device__ __noinline__ void fill(const RankSet &S, uint64_t *fin) {
 // zero (n_zero 16-byte words): the work words and sample histograms that the
 // stream's previous call used, zeroed here for its next one.
 // cmap (grouped launches): CTA b serves set cmap[b] & 0xFFFF, whose tables are
-// tabs[cmap[b] >> 16]; null for a sequential launch.  A call of one set brings
-// its descriptor and tables as a parameter (sets null): no upload precedes it.
-struct RankOne {
-  RankSet set;
-  RankTab tab;
+// tabs[cmap[b] >> 16]; null for a sequential launch.
+// pack (d_sets null): the call's descriptors, tables and CTA map as a launch
+// parameter, so that no upload precedes the kernel (it took 5 to 8 us of a
+// call).  Calls of one set take a pack of one, up to 64 sets with at most two
+// distinct tables a pack of 64 (about 20 KB of the 32 KB that a launch may
+// bring); others upload theirs.
+constexpr int kPackSets = 64, kPackTabs = 2;
+template <int kSets>
+struct RankPack {
+  RankSet set[kSets];
+  RankTab tab[kSets > 1 ? kPackTabs : 1];
+  uint8_t of_cta[kSets > 1 ? kMaxGroup : 8];  // the set of each CTA
+  uint8_t tab_of[kSets > 1 ? kSets : 8];
 };
+static_assert(sizeof(RankPack<kPackSets>) <= 30000, "a launch's parameters");
+template <int kSets>
 __global__ void __launch_bounds__(kCtaThreads, 3)
     rank_kernel(const RankSet *d_sets, int n_sets, int sequential, const uint32_t *cmap, const RankTab *tabs,
-                uint4 *zero, uint32_t n_zero, const __grid_constant__ RankOne one) {
+                uint4 *zero, uint32_t n_zero, const __grid_constant__ RankPack<kSets> pack) {
   extern __shared__ __align__(128) unsigned char dsm[];
   FilterStage *stage = reinterpret_cast<FilterStage *>(dsm);
   uint64_t *fin = reinterpret_cast<uint64_t *>(dsm);
@@ -1476,16 +1487,16 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
     const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
     for (uint32_t w = g; w < n_zero; w += gs) zero[w] = make_uint4(0u, 0u, 0u, 0u);
   }
-  const RankSet *const sets = d_sets ? d_sets : &one.set;
+  const RankSet *const sets = d_sets ? d_sets : pack.set;
   int s0, sstep;
   const RankTab *tab0 = nullptr;  // the first set's tables, when the map names them
   if (sequential) {
     s0 = blockIdx.x;
     sstep = gridDim.x;
   } else if (!d_sets) {
-    s0 = 0;
-    tab0 = &one.tab;
-    sstep = 1;
+    s0 = kSets > 1 ? pack.of_cta[blockIdx.x] : 0;
+    tab0 = &pack.tab[kSets > 1 ? pack.tab_of[s0] : 0];
+    sstep = n_sets;  // one set
   } else {
     const uint32_t e = __ldg(cmap + blockIdx.x);
     s0 = (int)(e & 0xFFFFu);
@@ -1955,14 +1966,17 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
 // each): CTA L selects list L's global top M (narrowed and sorted as in the
 // finish, carrying the sizes), writes it as the finish does, and the last list's CTA runs the
 // fill.  One CTA per list, consumer-sized (256 threads).
-__global__ void __launch_bounds__(kConsumers) rank_merge_kernel(const RankSet *Sp, const unsigned char *gathered,
-                                                                int n_shards, uint64_t stride) {
+__global__ void __launch_bounds__(kConsumers) rank_merge_kernel(const __grid_constant__ RankSet desc,
+                                                                const unsigned char *gathered, int n_shards,
+                                                                uint64_t stride, uint4 *zero, uint32_t n_zero) {
   extern __shared__ __align__(128) unsigned char dsm[];
   uint64_t *fin = reinterpret_cast<uint64_t *>(dsm);
   __shared__ SelectScratch ss;
   __shared__ unsigned int pre[kMaxShards + 1];
   __shared__ unsigned int last;
-  const RankSet &S = *Sp;
+  const RankSet &S = desc;
+  for (uint32_t w = blockIdx.x * kConsumers + threadIdx.x; w < n_zero; w += kLists * kConsumers)
+    zero[w] = make_uint4(0u, 0u, 0u, 0u);
   const int L = blockIdx.x;
   const uint32_t Mw = L == 0 ? S.k : S.max_moves;
   const bool active = (S.act >> L) & 1;
@@ -2108,6 +2122,8 @@ struct RankPlan {
   size_t zero_b = 0;  // bytes of a block that the call uses
   uint32_t grid = 0;
   int sequential = 0;
+  bool packed = false;
+  RankPack<kPackSets> pack[2];  // for each block
 };
 struct StreamState {
   std::mutex mu;  // held from the choice of a block to the launch that uses it
@@ -2239,16 +2255,20 @@ const LaunchCfg &launch_cfg() {
   std::lock_guard<std::mutex> lock(mu);
   if (!done[dev]) {
     LaunchCfg c;
-    int n_sm = 0, per_sm = 0, coop = 0;
+    int n_sm = 0, per_sm = 0, per_sm64 = 0, coop = 0;
     c.ok = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
            cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-           cudaFuncSetAttribute(rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem) ==
+           cudaFuncSetAttribute(rank_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem) ==
+               cudaSuccess &&
+           cudaFuncSetAttribute(rank_kernel<kPackSets>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem) ==
                cudaSuccess &&
            cudaFuncSetAttribute(rank_merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMergeSmem) ==
                cudaSuccess &&
-           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rank_kernel, kCtaThreads, kDynSmem) ==
+           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rank_kernel<1>, kCtaThreads, kDynSmem) ==
                cudaSuccess &&
-           per_sm > 0;
+           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm64, rank_kernel<kPackSets>, kCtaThreads, kDynSmem) ==
+               cudaSuccess &&
+           per_sm > 0 && per_sm64 >= per_sm;
     if (!c.ok) cudaGetLastError();
     c.ctas = (uint32_t)std::min(std::max(1, n_sm * per_sm), (int)kMaxGroup);
     cfgs[dev] = c;
@@ -2299,8 +2319,10 @@ void plan_key(std::vector<unsigned char> &k, const unison_records *sets, const u
 // the call uses), zeroing the other.  The caller holds st.mu and has passed
 // that block (next_block) to the descriptors.
 int next_block(const StreamState &st) { return st.dirty[0] == 0 ? 0 : 1; }
+template <int kSets>
 int launch_rank_kernel(StreamState &st, uint32_t grid, const RankSet *d_sets, int n_sets, int sequential,
-                       const uint32_t *cmap, const RankTab *tabs, const RankOne &one, size_t zb, cudaStream_t stream) {
+                       const uint32_t *cmap, const RankTab *tabs, const RankPack<kSets> &pack, size_t zb,
+                       cudaStream_t stream) {
   const int p = next_block(st);
   cudaError_t e;
   {
@@ -2315,8 +2337,8 @@ int launch_rank_kernel(StreamState &st, uint32_t grid, const RankSet *d_sets, in
     lc.stream = stream;
     lc.attrs = coop;
     lc.numAttrs = 1;
-    e = cudaLaunchKernelEx(&lc, rank_kernel, d_sets, n_sets, sequential, cmap, tabs,
-                           reinterpret_cast<uint4 *>(st.zero[1 - p].p), (uint32_t)(st.dirty[1 - p] / 16), one);
+    e = cudaLaunchKernelEx(&lc, rank_kernel<kSets>, d_sets, n_sets, sequential, cmap, tabs,
+                           reinterpret_cast<uint4 *>(st.zero[1 - p].p), (uint32_t)(st.dirty[1 - p] / 16), pack);
   }
   count_launches(1);
   if (e == cudaSuccess) e = cudaGetLastError();
@@ -2336,12 +2358,15 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
   if (!state) return UNISON_ERR_CUDA;
   StreamState &st = *state;
   std::lock_guard<std::mutex> lock(st.mu);
-  static const RankOne none{};
+  static const RankPack<1> none{};
   thread_local std::vector<unsigned char> key;
   if (n_sets > 1) {
     plan_key(key, sets, params, outs, n_sets, off, cands);
     if (st.planned && st.plan.key == key) {
       const RankPlan &pl = st.plan;
+      if (pl.packed)
+        return launch_rank_kernel(st, pl.grid, nullptr, n_sets, 0, nullptr, nullptr, pl.pack[next_block(st)], pl.zero_b,
+                                  stream);
       return launch_rank_kernel(
           st, pl.grid, reinterpret_cast<const RankSet *>(st.main.p + next_block(st) * pl.desc_b), n_sets, pl.sequential,
           pl.sequential ? nullptr : reinterpret_cast<const uint32_t *>(st.main.p + pl.cmap_off),
@@ -2473,10 +2498,12 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
               align_up(sizeof(uint64_t) * kLists * s.nctas * s.cr, 256);
     if (s.ns) hist_b += hist_set;
   }
-  const bool single = n_sets == 1;  // one descriptor goes as a launch parameter
-  const size_t desc_b = single ? 0 : align_up(sizeof(RankSet) * n_sets, 256);
-  const size_t cmap_b = sequential || single ? 0 : align_up(sizeof(uint32_t) * grid, 256);
-  const size_t tab_b = single ? 0 : align_up(sizeof(RankTab) * tabs.size(), 256);
+  // descriptors go as a launch parameter where they fit
+  const bool single = n_sets == 1;
+  const bool packed = single || (!sequential && n_sets <= kPackSets && tabs.size() <= (size_t)kPackTabs);
+  const size_t desc_b = packed ? 0 : align_up(sizeof(RankSet) * n_sets, 256);
+  const size_t cmap_b = sequential || packed ? 0 : align_up(sizeof(uint32_t) * grid, 256);
+  const size_t tab_b = packed ? 0 : align_up(sizeof(RankTab) * tabs.size(), 256);
   const size_t work_b = align_up(sizeof(RankWork) * n_sets, 256);
   const size_t zero_b = work_b + hist_b;
   st.planned = false;  // the scratch is rewritten below; the plan returns only if the launch succeeds
@@ -2514,10 +2541,33 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
   };
   if (single) {
     in_block(next_block(st));
-    RankOne one;
-    one.set = hs[0];
-    one.tab = tabs[0];
+    RankPack<1> one;
+    one.set[0] = hs[0];
+    one.tab[0] = tabs[0];
     return launch_rank_kernel(st, grid, nullptr, 1, 0, nullptr, nullptr, one, zero_b, stream);
+  }
+  if (packed) {
+    RankPlan &pl = st.plan;
+    for (int b = 0; b < 2; b++) {
+      in_block(b);
+      RankPack<kPackSets> &pk = pl.pack[b];
+      std::memcpy(pk.set, hs.data(), sizeof(RankSet) * n_sets);
+      std::memcpy(pk.tab, tabs.data(), sizeof(RankTab) * tabs.size());
+      for (int i = 0; i < n_sets; i++) {
+        pk.tab_of[i] = (uint8_t)tab_of[i];
+        std::memset(pk.of_cta + hs[i].cta0, i, hs[i].nctas);
+      }
+    }
+    rc = launch_rank_kernel(st, grid, nullptr, n_sets, 0, nullptr, nullptr, pl.pack[next_block(st)], zero_b, stream);
+    if (rc == UNISON_OK) {
+      pl.key = key;
+      pl.zero_b = zero_b;
+      pl.grid = grid;
+      pl.sequential = 0;
+      pl.packed = true;
+      st.planned = true;
+    }
+    return rc;
   }
   // one copy from pinned staging
   {
@@ -2556,6 +2606,7 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
     pl.zero_b = zero_b;
     pl.grid = grid;
     pl.sequential = sequential;
+    pl.packed = false;
     st.planned = true;
   }
   return rc;
@@ -2610,43 +2661,30 @@ extern "C" int unison_rank_merge(const void *gathered_dev, int n_shards, const u
   s.counts = o.counts;
   s.moved = o.moved_bytes;
   for (int L = 0; L < kLists; L++) s.act |= list_active(s, L) ? 1u << L : 0u;
-  // scratch: descriptor and work words (one upload), sorted lists
-  const size_t desc_b = align_up(sizeof(RankSet), 256), work_b = align_up(sizeof(RankWork), 256);
-  const size_t lists_b = align_up(sizeof(uint64_t) * kLists * kMaxSel, 256) + align_up(sizeof(uint32_t) * kLists * kMaxSel, 256);
-  StreamState *const state = stream_state(stream);
-  if (!state) return UNISON_ERR_CUDA;
-  std::lock_guard<std::mutex> lock(state->mu);
-  state->planned = false;  // the descriptor area is rewritten below
-  {
-    const int ar = grow(state->main, desc_b + work_b + lists_b, false, stream);
-    if (ar != UNISON_OK) return ar;
-  }
-  char *const scratch = state->main.p;
-  s.work = reinterpret_cast<RankWork *>(scratch + desc_b);
-  s.sorted = reinterpret_cast<uint64_t *>(scratch + desc_b + work_b);
-  s.ssz = reinterpret_cast<uint32_t *>(scratch + desc_b + work_b + align_up(sizeof(uint64_t) * kLists * kMaxSel, 256));
+  // scratch: sorted lists; work words in the zero block whose turn it is
+  const size_t work_b = align_up(sizeof(RankWork), 256);
+  const size_t vals_b = align_up(sizeof(uint64_t) * kLists * kMaxSel, 256);
+  const size_t lists_b = vals_b + align_up(sizeof(uint32_t) * kLists * kMaxSel, 256);
   const LaunchCfg &cfg = launch_cfg();
   if (!cfg.ok) return UNISON_ERR_CUDA;
-  int rc = UNISON_OK;
-  auto ck = [&](cudaError_t e) {
-    if (e != cudaSuccess && rc == UNISON_OK) rc = UNISON_ERR_CUDA;
-  };
-  {
-    const size_t up = desc_b + work_b;
-    unsigned char *h = nullptr;
-    cudaEvent_t done = nullptr;
-    const int sr = staging_acquire(up, &h, &done);
-    if (sr != UNISON_OK) return sr;
-    std::memset(h, 0, up);
-    std::memcpy(h, &s, sizeof(RankSet));
-    ck(cudaMemcpyAsync(scratch, h, up, cudaMemcpyHostToDevice, stream));
-    ck(cudaEventRecord(done, stream));
-    staging_release();
-  }
-  rank_merge_kernel<<<kLists, kConsumers, kMergeSmem, stream>>>(reinterpret_cast<const RankSet *>(scratch),
-                                                             static_cast<const unsigned char *>(gathered_dev), n_shards,
-                                                             (uint64_t)cand_bytes(p.k, p.max_moves));
+  StreamState *const state = stream_state(stream);
+  if (!state) return UNISON_ERR_CUDA;
+  StreamState &st = *state;
+  std::lock_guard<std::mutex> lock(st.mu);
+  st.planned = false;  // the scratch is rewritten below
+  int rc = grow(st.main, lists_b, false, stream);
+  if (rc == UNISON_OK) rc = grow_zero(st, work_b, stream);
+  if (rc != UNISON_OK) return rc;
+  const int b = next_block(st);
+  s.work = reinterpret_cast<RankWork *>(st.zero[b].p);
+  s.sorted = reinterpret_cast<uint64_t *>(st.main.p);
+  s.ssz = reinterpret_cast<uint32_t *>(st.main.p + vals_b);
+  rank_merge_kernel<<<kLists, kConsumers, kMergeSmem, stream>>>(
+      s, static_cast<const unsigned char *>(gathered_dev), n_shards, (uint64_t)cand_bytes(p.k, p.max_moves),
+      reinterpret_cast<uint4 *>(st.zero[1 - b].p), (uint32_t)(st.dirty[1 - b] / 16));
   count_launches(1);
-  ck(cudaGetLastError());
-  return rc;
+  if (cudaGetLastError() != cudaSuccess) return UNISON_ERR_CUDA;  // nothing ran: the blocks are as they were
+  st.dirty[b] = work_b;
+  st.dirty[1 - b] = 0;
+  return UNISON_OK;
 }

@@ -190,6 +190,18 @@ def test_selection_of_crowded_values(B, sigma, n):
         check(r, rec, p)
 
 
+@pytest.mark.parametrize("n_sets,n_tabs", [(2, 2), (64, 2), (65, 1), (64, 3)])
+def test_descriptors_with_the_launch_or_uploaded(B, sigma, n_sets, n_tabs):
+    """The most sets and distinct survival tables whose descriptors go with the
+    launch (64 and 2), and one more of each, which are uploaded."""
+    rng = np.random.default_rng(n_sets)
+    sigs = [np.clip(sigma.astype(np.int64) - 37 * j, 41, 4095).astype(np.uint16) for j in range(n_tabs)]
+    recs = [synth.make_records(200 + i, int(rng.integers(1, 6000))) for i in range(n_sets)]
+    ps = [prm(sigs[i % n_tabs], k=20, budget=4 * GIB, max_moves=30, free_s=5000) for i in range(n_sets)]
+    for r, rec, p in zip(run(B, recs, ps), recs, ps):
+        check(r, rec, p)
+
+
 def test_calls_of_changing_size_on_one_stream(B, sigma):
     """Single sets, which bring their descriptor with the launch, and batches,
     sampled and not, growing and shrinking in turn on one stream: each call

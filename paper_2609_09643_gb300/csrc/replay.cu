@@ -211,7 +211,7 @@ __global__ void key_stream_kernel(const ComboDesc *combos) {
       } else if (k + 1 < ts) {
         c.rk.a[c.rk.n - (b + ts - (s + 1)) + k] = key << 24 | ec;
       }
-      if (k + 1 == ts) c.rk.rank[ec] = c.rk.n + (c.n_sessions - 1 - s);
+      if (k + 1 == ts) c.rk.rank[ec] = c.rk.n + (c.n_sessions - 1 - s) + 1;
     }
   }
 }
@@ -1257,8 +1257,8 @@ __global__ void __launch_bounds__(32) replay_kernel(const ReplayDesc *descs, con
 
 // Replays of the slot form.  kOnly >= 0: every replay of the launch is a lean
 // one of that policy (no log, no slot limit); else each takes its own body.
-// kMap8: the launch's session maps hold one byte a session, else two.
-template <int kOnly, bool kMap8>
+// kForm: the launch's form (slot_maps).
+template <int kOnly, int kForm>
 __global__ void __launch_bounds__(32) slot_kernel(const ReplayDesc *descs, const uint32_t *order) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ReplayDesc Dsh;
@@ -1267,24 +1267,24 @@ __global__ void __launch_bounds__(32) slot_kernel(const ReplayDesc *descs, const
   if (lane == 0) Dsh = descs[order[blockIdx.x]];
   __syncwarp();
   if constexpr (kOnly >= 0) {
-    unison_slots::slot_replay<unison_slots::kRanked, kOnly, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+    unison_slots::slot_replay<unison_slots::kRanked, kOnly, true, kForm>(Dsh, Dsh.slot, bufs, smem, lane);
   } else {
     using unison_slots::kRanked;
     using unison_slots::slot_replay;
     if (Dsh.policy == UNISON_SPEAR_TIDE)
-      slot_replay<kRanked, UNISON_SPEAR_TIDE, false, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_SPEAR_TIDE, false, kForm>(Dsh, Dsh.slot, bufs, smem, lane);
     else if (Dsh.log || Dsh.max_sessions)
-      slot_replay<kRanked, -1, false, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, -1, false, kForm>(Dsh, Dsh.slot, bufs, smem, lane);
     else if (Dsh.policy == UNISON_SPEAR)
-      slot_replay<kRanked, UNISON_SPEAR, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_SPEAR, true, kForm>(Dsh, Dsh.slot, bufs, smem, lane);
     else if (Dsh.policy == UNISON_LRU)
-      slot_replay<kRanked, UNISON_LRU, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_LRU, true, kForm>(Dsh, Dsh.slot, bufs, smem, lane);
     else if (Dsh.policy == UNISON_BELADY)
-      slot_replay<kRanked, UNISON_BELADY, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_BELADY, true, kForm>(Dsh, Dsh.slot, bufs, smem, lane);
     else if (Dsh.policy == UNISON_TIMEOUT)
-      slot_replay<kRanked, UNISON_TIMEOUT, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_TIMEOUT, true, kForm>(Dsh, Dsh.slot, bufs, smem, lane);
     else
-      slot_replay<kRanked, UNISON_LRU_TIDE, true, kMap8>(Dsh, Dsh.slot, bufs, smem, lane);
+      slot_replay<kRanked, UNISON_LRU_TIDE, true, kForm>(Dsh, Dsh.slot, bufs, smem, lane);
   }
 }
 
@@ -1297,10 +1297,12 @@ __global__ void __launch_bounds__(32) slot_variant_kernel(const ReplayDesc *desc
   const int lane = threadIdx.x & 31;
   if (lane == 0) Dsh = descs[order[blockIdx.x]];
   __syncwarp();
-  if (Dsh.log || Dsh.max_sessions)
-    unison_slots::slot_replay<kMode, -1, false, false>(Dsh, Dsh.slot, bufs, smem, lane);
-  else
-    unison_slots::slot_replay<kMode, -1, true, false>(Dsh, Dsh.slot, bufs, smem, lane);
+  using namespace unison_slots;
+  const bool lean = !Dsh.log && !Dsh.max_sessions, st = Dsh.policy == UNISON_SPEAR_TIDE;
+  if (lean && st) slot_replay<kMode, UNISON_SPEAR_TIDE, true, kFormPlain>(Dsh, Dsh.slot, bufs, smem, lane);
+  else if (lean) slot_replay<kMode, UNISON_SPEAR, true, kFormPlain>(Dsh, Dsh.slot, bufs, smem, lane);
+  else if (st) slot_replay<kMode, UNISON_SPEAR_TIDE, false, kFormPlain>(Dsh, Dsh.slot, bufs, smem, lane);
+  else slot_replay<kMode, UNISON_SPEAR, false, kFormPlain>(Dsh, Dsh.slot, bufs, smem, lane);
 }
 
 // Lower median (element floor((n-1)/2) in sorted order) by MSB-first radix select.
@@ -1572,32 +1574,45 @@ uint64_t rank_values(const ReplayPlan &P, size_t c, const unison_trace *tr) {
   return std::get<6>(P.combos[c]) ? tr->n_events : tr->n_turns - tr->n_sessions;
 }
 
-ReplayKernel slot_kernel_of(bool lean_st, bool map8) {
-  if (lean_st) return map8 ? slot_kernel<UNISON_SPEAR_TIDE, true> : slot_kernel<UNISON_SPEAR_TIDE, false>;
-  return map8 ? slot_kernel<-1, true> : slot_kernel<-1, false>;
+ReplayKernel slot_kernel_of(bool lean_st, uint32_t form) {
+  using namespace unison_slots;
+  if (lean_st) {
+    if (form == kFormMap8) return slot_kernel<UNISON_SPEAR_TIDE, kFormMap8>;
+    return form == kFormDeep ? slot_kernel<UNISON_SPEAR_TIDE, kFormDeep> : slot_kernel<UNISON_SPEAR_TIDE, kFormPlain>;
+  }
+  if (form == kFormMap8) return slot_kernel<-1, kFormMap8>;
+  return form == kFormDeep ? slot_kernel<-1, kFormDeep> : slot_kernel<-1, kFormPlain>;
 }
 
-// The session maps of a slot group: two bytes a session name the slot
-// directly; one byte (its low eight bits, the slot told apart by the session
-// it holds) when two would not fit or would need more waves of CTAs.
+// The form of a slot group's launch.  Session maps: two bytes a session name
+// the slot directly; one byte (its low eight bits, the slot told apart by the
+// session it holds) when two would not fit or would need more waves of CTAs.
+// Passes over the words are deep when every replay's trace has at least four
+// sessions a slot: its tiers then fill with sessions, where otherwise far fewer
+// than the slots are ever in use (40,000 sessions over 547 slots: 574 ms plain,
+// 500 ms deep; the sweep's 1,415 over up to 527, of which about 160 are used:
+// 27.4 ms plain, 28.2 ms deep).
 void slot_maps(const unison_trace *const *traces, const unison_replay_params *params, size_t smem_limit,
                std::vector<uint32_t> &group, bool lean_st, size_t &smem, ReplayPlan &P) {
+  using namespace unison_slots;
   size_t most16 = 0, most8 = 0;
+  bool deep = true;
   for (uint32_t r : group) {
     const uint32_t S = traces[params[r].trace_idx]->n_sessions, n = P.slot[r].nslots;
     const bool wide = params[r].policy != UNISON_SPEAR_TIDE;
-    most16 = std::max(most16, unison_slots::slot_bytes(n, S, wide, false));
-    most8 = std::max(most8, unison_slots::slot_bytes(n, S, wide, true));
+    most16 = std::max(most16, slot_bytes(n, S, wide, false));
+    most8 = std::max(most8, slot_bytes(n, S, wide, true));
+    deep &= n > 128 && S / 4 >= n;
   }
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const bool narrow =
-      most16 > smem_limit ||
-      (group.size() > (size_t)sms && smem_waves(slot_kernel_of(lean_st, false), group.size(), most16) >
-                                         smem_waves(slot_kernel_of(lean_st, true), group.size(), most8));
-  for (uint32_t r : group) P.slot[r].map8 = narrow ? 1u : 0u;
-  smem = narrow ? most8 : most16;
+  uint32_t form = deep ? kFormDeep : kFormPlain;
+  if (most16 > smem_limit || (group.size() > (size_t)sms && smem_waves(slot_kernel_of(lean_st, form), group.size(), most16) >
+                                                               smem_waves(slot_kernel_of(lean_st, kFormMap8), group.size(), most8)))
+    form = kFormMap8;
+  for (uint32_t r : group) P.slot[r].form = form;
+  smem = form == kFormMap8 ? most8 : most16;
 }
 
 // slots: whether replays may take the slot form (false: the layout of the
@@ -1902,10 +1917,10 @@ int launch_replays(const ReplayPlan &P, char *scratch, const std::vector<ComboDe
       ReplayKernel k;
       size_t n, smem;
     };
-    auto map8 = [&](const std::vector<uint32_t> &g) { return !g.empty() && P.slot[g[0]].map8; };
+    auto form = [&](const std::vector<uint32_t> &g) { return g.empty() ? 0u : P.slot[g[0]].form; };
     const Launch all[] = {
-        {slot_kernel_of(true, map8(P.in_slot_st)), P.in_slot_st.size(), P.smem_slot_st},
-        {slot_kernel_of(false, map8(P.in_slot_mix)), P.in_slot_mix.size(), P.smem_slot_mix},
+        {slot_kernel_of(true, form(P.in_slot_st)), P.in_slot_st.size(), P.smem_slot_st},
+        {slot_kernel_of(false, form(P.in_slot_mix)), P.in_slot_mix.size(), P.smem_slot_mix},
         {slot_variant_kernel<unison_slots::kOnline>, P.in_slot_online.size(), P.smem_slot_online},
         {slot_variant_kernel<unison_slots::kStale>, P.in_slot_stale.size(), P.smem_slot_stale},
         {replay_kernel<false, kKeyStream>, P.in_list.size(), P.max_smem_list},

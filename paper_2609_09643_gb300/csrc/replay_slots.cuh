@@ -16,24 +16,28 @@
 //
 // What bounds it: the dependence chain of one warp.  The chain of a choice is
 // a 16-byte shared load a lane for up to 128 slots, three maxima, one REDUX
-// and the load of the winner's size.  158 warp instructions an event, and 842
-// cycles for the slowest of 152 sweep replays (27.3 ms): an instruction costs
-// about 2.7 cycles to issue and wait for, so what follows from an arrival's
-// class is left to account_arrivals and branches are kept few (188
-// instructions, 1,010 cycles, 32.8 ms with the accounting in the loop).
-// Sorted lists of 64-bit keys in the warp's registers, which this replaced,
-// took 375 and 1,513 (49.2 ms).  Tried and not kept: the words' extremes found
-// at the top of every event, beside the session's lookup (185 instructions,
-// sweep 32.5 -> 34.3 ms); 256 words loaded at once (34.0 ms).
+// and the load of the winner's size.  An instruction costs about 2.7 cycles to
+// issue and wait for, and the event loop runs from the instruction cache beside
+// the scheduler only while it is short.  So what follows from an arrival's
+// class is left to account_arrivals, branches and rarely taken tests are kept
+// few, and loops stay rolled.  The 1,024-replay sweep's launch, one GB300: 57.5
+// ms with sorted lists of 64-bit keys in the warp's registers (375 instructions
+// an event), 38.7 with slots (188), 32.1 with the accounting taken out (158),
+// 27.9 with loops rolled, errors leaving by a jump, the bypass apart and each
+// event's record found by a pointer.  Tried and not kept: the words' extremes
+// found at the top of every event, beside the session's lookup (34.3 against
+// 32.5 ms); 256 words loaded at once in every pass (34.0); HBM's making of room
+// out of line for its second caller (48 against 31); the fast tier's payload
+// loaded only when a swap is tried (31.6 against 31.2).
 //
 // Two variants keep a second array of words.  A stale-snapshot replay ranks by
 // the snapshot's ranks and keeps the live ones beside them, so a choice is
 // compared with the live one by a second pass and a sync rewrites the words of
 // the sessions that changed, a lane each (16 replays over the four sync modes
-// 151 -> 55 ms).  Under the online hazard table keys change while sessions are
+// 151 -> 46 ms).  Under the online hazard table keys change while sessions are
 // resident, so a word is the key itself in 64 bits, and a rebuilt table rewrites
 // every word in place where sorted lists had to be sorted again (6 online, 6
-// offline and 6 LRU replays with logs 116 -> 51 ms).
+// offline and 6 LRU replays with logs 116 -> 49 ms).
 #pragma once
 
 #include "common.cuh"
@@ -70,7 +74,7 @@ struct SlotEvent {
 };
 constexpr uint32_t kRing = 128;
 struct SlotBufs {
-  SlotEvent e[kRing];
+  SlotEvent e[kRing + 1];  // the last mirrors the first event's word, so that a batch's end reads on
 };
 
 // What one replay of the slot form reads besides its ReplayDesc.
@@ -79,9 +83,13 @@ struct SlotDesc {
   uint32_t cap_s, cap_h;  // tokens, at most the sum of every session's largest size (< 2^31)
   uint32_t nslots;        // slots the replay can need
   uint32_t sbits;         // slot bits of a word
-  uint32_t map8;          // 1: the session map holds the slot's low byte only
+  uint32_t form;          // kForm*
   uint32_t serial;        // 1: the prefill queue's times may pass 2^63 ns (account_arrivals)
 };
+
+// Forms of a launch: the session map's width, and how the words are passed over
+// (see slot_maps in replay.cu).
+constexpr int kFormPlain = 0, kFormDeep = 1, kFormMap8 = 2;
 
 // What the event loop notes of each arrival, one byte in arrival order: the
 // request class, whether TIDE had promoted the session, and where it was
@@ -91,7 +99,9 @@ constexpr uint32_t kClassCold = 0, kClassFast = 1, kClassHbm = 2, kClassMiss = 3
 constexpr uint32_t kNotePromoted = 4, kNotePlaceShift = 3;  // bits 3-4: 0 fast tier, 1 HBM, 2 bypassed
 
 // Bytes of shared memory of one replay: words, payloads, free slots, map.
-__host__ __device__ inline size_t slot_words(uint32_t nslots) { return ((size_t)nslots + 127) / 128 * 128; }
+__host__ __device__ inline size_t slot_words(uint32_t nslots) {
+  return nslots <= 128 ? 128 : 128 + ((size_t)nslots - 128 + 255) / 256 * 256;
+}
 __host__ inline size_t slot_bytes(uint32_t nslots, uint32_t n_sessions, bool wide, bool map8) {
   const size_t pay = (size_t)nslots * (wide ? 16 : 8), fr = ((size_t)nslots * 2 + 15) / 16 * 16;
   const size_t map = ((size_t)n_sessions * (map8 ? 1 : 2) + 15) / 16 * 16;
@@ -109,7 +119,7 @@ constexpr int kStale = 1;   // ranks of a register-file snapshot (eq. stale)
 constexpr int kOnline = 2;  // keys under the online hazard table (Sec. V-F)
 
 // The replay's state.  kLean: no decision log and no slot limit.
-template <int kMode, bool kLean, bool kWide>
+template <int kMode, bool kLean, bool kWide, bool kDeep>
 struct Slots {
   uint32_t *W;
   uint32_t *L;            // kStale: the words by live ranks; kOnline: the words' low halves
@@ -130,13 +140,16 @@ struct Slots {
 };
 
 // h = (h ^ (event << 32 | kind << 24 | session)) * 0x100000001B3 mod 2^64.
-template <int kMode, bool kLean, bool kWide>
-__device__ __forceinline__ void decide(Slots<kMode, kLean, kWide> &st, uint32_t kind, uint32_t s, int lane) {
+template <int kMode, bool kLean, bool kWide, bool kDeep>
+__device__ __forceinline__ void decide(Slots<kMode, kLean, kWide, kDeep> &st, uint32_t kind, uint32_t s, int lane) {
   static_assert(kFnvPrime == (1ull << 40 | 0x1B3u), "the multiplication below");
   const uint32_t lo = st.h_lo ^ (s | kind << 24), hi = st.h_hi ^ st.e;
   const uint64_t m = (uint64_t)lo * 0x1B3u;
   st.h_lo = (uint32_t)m;
-  st.h_hi = (uint32_t)(m >> 32) + hi * 0x1B3u + (lo << 8);
+  // (one multiply-add each; written as a shift, lo << 8 took an instruction more)
+  uint32_t t = (uint32_t)(m >> 32) + hi * 0x1B3u;
+  asm("mad.lo.u32 %0, %1, 256, %0;" : "+r"(t) : "r"(lo));
+  st.h_hi = t;
   if constexpr (!kLean) {
     static_assert(sizeof(unison_decision) == sizeof(uint2), "a log entry: event, kind << 24 | session");
     if (st.log_left) {
@@ -146,43 +159,77 @@ __device__ __forceinline__ void decide(Slots<kMode, kLean, kWide> &st, uint32_t 
   }
 }
 
-// Extremes over the words of every slot handed out so far (a multiple of 128
-// words; the words past them are 0).
+// Extremes over the words of every slot handed out so far; the words past them
+// are 0.  A pass takes 128 words, 4 a lane; past the first 128, kDeep takes 256
+// at a time, two loads in flight.  Loops are kept rolled: unrolled by the
+// compiler they made the event loop 1,400 instructions long instead of 816,
+// past what the instruction cache next to the scheduler holds (30 paper-scale
+// replays 31.6 -> 28.0 ms).
+__device__ __forceinline__ uint32_t max4(uint4 v) { return max(max(v.x, v.y), max(v.z, v.w)); }
+__device__ __forceinline__ uint32_t max4(uint32_t m, uint4 v) { return max(max(m, max(v.x, v.y)), max(v.z, v.w)); }
+__device__ __forceinline__ uint4 flip4(uint4 v) {
+  return make_uint4(v.x ^ kFastBit, v.y ^ kFastBit, v.z ^ kFastBit, v.w ^ kFastBit);
+}
+__device__ __forceinline__ uint32_t min4_less1(uint4 v) {
+  return min(min(v.x - 1u, v.y - 1u), min(v.z - 1u, v.w - 1u));
+}
+__device__ __forceinline__ uint32_t min4_less1(uint32_t m, uint4 v) {
+  return min(min(m, min(v.x - 1u, v.y - 1u)), min(v.z - 1u, v.w - 1u));
+}
+template <bool kDeep>
 __device__ __forceinline__ uint32_t max_of(const uint32_t *W, uint32_t fresh, int lane) {
   const uint4 *w4 = reinterpret_cast<const uint4 *>(W) + lane;
   uint4 v = w4[0];
-  uint32_t m = max(max(v.x, v.y), max(v.z, v.w));
-  for (uint32_t q = 128; q < fresh; q += 128) {
+  uint32_t m = max4(v);
+#pragma unroll 1
+  for (uint32_t q = 128; q < fresh; q += kDeep ? 256 : 128) {
     w4 += 32;
     v = *w4;
-    m = max(max(m, max(v.x, v.y)), max(v.z, v.w));
+    if constexpr (kDeep) {
+      w4 += 32;
+      m = max4(m, *w4);
+    }
+    m = max4(m, v);
   }
   return __reduce_max_sync(kAll, m);
 }
 // The largest word with the tier bit flipped: > kFastBit if there is an HBM word.
+template <bool kDeep>
 __device__ __forceinline__ uint32_t max_hbm_of(const uint32_t *W, uint32_t fresh, int lane) {
   const uint4 *w4 = reinterpret_cast<const uint4 *>(W) + lane;
   uint4 v = w4[0];
-  uint32_t m = max(max(v.x ^ kFastBit, v.y ^ kFastBit), max(v.z ^ kFastBit, v.w ^ kFastBit));
-  for (uint32_t q = 128; q < fresh; q += 128) {
+  uint32_t m = max4(flip4(v));
+#pragma unroll 1
+  for (uint32_t q = 128; q < fresh; q += kDeep ? 256 : 128) {
     w4 += 32;
     v = *w4;
-    m = max(max(m, max(v.x ^ kFastBit, v.y ^ kFastBit)), max(v.z ^ kFastBit, v.w ^ kFastBit));
+    if constexpr (kDeep) {
+      w4 += 32;
+      m = max4(m, flip4(*w4));
+    }
+    m = max4(m, flip4(v));
   }
   return __reduce_max_sync(kAll, m);
 }
 // The largest word, and the smallest word above 0 less 1 (below
 // kFastBit - 1 if there is an HBM word).
+template <bool kDeep>
 __device__ __forceinline__ void extremes_of(const uint32_t *W, uint32_t fresh, uint32_t &mx, uint32_t &mn, int lane) {
   const uint4 *w4 = reinterpret_cast<const uint4 *>(W) + lane;
   uint4 v = w4[0];
-  uint32_t a = max(max(v.x, v.y), max(v.z, v.w));
-  uint32_t b = min(min(v.x - 1u, v.y - 1u), min(v.z - 1u, v.w - 1u));
-  for (uint32_t q = 128; q < fresh; q += 128) {
+  uint32_t a = max4(v), b = min4_less1(v);
+#pragma unroll 1
+  for (uint32_t q = 128; q < fresh; q += kDeep ? 256 : 128) {
     w4 += 32;
     v = *w4;
-    a = max(max(a, max(v.x, v.y)), max(v.z, v.w));
-    b = min(min(b, min(v.x - 1u, v.y - 1u)), min(v.z - 1u, v.w - 1u));
+    if constexpr (kDeep) {
+      w4 += 32;
+      const uint4 u = *w4;
+      a = max4(a, u);
+      b = min4_less1(b, u);
+    }
+    a = max4(a, v);
+    b = min4_less1(b, v);
   }
   mx = __reduce_max_sync(kAll, a);
   mn = __reduce_min_sync(kAll, b);
@@ -202,27 +249,36 @@ __device__ __forceinline__ uint64_t online_word(uint64_t key, uint32_t s) {
 // kOnlineLive and L (the first below kOnlineLive if there is one).
 __device__ __forceinline__ uint64_t online_max(const uint32_t *W, const uint32_t *L, uint32_t fresh, uint32_t flip,
                                                int lane) {
-  uint64_t m = 0;
-  for (uint32_t i = 4 * lane, q = 0; q == 0 || q < fresh; q += 128, i += 128) {
-    const uint4 w = *reinterpret_cast<const uint4 *>(W + i), l = *reinterpret_cast<const uint4 *>(L + i);
-    const uint64_t a = max((uint64_t)(w.x ^ flip) << 32 | l.x, (uint64_t)(w.y ^ flip) << 32 | l.y);
-    const uint64_t b = max((uint64_t)(w.z ^ flip) << 32 | l.z, (uint64_t)(w.w ^ flip) << 32 | l.w);
-    m = max(m, max(a, b));
-  }
+  const uint4 *w4 = reinterpret_cast<const uint4 *>(W) + lane, *l4 = reinterpret_cast<const uint4 *>(L) + lane;
+  auto of = [&](uint4 w, uint4 l) {
+    return max(max((uint64_t)(w.x ^ flip) << 32 | l.x, (uint64_t)(w.y ^ flip) << 32 | l.y),
+               max((uint64_t)(w.z ^ flip) << 32 | l.z, (uint64_t)(w.w ^ flip) << 32 | l.w));
+  };
+  uint64_t m = of(*w4, *l4);
+#pragma unroll 1
+  for (uint32_t q = 128; q < fresh; q += 128) m = max(m, of(*(w4 += 32), *(l4 += 32)));
   const uint32_t hi = __reduce_max_sync(kAll, (uint32_t)(m >> 32));
   return (uint64_t)hi << 32 | __reduce_max_sync(kAll, (uint32_t)(m >> 32) == hi ? (uint32_t)m : 0u);
 }
 // Both at once: the most evictable fast-tier word and the least evictable HBM one.
 __device__ __forceinline__ void online_ends(const uint32_t *W, const uint32_t *L, uint32_t fresh, uint64_t &top,
                                             uint64_t &low, int lane) {
-  uint64_t m = 0, n = ~0ull;
-  for (uint32_t i = 4 * lane, q = 0; q == 0 || q < fresh; q += 128, i += 128) {
-    const uint4 w = *reinterpret_cast<const uint4 *>(W + i), l = *reinterpret_cast<const uint4 *>(L + i);
-    constexpr uint32_t x = kOnlineLive;
-    m = max(m, max(max((uint64_t)w.x << 32 | l.x, (uint64_t)w.y << 32 | l.y),
-                   max((uint64_t)w.z << 32 | l.z, (uint64_t)w.w << 32 | l.w)));
-    n = min(n, min(min((uint64_t)(w.x ^ x) << 32 | l.x, (uint64_t)(w.y ^ x) << 32 | l.y),
-                   min((uint64_t)(w.z ^ x) << 32 | l.z, (uint64_t)(w.w ^ x) << 32 | l.w)));
+  const uint4 *w4 = reinterpret_cast<const uint4 *>(W) + lane, *l4 = reinterpret_cast<const uint4 *>(L) + lane;
+  constexpr uint32_t x = kOnlineLive;
+  auto most = [&](uint4 w, uint4 l) {
+    return max(max((uint64_t)w.x << 32 | l.x, (uint64_t)w.y << 32 | l.y),
+               max((uint64_t)w.z << 32 | l.z, (uint64_t)w.w << 32 | l.w));
+  };
+  auto least = [&](uint4 w, uint4 l) {
+    return min(min((uint64_t)(w.x ^ x) << 32 | l.x, (uint64_t)(w.y ^ x) << 32 | l.y),
+               min((uint64_t)(w.z ^ x) << 32 | l.z, (uint64_t)(w.w ^ x) << 32 | l.w));
+  };
+  uint64_t m = most(*w4, *l4), n = least(*w4, *l4);
+#pragma unroll 1
+  for (uint32_t q = 128; q < fresh; q += 128) {
+    const uint4 w = *(w4 += 32), l = *(l4 += 32);
+    m = max(m, most(w, l));
+    n = min(n, least(w, l));
   }
   const uint32_t hi = __reduce_max_sync(kAll, (uint32_t)(m >> 32)), lo = __reduce_min_sync(kAll, (uint32_t)(n >> 32));
   top = (uint64_t)hi << 32 | __reduce_max_sync(kAll, (uint32_t)(m >> 32) == hi ? (uint32_t)m : 0u);
@@ -301,33 +357,33 @@ struct Choice {
   uint32_t slot;
   uint64_t order;
 };
-template <int kMode, bool kLean, bool kWide>
-__device__ __forceinline__ Choice most_evictable_fast(const Slots<kMode, kLean, kWide> &st, const uint16_t *map,
+template <int kMode, bool kLean, bool kWide, bool kDeep>
+__device__ __forceinline__ Choice most_evictable_fast(const Slots<kMode, kLean, kWide, kDeep> &st, const uint16_t *map,
                                                       int lane) {
   if constexpr (kMode == kOnline) {
     const uint64_t m = online_max(st.W, st.L, st.fresh, 0u, lane);
     const bool any = m >> 63 != 0;
     return {any, any ? map[kOnlineIds - ((uint32_t)m & kOnlineIds)] : 0u, m & ~(1ull << 63)};
   } else {
-    const uint32_t w = max_of(st.W, st.fresh, lane);
+    const uint32_t w = max_of<kDeep>(st.W, st.fresh, lane);
     return {(w & kFastBit) != 0, w & st.smask, w & ~kFastBit};
   }
 }
-template <int kMode, bool kLean, bool kWide>
-__device__ __forceinline__ Choice most_evictable_hbm(const Slots<kMode, kLean, kWide> &st, const uint16_t *map,
+template <int kMode, bool kLean, bool kWide, bool kDeep>
+__device__ __forceinline__ Choice most_evictable_hbm(const Slots<kMode, kLean, kWide, kDeep> &st, const uint16_t *map,
                                                      int lane) {
   if constexpr (kMode == kOnline) {
     const uint64_t m = online_max(st.W, st.L, st.fresh, kFastBit, lane);  // (an empty slot: kFastBit, 0)
     const bool any = m > (1ull << 63);
     return {any, any ? map[kOnlineIds - ((uint32_t)m & kOnlineIds)] : 0u, m & ~(1ull << 63)};
   } else {
-    const uint32_t m = max_hbm_of(st.W, st.fresh, lane);
+    const uint32_t m = max_hbm_of<kDeep>(st.W, st.fresh, lane);
     return {m > kFastBit, m & st.smask, m & ~kFastBit};
   }
 }
 // The words of a choice in the other tier, or none.
-template <int kMode, bool kLean, bool kWide>
-__device__ __forceinline__ void set_word(Slots<kMode, kLean, kWide> &st, uint32_t slot, bool fast, uint64_t order) {
+template <int kMode, bool kLean, bool kWide, bool kDeep>
+__device__ __forceinline__ void set_word(Slots<kMode, kLean, kWide, kDeep> &st, uint32_t slot, bool fast, uint64_t order) {
   const uint32_t bit = fast ? kFastBit : 0u;
   if constexpr (kMode == kOnline) {
     st.W[slot] = (uint32_t)(order >> 32) | bit;
@@ -337,15 +393,15 @@ __device__ __forceinline__ void set_word(Slots<kMode, kLean, kWide> &st, uint32_
     if constexpr (kMode == kStale) st.L[slot] = (st.L[slot] & ~kFastBit) | bit;
   }
 }
-template <int kMode, bool kLean, bool kWide>
-__device__ __forceinline__ void clear_word(Slots<kMode, kLean, kWide> &st, uint32_t slot) {
+template <int kMode, bool kLean, bool kWide, bool kDeep>
+__device__ __forceinline__ void clear_word(Slots<kMode, kLean, kWide, kDeep> &st, uint32_t slot) {
   st.W[slot] = 0u;
   if constexpr (kMode != kRanked) st.L[slot] = 0u;
 }
 
 // kStale: a choice (slot) against the live ranks' over the same sessions.
-template <int kMode, bool kLean, bool kWide>
-__device__ __forceinline__ void count_victim(Slots<kMode, kLean, kWide> &st, uint32_t slot, uint32_t live_word) {
+template <int kMode, bool kLean, bool kWide, bool kDeep>
+__device__ __forceinline__ void count_victim(Slots<kMode, kLean, kWide, kDeep> &st, uint32_t slot, uint32_t live_word) {
   if constexpr (kMode == kStale) {
     st.vict_n++;
     st.vict_diff += (live_word & st.smask) != slot;
@@ -373,15 +429,15 @@ __device__ __forceinline__ uint2 payload(const St &st, uint32_t slot) {
 // Room in HBM for `size` tokens against its unpinned residents: evicts the
 // most evictable ones, only those above `d` (a session demoted out of the fast
 // tier; without one every resident is above).  False when the next one is not.
-template <int kMode, bool kLean, bool kWide>
-__device__ __forceinline__ bool make_hbm_room(Slots<kMode, kLean, kWide> &st, const uint16_t *map, uint32_t size,
+template <int kMode, bool kLean, bool kWide, bool kDeep>
+__device__ __forceinline__ bool make_hbm_room(Slots<kMode, kLean, kWide, kDeep> &st, const uint16_t *map, uint32_t size,
                                               const Choice &d, int lane) {
   while (size > st.free_h) {
     const Choice v = most_evictable_hbm(st, map, lane);
     const bool drop = !v.any || (d.any && d.order > v.order);
     if constexpr (kMode == kStale) {
       // the live choice: among HBM's sessions and the demoted one
-      uint32_t live = max_hbm_of(st.L, st.fresh, lane);
+      uint32_t live = max_hbm_of<kDeep>(st.L, st.fresh, lane);
       live = live > kFastBit ? live & ~kFastBit : 0u;
       if (d.any) live = max(live, st.L[d.slot] & ~kFastBit);
       count_victim(st, drop ? d.slot : v.slot, live);
@@ -451,8 +507,8 @@ __device__ __forceinline__ void expire_slots(St &st, uint32_t now, uint32_t ttl,
 // of Algorithm 1 has it: phase 1 promotes the least evictable HBM sessions
 // into free fast-tier space, phase 2 swaps the least evictable HBM session
 // with the most evictable fast-tier one.  Returns the bytes moved.
-template <int kMode, bool kLean, bool kWide>
-__device__ __forceinline__ uint64_t tide_slots(Slots<kMode, kLean, kWide> &st, const uint16_t *map, uint64_t budget,
+template <int kMode, bool kLean, bool kWide, bool kDeep>
+__device__ __forceinline__ uint64_t tide_slots(Slots<kMode, kLean, kWide, kDeep> &st, const uint16_t *map, uint64_t budget,
                                                uint32_t kvb, int lane) {
   uint64_t rem = budget;
   bool fill = true;  // phase 1
@@ -466,44 +522,37 @@ __device__ __forceinline__ uint64_t tide_slots(Slots<kMode, kLean, kWide> &st, c
       dc = {fast, fast ? map[kOnlineIds - ((uint32_t)top & kOnlineIds)] : 0u, top & ~(1ull << 63)};
     } else {
       uint32_t mx, mn;
-      extremes_of(st.W, st.fresh, mx, mn, lane);
+      extremes_of<kDeep>(st.W, st.fresh, mx, mn, lane);
       pc = {mn < kFastBit - 1u, (mn + 1u) & st.smask, mn + 1u};
       dc = {(mx & kFastBit) != 0, mx & st.smask, mx & ~kFastBit};  // (a valid slot even when mx names none)
     }
-    if (!pc.any) break;
+    // (without an HBM session pc names a valid slot all the same)
     const uint2 p = *reinterpret_cast<const uint2 *>(&st.P[pc.slot]);
     const uint2 d = payload(st, dc.slot);
     const uint32_t sp = p.x & kSizeBits, pid = p.y & kIdMask;
+    const uint32_t sd = d.x & kSizeBits, did = d.y & kIdMask;
     uint64_t by = (uint64_t)sp * kvb;
-    fill = fill && by <= rem && sp <= st.free_s;
+    fill = fill && pc.any && by <= rem && sp <= st.free_s;
     if (!fill) {
       // phase 2: the swap is legal and the demoted session the more evictable
-      const uint32_t sd = d.x & kSizeBits, did = d.y & kIdMask;
       by += (uint64_t)sd * kvb;
-      const bool swap = dc.any && dc.order > pc.order && by <= rem && sp <= st.free_s + sd && sd <= st.free_h + sp;
-      if (!swap) break;
-      if constexpr (kMode == kStale) {
-        uint32_t mx, mn;
-        extremes_of(st.L, st.fresh, mx, mn, lane);
-        st.prom_n++;
-        st.prom_diff += ((mn + 1u) & st.smask) != pc.slot;
-        count_victim(st, dc.slot, mx);
-      }
+      if (!(pc.any && dc.any && dc.order > pc.order && by <= rem && sp <= st.free_s + sd && sd <= st.free_h + sp)) break;
+    }
+    if constexpr (kMode == kStale) {
+      uint32_t mx, mn;
+      extremes_of<kDeep>(st.L, st.fresh, mx, mn, lane);
+      st.prom_n++;
+      st.prom_diff += ((mn + 1u) & st.smask) != pc.slot;
+      if (!fill) count_victim(st, dc.slot, mx);
+    }
+    decide(st, UNISON_KIND_PROMOTE, pid, lane);
+    if (!fill) {
       set_word(st, dc.slot, false, dc.order);
       st.P[dc.slot].v.y = did;
       st.free_s += sd;
       st.free_h -= sd;
       st.n_tide_demote++;
-      decide(st, UNISON_KIND_PROMOTE, pid, lane);
       decide(st, UNISON_KIND_TIDE_DEMOTE, did, lane);
-    } else {
-      if constexpr (kMode == kStale) {
-        uint32_t mx, mn;
-        extremes_of(st.L, st.fresh, mx, mn, lane);
-        st.prom_n++;
-        st.prom_diff += ((mn + 1u) & st.smask) != pc.slot;
-      }
-      decide(st, UNISON_KIND_PROMOTE, pid, lane);
     }
     rem -= by;
     st.free_s -= sp;
@@ -520,17 +569,17 @@ __device__ __forceinline__ uint64_t tide_slots(Slots<kMode, kLean, kWide> &st, c
 // few (each costs an issue slot and a fetch, and one warp hides neither):
 // classes and tiers are selected, and the loops that make room and migrate are
 // the only ones an ordinary event passes.
-template <int kMode, int kPol, bool kLean, bool kMap8, class Desc>
+template <int kMode, int kPol, bool kLean, int kForm, class Desc>
 __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, SlotBufs &bufs, unsigned char *smem,
                                             int lane) {
-  constexpr bool kWide = kPol != UNISON_SPEAR_TIDE;
+  constexpr bool kWide = kMode != kRanked || kPol != UNISON_SPEAR_TIDE, kMap8 = kForm == kFormMap8, kDeep = kForm != kFormPlain;
   const uint32_t policy = kPol >= 0 ? (uint32_t)kPol : D.policy;
   const bool spear = kMode != kRanked || policy == UNISON_SPEAR || policy == UNISON_SPEAR_TIDE;
   const bool tide_on = policy == UNISON_SPEAR_TIDE || policy == UNISON_LRU_TIDE;
   const bool belady = kMode == kRanked && policy == UNISON_BELADY;
   const bool timeout = kMode == kRanked && policy == UNISON_TIMEOUT && D.ttl != 0xFFFFFFFFu;
 
-  Slots<kMode, kLean, kWide> st;
+  Slots<kMode, kLean, kWide, kDeep> st;
   const uint32_t nslots = Q.nslots;
   st.sbits = Q.sbits;
   st.smask = (1u << Q.sbits) - 1u;
@@ -543,7 +592,7 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
   p += ((size_t)Q.nslots * 2 + 15) / 16 * 16;
   uint8_t *const map8 = p;
   uint16_t *const map16 = reinterpret_cast<uint16_t *>(p);
-  static_assert(kMode == kRanked || (!kMap8 && kPol < 0), "stale and online replays: SPEAR or SPEAR+TIDE, two-byte maps");
+  static_assert(kMode == kRanked || kForm == kFormPlain, "stale and online replays: SPEAR or SPEAR+TIDE, two-byte maps");
   // kStale: every session's live and snapshot rank, sessions changed since the
   // last sync; kOnline: every session's arrivals so far (saturating far above
   // the table's last row), the table
@@ -560,7 +609,7 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
       snap = live + D.n_sessions;
       dirty = snap + D.n_sessions;
       // a zero register row (gap average 0, turn 0, not done)
-      for (uint32_t i = lane; i < D.n_sessions; i += 32) live[i] = snap[i] = Q.rank[D.n_events + i] + 1u;
+      for (uint32_t i = lane; i < D.n_sessions; i += 32) live[i] = snap[i] = Q.rank[D.n_events + i];
     } else {
       table = reinterpret_cast<OnlineTable *>(q);
       turns = reinterpret_cast<uint16_t *>(q + round16(sizeof(OnlineTable)));
@@ -570,12 +619,15 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
   }
   {
     uint4 *w4 = reinterpret_cast<uint4 *>(st.W);
+#pragma unroll 1
     for (uint32_t i = lane; i < slot_words(Q.nslots) / 4; i += 32) w4[i] = make_uint4(0u, 0u, 0u, 0u);
     uint4 *m4 = reinterpret_cast<uint4 *>(p);
     const uint32_t mq = (D.n_sessions * (kMap8 ? 1u : 2u) + 15) / 16;
+#pragma unroll 1
     for (uint32_t i = lane; i < mq; i += 32) m4[i] = make_uint4(0u, 0u, 0u, 0u);
     // the ring past the last event names session 0
-    for (uint32_t i = lane; i < kRing; i += 32) bufs.e[i].ev = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 1
+    for (uint32_t i = lane; i <= kRing; i += 32) bufs.e[i].ev = make_uint4(0u, 0u, 0u, 0u);
     if (lane == 0) {
       st.P[0].v.y = kIdMask;  // a zero map entry finds no session
       st.F[0] = 0;
@@ -598,9 +650,10 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
   const uint32_t n_turns = D.n_turns;
   uint8_t *note_out = reinterpret_cast<uint8_t *>(D.ttft) + 7ull * n_turns;
   // the DMA's last batch: its bytes (0: none in flight) and the time since it
-  // began, advanced from completion to completion, which are less than 2^32
-  // us apart (the next event, and a turn, take less than 2^31)
-  uint64_t busy_bytes = 0, busy_us = 0;
+  // began (saturating), advanced from completion to completion, which are less
+  // than 2^32 us apart (the next event, and a turn, take less than 2^31)
+  uint64_t busy_bytes = 0;
+  uint32_t busy_us = 0;
   uint32_t oldest = 0;  // Timeout: see expire_slots
   const uint32_t kvb = D.kvb, max_sessions = D.max_sessions, dma = (uint32_t)D.dma;
 
@@ -610,6 +663,7 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
     if (i < E) {
       SlotEvent &d = bufs.e[i & (kRing - 1)];
       async16(&d.ev, &D.ev[i]);
+      if ((i & (kRing - 1)) == 0) async16(&bufs.e[kRing].ev, &D.ev[i]);
       if (spear && kMode != kOnline) async4(&d.aux.x, &Q.rank[i]);
       if (tide_on || kMode == kOnline) async4(&d.aux.y, &D.gq[i]);
       if (belady) async4(&d.aux.z, &D.nref[i]);
@@ -627,16 +681,17 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
   // processed; a map entry changes only when its session is placed
   uint32_t nw = bufs.e[0].ev.y, nmap = map_of(nw & kIdMask), e = 0;
 
-  while (e < E && st.status != UNISON_ERR_CAPACITY) {
+  while (e < E) {
     fetch(e + 64);
     async_wait<1>();  // the batch after this one has landed
     __syncwarp();
     const uint32_t end = min(E, e + 32);
+    const SlotEvent *next = &bufs.e[e & (kRing - 1)];
     for (; e < end; e++) {
-      const SlotEvent &rec = bufs.e[e & (kRing - 1)];
+      const SlotEvent &rec = *next++;
       const uint32_t w1 = nw, s = w1 & kIdMask;
       uint32_t slot = nmap;
-      nw = bufs.e[(e + 1) & (kRing - 1)].ev.y;
+      nw = next->ev.y;
       const uint32_t ns = nw & kIdMask;
       st.e = e;
       if (timeout) {
@@ -662,8 +717,9 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
         uint32_t note = cls | (pl.x >> 31) * kNotePromoted;  // (the bit counts for fast-tier hits only)
         if (found) {
           clear_word(st, slot);
-          st.free_s += fast ? size : 0u;
-          st.free_h += fast ? 0u : size;
+          const uint32_t in_s = size & (uint32_t)((int32_t)pl.y >> 31);
+          st.free_s += in_s;
+          st.free_h += size - in_s;
         }
         // placement; a session that was resident keeps its slot
         uint32_t tier = 0;  // 0 fast, 1 HBM, 2 bypassed
@@ -679,9 +735,9 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
             const Choice c = most_evictable_fast(st, map16, lane);
             if (!c.any) {
               st.status = UNISON_ERR_CAPACITY;
-              break;
+              goto out;
             }
-            if constexpr (kMode == kStale) count_victim(st, c.slot, max_of(st.L, st.fresh, lane));
+            if constexpr (kMode == kStale) count_victim(st, c.slot, max_of<kDeep>(st.L, st.fresh, lane));
             // it is demoted into HBM, displacing more evictable sessions
             // there, or dropped
             const uint2 d = payload(st, c.slot);
@@ -703,17 +759,22 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
           st.room_s -= n;
         } else if (n <= st.room_h) {
           tier = 1;
-          if (!make_hbm_room(st, map16, n, Choice{false, 0u, 0ull}, lane)) st.status = UNISON_ERR_CAPACITY;
+          if (!make_hbm_room(st, map16, n, Choice{false, 0u, 0ull}, lane)) {
+            st.status = UNISON_ERR_CAPACITY;
+            goto out;
+          }
           st.free_h -= n;
           st.room_h -= n;
         } else {
           tier = 2;
         }
-        if (st.status == UNISON_ERR_CAPACITY) break;
         static_assert(UNISON_KIND_PLACE_H == UNISON_KIND_PLACE_S + 1 && UNISON_KIND_BYPASS == UNISON_KIND_PLACE_S + 2,
                       "placement kinds");
-        decide(st, UNISON_KIND_PLACE_S + tier, s, lane);
-        if (tier < 2) {
+        if (tier == 2) {
+          decide(st, UNISON_KIND_BYPASS, s, lane);
+          if (found) release_slot(st, slot);
+        } else {
+          decide(st, UNISON_KIND_PLACE_S + tier, s, lane);
           if (!found) {
             // the last slot freed, else a new one
             const bool reuse = st.nfree != 0;
@@ -724,7 +785,7 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
             st.n_res++;
             if (slot >= nslots) {
               st.status = UNISON_ERR_CAPACITY;
-              break;
+              goto out;
             }
             __syncwarp();
             if (kMap8) map8[s] = (uint8_t)slot;
@@ -746,11 +807,11 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
               const Choice f = most_evictable_fast(st, map16, lane), h = most_evictable_hbm(st, map16, lane);
               if (!f.any && !h.any) {
                 st.status = UNISON_ERR_CAPACITY;
-                break;
+                goto out;
               }
               const uint32_t vs = f.any && (!h.any || f.order > h.order) ? f.slot : h.slot, vw = st.W[vs];
               if constexpr (kMode == kStale) {
-                const uint32_t lh = max_hbm_of(st.L, st.fresh, lane), lf = max_of(st.L, st.fresh, lane);
+                const uint32_t lh = max_hbm_of<kDeep>(st.L, st.fresh, lane), lf = max_of<kDeep>(st.L, st.fresh, lane);
                 count_victim(st, vs, max(lh > kFastBit ? lh & ~kFastBit : 0u, lf & kFastBit ? lf & ~kFastBit : 0u));
               }
               const uint2 v = payload(st, vs);
@@ -762,10 +823,7 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
               release_slot(st, vs);
               __syncwarp();
             }
-            if (st.status == UNISON_ERR_CAPACITY) break;
           }
-        } else if (found) {
-          release_slot(st, slot);
         }
         *note_out++ = (uint8_t)(note | tier << kNotePlaceShift);  // (every lane the same byte)
         if constexpr (kMode == kOnline) {
@@ -777,7 +835,8 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
         // completion: the session is unpinned (if resident) with its new rank
         n_done++;
         const uint32_t now = rec.ev.x;
-        busy_us += (uint32_t)(now - last_done);
+        const uint32_t el = busy_us + (now - last_done);
+        busy_us = el < busy_us ? kAll : el;
         last_done = now;
         if (found) {
           if constexpr (kMode == kOnline) {
@@ -789,17 +848,18 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
           } else {
             uint32_t rk;
             if (kMode == kStale) rk = snap[s];  // residents rank by their snapshot rows
-            else if (spear) rk = rec.aux.x + 1u;
+            else if (spear) rk = rec.aux.x;
             else rk = n_turns - n_done + 1u;  // the later the touch, the less evictable
             if constexpr (kWide) {
               if (belady) rk = st.P[slot].v.z;
               if (timeout) st.P[slot].v.w = now;
             }
             st.W[slot] = rk << st.sbits | slot | (pl.y & kFastBit);
-            if constexpr (kMode == kStale) st.L[slot] = (rec.aux.x + 1u) << st.sbits | slot | (pl.y & kFastBit);
+            if constexpr (kMode == kStale) st.L[slot] = rec.aux.x << st.sbits | slot | (pl.y & kFastBit);
           }
-          st.room_s += fast ? size : 0u;
-          st.room_h += fast ? 0u : size;
+          const uint32_t in_s = size & (uint32_t)((int32_t)pl.y >> 31);
+          st.room_s += in_s;
+          st.room_h += size - in_s;
         }
         if constexpr (kMode == kOnline) {
           // Sec. V-F: the finished session's turn count joins the table, and
@@ -816,12 +876,12 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
             __syncwarp();
           }
         }
-        if (tide_on && !(w1 & kEvEdge)) {
+        if (tide_on) {
           // the DMA is free again from start + ceil(bytes / rate) us on, i.e.
           // once the elapsed us times the rate cover the bytes.  A batch's
-          // bytes are at most 2^31 us of the rate.
-          const bool busy = busy_us >> 31 == 0 && (uint64_t)(uint32_t)busy_us * dma < busy_bytes;
-          if (!busy) {
+          // bytes are at most 2^31 us of the rate, so the saturated time does.
+          const bool busy = (uint64_t)busy_us * dma < busy_bytes;
+          if (!busy && !(w1 & kEvEdge)) {
             st.n_tide_calls++;
             busy_bytes = tide_slots(st, map16, (uint64_t)rec.aux.y * dma, kvb, lane);  // (0 at rate 0: no budget)
             dma_bytes += busy_bytes;
@@ -830,7 +890,7 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
         }
       }
       if constexpr (kMode == kStale) {
-        live[s] = rec.aux.x + 1u;
+        live[s] = rec.aux.x;
         __syncwarp();
         if (n_dirty < kDirtySlots) dirty[n_dirty] = s;
         n_dirty++;
@@ -859,6 +919,7 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
       }
     }
   }
+out:
   async_wait<0>();
   if (lane == 0) {
     // the counters that follow from the arrivals' notes are account_arrivals'
@@ -1205,7 +1266,7 @@ __device__ void rank_keys_body(const RankDesc &d, uint32_t (*cnt)[256], SortShar
     src = dst;
     dst = t;
   }
-  for (uint32_t i = tid; i < n; i += kSortThreads) d.rank[(uint32_t)(src[i] & 0xFFFFFFull)] = i;
+  for (uint32_t i = tid; i < n; i += kSortThreads) d.rank[(uint32_t)(src[i] & 0xFFFFFFull)] = i + 1;
 }
 
 }  // namespace unison_slots

@@ -23,8 +23,9 @@
 // few, and loops stay rolled.  The 1,024-replay sweep's launch, one GB300: 57.5
 // ms with sorted lists of 64-bit keys in the warp's registers (375 instructions
 // an event), 38.7 with slots (188), 32.1 with the accounting taken out (158),
-// 27.9 with loops rolled, errors leaving by a jump, the bypass apart and each
-// event's record found by a pointer.  Tried and not kept: the words' extremes
+// 26.8 with loops rolled, errors leaving by a jump, the bypass apart, each
+// event's record found by a pointer and room in HBM for a demoted session tested
+// in place.  Tried and not kept: the words' extremes
 // found at the top of every event, beside the session's lookup (34.3 against
 // 32.5 ms); 256 words loaded at once in every pass (34.0); HBM's making of room
 // out of line for its second caller (48 against 31); the fast tier's payload
@@ -733,24 +734,25 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
         } else if (n <= st.room_s) {
           while (n > st.free_s) {
             const Choice c = most_evictable_fast(st, map16, lane);
-            if (!c.any) {
-              st.status = UNISON_ERR_CAPACITY;
-              goto out;
-            }
             if constexpr (kMode == kStale) count_victim(st, c.slot, max_of<kDeep>(st.L, st.fresh, lane));
             // it is demoted into HBM, displacing more evictable sessions
             // there, or dropped
             const uint2 d = payload(st, c.slot);
             const uint32_t sd = d.x & kSizeBits, did = d.y & kIdMask;
             st.free_s += sd;
-            const bool keep = sd <= st.room_h && make_hbm_room(st, map16, sd, c, lane);
+            const bool keep =
+                sd <= st.free_h || (c.any && sd <= st.room_h && make_hbm_room(st, map16, sd, c, lane));
             decide(st, keep ? (uint32_t)UNISON_KIND_DEMOTE : (uint32_t)UNISON_KIND_EVICT, did, lane);
-            if (keep) {
+            if (keep && c.any) {
               set_word(st, c.slot, false, c.order);
               st.P[c.slot].v.y = did;
               st.free_h -= sd;
               st.n_demote++;
             } else {
+              if (!c.any) {  // no unpinned session although the tier is short of space
+                st.status = UNISON_ERR_CAPACITY;
+                goto out;
+              }
               st.n_evict++;
               release_slot(st, c.slot);
             }
@@ -790,8 +792,8 @@ __device__ __forceinline__ void slot_replay(const Desc &D, const SlotDesc &Q, Sl
             __syncwarp();
             if (kMap8) map8[s] = (uint8_t)slot;
             else map16[s] = (uint16_t)slot;
+            if (ns == s) nmap = kMap8 ? (slot & 255u) : slot;  // read before it was set
           }
-          if (ns == s) nmap = kMap8 ? (slot & 255u) : slot;  // read before it was set
           *reinterpret_cast<uint2 *>(&st.P[slot]) = make_uint2(n, s | (tier ? 0u : kFastBit));
           if constexpr (kWide) {
             // a session with no next arrival ranks above every event index,

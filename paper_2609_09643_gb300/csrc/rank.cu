@@ -64,7 +64,7 @@ constexpr uint32_t kCandCap = 65536;     // candidate slots per list and set
 constexpr uint32_t kMaxGroup = 512;       // CTAs of one launch, at most (152 SMs x 3)
 constexpr uint32_t kMaxSel = 4096;       // largest k and max_moves
 constexpr uint32_t kFull = 0xFFFFFFFFu;
-constexpr uint32_t kSampleCtas = 64;     // sampling CTAs per set, at most
+constexpr uint32_t kSampleCtas = 63;     // sampling CTAs per set, at most
 constexpr uint32_t kSampleQ = 4;         // samples per consumer thread
 constexpr uint32_t kLaunchSamples = 131072;  // samples per launch, about,
 constexpr uint32_t kSmallSample = 4096;  // the shortest lists, where this many samples give them
@@ -87,6 +87,8 @@ constexpr uint32_t kIpt = kMaxSel / kConsumers;        // fill items per consume
 static_assert(kConsumers >= kLutN * 5, "one consumer thread per bound-table entry");
 static_assert(kMaxSel % kConsumers == 0 && kIpt % 4 == 0, "fill layout");
 static_assert(kBins == 16 * kConsumers, "histogram cut layout");
+constexpr uint32_t kMaxSample = kSampleCtas * kPerCtaSamples;
+static_assert(kMaxSample < 65536, "16-bit counts");
 
 struct __align__(128) FilterStage {
   uint32_t gap[kBigTile];
@@ -177,7 +179,7 @@ struct RankSet {
   uint32_t cr;       // region size
   uint64_t *sorted;  // [3][kMaxSel]
   uint32_t *ssz;     // [3][kMaxSel] KV tokens of the sorted entries (D and P)
-  unsigned int *shist;  // [3][kBins] sample histogram (zero between calls)
+  uint16_t *shist;      // [3][kBins] sample histogram (zero between calls)
 };
 
 // A shard's candidate lists (unison_rank_shard): a 64-byte header, then its
@@ -492,9 +494,12 @@ __device__ uint64_t block_select_rank(Get get, uint32_t n, uint32_t rank, Select
   return prefix;
 }
 
-// hist_cut over the kLists histograms hist[L * kBins ..] at once (their
-// loads in flight together): cut[L] for need[L] > 0, -1 for need[L] == 0.
-__device__ void hist_cut3(unsigned int *hist, const uint32_t (&need)[kLists], int (&cut)[kLists]) {
+// Cut of the kLists histograms hist[L * kBins ..] of 16-bit counts at once
+// (their loads in flight together): the bin holding the need[L]-th value from
+// the top, -1 for need[L] == 0 or too few values.  Every CTA of a group reads
+// them, 24 KB from L2 (with 32-bit counts, 48 KB, one set of 2^20 records took
+// 2 us more and 33 of them 4.5 us).
+__device__ void hist_cut3(const uint16_t *hist, const uint32_t (&need)[kLists], int (&cut)[kLists]) {
   __shared__ unsigned int wtot[kLists][kConsumers / 32];
   __shared__ int scut[kLists];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -502,11 +507,16 @@ __device__ void hist_cut3(unsigned int *hist, const uint32_t (&need)[kLists], in
   uint32_t c[kLists][16], tot[kLists], ex[kLists];
 #pragma unroll
   for (int L = 0; L < kLists; L++) {
-    uint4 *h4 = reinterpret_cast<uint4 *>(hist + L * kBins + lo);
+    const uint4 *h4 = reinterpret_cast<const uint4 *>(hist + L * kBins + lo);
 #pragma unroll
-    for (int q = 0; q < 4; q++) {
+    for (int q = 0; q < 2; q++) {
       const uint4 x = __ldcg(h4 + q);
-      c[L][4 * q] = x.x; c[L][4 * q + 1] = x.y; c[L][4 * q + 2] = x.z; c[L][4 * q + 3] = x.w;
+      const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        c[L][8 * q + 2 * u] = w[u] & 0xFFFFu;
+        c[L][8 * q + 2 * u + 1] = w[u] >> 16;
+      }
     }
   }
 #pragma unroll
@@ -941,7 +951,10 @@ __device__ __noinline__ void sample_share(const RankSet &S, uint32_t r, const ui
       const int first = who ? __ffs(who) - 1 : 0;
       const uint32_t b0 = __shfl_sync(kFull, b, first);
       const bool one = __ballot_sync(kFull, in && b == b0) == who;
-      if (in && (!one || (int)(tid & 31) == first)) atomicAdd(&S.shist[L * kBins + b], one ? (unsigned)__popc(who) : 1u);
+      if (in && (!one || (int)(tid & 31) == first))
+        // two counts a word: neither can pass 16 bits (kMaxSample)
+        atomicAdd(reinterpret_cast<unsigned int *>(S.shist) + (L * kBins + b) / 2,
+                  (one ? (unsigned)__popc(who) : 1u) << 16 * (b & 1));
     }
   }
   if (tid == 0) atomicAdd(&S.work->gathered, 1u);  // the group's copies may start now
@@ -2485,7 +2498,7 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
   // candidates; and the per-set histograms in their own block
   const size_t fixed_set = align_up(sizeof(uint64_t) * kLists * kMaxSel, 256) +
                            align_up(sizeof(uint32_t) * kLists * kMaxSel, 256);
-  const size_t hist_set = sizeof(unsigned int) * kLists * kBins;
+  const size_t hist_set = sizeof(uint16_t) * kLists * kBins;
   size_t sets_b = 0, hist_b = 0;  // hist_b: one parity's histograms (sampled sets only)
   for (int i = 0; i < n_sets; i++) {
     RankSet &s = hs[i];
@@ -2535,7 +2548,7 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
     for (int i = 0; i < n_sets; i++) {
       RankSet &s = hs[i];
       s.work = reinterpret_cast<RankWork *>(z) + i;
-      s.shist = s.ns ? reinterpret_cast<unsigned int *>(z + hoff) : nullptr;
+      s.shist = s.ns ? reinterpret_cast<uint16_t *>(z + hoff) : nullptr;
       if (s.ns) hoff += hist_set;
     }
   };

@@ -27,6 +27,8 @@
 //            exact values of the records that pass are appended per list to
 //            the CTA's own region, which moves into the set's list when the
 //            CTA is done.
+//            A set of at most 4,096 records streams nothing: three CTAs collect
+//            one list's values each, from every eligible record.
 //   finish   the last three CTAs of the group to finish streaming take one
 //            list each: cuts into 256 buckets below the common prefix narrow the
 //            candidates to few beyond the first M, which are sorted and the
@@ -171,6 +173,7 @@ struct RankSet {
   uint32_t rL[kLists];           // sample rank of each list's threshold
   uint32_t ccap;                 // candidate slots per list (kCandCap, or n rounded up for a set too small to sample)
   uint32_t off;                  // index of record 0 in the whole set (a shard's slice), else 0
+  uint32_t direct;               // small set, one CTA a list: each collects its list's values itself
   unsigned char *cands;          // a shard's candidate lists (unison_rank_shard), else null
   // scratch (per set)
   RankWork *work;
@@ -874,7 +877,7 @@ __host__ uint64_t sample_size(const RankSet &S, int o) {
 
 // CTAs a set can use: one a tile, and one a list for the finish (a set of
 // 1,000 records whose one CTA finished its lists in turn took 58 us, with three
-// 29 us).
+// 29 us, and 17 us when each collects its list's values itself).
 __host__ __forceinline__ uint32_t most_ctas(const RankSet &S) { return std::max<uint32_t>(S.ntiles, kLists); }
 
 // The sample plan of a set whose group (cta0, nctas) is fixed.
@@ -888,6 +891,7 @@ void plan_sample(RankSet &s, int n_sets) {
   ns = umin64(ns, cap);
   // half a CTA's most a CTA where there are enough: the samples' latency is the
   // call's head
+  s.direct = ns == 0 && s.n <= kSmemCand && s.nctas == kLists ? 1u : 0u;
   s.sctas = ns ? (uint32_t)umin64(most, (ns + kPerCtaSamples / 2 - 1) / (kPerCtaSamples / 2)) : 0u;
   if (ns) ns = (ns + 8ull * s.sctas - 1) / (8ull * s.sctas) * (8ull * s.sctas);  // whole runs, evenly split
   ns = umin64(ns, (uint64_t)kPerCtaSamples * s.sctas);
@@ -1076,11 +1080,67 @@ __device__ __noinline__ uint32_t stream_topM(const RankSet &S, int L, uint32_t M
   return got;
 }
 
+// Every eligible record's value of list L into buf (room for the set's
+// records), and, for list 0, the keys when asked for.  Returns the count.
+__device__ __noinline__ uint32_t collect_list(const RankSet &S, int L, uint64_t *buf, const uint64_t *t2s,
+                                              const uint64_t *mgs, SelectScratch &ss) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, n = S.n;
+  const bool active = (S.act >> L) & 1, keys = L == 0 && S.keys;
+  if (tid == 0) ss.cnt = 0;
+  consumers_sync();
+  for (uint32_t b = 0; b < n; b += 4 * kConsumers) {
+    const uint32_t i = b + 4 * tid;
+    uint32_t g[4], t[4], fl[4], tr[4];
+    if (i + 4 <= n) {
+      const uint4 gq = *reinterpret_cast<const uint4 *>(S.gap + i);
+      const uint2 tq = *reinterpret_cast<const uint2 *>(S.turn + i);
+      const uint32_t fq = *reinterpret_cast<const uint32_t *>(S.flags + i);
+      const uint32_t rq = *reinterpret_cast<const uint32_t *>(S.tier + i);
+      g[0] = gq.x; g[1] = gq.y; g[2] = gq.z; g[3] = gq.w;
+      t[0] = tq.x & 0xFFFFu; t[1] = tq.x >> 16; t[2] = tq.y & 0xFFFFu; t[3] = tq.y >> 16;
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        fl[k] = fq >> 8 * k & 0xFFu;
+        tr[k] = rq >> 8 * k & 0xFFu;
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const bool in = i + k < n;
+        g[k] = in ? S.gap[i + k] : 0u;
+        t[k] = in ? S.turn[i + k] : 0u;
+        fl[k] = in ? S.flags[i + k] : 1u;  // padding reads as pinned: never eligible
+        tr[k] = in ? S.tier[i + k] : 0u;
+      }
+    }
+    uint64_t v[4];
+    unsigned bal[4], at = 0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      const uint64_t sc = score_of(g[k], min(t[k], kTMax), (fl[k] & 2) != 0, t2s, mgs);
+      if (keys && i + k < n) S.keys[i + k] = sc;
+      v[k] = list_val(ck_of(sc, S.off + i + k), L);
+      bal[k] = __ballot_sync(kFull, active && ((elig_mask((uint8_t)fl[k], (uint8_t)tr[k]) >> L) & 1));
+    }
+    const uint32_t n0 = __popc(bal[0]), n1 = n0 + __popc(bal[1]), n2 = n1 + __popc(bal[2]);
+    if (lane == 0) at = atomicAdd(&ss.cnt, n2 + __popc(bal[3]));
+    at = __shfl_sync(kFull, at, 0);
+    const uint32_t before[4] = {0u, n0, n1, n2};
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+      if (bal[k] >> lane & 1) buf[at + before[k] + __popc(bal[k] & ((1u << lane) - 1))] = v[k];
+  }
+  consumers_sync();
+  return ss.cnt;
+}
+
 // List L of set S: the exact top-M of its candidates, sorted, with the moved
 // records' sizes; victims are written out directly.  fin: the 64 KB dynamic
 // area (the stages are idle).  Returns true when this was the set's last list.
+// local >= 0: the area already holds that many candidates, every eligible
+// record's (collect_list).
 __device__ __noinline__ bool finish_list(const RankSet &S, int L, uint64_t *fin, const uint64_t *t2s, const uint64_t *mgs,
-                                         SelectScratch &ss, const SetConst &cs) {
+                                         SelectScratch &ss, const SetConst &cs, int local = -1) {
   __shared__ __align__(8) uint64_t cbar;
   __shared__ unsigned int last, sh_emitted, sh_flags, nsurv;
   const uint32_t Mw = (L == 0) ? S.k : S.max_moves;
@@ -1093,8 +1153,8 @@ __device__ __noinline__ bool finish_list(const RankSet &S, int L, uint64_t *fin,
   // one thread reads the other CTAs' results, so that every consumer thread
   // takes the same path through the barriers below
   if (tid == 0) {
-    sh_emitted = __ldcg(&S.work->cand[L]);
-    sh_flags = ((cs.act >> L) & 1u) | (cs.thr[L] == 0 ? 2u : 0u);
+    sh_emitted = local >= 0 ? (unsigned)local : __ldcg(&S.work->cand[L]);
+    sh_flags = local >= 0 ? ((S.act >> L) & 1u) | 2u : ((cs.act >> L) & 1u) | (cs.thr[L] == 0 ? 2u : 0u);
   }
   consumers_sync();
   const bool active = sh_flags & 1;
@@ -1113,7 +1173,7 @@ __device__ __noinline__ bool finish_list(const RankSet &S, int L, uint64_t *fin,
     if (certified) {
       const uint32_t c = emitted;
       const bool in_smem = c <= bufcap;
-      if (in_smem) {
+      if (in_smem && local < 0) {
         // one bulk copy (an even count: a 16-byte multiple; ccap is even, so
         // the list holds c + 1 entries when c is odd, and so does the area)
         const uint32_t bytes = ((c + 1) & ~1u) * 8u;
@@ -1448,6 +1508,20 @@ __device__ __noinline__ void fill(const RankSet &S, uint64_t *fin) {
   consumers_sync();
 }
 
+// The set's last list is done: the fill, or a shard's header.
+__device__ __forceinline__ void finish_set(const RankSet &S, uint64_t *fin) {
+  if (!S.cands) {
+    fill(S, fin);
+  } else if (threadIdx.x == 0) {
+    CandHeader *h = reinterpret_cast<CandHeader *>(S.cands);
+    h->n = S.n;
+    h->off = S.off;
+    h->k = S.k;
+    h->max_moves = S.max_moves;
+    h->status = *(volatile unsigned int *)&S.work->status;
+  }
+}
+
 // ------------------------------------------------------------- kernel ----
 // Grouped (sequential == 0): CTA c serves the set whose group holds it.
 // Sequential: CTA c serves sets c, c + G, c + 2G, ... one after another, each
@@ -1541,6 +1615,7 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
     int sfail = s0;
     for (int s = s0; s < n_sets && !failed; s += sstep) {
       const RankSet &T = sets[s];
+      if (T.direct) return;  // (a grouped launch: this CTA's only set)
       const uint32_t r = sequential ? 0u : blockIdx.x - T.cta0, nct = sequential ? 1u : T.nctas;
       if (T.ns) {
         // The sample's random reads go first: the group's bulk copies would
@@ -1638,6 +1713,14 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
         sgs[ct] = S.tab->sigma[ct];
       }
       consumers_sync();
+    }
+    if (S.direct) {
+      // no thresholds and no streaming: CTA r collects every eligible record's
+      // value of list r and finishes the list
+      const int local = (int)collect_list(S, (int)r, fin, t2s, mgs, u.s);
+      const bool last = finish_list(S, (int)r, fin, t2s, mgs, u.s, c, local);
+      if (last) finish_set(S, fin);
+      return;
     }
     // 1. thresholds: the sampling CTAs sample; every CTA cuts the histograms
     if (r < S.sctas) sample_share(S, r, t2s, mgs);
@@ -1958,15 +2041,7 @@ __global__ void __launch_bounds__(kCtaThreads, 3)
 #pragma unroll 1
       for (int L = 0; L < kLists; L++)
         if ((mine >> L) & 1) last = finish_list(S, L, fin, t2s, mgs, u.s, c);
-      if (last && !S.cands) fill(S, fin);
-      if (last && S.cands && ct == 0) {  // a shard: the header closes its lists
-        CandHeader *h = reinterpret_cast<CandHeader *>(S.cands);
-        h->n = S.n;
-        h->off = S.off;
-        h->k = S.k;
-        h->max_moves = S.max_moves;
-        h->status = *(volatile unsigned int *)&S.work->status;
-      }
+      if (last) finish_set(S, fin);
     }
     // 4. the stage memory is free for the next set's copies
     consumers_sync();

@@ -190,6 +190,30 @@ def test_selection_of_crowded_values(B, sigma, n):
         check(r, rec, p)
 
 
+@pytest.mark.parametrize("n", [1, 5, 1023, 1025, 4095, 4096, 4097])
+def test_small_sets_with_keys_and_as_shards(B, sigma, n):
+    """Sets of up to 4,096 records, whose lists are collected by one CTA each:
+    sizes beside a thread's four records and a pass of 1,024, every score
+    wanted, lists of none, few and more than the set holds; and the same set as
+    three shards, merged."""
+    import torch
+    rec = synth.make_records(900 + n, n)
+    ps = [prm(sigma, k=k, budget=b * GIB, max_moves=m, free_s=fs)
+          for k, b, m, fs in ((0, 1, 4096, 9000), (16, 64, 64, 0), (4096, 0, 300, 0), (300, 64, 4096, 1 << 30))]
+    for r, p in zip(run(B, [rec] * len(ps), ps, keys=True), ps):
+        check(r, rec, p, keys=True)
+    dev, p = B.records_to_device(rec), ps[1]
+    cuts = sorted({0, n // 48 * 16, n // 24 * 16, n})
+    parts = []
+    for a, b in zip(cuts, cuts[1:]):
+        parts.append(B.rank_cands(p["k"], p["max_moves"]))
+        B.rank_shard({k: v[a:b] for k, v in dev.items()}, a, p, parts[-1])
+    out = B.rank_outputs(n, p["k"], p["max_moves"])
+    B.rank_merge(torch.cat(parts), len(parts), p, out)
+    torch.cuda.synchronize()
+    check(B.rank_result(out), rec, p)
+
+
 @pytest.mark.parametrize("n_sets,n_tabs", [(2, 2), (64, 2), (65, 1), (64, 3)])
 def test_descriptors_with_the_launch_or_uploaded(B, sigma, n_sets, n_tabs):
     """The most sets and distinct survival tables whose descriptors go with the

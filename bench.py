@@ -914,25 +914,25 @@ def main():
     # 16 B event + 4 B previous size + 8 B key + 4 B gap average + 8 B key
     # before each arrival (half the events): 36 B/event
     alg_bytes = events_per_step * 36
-    replay_roof = None if not rep_n else {"bound": "latency", "kernel": "replay_kernel", "avg_ms": avg_rep_ms,
+    replay_roof = None if not rep_n else {"bound": "latency", "kernel": "slot_kernel", "avg_ms": avg_rep_ms,
                    "ns_per_event_per_replay": 1e6 * avg_rep_ms / (events_per_step / n_rep),
                    "hbm_gbs": alg_bytes / (avg_rep_ms / 1e3) / 1e9, "launches_timed": rep_n,
                    "share_of_step": avg_rep_ms * args.steps / ms if ms else None,
                    "key_stream_avg_ms": ks_ms / max(ks_n, 1), "ttft_median_avg_ms": md_ms / max(md_n, 1)}
     if replay_roof is not None:
         # The launch ends with its slowest replay: its cycles per event, against
-        # the chain an event needs with both tiers in the warp's registers and
-        # the pin list in shared memory (about 17 dependent steps of about 30
-        # cycles each: the event's and its key's loads, the lookup ballot and
-        # entry shuffle, the erase shuffle, pin slot, pin entry and its store,
-        # a demotion's pop, the HBM search ballot and insert shuffle, TIDE's
-        # two heads and its insert's ballot and shuffle).
+        # the chain an event needs with its residents in shared-memory slots
+        # (about 12 dependent steps of about 30 cycles each, the mean of an
+        # arrival and a completion: the event's record, the session's slot, its
+        # payload, the test of room, one pass over the words (load, reduction,
+        # the winner's payload) for a demotion or for TIDE's first choice, a
+        # second pass, the word's store).
         mhz = (clocks or {}).get("sm_mhz") or 2070.0
         replay_roof["cycles_per_event_slowest_replay"] = avg_rep_ms * 1e3 * mhz / (events_per_step / n_rep)
-        replay_roof["floor_cycles_per_event"] = 17 * 30
-        replay_roof["floor_basis"] = ("17 dependent steps per event x ~30 cycles: shared-memory loads (event, key, "
-                                      "pin slot and entry) and the register tiers' ballots and shuffles (lookup, "
-                                      "erase, demotion, HBM insert, TIDE heads and insert)")
+        replay_roof["floor_cycles_per_event"] = 12 * 30
+        replay_roof["floor_basis"] = ("12 dependent steps per event x ~30 cycles: shared-memory loads (event, session's "
+                                      "slot, payload), the test of room, two passes over the slot words (load, "
+                                      "reduction, payload) and a store")
     avg_rk = rk_ms / max(rk_n, 1) if rk_n else float("nan")
     achieved = rank_bytes / (avg_rk / 1e3) / 1e9 if rk_n else float("nan")
     n_rec = len(r_params) * RANK_N

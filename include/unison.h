@@ -459,13 +459,13 @@ typedef struct {
  * sample, and a set whose candidates fall short is re-selected exactly on
  * the device.  sets, params, outs: host arrays [n_sets].  Asynchronous: the
  * call queues one cooperative kernel on cuda_stream, after one upload of its
- * descriptors when it has several sets (every CTA of the grid resident at once; each set is ranked
- * by a group of CTAs, or, with more sets than resident CTAs, each CTA takes
- * whole sets in turn).  Any n_sets >= 0 that fits in memory is accepted.
- * Memory: the call's device scratch (about 1.7 MB per set) is kept per
+ * descriptors when they are too many for the launch's parameters (every CTA
+ * of the grid resident at once; each set is ranked by a group of CTAs, or,
+ * with more sets than resident CTAs, each CTA takes whole sets in turn).  Any n_sets >= 0 that fits in memory is accepted.
+ * Memory: the call's device scratch (up to about 3.4 MB per set) is kept per
  * (device, stream) and grown when a call needs more, and the per-call
- * descriptors go up from a small pinned host ring; both are held for the
- * life of the process.  Calls on one stream run in order and share that
+ * descriptors that are uploaded go from a small pinned host ring; both are
+ * held for the life of the process.  Calls on one stream run in order and share that
  * stream's scratch; calls on different streams use different scratch.  The
  * scratch is found by the stream's handle, so a stream must outlive the
  * ranking calls queued on it.

@@ -12,7 +12,7 @@
 // One cooperative, persistent kernel does a whole call.  Each set owns a
 // group of CTAs (in proportion to its records; with more sets than CTAs,
 // each CTA takes whole sets in turn).  Per set, inside the group:
-//   sample   up to 16 CTAs gather a jittered stratified sample, count it in
+//   sample   up to 63 CTAs gather a jittered stratified sample, count it in
 //            shared memory and add it to a 4,096-bin histogram per list (bins
 //            monotone in the list value).  Once every sampling CTA's counts
 //            are in, each CTA of the group cuts the histograms at the lists'
@@ -824,7 +824,8 @@ __device__ __forceinline__ void sort_desc(uint64_t *a, uint32_t n, uint64_t *tmp
 // of kLaunchSamples and kSetSamples, because a sample's runs are random rows of
 // DRAM.  Measured, whole call: 33 sets of 2^20 records 118 us at 9,800 samples
 // a set, 139 us at 4,096 (18,000 candidates a set in place of 13,000, and a
-// longer last set); 7 sets of 2^24 199 us at 18,000 a set, 205 us at 35,000.
+// longer last set); 7 sets of 2^24 199 us at 18,000 a set, 205 us at 35,000 (the
+// calls took 8 to 12 us longer then than they do with 16-bit histograms).
 // The threshold is the floor of the histogram bin holding the rank-r sample, so
 // it admits a few more.
 __host__ __forceinline__ uint64_t umin64(uint64_t a, uint64_t b) { return a < b ? a : b; }
@@ -2190,9 +2191,9 @@ bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) %
 // the process.  The stream handle is the key: a stream must outlive the
 // ranking calls queued on it (a new stream that reuses a destroyed one's
 // handle would otherwise share its scratch without being ordered after it).
-// Per key: the calls' working scratch, and two blocks for the state that a
-// call must find zero (work words, then the sampled sets' histograms).  Calls
-// alternate between the two; each zeroes what the one before it used, so a
+// Per key: the calls' working scratch, and blocks for the state that a call
+// must find zero (work words, then the sampled sets' histograms).  Calls
+// alternate between two; each zeroes what the one before it used, so a
 // block is all zero when its turn comes, whatever the calls' sizes, and no
 // clearing precedes a launch (a memset and the upload of a single set's
 // descriptor took about 10 of a call's 52 us at 2^20 records).
@@ -2215,7 +2216,7 @@ struct RankPlan {
 };
 struct StreamState {
   std::mutex mu;  // held from the choice of a block to the launch that uses it
-  Scratch main, zero[2];
+  Scratch main, zero[3];  // zero[2]: of captured calls (block_for)
   size_t dirty[2] = {0, 0};  // bytes from a block's start that are not zero
   bool planned = false;
   RankPlan plan;
@@ -2260,11 +2261,11 @@ int grow(Scratch &e, size_t bytes, bool zero, cudaStream_t stream) {
   return UNISON_OK;
 }
 
-// Both zero blocks at least `bytes` long (a new block is zero).
+// The zero blocks at least `bytes` long (a new block is zero).
 int grow_zero(StreamState &st, size_t bytes, cudaStream_t stream) {
-  for (int i = 0; i < 2; i++) {
+  for (int i = 0; i < 3; i++) {
     if (st.zero[i].bytes >= bytes) continue;
-    st.dirty[i] = 0;
+    if (i < 2) st.dirty[i] = 0;
     st.planned = false;  // the plan's descriptors name the old block
     const int rc = grow(st.zero[i], bytes, true, stream);
     if (rc != UNISON_OK) return rc;
@@ -2406,12 +2407,30 @@ void plan_key(std::vector<unsigned char> &k, const unison_records *sets, const u
 // Launches a call on the zero block whose turn it is (zb: the bytes of it that
 // the call uses), zeroing the other.  The caller holds st.mu and has passed
 // that block (next_block) to the descriptors.
+// A call captured into a graph runs whenever the graph does, any number of
+// times, so it takes a block apart from the ordinary calls' and clears it by a
+// node of its own.
 int next_block(const StreamState &st) { return st.dirty[0] == 0 ? 0 : 1; }
+int block_for(const StreamState &st, bool captured) { return captured ? 2 : next_block(st); }
+bool is_capturing(cudaStream_t stream) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &s) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return s != cudaStreamCaptureStatusNone;
+}
 template <int kSets>
 int launch_rank_kernel(StreamState &st, uint32_t grid, const RankSet *d_sets, int n_sets, int sequential,
                        const uint32_t *cmap, const RankTab *tabs, const RankPack<kSets> &pack, size_t zb,
-                       cudaStream_t stream) {
-  const int p = next_block(st);
+                       bool captured, cudaStream_t stream) {
+  const int p = block_for(st, captured);
+  if (captured && cudaMemsetAsync(st.zero[p].p, 0, zb, stream) != cudaSuccess) {
+    cudaGetLastError();
+    return UNISON_ERR_CUDA;
+  }
+  char *const other = captured ? nullptr : st.zero[1 - p].p;
+  const uint32_t n_other = captured ? 0u : (uint32_t)(st.dirty[1 - p] / 16);
   cudaError_t e;
   {
     ProfSpan span("rank", stream);
@@ -2426,7 +2445,7 @@ int launch_rank_kernel(StreamState &st, uint32_t grid, const RankSet *d_sets, in
     lc.attrs = coop;
     lc.numAttrs = 1;
     e = cudaLaunchKernelEx(&lc, rank_kernel<kSets>, d_sets, n_sets, sequential, cmap, tabs,
-                           reinterpret_cast<uint4 *>(st.zero[1 - p].p), (uint32_t)(st.dirty[1 - p] / 16), pack);
+                           reinterpret_cast<uint4 *>(other), n_other, pack);
   }
   count_launches(1);
   if (e == cudaSuccess) e = cudaGetLastError();
@@ -2435,6 +2454,7 @@ int launch_rank_kernel(StreamState &st, uint32_t grid, const RankSet *d_sets, in
     st.planned = false;
     return UNISON_ERR_CUDA;  // nothing ran: the blocks are as they were
   }
+  if (captured) return UNISON_OK;
   st.dirty[p] = zb;
   st.dirty[1 - p] = 0;
   return UNISON_OK;
@@ -2446,19 +2466,20 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
   if (!state) return UNISON_ERR_CUDA;
   StreamState &st = *state;
   std::lock_guard<std::mutex> lock(st.mu);
+  const bool captured = is_capturing(stream);
   static const RankPack<1> none{};
   thread_local std::vector<unsigned char> key;
   if (n_sets > 1) {
     plan_key(key, sets, params, outs, n_sets, off, cands);
-    if (st.planned && st.plan.key == key) {
+    if (!captured && st.planned && st.plan.key == key) {
       const RankPlan &pl = st.plan;
       if (pl.packed)
         return launch_rank_kernel(st, pl.grid, nullptr, n_sets, 0, nullptr, nullptr, pl.pack[next_block(st)], pl.zero_b,
-                                  stream);
+                                  false, stream);
       return launch_rank_kernel(
           st, pl.grid, reinterpret_cast<const RankSet *>(st.main.p + next_block(st) * pl.desc_b), n_sets, pl.sequential,
           pl.sequential ? nullptr : reinterpret_cast<const uint32_t *>(st.main.p + pl.cmap_off),
-          reinterpret_cast<const RankTab *>(st.main.p + pl.tabs_off), none, pl.zero_b, stream);
+          reinterpret_cast<const RankTab *>(st.main.p + pl.tabs_off), none, pl.zero_b, false, stream);
     }
   }
   std::vector<RankSet> hs(n_sets);
@@ -2568,13 +2589,13 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
     }
   }
   for (int i = 0; i < n_sets; i++) plan_sample(hs[i], n_sets);
-  // scratch: descriptors, tables, every set's work words (zeroed by the
-  // upload), then per set: thresholds, tables, sorted lists and sizes,
-  // candidates; and the per-set histograms in their own block
+  // scratch: the descriptors, CTA map and tables of a call that uploads them,
+  // then per set: sorted lists and sizes, candidates.  In a zero block: every
+  // set's work words, then the sampled sets' histograms
   const size_t fixed_set = align_up(sizeof(uint64_t) * kLists * kMaxSel, 256) +
                            align_up(sizeof(uint32_t) * kLists * kMaxSel, 256);
   const size_t hist_set = sizeof(uint16_t) * kLists * kBins;
-  size_t sets_b = 0, hist_b = 0;  // hist_b: one parity's histograms (sampled sets only)
+  size_t sets_b = 0, hist_b = 0;  // hist_b: one block's histograms (sampled sets only)
   for (int i = 0; i < n_sets; i++) {
     RankSet &s = hs[i];
     // without a sample every eligible record is a candidate: at most n
@@ -2628,16 +2649,16 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
     }
   };
   if (single) {
-    in_block(next_block(st));
+    in_block(block_for(st, captured));
     RankPack<1> one;
     one.set[0] = hs[0];
     one.tab[0] = tabs[0];
-    return launch_rank_kernel(st, grid, nullptr, 1, 0, nullptr, nullptr, one, zero_b, stream);
+    return launch_rank_kernel(st, grid, nullptr, 1, 0, nullptr, nullptr, one, zero_b, captured, stream);
   }
   if (packed) {
     RankPlan &pl = st.plan;
     for (int b = 0; b < 2; b++) {
-      in_block(b);
+      in_block(captured ? 2 : b);
       RankPack<kPackSets> &pk = pl.pack[b];
       std::memcpy(pk.set, hs.data(), sizeof(RankSet) * n_sets);
       std::memcpy(pk.tab, tabs.data(), sizeof(RankTab) * tabs.size());
@@ -2646,8 +2667,9 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
         std::memset(pk.of_cta + hs[i].cta0, i, hs[i].nctas);
       }
     }
-    rc = launch_rank_kernel(st, grid, nullptr, n_sets, 0, nullptr, nullptr, pl.pack[next_block(st)], zero_b, stream);
-    if (rc == UNISON_OK) {
+    rc = launch_rank_kernel(st, grid, nullptr, n_sets, 0, nullptr, nullptr, pl.pack[next_block(st)], zero_b, captured,
+                            stream);
+    if (rc == UNISON_OK && !captured) {
       pl.key = key;
       pl.zero_b = zero_b;
       pl.grid = grid;
@@ -2665,7 +2687,7 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
     const int sr = staging_acquire(up, &h, &done);
     if (sr != UNISON_OK) return sr;
     for (int b = 0; b < 2; b++) {
-      in_block(b);
+      in_block(captured ? 2 : b);
       std::memcpy(h + b * desc_b, hs.data(), sizeof(RankSet) * n_sets);
     }
     if (!sequential) {
@@ -2684,8 +2706,8 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
   }
   rc = launch_rank_kernel(st, grid, reinterpret_cast<const RankSet *>(scratch + next_block(st) * desc_b), n_sets,
                           sequential, sequential ? nullptr : reinterpret_cast<const uint32_t *>(scratch + cmap_off),
-                          d_tabs, none, zero_b, stream);
-  if (rc == UNISON_OK) {
+                          d_tabs, none, zero_b, captured, stream);
+  if (rc == UNISON_OK && !captured) {
     RankPlan &pl = st.plan;
     pl.key = key;
     pl.desc_b = desc_b;
@@ -2763,15 +2785,22 @@ extern "C" int unison_rank_merge(const void *gathered_dev, int n_shards, const u
   int rc = grow(st.main, lists_b, false, stream);
   if (rc == UNISON_OK) rc = grow_zero(st, work_b, stream);
   if (rc != UNISON_OK) return rc;
-  const int b = next_block(st);
+  const bool captured = is_capturing(stream);
+  const int b = block_for(st, captured);
+  if (captured && cudaMemsetAsync(st.zero[b].p, 0, work_b, stream) != cudaSuccess) {
+    cudaGetLastError();
+    return UNISON_ERR_CUDA;
+  }
   s.work = reinterpret_cast<RankWork *>(st.zero[b].p);
   s.sorted = reinterpret_cast<uint64_t *>(st.main.p);
   s.ssz = reinterpret_cast<uint32_t *>(st.main.p + vals_b);
   rank_merge_kernel<<<kLists, kConsumers, kMergeSmem, stream>>>(
       s, static_cast<const unsigned char *>(gathered_dev), n_shards, (uint64_t)cand_bytes(p.k, p.max_moves),
-      reinterpret_cast<uint4 *>(st.zero[1 - b].p), (uint32_t)(st.dirty[1 - b] / 16));
+      reinterpret_cast<uint4 *>(captured ? nullptr : st.zero[1 - b].p),
+      captured ? 0u : (uint32_t)(st.dirty[1 - b] / 16));
   count_launches(1);
   if (cudaGetLastError() != cudaSuccess) return UNISON_ERR_CUDA;  // nothing ran: the blocks are as they were
+  if (captured) return UNISON_OK;
   st.dirty[b] = work_b;
   st.dirty[1 - b] = 0;
   return UNISON_OK;

@@ -35,10 +35,10 @@
 // the snapshot's ranks and keeps the live ones beside them, so a choice is
 // compared with the live one by a second pass and a sync rewrites the words of
 // the sessions that changed, a lane each (16 replays over the four sync modes
-// 151 -> 46 ms).  Under the online hazard table keys change while sessions are
+// 148 -> 45 ms).  Under the online hazard table keys change while sessions are
 // resident, so a word is the key itself in 64 bits, and a rebuilt table rewrites
 // every word in place where sorted lists had to be sorted again (6 online, 6
-// offline and 6 LRU replays with logs 116 -> 49 ms).
+// offline and 6 LRU replays with logs 111 -> 47 ms).
 #pragma once
 
 #include "common.cuh"
@@ -956,7 +956,10 @@ out:
 // of requests is q' = max(q + P, M), and two runs compose to P1 + P2 and
 // max(M1 + P2, M2), so the block scans 1,024 events at a time.  The event loop
 // is a serial chain and the queue took about 22 of an arrival's instructions
-// in it; here it costs 0.2-0.4 ms for the 1,024-replay sweep.  Times that
+// in it; here it takes about 0.85 of ttft_median_kernel's 1.22 ms over the
+// 1,024-replay sweep, where leaving it out of the loop saved 6.6.  Not faster:
+// 512 threads (1.44 ms), the next chunk's events loaded ahead (1.35 to 1.41),
+// counters packed in 16 bits (1.24).  Times that
 // could pass 2^63 ns (D.slot.serial) wrap as the recurrence does when one
 // thread walks it.
 // Values overwrite the notes in place: the 8-byte values of arrivals up to i

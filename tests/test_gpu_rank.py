@@ -472,3 +472,47 @@ def test_record_sharded_ranking_equals_whole_set(B, sigma, world):
         B.rank_merge(torch.cat(parts), world, p, out)
         torch.cuda.synchronize()
         check(B.rank_result(out), rec, p)
+
+
+def test_captured_calls_replay_beside_ordinary_ones(B, sigma):
+    """A single set, a batch and a merge captured into a graph: each replay of
+    it ranks exactly, and so do ordinary calls on the stream after the capture
+    and between replays (a captured call clears work words of its own)."""
+    import torch
+    recs = [synth.make_records(81, 3_000), synth.make_records(82, 50_000)]
+    ps = [prm(sigma, k=100, budget=GIB, max_moves=64), prm(sigma, k=300, budget=4 * GIB, max_moves=200)]
+    devs = [B.records_to_device(r) for r in recs]
+    outs = [[B.rank_outputs(r.n, p["k"], p["max_moves"]) for r, p in zip(recs, ps)] for _ in range(2)]
+    mout = B.rank_outputs(recs[1].n, ps[1]["k"], ps[1]["max_moves"])
+    sout = B.rank_outputs(recs[1].n, ps[1]["k"], ps[1]["max_moves"])
+    cands = B.rank_cands(ps[1]["k"], ps[1]["max_moves"])
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    calls = [B.rank_prepare(devs, ps, o) for o in outs]  # the graph's outputs, the ordinary calls'
+    single = B.rank_prepare(devs[1:], ps[1:], [sout])
+    torch.cuda.synchronize()
+
+    def graphed():
+        single.run(stream)
+        calls[0].run(stream)
+        B.rank_shard(devs[1], 0, ps[1], cands, stream=stream)
+        B.rank_merge(cands, 1, ps[1], mout, stream=stream)
+
+    calls[1].run(stream)
+    graphed()  # scratch grown before the capture
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        graphed()
+    for _ in range(3):
+        for o in outs[0] + outs[1] + [mout, sout]:
+            o["counts"].zero_()
+        torch.cuda.synchronize()
+        calls[1].run(stream)
+        with torch.cuda.stream(stream):
+            graph.replay()
+        calls[1].run(stream)
+        torch.cuda.synchronize()
+        for o in outs:
+            for oo, rec, p in zip(o, recs, ps):
+                check(B.rank_result(oo), rec, p)
+        for oo in (mout, sout):
+            check(B.rank_result(oo), recs[1], ps[1])

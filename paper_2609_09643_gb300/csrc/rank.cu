@@ -70,7 +70,7 @@ constexpr uint32_t kSampleCtas = 63;     // sampling CTAs per set, at most
 constexpr uint32_t kSampleQ = 4;         // samples per consumer thread
 constexpr uint32_t kLaunchSamples = 131072;  // samples per launch, about,
 constexpr uint32_t kSmallSample = 4096;  // the shortest lists, where this many samples give them
-constexpr uint32_t kSetSamples = 12288;      // or this many a set
+constexpr uint32_t kSetSamples = 16384;      // or this many a set
 constexpr uint32_t kBins = 4096;         // histogram bins per list
 constexpr uint32_t kEndTile = 0xFFFFFFFFu;
 
@@ -817,10 +817,10 @@ __device__ __forceinline__ void sort_desc(uint64_t *a, uint32_t n, uint64_t *tmp
 // P(Gamma(r) < r M / target) = P(Poisson(r M / target) >= r): r is large enough
 // when that is below 1e-6 (sample_rank).  A shortfall costs time, never
 // exactness (the finish re-selects the list).  A larger target needs a smaller
-// rank, hence a smaller sample (28, 17, 13, 10 for M = 1,024 at the targets
-// below: 0.9, 0.37, 0.21, 0.11 % of the records), but leaves more candidates to
+// rank, hence a smaller sample (28, 17, 13, 10 for M = 1,024 at the last four
+// targets below: 0.9, 0.37, 0.21, 0.11 % of the records), but leaves more candidates to
 // the streaming tests and the finish.  A set takes the smallest target whose
-// sample is within its cap: 1,024 a sampling CTA, and the larger of its share
+// sample is within its cap (plan_sample): 1,024 a sampling CTA, and the larger of its share
 // of kLaunchSamples and kSetSamples, because a sample's runs are random rows of
 // DRAM.  Measured, whole call: 33 sets of 2^20 records 118 us at 9,800 samples
 // a set, 139 us at 4,096 (18,000 candidates a set in place of 13,000, and a
@@ -833,10 +833,10 @@ __host__ __forceinline__ bool list_active(const RankSet &S, int L) {
   const uint32_t M = (L == 0) ? S.k : S.max_moves;
   return M > 0 && (L == 0 || S.budget > 0);
 }
-constexpr int kTargets = 5;
-__host__ __forceinline__ uint64_t list_target_of(const RankSet &S, int L, int o) {
-  const uint64_t M = (L == 0) ? S.k : S.max_moves;
-  const uint64_t mul[kTargets] = {2, 2, 3, 4, 6}, add[kTargets] = {128, 512, 512, 512, 512};
+constexpr int kTargets = 6;
+__host__ __forceinline__ uint64_t list_wanted(const RankSet &S, int L) { return (L == 0) ? S.k : S.max_moves; }
+__host__ __forceinline__ uint64_t target_of(uint64_t M, int o) {
+  const uint64_t mul[kTargets] = {2, 2, 2, 3, 4, 6}, add[kTargets] = {128, 256, 512, 512, 512, 512};
   return mul[o] * (M + add[o]);
 }
 // The smallest rank whose chance of a shortfall is below 1e-6, for a ratio M /
@@ -859,21 +859,10 @@ __host__ uint32_t sample_rank(uint64_t M, uint64_t target) {
   static const SampleRanks ranks;
   return ranks.r[std::min<uint64_t>((64 * M + target - 1) / target, 32)];
 }
-// Samples that target choice o needs, 0 for none.
-__host__ uint64_t sample_size(const RankSet &S, int o) {
-  // up to 4,096 records, the finish holds every record's value in shared
-  // memory; a set of 16,000 takes 42 us with a sample, and about 75 us when
-  // every record is a candidate
-  if (S.n <= kSmemCand) return 0;
-  uint64_t ns = 0, tmax = 0;
-  for (int L = 0; L < kLists; L++) {
-    if (!list_active(S, L)) continue;
-    const uint64_t M = (L == 0) ? S.k : S.max_moves, t = list_target_of(S, L, o);
-    tmax = std::max(tmax, t);
-    ns = std::max(ns, ((uint64_t)sample_rank(M, t) * S.n + t - 1) / t);
-  }
-  if (S.n <= kSample && 2 * tmax > S.n) return 0;  // a sample would leave most records candidates
-  return ns;
+// Samples that target choice o of a list of M needs.
+__host__ uint64_t sample_size(const RankSet &S, uint64_t M, int o) {
+  const uint64_t t = target_of(M, o);
+  return ((uint64_t)sample_rank(M, t) * S.n + t - 1) / t;
 }
 
 // CTAs a set can use: one a tile, and one a list for the finish (a set of
@@ -881,14 +870,38 @@ __host__ uint64_t sample_size(const RankSet &S, int o) {
 // 29 us, and 17 us when each collects its list's values itself).
 __host__ __forceinline__ uint32_t most_ctas(const RankSet &S) { return std::max<uint32_t>(S.ntiles, kLists); }
 
-// The sample plan of a set whose group (cta0, nctas) is fixed.
+// The sample plan of a set whose group (cta0, nctas) is fixed.  The longest
+// list decides the sample; each other list takes the smallest target that this
+// sample allows it (a short list needs more samples for a target of its size
+// than a long one, and chosen for all lists together it put the long lists on
+// larger targets: 9 sets of 2^22, k from 1 to 1,024, 100.3 us, 94.4 with a
+// target a list and 16,384 samples a set in place of 12,288).
+// The second target only where a set has few CTAs to share its candidates
+// among (64 sets of 2^18 93.0 -> 91.3 us; one set of 2^20 has 256 CTAs and
+// lost 1 us of 35 to the larger sample).
+constexpr uint32_t kFewCtas = 64;
 void plan_sample(RankSet &s, int n_sets) {
   const uint32_t most = std::min(s.nctas, kSampleCtas);
   const uint64_t share = std::max<uint64_t>(kLaunchSamples / n_sets, kSetSamples);
   const uint64_t cap = umin64((uint64_t)kPerCtaSamples * most, share);
-  int o = 0;
-  uint64_t ns = sample_size(s, 0);
-  while (ns > (o == 0 ? umin64(cap, kSmallSample) : cap) && o + 1 < kTargets) ns = sample_size(s, ++o);
+  uint64_t longest = 0, ns = 0;
+  for (int L = 0; L < kLists; L++)
+    if (list_active(s, L)) longest = std::max(longest, list_wanted(s, L));
+  // up to 4,096 records, the finish holds every record's value in shared
+  // memory; a set of 16,000 takes 42 us with a sample, and about 75 us when
+  // every record is a candidate
+  if (s.n > kSmemCand && longest) {
+    int o = 0;
+    for (;; o++) {
+      ns = sample_size(s, longest, o);
+      const bool fits = ns <= (o == 0 ? umin64(cap, kSmallSample) : cap) && (o != 1 || s.nctas < kFewCtas);
+      if (fits || o + 1 == kTargets) break;
+    }
+    if (s.n <= kSample && 2 * target_of(longest, o) > s.n) ns = 0;  // a sample would leave most records candidates
+  }
+  if (ns)
+    for (int L = 0; L < kLists; L++)
+      if (list_active(s, L)) ns = std::max(ns, sample_size(s, list_wanted(s, L), kTargets - 1));
   ns = umin64(ns, cap);
   // half a CTA's most a CTA where there are enough: the samples' latency is the
   // call's head
@@ -899,8 +912,14 @@ void plan_sample(RankSet &s, int n_sets) {
   s.ns = (uint32_t)ns;
   s.nruns = s.ns / 8;
   s.sstep = s.nruns ? ((uint64_t)s.n << 16) / s.nruns : 0;
-  for (int L = 0; L < kLists; L++)
-    s.rL[L] = (s.ns && list_active(s, L)) ? (uint32_t)((list_target_of(s, L, o) * s.ns + s.n - 1) / s.n) : 0u;
+  for (int L = 0; L < kLists; L++) {
+    s.rL[L] = 0;
+    if (!s.ns || !list_active(s, L)) continue;
+    const uint64_t M = list_wanted(s, L);
+    int o = 0;
+    while (o + 1 < kTargets && sample_size(s, M, o) > s.ns) o++;
+    s.rL[L] = (uint32_t)((target_of(M, o) * s.ns + s.n - 1) / s.n);
+  }
 }
 
 // Sampling CTA r of set S (consumer threads): samples j = r * per + jt of

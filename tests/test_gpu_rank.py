@@ -516,3 +516,17 @@ def test_captured_calls_replay_beside_ordinary_ones(B, sigma):
                 check(B.rank_result(oo), rec, p)
         for oo in (mout, sout):
             check(B.rank_result(oo), recs[1], ps[1])
+
+
+@pytest.mark.parametrize("n", [4_097, 40_001, 1 << 20])
+def test_lists_of_unlike_lengths_share_a_sample(B, sigma, n):
+    """One sample serves lists of 1 to 4,096 wanted: sets whose shortest list
+    is the victims', the moves' or neither, few CTAs a set and many."""
+    ks = [(1, 4096), (4096, 1), (64, 1024), (1024, 64), (300, 0), (2, 2)]
+    recs = [synth.make_records(90 + i, n) for i in range(2)]
+    recs = [recs[i % 2] for i in range(len(ks))]
+    ps = [prm(sigma, k=k, budget=16 * GIB, max_moves=m, free_s=10_000) for k, m in ks]
+    for r, rec, p in zip(run(B, recs, ps), recs, ps):
+        check(r, rec, p)
+    for rec, p in zip(recs[:2], ps[:2]):
+        check(run(B, [rec], [p])[0], rec, p)

@@ -870,6 +870,43 @@ __host__ uint64_t sample_size(const RankSet &S, uint64_t M, int o) {
 // 29 us, and 17 us when each collects its list's values itself).
 __host__ __forceinline__ uint32_t most_ctas(const RankSet &S) { return std::max<uint32_t>(S.ntiles, kLists); }
 
+// Groups of a launch of at most `ctas` sets: each set gets CTAs in proportion
+// to its tiles (at least 1, at most most_ctas); CTAs left over go to the sets
+// with the most tiles per CTA, and where the sets of less than a CTA's share
+// took more than there are, the sets with the fewest tiles per CTA give theirs
+// back.  Returns the CTAs of all groups: never more than `ctas`, which are
+// resident at once (a cooperative launch of more is refused).
+uint32_t share_ctas(std::vector<RankSet> &sets, uint32_t ctas, uint64_t tiles) {
+  uint64_t used = 0;
+  for (RankSet &s : sets) {
+    s.nctas = (uint32_t)std::max<uint64_t>(1, (uint64_t)ctas * s.ntiles / tiles);
+    s.nctas = std::min(s.nctas, most_ctas(s));
+    used += s.nctas;
+  }
+  auto denser = [](const RankSet &a, const RankSet &b) {  // more tiles per CTA
+    return (uint64_t)a.ntiles * b.nctas > (uint64_t)b.ntiles * a.nctas;
+  };
+  for (; used < ctas; used++) {
+    RankSet *most = nullptr;
+    for (RankSet &s : sets)
+      if (s.nctas < most_ctas(s) && (!most || denser(s, *most))) most = &s;
+    if (!most) break;
+    most->nctas++;
+  }
+  for (; used > ctas; used--) {
+    RankSet *least = nullptr;  // there is one: `ctas` sets or fewer hold more than `ctas`
+    for (RankSet &s : sets)
+      if (s.nctas > 1 && (!least || denser(*least, s))) least = &s;
+    least->nctas--;
+  }
+  uint32_t cta = 0;
+  for (RankSet &s : sets) {
+    s.cta0 = cta;
+    cta += s.nctas;
+  }
+  return cta;
+}
+
 // The sample plan of a set whose group (cta0, nctas) is fixed.  The longest
 // list decides the sample; each other list takes the smallest target that this
 // sample allows it (a short list needs more samples for a target of its size
@@ -2572,35 +2609,11 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
   }
   const LaunchCfg &cfg = launch_cfg();
   if (!cfg.ok) return UNISON_ERR_CUDA;
-  // Groups: each set gets CTAs in proportion to its tiles (at least 1, at
-  // most one a tile, or one a list); CTAs left over go to the sets with the most tiles
-  // per CTA.  With more sets than CTAs, CTA c takes sets c, c + G, ...
+  // Groups; with more sets than CTAs, CTA c takes sets c, c + G, ...
   const int sequential = (uint64_t)n_sets > cfg.ctas ? 1 : 0;
   uint32_t grid = cfg.ctas;
   if (!sequential) {
-    uint64_t used = 0;
-    for (int i = 0; i < n_sets; i++) {
-      RankSet &s = hs[i];
-      s.nctas = (uint32_t)std::max<uint64_t>(1, (uint64_t)cfg.ctas * s.ntiles / tiles);
-      s.nctas = std::min(s.nctas, most_ctas(s));
-      used += s.nctas;
-    }
-    while (used < cfg.ctas) {
-      int best = -1;
-      for (int i = 0; i < n_sets; i++)
-        if (hs[i].nctas < most_ctas(hs[i]) &&
-            (best < 0 || (uint64_t)hs[i].ntiles * hs[best].nctas > (uint64_t)hs[best].ntiles * hs[i].nctas))
-          best = i;
-      if (best < 0) break;
-      hs[best].nctas++;
-      used++;
-    }
-    uint32_t cta = 0;
-    for (int i = 0; i < n_sets; i++) {
-      hs[i].cta0 = cta;
-      cta += hs[i].nctas;
-    }
-    grid = cta;
+    grid = share_ctas(hs, cfg.ctas, tiles);
   } else {
     for (int i = 0; i < n_sets; i++) {
       hs[i].cta0 = (uint32_t)(i % cfg.ctas);

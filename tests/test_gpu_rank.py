@@ -314,6 +314,24 @@ def test_batch_of_mixed_sets(B, sigma):
         check(r, rec, p, keys=True)
 
 
+@pytest.mark.parametrize("large,small", [(1, 2), (1, 63), (2, 62), (3, 100)])
+def test_large_sets_beside_small_ones(B, sigma, large, small):
+    """Sets of 2^22 records beside sets of one tile: every small set's CTA is
+    one that the large sets' shares must leave, or the groups come to more CTAs
+    than are resident at once and the launch is refused."""
+    big = synth.make_records(61, 1 << 22)
+    recs = [synth.make_records(300 + i, 1000 + 13 * i) for i in range(small)]
+    for i in range(large):
+        recs.insert(i * small // large, big)
+    ps = [prm(sigma, k=40 + i % 3, budget=(1 + i % 5) * GIB, max_moves=50, free_s=5000) for i in range(len(recs))]
+    res = run(B, recs, ps)
+    whole = [i for i, r in enumerate(recs) if r is big][:1]
+    for i in whole + [i for i, r in enumerate(recs) if r is not big]:
+        check(res[i], recs[i], ps[i])
+    for i, r in enumerate(recs):
+        assert res[i]["status"] == 0 and len(res[i]["victims"]) == ps[i]["k"]
+
+
 def test_keys_exact_at_division_boundaries(B):
     """Every sigma in [41, 4095] (through a table of 51 distinct values per
     run), gaps at multiples of sigma and just below, and the largest gap."""

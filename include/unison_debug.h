@@ -5,10 +5,11 @@
  * the ranking call compiled with UNISON_DEBUG_HOOKS).  The default library,
  * libunison.so, neither exports them nor contains the hooks.  The paper has
  * no counterpart: they let a test show that a bounded device wait of the
- * ranking kernel runs out, reports itself, and leaves the GPU usable.
+ * ranking kernel runs out, reports itself, and leaves the GPU usable, and
+ * that a ranking call is not misled by an older call's error.
  *
- * In the test library every bounded wait of the ranking kernel gives up
- * after a few thousand polls instead of more than a second.
+ * In the test library the ranking kernel's bounded waits give up after 2 ms
+ * (on another CTA) and 50 ms (on a CTA's own copies) instead of 2 and 4 s.
  */
 #ifndef UNISON_DEBUG_H
 #define UNISON_DEBUG_H
@@ -25,6 +26,11 @@ extern "C" {
  * its other outputs are still the exact ranking.  -1 turns a hook off.
  * Returns UNISON_OK, or UNISON_ERR_CUDA if the hooks could not be set. */
 int unison_debug_rank_wait_hooks(int flag_set, int mbar_set);
+
+/* Makes a failing CUDA call (an invalid device number; nothing reaches the
+ * device) and leaves its error pending in the library's CUDA runtime.  The
+ * current device stays as it was.  Returns UNISON_OK if an error is pending. */
+int unison_debug_leave_error(void);
 
 #ifdef __cplusplus
 }

@@ -92,7 +92,7 @@ _lib = None
 
 # Every symbol include/unison.h declares (checked by the ABI tests).
 # the test library of native.build_debug() (include/unison_debug.h) adds these
-DEBUG_EXPORTS = ["unison_debug_rank_wait_hooks"]
+DEBUG_EXPORTS = ["unison_debug_rank_wait_hooks", "unison_debug_leave_error"]
 EXPORTS = ["unison_strerror", "unison_version", "unison_trace_create", "unison_trace_load",
            "unison_trace_upload", "unison_trace_free", "unison_trace_info", "unison_trace_device_bytes",
            "unison_replay_batch", "unison_stats", "unison_hazard_lut", "unison_rank_batch", "unison_rank",
@@ -131,6 +131,7 @@ def debug_lib():
                 raise RuntimeError(f"{LIB_DEBUG} is missing: run native.build_debug() first")
             L = _bind_rank(C.CDLL(LIB_DEBUG))
             L.unison_debug_rank_wait_hooks.argtypes = [C.c_int, C.c_int]
+            L.unison_debug_leave_error.argtypes = []
             _debug_lib = L
     return _debug_lib
 

@@ -2438,6 +2438,12 @@ extern "C" int unison_debug_rank_wait_hooks(int flag_set, int mbar_set) {
   }
   return UNISON_OK;
 }
+
+// Leaves an error pending in the library's CUDA runtime, as a call that failed
+// without clearing it would.  Nothing reaches the device.
+extern "C" int unison_debug_leave_error(void) {
+  return cudaSetDevice(-1) != cudaSuccess && cudaPeekAtLastError() != cudaSuccess ? UNISON_OK : UNISON_ERR_CUDA;
+}
 #endif
 
 namespace {
@@ -2504,7 +2510,8 @@ int launch_rank_kernel(StreamState &st, uint32_t grid, const RankSet *d_sets, in
                            reinterpret_cast<uint4 *>(other), n_other, pack);
   }
   count_launches(1);
-  if (e == cudaSuccess) e = cudaGetLastError();
+  // The launch's own verdict: cudaGetLastError() could name an older call's
+  // error although the kernel is queued and will leave its block dirty.
   if (e != cudaSuccess) {
     cudaGetLastError();
     st.planned = false;
@@ -2826,12 +2833,20 @@ extern "C" int unison_rank_merge(const void *gathered_dev, int n_shards, const u
   s.work = reinterpret_cast<RankWork *>(st.zero[b].p);
   s.sorted = reinterpret_cast<uint64_t *>(st.main.p);
   s.ssz = reinterpret_cast<uint32_t *>(st.main.p + vals_b);
-  rank_merge_kernel<<<kLists, kConsumers, kMergeSmem, stream>>>(
-      s, static_cast<const unsigned char *>(gathered_dev), n_shards, (uint64_t)cand_bytes(p.k, p.max_moves),
-      reinterpret_cast<uint4 *>(captured ? nullptr : st.zero[1 - b].p),
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(kLists);
+  lc.blockDim = dim3(kConsumers);
+  lc.dynamicSmemBytes = kMergeSmem;
+  lc.stream = stream;
+  const cudaError_t e = cudaLaunchKernelEx(
+      &lc, rank_merge_kernel, s, static_cast<const unsigned char *>(gathered_dev), n_shards,
+      (uint64_t)cand_bytes(p.k, p.max_moves), reinterpret_cast<uint4 *>(captured ? nullptr : st.zero[1 - b].p),
       captured ? 0u : (uint32_t)(st.dirty[1 - b] / 16));
   count_launches(1);
-  if (cudaGetLastError() != cudaSuccess) return UNISON_ERR_CUDA;  // nothing ran: the blocks are as they were
+  if (e != cudaSuccess) {  // (its own verdict, as in launch_rank_kernel)
+    cudaGetLastError();
+    return UNISON_ERR_CUDA;  // nothing ran: the blocks are as they were
+  }
   if (captured) return UNISON_OK;
   st.dirty[b] = work_b;
   st.dirty[1 - b] = 0;

@@ -467,6 +467,41 @@ def test_bounded_waits_report_timeout_and_recover(B, sigma):
         check(B.rank_result(o), rec, p)
 
 
+def test_older_error_does_not_mislead_ranking_calls(B, sigma):
+    """An error that an earlier call left pending is not taken for the launch's:
+    each ranking call (batch, shard, merge) reports its own verdict, queues its
+    work once and leaves its zero blocks in the state the next call expects."""
+    import ctypes
+    import torch
+    from paper_2609_09643_gb300 import native
+    native.build_debug()
+    D = B.debug_lib()
+    rec, p = synth.make_records(47, 60_000), prm(sigma, k=200, budget=4 * GIB, max_moves=100, free_s=9000)
+    dev = B.records_to_device(rec)
+    stream = torch.cuda.Stream()
+    handle = ctypes.c_void_p(stream.cuda_stream)
+    cands = [B.rank_cands(p["k"], p["max_moves"]) for _ in range(2)]
+    outs = [B.rank_outputs(rec.n, p["k"], p["max_moves"]) for _ in range(4)]
+    torch.cuda.synchronize()
+    cp, half = B._rank_params(p), rec.n // 32 * 16
+    for o in outs[:2]:  # two calls in a row, then shards and a merge, then one more
+        assert D.unison_debug_leave_error() == B.OK
+        B.RankCall([dev], [p], [o], lib_=D).run(stream)
+    for i, (a, b) in enumerate(((0, half), (half, rec.n))):
+        part = B._records({f: v[a:b] for f, v in dev.items()})
+        assert D.unison_debug_leave_error() == B.OK
+        assert D.unison_rank_shard(ctypes.byref(part), a, ctypes.byref(cp), cands[i].data_ptr(), handle) == B.OK
+    stream.synchronize()
+    both, mo = torch.cat(cands), B._rank_out(outs[2])
+    torch.cuda.synchronize()
+    assert D.unison_debug_leave_error() == B.OK
+    assert D.unison_rank_merge(both.data_ptr(), 2, ctypes.byref(cp), ctypes.byref(mo), handle) == B.OK
+    B.RankCall([dev], [p], [outs[3]], lib_=D).run(stream)
+    stream.synchronize()
+    for o in outs:
+        check(B.rank_result(o), rec, p)
+
+
 @pytest.mark.parametrize("world", [2, 4])
 def test_record_sharded_ranking_equals_whole_set(B, sigma, world):
     """Sec. IV-D's scan split by records: each slice ranked into its candidate

@@ -469,6 +469,15 @@ typedef struct {
  * stream's scratch; calls on different streams use different scratch.  The
  * scratch is found by the stream's handle, so a stream must outlive the
  * ranking calls queued on it.
+ * Capture: a call on a stream that is being captured becomes part of the
+ * graph, which may then run at any time, on any stream and any number of
+ * times, beside other calls; two executables of one graph must not run at the
+ * same time, as they share the call's scratch.  Each captured call (of this and
+ * of the three entry points below) has device memory of its own, held by the
+ * graph and its executables and freed by a ranking call made after they are
+ * gone.  The arrays must stay valid as long as the graph may run; params are
+ * read at the capture.  (Replay calls copy from host memory of the call and
+ * are not for capture.)
  * Errors: UNISON_ERR_ARG (null or misaligned arrays), UNISON_ERR_RANGE
  * (limits above), UNISON_ERR_OOM (scratch or staging), UNISON_ERR_CUDA
  * (launch; a device without cooperative launch); a bounded device wait that

@@ -43,11 +43,13 @@
 // to the end of the kernel.  A cooperative launch keeps every CTA of the grid
 // resident, so the waits on other CTAs end.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <map>
 #include <memory>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "common.cuh"
@@ -2271,8 +2273,9 @@ struct RankPlan {
   RankPack<kPackSets> pack[2];  // for each block
 };
 struct StreamState {
+  int dev = 0;
   std::mutex mu;  // held from the choice of a block to the launch that uses it
-  Scratch main, zero[3];  // zero[2]: of captured calls (block_for)
+  Scratch main, zero[2];
   size_t dirty[2] = {0, 0};  // bytes from a block's start that are not zero
   bool planned = false;
   RankPlan plan;
@@ -2293,7 +2296,10 @@ StreamState *stream_state(cudaStream_t stream) {
   }
   std::lock_guard<std::mutex> lock(g_state_mu);
   auto &e = g_state[std::make_pair(dev, stream)];
-  if (!e) e.reset(new StreamState());
+  if (!e) {
+    e.reset(new StreamState());
+    e->dev = dev;
+  }
   return e.get();
 }
 
@@ -2319,13 +2325,162 @@ int grow(Scratch &e, size_t bytes, bool zero, cudaStream_t stream) {
 
 // The zero blocks at least `bytes` long (a new block is zero).
 int grow_zero(StreamState &st, size_t bytes, cudaStream_t stream) {
-  for (int i = 0; i < 3; i++) {
+  for (int i = 0; i < 2; i++) {
     if (st.zero[i].bytes >= bytes) continue;
-    if (i < 2) st.dirty[i] = 0;
+    st.dirty[i] = 0;
     st.planned = false;  // the plan's descriptors name the old block
     const int rc = grow(st.zero[i], bytes, true, stream);
     if (rc != UNISON_OK) return rc;
   }
+  return UNISON_OK;
+}
+
+// Memory of captured calls.  A call captured into a graph runs whenever the
+// graph does, any number of times, on any stream and between any other calls,
+// so it shares nothing with them: its scratch, its work words and histograms
+// (cleared by a node of the graph) and the descriptors, tables and CTA map that
+// do not go with the launch (written once, here: they never change) lie in
+// memory of its own, which stays where it is.  The graph and every executable
+// made from it hold that memory by a user object; when the last of them is gone
+// its destructor, which may not call CUDA, leaves the memory on a list that the
+// device's next ranking call frees.
+struct GraphMem {
+  char *p;
+  int dev;
+  GraphMem *next;
+};
+struct GraphPool {
+  std::mutex mu;
+  GraphMem *unused = nullptr;
+  std::atomic<bool> any{false};  // something in the list
+  cudaStream_t side[64] = {};    // for the memory's allocation and uploads
+};
+GraphPool &graph_pool() {
+  static GraphPool *const g = new GraphPool;  // outlives the last graph
+  return *g;
+}
+void CUDART_CB graph_gone(void *mem) {
+  GraphPool &g = graph_pool();
+  GraphMem *const m = static_cast<GraphMem *>(mem);
+  std::lock_guard<std::mutex> lock(g.mu);
+  m->next = g.unused;
+  g.unused = m;
+  g.any.store(true, std::memory_order_release);
+}
+
+// Frees, in `stream`'s order, the memory of the device's graphs that are gone.
+void free_unused(int dev, cudaStream_t stream) {
+  GraphPool &g = graph_pool();
+  if (!g.any.load(std::memory_order_acquire)) return;
+  GraphMem *mine = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g.mu);
+    for (GraphMem **at = &g.unused; *at;) {
+      GraphMem *const m = *at;
+      if (m->dev != dev) {
+        at = &m->next;
+        continue;
+      }
+      *at = m->next;
+      m->next = mine;
+      mine = m;
+    }
+    g.any.store(g.unused != nullptr, std::memory_order_release);
+  }
+  while (mine) {
+    GraphMem *const m = mine;
+    mine = m->next;
+    if (cudaFreeAsync(m->p, stream) != cudaSuccess) cudaGetLastError();
+    delete m;
+  }
+}
+
+// While a capture is under way its thread may allocate and wait only in this
+// mode, on streams that are not captured.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// Memory for one captured call, held by `graph`.
+int graph_alloc(size_t bytes, cudaGraph_t graph, char **out) {
+  GraphPool &g = graph_pool();
+  RelaxedCapture relaxed;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    return UNISON_ERR_CUDA;
+  }
+  cudaStream_t side = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g.mu);
+    if (!g.side[dev] && cudaStreamCreateWithFlags(&g.side[dev], cudaStreamNonBlocking) != cudaSuccess) {
+      cudaGetLastError();
+      g.side[dev] = nullptr;
+      return UNISON_ERR_CUDA;
+    }
+    side = g.side[dev];
+  }
+  free_unused(dev, side);
+  GraphMem *const m = new (std::nothrow) GraphMem{nullptr, dev, nullptr};
+  if (!m) return UNISON_ERR_OOM;
+  if (unison_fault_alloc() || cudaMallocAsync(reinterpret_cast<void **>(&m->p), bytes, side) != cudaSuccess) {
+    cudaGetLastError();
+    delete m;
+    return UNISON_ERR_OOM;
+  }
+  cudaUserObject_t held = nullptr;
+  if (cudaStreamSynchronize(side) != cudaSuccess ||
+      cudaUserObjectCreate(&held, m, graph_gone, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFreeAsync(m->p, side);
+    delete m;
+    return UNISON_ERR_CUDA;
+  }
+  if (cudaGraphRetainUserObject(graph, held, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+    cudaGetLastError();
+    cudaUserObjectRelease(held, 1);  // its destructor takes the memory
+    return UNISON_ERR_CUDA;
+  }
+  *out = m->p;
+  return UNISON_OK;
+}
+
+// Fills [dst, dst + bytes) of a captured call's memory from host memory, now.
+int graph_write(char *dst, const void *src, size_t bytes) {
+  RelaxedCapture relaxed;
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
+    cudaStream_t side = nullptr;
+    {
+      std::lock_guard<std::mutex> lock(graph_pool().mu);
+      side = graph_pool().side[dev];  // made by graph_alloc
+    }
+    if (side && cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, side) == cudaSuccess &&
+        cudaStreamSynchronize(side) == cudaSuccess)
+      return UNISON_OK;
+  }
+  cudaGetLastError();
+  return UNISON_ERR_CUDA;
+}
+
+// Whether `stream` is being captured, and into which graph.
+int capture_of(cudaStream_t stream, bool *captured, cudaGraph_t *graph) {
+  *captured = false;
+  *graph = nullptr;
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &s) != cudaSuccess) {
+    cudaGetLastError();  // (the legacy stream beside a capture: its launches are refused)
+    return UNISON_OK;
+  }
+  if (s == cudaStreamCaptureStatusNone) return UNISON_OK;
+  if (s != cudaStreamCaptureStatusActive ||
+      cudaStreamGetCaptureInfo(stream, &s, nullptr, graph, nullptr, nullptr, nullptr) != cudaSuccess || !*graph) {
+    cudaGetLastError();
+    return UNISON_ERR_CUDA;  // a capture that failed already
+  }
+  *captured = true;
   return UNISON_OK;
 }
 
@@ -2466,33 +2621,13 @@ void plan_key(std::vector<unsigned char> &k, const unison_records *sets, const u
   if (!cands) put(outs, sizeof(unison_rank_out) * n_sets);
 }
 
-// Launches a call on the zero block whose turn it is (zb: the bytes of it that
-// the call uses), zeroing the other.  The caller holds st.mu and has passed
-// that block (next_block) to the descriptors.
-// A call captured into a graph runs whenever the graph does, any number of
-// times, so it takes a block apart from the ordinary calls' and clears it by a
-// node of its own.
-int next_block(const StreamState &st) { return st.dirty[0] == 0 ? 0 : 1; }
-int block_for(const StreamState &st, bool captured) { return captured ? 2 : next_block(st); }
-bool is_capturing(cudaStream_t stream) {
-  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(stream, &s) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return s != cudaStreamCaptureStatusNone;
-}
+// Queues the kernel.  The verdict is the launch's own: cudaGetLastError() could
+// name an older call's error although the kernel is queued and will leave its
+// block dirty.
 template <int kSets>
-int launch_rank_kernel(StreamState &st, uint32_t grid, const RankSet *d_sets, int n_sets, int sequential,
-                       const uint32_t *cmap, const RankTab *tabs, const RankPack<kSets> &pack, size_t zb,
-                       bool captured, cudaStream_t stream) {
-  const int p = block_for(st, captured);
-  if (captured && cudaMemsetAsync(st.zero[p].p, 0, zb, stream) != cudaSuccess) {
-    cudaGetLastError();
-    return UNISON_ERR_CUDA;
-  }
-  char *const other = captured ? nullptr : st.zero[1 - p].p;
-  const uint32_t n_other = captured ? 0u : (uint32_t)(st.dirty[1 - p] / 16);
+int queue_rank_kernel(uint32_t grid, const RankSet *d_sets, int n_sets, int sequential, const uint32_t *cmap,
+                      const RankTab *tabs, const RankPack<kSets> &pack, char *other, size_t other_b,
+                      cudaStream_t stream) {
   cudaError_t e;
   {
     ProfSpan span("rank", stream);
@@ -2507,20 +2642,44 @@ int launch_rank_kernel(StreamState &st, uint32_t grid, const RankSet *d_sets, in
     lc.attrs = coop;
     lc.numAttrs = 1;
     e = cudaLaunchKernelEx(&lc, rank_kernel<kSets>, d_sets, n_sets, sequential, cmap, tabs,
-                           reinterpret_cast<uint4 *>(other), n_other, pack);
+                           reinterpret_cast<uint4 *>(other), (uint32_t)(other_b / 16), pack);
   }
   count_launches(1);
-  // The launch's own verdict: cudaGetLastError() could name an older call's
-  // error although the kernel is queued and will leave its block dirty.
-  if (e != cudaSuccess) {
-    cudaGetLastError();
+  if (e == cudaSuccess) return UNISON_OK;
+  cudaGetLastError();
+  return UNISON_ERR_CUDA;  // nothing ran
+}
+
+// Launches a call on the zero block whose turn it is (zb: the bytes of it that
+// the call uses), zeroing the other.  The caller holds st.mu and has passed
+// that block (next_block) to the descriptors.
+int next_block(const StreamState &st) { return st.dirty[0] == 0 ? 0 : 1; }
+template <int kSets>
+int launch_rank_kernel(StreamState &st, uint32_t grid, const RankSet *d_sets, int n_sets, int sequential,
+                       const uint32_t *cmap, const RankTab *tabs, const RankPack<kSets> &pack, size_t zb,
+                       cudaStream_t stream) {
+  const int p = next_block(st);
+  const int rc = queue_rank_kernel(grid, d_sets, n_sets, sequential, cmap, tabs, pack, st.zero[1 - p].p,
+                                   st.dirty[1 - p], stream);
+  if (rc != UNISON_OK) {
     st.planned = false;
-    return UNISON_ERR_CUDA;  // nothing ran: the blocks are as they were
+    return rc;  // the blocks are as they were
   }
-  if (captured) return UNISON_OK;
   st.dirty[p] = zb;
   st.dirty[1 - p] = 0;
   return UNISON_OK;
+}
+
+// A captured call: its own words are cleared by a node before the kernel's.
+template <int kSets>
+int capture_rank_kernel(uint32_t grid, const RankSet *d_sets, int n_sets, int sequential, const uint32_t *cmap,
+                        const RankTab *tabs, const RankPack<kSets> &pack, char *words, size_t zb,
+                        cudaStream_t stream) {
+  if (cudaMemsetAsync(words, 0, zb, stream) != cudaSuccess) {
+    cudaGetLastError();
+    return UNISON_ERR_CUDA;
+  }
+  return queue_rank_kernel(grid, d_sets, n_sets, sequential, cmap, tabs, pack, nullptr, 0, stream);
 }
 
 int rank_launch(const unison_records *sets, const unison_rank_params *params, const unison_rank_out *outs,
@@ -2528,21 +2687,25 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
   StreamState *const state = stream_state(stream);
   if (!state) return UNISON_ERR_CUDA;
   StreamState &st = *state;
+  bool captured = false;
+  cudaGraph_t graph = nullptr;
+  int rc = capture_of(stream, &captured, &graph);
+  if (rc != UNISON_OK) return rc;
   std::lock_guard<std::mutex> lock(st.mu);
-  const bool captured = is_capturing(stream);
+  if (!captured) free_unused(st.dev, stream);
   static const RankPack<1> none{};
   thread_local std::vector<unsigned char> key;
-  if (n_sets > 1) {
+  if (n_sets > 1 && !captured) {
     plan_key(key, sets, params, outs, n_sets, off, cands);
-    if (!captured && st.planned && st.plan.key == key) {
+    if (st.planned && st.plan.key == key) {
       const RankPlan &pl = st.plan;
       if (pl.packed)
         return launch_rank_kernel(st, pl.grid, nullptr, n_sets, 0, nullptr, nullptr, pl.pack[next_block(st)], pl.zero_b,
-                                  false, stream);
+                                  stream);
       return launch_rank_kernel(
           st, pl.grid, reinterpret_cast<const RankSet *>(st.main.p + next_block(st) * pl.desc_b), n_sets, pl.sequential,
           pl.sequential ? nullptr : reinterpret_cast<const uint32_t *>(st.main.p + pl.cmap_off),
-          reinterpret_cast<const RankTab *>(st.main.p + pl.tabs_off), none, pl.zero_b, false, stream);
+          reinterpret_cast<const RankTab *>(st.main.p + pl.tabs_off), none, pl.zero_b, stream);
     }
   }
   std::vector<RankSet> hs(n_sets);
@@ -2628,9 +2791,10 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
     }
   }
   for (int i = 0; i < n_sets; i++) plan_sample(hs[i], n_sets);
-  // scratch: the descriptors, CTA map and tables of a call that uploads them,
-  // then per set: sorted lists and sizes, candidates.  In a zero block: every
-  // set's work words, then the sampled sets' histograms
+  // scratch: the descriptors (for each zero block; a captured call has one),
+  // CTA map and tables of a call whose launch does not bring them, then per
+  // set: sorted lists and sizes, candidates.  In a zero block: every set's work
+  // words, then the sampled sets' histograms
   const size_t fixed_set = align_up(sizeof(uint64_t) * kLists * kMaxSel, 256) +
                            align_up(sizeof(uint32_t) * kLists * kMaxSel, 256);
   const size_t hist_set = sizeof(uint16_t) * kLists * kBins;
@@ -2654,16 +2818,24 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
   const size_t tab_b = packed ? 0 : align_up(sizeof(RankTab) * tabs.size(), 256);
   const size_t work_b = align_up(sizeof(RankWork) * n_sets, 256);
   const size_t zero_b = work_b + hist_b;
-  st.planned = false;  // the scratch is rewritten below; the plan returns only if the launch succeeds
-  int rc = grow(st.main, 2 * desc_b + cmap_b + tab_b + sets_b, false, stream);
-  if (rc == UNISON_OK) rc = grow_zero(st, zero_b, stream);
-  if (rc != UNISON_OK) return rc;
-  // image: descriptors for block 0 and 1, the CTA map, tables; then the
-  // per-set areas
-  const size_t cmap_off = 2 * desc_b, tabs_off = cmap_off + cmap_b;
-  char *const scratch = st.main.p;
+  const int images = captured ? 1 : 2;
+  const size_t cmap_off = images * desc_b, tabs_off = cmap_off + cmap_b, up_b = tabs_off + tab_b;
+  char *scratch = nullptr, *block[2] = {};
+  if (captured) {
+    rc = graph_alloc(up_b + sets_b + zero_b, graph, &scratch);
+    if (rc != UNISON_OK) return rc;
+    block[0] = scratch + up_b + sets_b;
+  } else {
+    st.planned = false;  // the scratch is rewritten below; the plan returns only if the launch succeeds
+    rc = grow(st.main, up_b + sets_b, false, stream);
+    if (rc == UNISON_OK) rc = grow_zero(st, zero_b, stream);
+    if (rc != UNISON_OK) return rc;
+    scratch = st.main.p;
+    for (int b = 0; b < 2; b++) block[b] = st.zero[b].p;
+  }
   RankTab *d_tabs = reinterpret_cast<RankTab *>(scratch + tabs_off);
-  char *p = scratch + tabs_off + tab_b;
+  const uint32_t *d_cmap = sequential ? nullptr : reinterpret_cast<const uint32_t *>(scratch + cmap_off);
+  char *p = scratch + up_b;
   for (int i = 0; i < n_sets; i++) {
     RankSet &s = hs[i];
     s.tab = d_tabs + tab_of[i];
@@ -2678,7 +2850,7 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
   }
   // the work words and histograms of the sets in block b
   auto in_block = [&](int b) {
-    char *const z = st.zero[b].p;
+    char *const z = block[b];
     size_t hoff = work_b;
     for (int i = 0; i < n_sets; i++) {
       RankSet &s = hs[i];
@@ -2688,27 +2860,35 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
     }
   };
   if (single) {
-    in_block(block_for(st, captured));
+    in_block(captured ? 0 : next_block(st));
     RankPack<1> one;
     one.set[0] = hs[0];
     one.tab[0] = tabs[0];
-    return launch_rank_kernel(st, grid, nullptr, 1, 0, nullptr, nullptr, one, zero_b, captured, stream);
+    if (captured) return capture_rank_kernel(grid, nullptr, 1, 0, nullptr, nullptr, one, block[0], zero_b, stream);
+    return launch_rank_kernel(st, grid, nullptr, 1, 0, nullptr, nullptr, one, zero_b, stream);
   }
   if (packed) {
-    RankPlan &pl = st.plan;
-    for (int b = 0; b < 2; b++) {
-      in_block(captured ? 2 : b);
-      RankPack<kPackSets> &pk = pl.pack[b];
+    auto fill_pack = [&](RankPack<kPackSets> &pk) {
       std::memcpy(pk.set, hs.data(), sizeof(RankSet) * n_sets);
       std::memcpy(pk.tab, tabs.data(), sizeof(RankTab) * tabs.size());
       for (int i = 0; i < n_sets; i++) {
         pk.tab_of[i] = (uint8_t)tab_of[i];
         std::memset(pk.of_cta + hs[i].cta0, i, hs[i].nctas);
       }
+    };
+    if (captured) {
+      RankPack<kPackSets> pk;
+      in_block(0);
+      fill_pack(pk);
+      return capture_rank_kernel(grid, nullptr, n_sets, 0, nullptr, nullptr, pk, block[0], zero_b, stream);
     }
-    rc = launch_rank_kernel(st, grid, nullptr, n_sets, 0, nullptr, nullptr, pl.pack[next_block(st)], zero_b, captured,
-                            stream);
-    if (rc == UNISON_OK && !captured) {
+    RankPlan &pl = st.plan;
+    for (int b = 0; b < 2; b++) {
+      in_block(b);
+      fill_pack(pl.pack[b]);
+    }
+    rc = launch_rank_kernel(st, grid, nullptr, n_sets, 0, nullptr, nullptr, pl.pack[next_block(st)], zero_b, stream);
+    if (rc == UNISON_OK) {
       pl.key = key;
       pl.zero_b = zero_b;
       pl.grid = grid;
@@ -2718,15 +2898,10 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
     }
     return rc;
   }
-  // one copy from pinned staging
-  {
-    const size_t up = tabs_off + tab_b;
-    unsigned char *h = nullptr;
-    cudaEvent_t done = nullptr;
-    const int sr = staging_acquire(up, &h, &done);
-    if (sr != UNISON_OK) return sr;
-    for (int b = 0; b < 2; b++) {
-      in_block(captured ? 2 : b);
+  // the image of what the launch does not bring
+  auto fill_image = [&](unsigned char *h) {
+    for (int b = 0; b < images; b++) {
+      in_block(b);
       std::memcpy(h + b * desc_b, hs.data(), sizeof(RankSet) * n_sets);
     }
     if (!sequential) {
@@ -2735,7 +2910,23 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
         for (uint32_t b = hs[i].cta0; b < hs[i].cta0 + hs[i].nctas; b++) cm[b] = (uint32_t)i | ((uint32_t)tab_of[i] << 16);
     }
     std::memcpy(h + tabs_off, tabs.data(), sizeof(RankTab) * tabs.size());
-    if (cudaMemcpyAsync(scratch, h, up, cudaMemcpyHostToDevice, stream) != cudaSuccess) rc = UNISON_ERR_CUDA;
+  };
+  if (captured) {
+    std::vector<uint64_t> image((up_b + 7) / 8);
+    fill_image(reinterpret_cast<unsigned char *>(image.data()));
+    rc = graph_write(scratch, image.data(), up_b);
+    if (rc != UNISON_OK) return rc;
+    return capture_rank_kernel(grid, reinterpret_cast<const RankSet *>(scratch), n_sets, sequential, d_cmap, d_tabs,
+                               none, block[0], zero_b, stream);
+  }
+  // one copy from pinned staging
+  {
+    unsigned char *h = nullptr;
+    cudaEvent_t done = nullptr;
+    const int sr = staging_acquire(up_b, &h, &done);
+    if (sr != UNISON_OK) return sr;
+    fill_image(h);
+    if (cudaMemcpyAsync(scratch, h, up_b, cudaMemcpyHostToDevice, stream) != cudaSuccess) rc = UNISON_ERR_CUDA;
     if (cudaEventRecord(done, stream) != cudaSuccess) rc = UNISON_ERR_CUDA;  // the buffer is reused after this copy
     staging_release();
     if (rc != UNISON_OK) {
@@ -2744,9 +2935,8 @@ int rank_launch(const unison_records *sets, const unison_rank_params *params, co
     }
   }
   rc = launch_rank_kernel(st, grid, reinterpret_cast<const RankSet *>(scratch + next_block(st) * desc_b), n_sets,
-                          sequential, sequential ? nullptr : reinterpret_cast<const uint32_t *>(scratch + cmap_off),
-                          d_tabs, none, zero_b, captured, stream);
-  if (rc == UNISON_OK && !captured) {
+                          sequential, d_cmap, d_tabs, none, zero_b, stream);
+  if (rc == UNISON_OK) {
     RankPlan &pl = st.plan;
     pl.key = key;
     pl.desc_b = desc_b;
@@ -2819,20 +3009,36 @@ extern "C" int unison_rank_merge(const void *gathered_dev, int n_shards, const u
   StreamState *const state = stream_state(stream);
   if (!state) return UNISON_ERR_CUDA;
   StreamState &st = *state;
-  std::lock_guard<std::mutex> lock(st.mu);
-  st.planned = false;  // the scratch is rewritten below
-  int rc = grow(st.main, lists_b, false, stream);
-  if (rc == UNISON_OK) rc = grow_zero(st, work_b, stream);
+  bool captured = false;
+  cudaGraph_t graph = nullptr;
+  int rc = capture_of(stream, &captured, &graph);
   if (rc != UNISON_OK) return rc;
-  const bool captured = is_capturing(stream);
-  const int b = block_for(st, captured);
-  if (captured && cudaMemsetAsync(st.zero[b].p, 0, work_b, stream) != cudaSuccess) {
-    cudaGetLastError();
-    return UNISON_ERR_CUDA;
+  std::lock_guard<std::mutex> lock(st.mu);
+  char *scratch = nullptr, *words = nullptr, *other = nullptr;
+  size_t other_b = 0;
+  const int b = next_block(st);
+  if (captured) {  // (memory of its own, as in rank_launch)
+    rc = graph_alloc(lists_b + work_b, graph, &scratch);
+    if (rc != UNISON_OK) return rc;
+    words = scratch + lists_b;
+    if (cudaMemsetAsync(words, 0, work_b, stream) != cudaSuccess) {
+      cudaGetLastError();
+      return UNISON_ERR_CUDA;
+    }
+  } else {
+    free_unused(st.dev, stream);
+    st.planned = false;  // the scratch is rewritten below
+    rc = grow(st.main, lists_b, false, stream);
+    if (rc == UNISON_OK) rc = grow_zero(st, work_b, stream);
+    if (rc != UNISON_OK) return rc;
+    scratch = st.main.p;
+    words = st.zero[b].p;
+    other = st.zero[1 - b].p;
+    other_b = st.dirty[1 - b];
   }
-  s.work = reinterpret_cast<RankWork *>(st.zero[b].p);
-  s.sorted = reinterpret_cast<uint64_t *>(st.main.p);
-  s.ssz = reinterpret_cast<uint32_t *>(st.main.p + vals_b);
+  s.work = reinterpret_cast<RankWork *>(words);
+  s.sorted = reinterpret_cast<uint64_t *>(scratch);
+  s.ssz = reinterpret_cast<uint32_t *>(scratch + vals_b);
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(kLists);
   lc.blockDim = dim3(kConsumers);
@@ -2840,10 +3046,9 @@ extern "C" int unison_rank_merge(const void *gathered_dev, int n_shards, const u
   lc.stream = stream;
   const cudaError_t e = cudaLaunchKernelEx(
       &lc, rank_merge_kernel, s, static_cast<const unsigned char *>(gathered_dev), n_shards,
-      (uint64_t)cand_bytes(p.k, p.max_moves), reinterpret_cast<uint4 *>(captured ? nullptr : st.zero[1 - b].p),
-      captured ? 0u : (uint32_t)(st.dirty[1 - b] / 16));
+      (uint64_t)cand_bytes(p.k, p.max_moves), reinterpret_cast<uint4 *>(other), (uint32_t)(other_b / 16));
   count_launches(1);
-  if (e != cudaSuccess) {  // (its own verdict, as in launch_rank_kernel)
+  if (e != cudaSuccess) {  // (its own verdict, as in queue_rank_kernel)
     cudaGetLastError();
     return UNISON_ERR_CUDA;  // nothing ran: the blocks are as they were
   }

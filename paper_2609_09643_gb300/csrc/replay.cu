@@ -270,11 +270,33 @@ __device__ __forceinline__ uint32_t lower_bound(const Sorted &T, uint64_t k, int
   return lo + __popc(__ballot_sync(kFull, i < hi && ekey(T.e[i]) < k));
 }
 
-// Move e[lo, hi) by delta places (delta > 0 toward the end), warp-parallel.
+// Move e[lo, hi) by delta places (delta > 0 toward the end), warp-parallel:
+// whole chunks of 256 entries, eight of a lane's in flight and no predicates,
+// then the rest four at a time.  A list of 6,000 in global memory took 192 to
+// 481 cycles per 128 entries four at a time, depending on the kernel around it
+// (99.9 and 95.4 % of the sectors found in L1), and takes 135 to 142 so; 2,800
+// residents in shared memory, lru, 411 -> 370 ms a replay.
 // Out of line on purpose: inlined at every call site, the shifts' register
 // demand crowds the event loop.
 __device__ __noinline__ void shift_block(uint4 *e, uint32_t lo, uint32_t hi, int32_t delta, int lane) {
   if (lo >= hi || delta == 0) return;
+  if (hi - lo >= 256) {
+    auto whole = [&](uint32_t bot) {
+      uint4 *const from = e + bot + lane, *const to = from + delta;
+      uint4 v[8];
+#pragma unroll
+      for (int j = 0; j < 8; j++) v[j] = from[32 * j];
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < 8; j++) to[32 * j] = v[j];
+      __syncwarp();
+    };
+    if (delta > 0) {
+      for (; hi - lo >= 256; hi -= 256) whole(hi - 256);
+    } else {
+      for (; hi - lo >= 256; lo += 256) whole(lo);
+    }
+  }
   if (delta > 0) {  // top chunk first
     uint32_t top = hi;
     while (top > lo) {
@@ -324,7 +346,11 @@ struct Hot {
   uint32_t max_sessions;
 };
 
+// kLean_: the replay keeps no decision log, has the tier map and pin slots, and
+// no slot limit -- known at compile time.
+template <bool kLean_>
 struct ReplayState {
+  static constexpr bool kLean = kLean_;
   Sorted S, H;      // unpinned residents per tier
   uint4 *pin;       // pinned residents
   uint32_t npin, pin_cap;
@@ -351,10 +377,11 @@ struct ReplayState {
 
 constexpr uint16_t kNoSlot = 0xFFFF;
 
-__device__ __forceinline__ void log_dec(ReplayState &st, uint32_t kind, uint32_t s, int lane) {
+template <class St>
+__device__ __forceinline__ void log_dec(St &st, uint32_t kind, uint32_t s, int lane) {
   const uint64_t w = ((uint64_t)st.e << 32) | ((uint64_t)kind << 24) | s;
   st.hash = (st.hash ^ w) * kFnvPrime;
-  if (st.log) {
+  if (!St::kLean && st.log) {
     if (st.log_len < st.log_cap) {
       if (lane == 0) {
         unison_decision d;
@@ -371,11 +398,13 @@ __device__ __forceinline__ void log_dec(ReplayState &st, uint32_t kind, uint32_t
 
 // Tier-map update: every lane stores the same byte, so each lane's later
 // reads see it without a warp barrier.
-__device__ __forceinline__ void set_tier(ReplayState &st, uint32_t id, uint32_t tier) {
-  if (st.tmap) st.tmap[id] = (uint8_t)tier;
+template <class St>
+__device__ __forceinline__ void set_tier(St &st, uint32_t id, uint32_t tier) {
+  if (St::kLean || st.tmap) st.tmap[id] = (uint8_t)tier;
 }
 
-__device__ __forceinline__ bool sorted_insert(ReplayState &st, Sorted &T, uint4 v, int lane, uint32_t tier) {
+template <class St>
+__device__ __forceinline__ bool sorted_insert(St &st, Sorted &T, uint4 v, int lane, uint32_t tier) {
   if (T.n >= T.cap) {
     st.status = UNISON_ERR_CAPACITY;
     return false;
@@ -403,7 +432,8 @@ __device__ __forceinline__ void drop_front(Sorted &T, uint32_t m, int lane) {
   T.n -= m;
 }
 
-__device__ __forceinline__ uint4 sorted_pop_back(ReplayState &st, Sorted &T) {
+template <class St>
+__device__ __forceinline__ uint4 sorted_pop_back(St &st, Sorted &T) {
   const uint4 v = T.e[T.n - 1];
   __syncwarp();
   T.n--;
@@ -427,23 +457,27 @@ __device__ __forceinline__ uint64_t warp_min_u64(uint64_t v) {
   for (int o = 16; o > 0; o >>= 1) v = min(v, (uint64_t)__shfl_xor_sync(kFull, (unsigned long long)v, o));
   return v;
 }
-__device__ __forceinline__ uint64_t live_max(const ReplayState &st, const Sorted &T, uint32_t lo, uint32_t hi,
+template <class St>
+__device__ __forceinline__ uint64_t live_max(const St &st, const Sorted &T, uint32_t lo, uint32_t hi,
                                              int lane) {
   uint64_t m = 0;
   for (uint32_t i = lo + lane; i < hi; i += 32) m = max(m, st.live[packed_id(ekey(T.e[i]))]);
   return warp_max_u64(m);
 }
-__device__ __forceinline__ uint64_t live_min(const ReplayState &st, const Sorted &T, uint32_t lo, uint32_t hi,
+template <class St>
+__device__ __forceinline__ uint64_t live_min(const St &st, const Sorted &T, uint32_t lo, uint32_t hi,
                                              int lane) {
   uint64_t m = ~0ull;
   for (uint32_t i = lo + lane; i < hi; i += 32) m = min(m, st.live[packed_id(ekey(T.e[i]))]);
   return warp_min_u64(m);
 }
-__device__ __forceinline__ void count_victim(ReplayState &st, uint32_t chosen, uint64_t live_best) {
+template <class St>
+__device__ __forceinline__ void count_victim(St &st, uint32_t chosen, uint64_t live_best) {
   st.vict_n++;
   st.vict_diff += packed_id(live_best) != chosen;
 }
-__device__ __forceinline__ void count_promotion(ReplayState &st, uint32_t chosen, uint64_t live_best) {
+template <class St>
+__device__ __forceinline__ void count_promotion(St &st, uint32_t chosen, uint64_t live_best) {
   st.prom_n++;
   st.prom_diff += packed_id(live_best) != chosen;
 }
@@ -451,8 +485,8 @@ __device__ __forceinline__ void count_promotion(ReplayState &st, uint32_t chosen
 // A session demoted out of the fast tier enters HBM, displacing the most
 // evictable unpinned HBM sessions, or is dropped when it is itself the most
 // evictable of (unpinned HBM) + {itself}.
-template <bool kStale>
-__device__ __forceinline__ bool admit_demoted(ReplayState &st, const Hot &D, uint4 d, int lane) {
+template <bool kStale, class St>
+__device__ __forceinline__ bool admit_demoted(St &st, const Hot &D, uint4 d, int lane) {
   const uint32_t id = packed_id(ekey(d));
   const uint32_t size = esize(d);
   if (st.pinned_h > D.cap_h || size > D.cap_h - st.pinned_h) {
@@ -483,24 +517,25 @@ __device__ __forceinline__ bool admit_demoted(ReplayState &st, const Hot &D, uin
   return true;
 }
 
-__device__ __forceinline__ bool pin_append(ReplayState &st, uint64_t pk, uint32_t size, uint32_t s, uint32_t tier,
+template <class St>
+__device__ __forceinline__ bool pin_append(St &st, uint64_t pk, uint32_t size, uint32_t s, uint32_t tier,
                                            int lane) {
   if (st.npin >= st.pin_cap) {
     st.status = UNISON_ERR_CAPACITY;
     return false;
   }
   if (lane == 0) st.pin[st.npin] = make_uint4((uint32_t)pk, (uint32_t)(pk >> 32), size, s | (tier << 30));
-  if (st.pslot) st.pslot[s] = (uint16_t)st.npin;  // every lane stores the same slot
+  if (St::kLean || st.pslot) st.pslot[s] = (uint16_t)st.npin;  // every lane stores the same slot
   __syncwarp();
   st.npin++;
   return true;
 }
 
 // Placement of the arriving (pinned) session s with n tokens.
-template <bool kStale>
-__device__ __forceinline__ bool place(ReplayState &st, const Hot &D, uint32_t s, uint64_t pk, uint32_t n,
+template <bool kStale, class St>
+__device__ __forceinline__ bool place(St &st, const Hot &D, uint32_t s, uint64_t pk, uint32_t n,
                                       int lane) {
-  if (D.max_sessions && st.npin >= D.max_sessions) {
+  if (!St::kLean && D.max_sessions && st.npin >= D.max_sessions) {
     log_dec(st, UNISON_KIND_BYPASS, s, lane);
     CNT(st, n_bypass, 1);
     return true;
@@ -544,7 +579,7 @@ __device__ __forceinline__ bool place(ReplayState &st, const Hot &D, uint32_t s,
     CNT(st, n_bypass, 1);
     return true;
   }
-  if (D.max_sessions) {
+  if (!St::kLean && D.max_sessions) {
     while (st.S.n + st.H.n + st.npin > D.max_sessions) {
       if (st.S.n == 0 && st.H.n == 0) {
         st.status = UNISON_ERR_CAPACITY;
@@ -572,8 +607,8 @@ __device__ __forceinline__ bool place(ReplayState &st, const Hot &D, uint32_t s,
 // free fast-tier space; phase 2: pair the next least evictable HBM session
 // with the most evictable fast-tier one), which makes the same moves as the
 // pair loop of Algorithm 1, and are then applied in bulk.
-template <bool kStale>
-__device__ __forceinline__ uint64_t tide(ReplayState &st, const Hot &D, uint64_t budget, uint32_t rcap_s,
+template <bool kStale, class St>
+__device__ __forceinline__ uint64_t tide(St &st, const Hot &D, uint64_t budget, uint32_t rcap_s,
                                          int lane) {
   const uint32_t sn = st.S.n;  // fast-tier entries; the fast tier changes only at the end
   uint64_t rem = budget;
@@ -668,7 +703,8 @@ __device__ __forceinline__ uint64_t tide(ReplayState &st, const Hot &D, uint64_t
 // Timeout: expire unpinned residents idle >= ttl, smallest session id first.
 // Under recency keys the last return time falls as the key grows, so the
 // expired sessions of a tier are a top suffix of its array.
-__device__ __forceinline__ void expire_idle(ReplayState &st, uint32_t now, uint32_t ttl, int lane) {
+template <class St>
+__device__ __forceinline__ void expire_idle(St &st, uint32_t now, uint32_t ttl, int lane) {
   for (;;) {
     // expired suffix lengths
     uint32_t cs = 0, ch = 0;
@@ -808,12 +844,12 @@ struct EventBufs {
 // One replay: Algorithm 1 over the trace's events.  kPol is the replay's
 // policy when the body is specialised for it (its policy tests then fold
 // away), or -1 for the body that reads the policy from the descriptor.
-template <bool kGlobalLists, int kKeys, int kPol>
+template <bool kGlobalLists, int kKeys, int kPol, bool kLean>
 __device__ __forceinline__ void replay_body(const ReplayDesc &D, EventBufs &bufs, unsigned char *smem, int lane) {
   constexpr bool kOnline = kKeys == kKeyOnline, kStale = kKeys == kKeyStale;
   const Hot hot{D.cap_s, D.cap_h, D.kvb, D.dma, D.max_sessions};
 
-  ReplayState st;
+  ReplayState<kLean> st;
   uint32_t *online_gs = nullptr;
   uint16_t *online_ks = nullptr;
   OnlineTable *online_tab = nullptr;
@@ -842,12 +878,12 @@ __device__ __forceinline__ void replay_body(const ReplayDesc &D, EventBufs &bufs
     p += 2 * D.rcap_s;
     st.tmap = nullptr;
     st.pslot = nullptr;
-    if (!kGlobalLists && D.tmap != kMapNone) {
+    if (!kGlobalLists && (kLean || D.tmap != kMapNone)) {
       // tier map (1 B per session), then pin slots (2 B per session)
       st.tmap = reinterpret_cast<uint8_t *>(p);
       uint32_t *m32 = reinterpret_cast<uint32_t *>(p);
       for (uint32_t i = lane; i < (D.n_sessions + 3) / 4; i += 32) m32[i] = 0u;
-      if (D.tmap == kMapSlots) {
+      if (kLean || D.tmap == kMapSlots) {
         st.pslot = reinterpret_cast<uint16_t *>(reinterpret_cast<unsigned char *>(p) + ((D.n_sessions + 15) & ~15u));
         uint32_t *s32 = reinterpret_cast<uint32_t *>(st.pslot);
         for (uint32_t i = lane; i < (D.n_sessions + 1) / 2; i += 32) s32[i] = 0xFFFFFFFFu;
@@ -1003,7 +1039,7 @@ __device__ __forceinline__ void replay_body(const ReplayDesc &D, EventBufs &bufs
             pkb = pack_key(0xFFFFFFFFull - spev[bi][j], s);
           // with the tier map only the session's own tier is searched (and
           // nothing for a session that is not resident)
-          const uint32_t mt = st.tmap ? st.tmap[s] : (kTierS | kTierH);
+          const uint32_t mt = kLean || st.tmap ? st.tmap[s] : (kTierS | kTierH);
           if (mt & kTierS) {
             pos = lower_bound(st.S, pkb, lane);
             if (pos < st.S.n && ekey(st.S.e[pos]) == pkb) {
@@ -1098,7 +1134,7 @@ __device__ __forceinline__ void replay_body(const ReplayDesc &D, EventBufs &bufs
           mark_dirty(s);
         }
         uint32_t pi = kNoSlot;
-        if (st.pslot) {
+        if (kLean || st.pslot) {
           pi = st.pslot[s];
         } else {
           int mine = -1;
@@ -1112,7 +1148,7 @@ __device__ __forceinline__ void replay_body(const ReplayDesc &D, EventBufs &bufs
           const uint4 last = st.pin[st.npin - 1];
           __syncwarp();
           if (lane == 0) st.pin[pi] = last;
-          if (st.pslot) {  // the last entry moves into the freed slot
+          if (kLean || st.pslot) {  // the last entry moves into the freed slot
             st.pslot[last.w & kIdMask] = (uint16_t)pi;
             st.pslot[s] = kNoSlot;
           }
@@ -1240,19 +1276,22 @@ __device__ __forceinline__ void replay_body(const ReplayDesc &D, EventBufs &bufs
   }
 }
 
-// One warp per replay.  SPEAR+TIDE replays run a body with the policy folded in.
-template <bool kGlobalLists, int kKeys>
-__global__ void __launch_bounds__(32) replay_kernel(const ReplayDesc *descs, const uint32_t *order) {
+// One warp per replay.  kOnly >= 0: every replay of the launch has that policy,
+// and the kernel holds only its body (and is sized for it alone); kLean: every
+// replay of the launch is lean (see ReplayState).  One kernel for all policies
+// took 922 ms for 8 SPEAR+TIDE replays of 2,800 residents, in global memory 187
+// for four of 6,000; with a kernel of their own 781 and 102 ms (152 lean
+// replays of 2,800: 210 -> 152).  At least 12 CTAs an SM: unbounded, the
+// kernels over global memory take 204 registers, which leaves room for 9.
+template <bool kGlobalLists, int kKeys, int kOnly, bool kLean>
+__global__ void __launch_bounds__(32, 12) replay_kernel(const ReplayDesc *descs, const uint32_t *order) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ ReplayDesc Dsh;
   __shared__ __align__(16) EventBufs bufs;
   const int lane = threadIdx.x & 31;
   if (lane == 0) Dsh = descs[order[blockIdx.x]];
   __syncwarp();
-  if (kKeys == kKeyStream && Dsh.policy == UNISON_SPEAR_TIDE)
-    replay_body<kGlobalLists, kKeys, UNISON_SPEAR_TIDE>(Dsh, bufs, smem, lane);
-  else
-    replay_body<kGlobalLists, kKeys, -1>(Dsh, bufs, smem, lane);
+  replay_body<kGlobalLists, kKeys, kOnly, kLean>(Dsh, bufs, smem, lane);
 }
 
 // Replays of the slot form.  kOnly >= 0: every replay of the launch is a lean
@@ -1445,13 +1484,17 @@ struct ReplayPlan {
   std::vector<size_t> off_lut, off_stream, off_ttft, off_glist;
   std::vector<char> need_keys, need_rank;  // per combination: packed keys (sorted lists), ranks (slot form)
   // Replay groups, one kernel launch each: the slot form (lean SPEAR+TIDE
-  // replays, the other policies, online hazard table, stale snapshot), sorted lists in shared memory, in global memory,
-  // online hazard table, stale snapshot.  The launches are independent and
-  // run concurrently.
-  std::vector<uint32_t> in_slot_st, in_slot_mix, in_slot_online, in_slot_stale, in_list, in_glist, in_online, in_stale;
+  // replays, the other policies, online hazard table, stale snapshot), sorted
+  // lists in shared memory (SPEAR+TIDE, the other policies), in global memory
+  // (the same), online hazard table, stale snapshot.  The launches are
+  // independent and run concurrently.
+  std::vector<uint32_t> in_slot_st, in_slot_mix, in_slot_online, in_slot_stale;
+  std::vector<uint32_t> in_list_st, in_list, in_glist_st, in_glist, in_online, in_stale;
   std::vector<uint32_t> rcap_s, rcap_h, tmap;
   std::vector<unison_slots::SlotDesc> slot;  // nslots 0: not of the slot form
-  size_t smem_slot_st = 0, smem_slot_mix = 0, smem_slot_online = 0, smem_slot_stale = 0, max_smem_list = 0, max_smem_online = 0, max_smem_stale = 0;
+  size_t smem_slot_st = 0, smem_slot_mix = 0, smem_slot_online = 0, smem_slot_stale = 0;
+  size_t max_smem_list_st = 0, max_smem_list = 0, max_smem_online = 0, max_smem_stale = 0;
+  bool list_lean = false;  // in_list_st is not empty and every replay of it is lean
 };
 
 // Resident-list capacity of a tier: at most one entry per session and no more
@@ -1488,6 +1531,12 @@ size_t online_bytes(uint32_t cs, uint32_t ch, uint32_t n_sessions) {
 }
 
 using ReplayKernel = void (*)(const ReplayDesc *, const uint32_t *);
+
+// The kernel of SPEAR+TIDE replays over sorted lists in shared memory.
+ReplayKernel list_st_kernel(bool lean) {
+  return lean ? replay_kernel<false, kKeyStream, UNISON_SPEAR_TIDE, true>
+              : replay_kernel<false, kKeyStream, UNISON_SPEAR_TIDE, false>;
+}
 
 // Waves of CTAs a group of n replays needs with `dyn` bytes per CTA.
 uint64_t smem_waves(ReplayKernel k, size_t n, size_t dyn) {
@@ -1697,11 +1746,13 @@ int plan_replays(const unison_trace *const *traces, const unison_replay_params *
       const bool lean_st = p.policy == UNISON_SPEAR_TIDE && p.max_sessions == 0 && !logged;
       (lean_st ? P.in_slot_st : P.in_slot_mix).push_back((uint32_t)r);
     } else if (lists <= smem_limit) {
-      P.in_list.push_back((uint32_t)r);
-      P.max_smem_list = std::max<size_t>(P.max_smem_list, lists + (P.tmap[r] == kMapSlots ? map : 0));
+      const bool st = p.policy == UNISON_SPEAR_TIDE;
+      (st ? P.in_list_st : P.in_list).push_back((uint32_t)r);
+      size_t &m = st ? P.max_smem_list_st : P.max_smem_list;
+      m = std::max<size_t>(m, lists + (P.tmap[r] == kMapSlots ? map : 0));
     } else {
       P.tmap[r] = kMapNone;
-      P.in_glist.push_back((uint32_t)r);
+      (p.policy == UNISON_SPEAR_TIDE ? P.in_glist_st : P.in_glist).push_back((uint32_t)r);
       P.off_glist[r] = off;
       off = align_up(off + lists, 256);
     }
@@ -1726,8 +1777,12 @@ int plan_replays(const unison_trace *const *traces, const unison_replay_params *
     if (P.need_rank[c]) off += align_up(4 * rank_entries(P, c, tr), 8) + 16 * rank_values(P, c, tr);
     off = align_up(off, 256);
   }
+  if (!P.in_list_st.empty())
+    add_tier_maps(traces, params, smem_limit, P.in_list_st, list_st_kernel(false), P.max_smem_list_st, P);
   if (!P.in_list.empty())
-    add_tier_maps(traces, params, smem_limit, P.in_list, replay_kernel<false, kKeyStream>, P.max_smem_list, P);
+    add_tier_maps(traces, params, smem_limit, P.in_list, replay_kernel<false, kKeyStream, -1, false>, P.max_smem_list, P);
+  P.list_lean = !P.in_list_st.empty() && !logged;
+  for (uint32_t r : P.in_list_st) P.list_lean &= P.tmap[r] == kMapSlots && params[r].max_sessions == 0;
   if (!P.in_slot_st.empty()) slot_maps(traces, params, slot_limit, P.in_slot_st, true, P.smem_slot_st, P);
   if (!P.in_slot_mix.empty()) slot_maps(traces, params, slot_limit, P.in_slot_mix, false, P.smem_slot_mix, P);
   off_res = 0;
@@ -1824,23 +1879,29 @@ void fill_descs(const unison_trace *const *traces, const unison_replay_params *p
     d.slot.rank = P.replay_combo[r] >= 0 ? hc[P.replay_combo[r]].rk.rank : nullptr;
   }
   order.clear();
-  for (const auto *g : {&P.in_slot_st, &P.in_slot_mix, &P.in_slot_online, &P.in_slot_stale, &P.in_list, &P.in_glist, &P.in_online, &P.in_stale})
+  for (const auto *g : {&P.in_slot_st, &P.in_slot_mix, &P.in_slot_online, &P.in_slot_stale, &P.in_list_st, &P.in_list,
+                        &P.in_glist_st, &P.in_glist, &P.in_online, &P.in_stale})
     order.insert(order.end(), g->begin(), g->end());
   // A launch lasts as long as its slowest replay, and CTAs start in index
-  // order: the SPEAR+TIDE launch takes its replays by predicted cost,
+  // order: the SPEAR+TIDE launches take their replays by predicted cost,
   // largest first, so the long ones start early and the short ones fill in.
   // The predictor is the product of the tiers' capacities (the larger both
   // tiers, the more tier moves a replay makes); decisions do not depend on
   // the order.
-  std::stable_sort(order.begin(), order.begin() + P.in_slot_st.size(), [&](uint32_t a, uint32_t b) {
-    return (double)hd[a].cap_s * (double)hd[a].cap_h > (double)hd[b].cap_s * (double)hd[b].cap_h;
-  });
+  auto dearest_first = [&](size_t from, size_t n) {
+    std::stable_sort(order.begin() + from, order.begin() + from + n, [&](uint32_t a, uint32_t b) {
+      return (double)hd[a].cap_s * (double)hd[a].cap_h > (double)hd[b].cap_s * (double)hd[b].cap_h;
+    });
+  };
+  dearest_first(0, P.in_slot_st.size());
+  dearest_first(P.in_slot_st.size() + P.in_slot_mix.size() + P.in_slot_online.size() + P.in_slot_stale.size(),
+                P.in_list_st.size());
 }
 
 // Side streams for the replay groups of one call, one set per device, made
 // on first use.  The caller holds the lock while it forks and joins, so two
 // host threads never interleave their events.
-constexpr int kSideStreams = 7;
+constexpr int kSideStreams = 9;
 struct SideStreams {
   cudaStream_t s[kSideStreams] = {};
   cudaEvent_t fork = nullptr, join[kSideStreams] = {};
@@ -1923,10 +1984,13 @@ int launch_replays(const ReplayPlan &P, char *scratch, const std::vector<ComboDe
         {slot_kernel_of(false, form(P.in_slot_mix)), P.in_slot_mix.size(), P.smem_slot_mix},
         {slot_variant_kernel<unison_slots::kOnline>, P.in_slot_online.size(), P.smem_slot_online},
         {slot_variant_kernel<unison_slots::kStale>, P.in_slot_stale.size(), P.smem_slot_stale},
-        {replay_kernel<false, kKeyStream>, P.in_list.size(), P.max_smem_list},
-        {replay_kernel<true, kKeyStream>, P.in_glist.size(), 0},
-        {replay_kernel<false, kKeyOnline>, P.in_online.size(), P.max_smem_online},
-        {replay_kernel<false, kKeyStale>, P.in_stale.size(), P.max_smem_stale}};
+        {list_st_kernel(P.list_lean), P.in_list_st.size(), P.max_smem_list_st},
+        {replay_kernel<false, kKeyStream, -1, false>, P.in_list.size(), P.max_smem_list},
+        {replay_kernel<true, kKeyStream, UNISON_SPEAR_TIDE, false>, P.in_glist_st.size(), 0},
+        {replay_kernel<true, kKeyStream, -1, false>, P.in_glist.size(), 0},
+        {replay_kernel<false, kKeyOnline, -1, false>, P.in_online.size(), P.max_smem_online},
+        {replay_kernel<false, kKeyStale, -1, false>, P.in_stale.size(), P.max_smem_stale}};
+    static_assert(sizeof all / sizeof all[0] <= kSideStreams + 1, "a stream for every group");
     std::vector<Launch> ls;
     std::vector<size_t> first;
     size_t off = 0;

@@ -290,30 +290,64 @@ def test_global_list_path_spear_tide_only(B):
         assert_same(res[i], oracle.replay(tr, to_oracle(p)), i)
 
 
-def test_all_six_launch_groups_in_one_call(B):
-    """One call with a replay in every launch group (SPEAR+TIDE and other
-    policies with lists in shared and in global memory, online table, stale
-    snapshot): the groups run concurrently on forked streams, and each replay
-    must still equal the oracle, with full decision logs."""
+def test_all_launch_groups_in_one_call(B):
+    """One call with a replay in every launch group (the slot form: lean
+    SPEAR+TIDE, other policies, online table, stale snapshot; sorted lists, for
+    traces with more residents than the slot form takes: SPEAR+TIDE and other
+    policies in shared and in global memory, online table, stale snapshot): the
+    groups run concurrently on forked streams, and each replay must still equal
+    the oracle.  With full decision logs too, where no SPEAR+TIDE replay is
+    lean."""
     big = synth.make_trace(3, np.full(6000, 4), 0.01, synth.GAP_MIX_CODING)
+    mid = synth.make_trace(37, np.full(2400, 3), 0.01, synth.GAP_MIX_CODING)
     small = synth.paper_scale_trace(2, "general")
-    reps = [(0, base("spear_tide", 1 << 60, 1 << 60, 1024)),            # global, SPEAR+TIDE
-            (0, base("lru", 1 << 60, 1 << 60, 1024)),                   # global, other
-            (1, base("spear_tide", 2 * GIB, 32 * GIB, 131072)),         # shared, SPEAR+TIDE
-            (1, base("belady", 2 * GIB, 32 * GIB, 131072)),             # shared, other
-            (1, base("spear_tide", 2 * GIB, 32 * GIB, 131072, online=True)),
-            (1, base("spear", 2 * GIB, 32 * GIB, 131072, stale="arrivals", stale_m=3))]
+    many = 60 * 2400 * 28672  # about 60 of mid's sessions
+    reps = [(0, base("spear_tide", 1 << 60, 1 << 60, 1024)),            # lists, global, SPEAR+TIDE
+            (0, base("lru", 1 << 60, 1 << 60, 1024)),                   # lists, global, other
+            (1, base("spear_tide", many, 1 << 60, 28672)),              # lists, shared, SPEAR+TIDE
+            (1, base("belady", many, 1 << 60, 28672)),                  # lists, shared, other
+            (1, base("spear_tide", many, 1 << 60, 28672, online=True)),
+            (1, base("spear", many, 1 << 60, 28672, stale="gap_start")),
+            (2, base("spear_tide", 2 * GIB, 32 * GIB, 131072)),         # slots, SPEAR+TIDE
+            (2, base("belady", 2 * GIB, 32 * GIB, 131072)),             # slots, other
+            (2, base("spear_tide", 2 * GIB, 32 * GIB, 131072, online=True)),
+            (2, base("spear", 2 * GIB, 32 * GIB, 131072, stale="arrivals", stale_m=3))]
     cap = 8 * max(big.n_events, small.n_events)
-    trs = [big, small]
+    trs = [big, mid, small]
     res, log, _ = run_gpu(B, trs, reps, log_capacity=cap)
+    lean, _, _ = run_gpu(B, trs, reps)
     for i, (ti, p) in enumerate(reps):
         o = oracle.replay(trs[ti], to_oracle(p), log=True)
         assert_same(res[i], o, i)
         assert_same_log(B, log[i], res[i], o, i)
+        assert_same(lean[i], o, i)
     # the same replays one per call give the same results
     for i, (ti, p) in enumerate(reps):
         one, _, _ = run_gpu(B, [trs[ti]], [(0, p)])
         assert_same(one[0], res[i], i)
+
+
+@pytest.mark.parametrize("n_sessions", [2048, 2200])
+@pytest.mark.parametrize("pol", POLS)
+def test_sorted_lists_in_shared_memory(B, pol, n_sessions):
+    """One session more than the slot form's most, and 150 more: lists of one
+    policy, so that SPEAR+TIDE takes its lean kernel (and with a log or a slot
+    limit the other).  Tiers of a handful, of a few chunks of a shift (256
+    entries) and of every session."""
+    tr = synth.make_trace(38, np.full(n_sessions, 4), 0.01, synth.GAP_MIX_CODING)
+    one = int(tr.out_tok.min()) * 28672
+    reps = [(0, base(pol, cs * one, ch, 28672, ttl=3_000_000)) for cs, ch in
+            ((20, 1 << 60), (600, 1 << 60), (1500, 1 << 60), (3000, 1 << 60))]
+    res, _, _ = run_gpu(B, [tr], reps)
+    limited = reps + [(0, dict(reps[0][1], max_sessions=700))]
+    cap = 8 * tr.n_events
+    res2, log, _ = run_gpu(B, [tr], limited, log_capacity=cap)
+    for i, (_, p) in enumerate(limited):
+        o = oracle.replay(tr, to_oracle(p), log=True, log_capacity=cap)
+        assert_same(res2[i], o, (pol, i))
+        assert_same_log(B, log[i], res2[i], o, (pol, i))
+        if i < len(reps):
+            assert_same(res[i], o, (pol, i))
 
 
 def test_mixed_calls_from_two_host_threads(B):

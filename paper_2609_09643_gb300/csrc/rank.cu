@@ -280,6 +280,7 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
 }
 __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 __device__ __forceinline__ uint64_t now_ns() {
   uint64_t t;
@@ -1239,6 +1240,9 @@ __device__ __noinline__ bool finish_list(const RankSet &S, int L, uint64_t *fin,
         fence_proxy_async();  // earlier generic accesses to the area before the async copy
         consumers_sync();
         if (tid == 0) {
+          // the candidates are ordinary stores of every CTA of the group, seen
+          // by this thread's wait; the copy reads them by another route
+          fence_proxy_async_global();
           mbar_init(&cbar, 1);
           fence_mbar_init();
           mbar_expect_tx(&cbar, bytes);

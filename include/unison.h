@@ -461,14 +461,17 @@ typedef struct {
  * call queues one cooperative kernel on cuda_stream, after one upload of its
  * descriptors when they are too many for the launch's parameters (every CTA
  * of the grid resident at once; each set is ranked by a group of CTAs, or,
- * with more sets than resident CTAs, each CTA takes whole sets in turn).  Any n_sets >= 0 that fits in memory is accepted.
- * Memory: the call's device scratch (up to about 3.4 MB per set) is kept per
- * (device, stream) and grown when a call needs more, and the per-call
- * descriptors that are uploaded go from a small pinned host ring; both are
- * held for the life of the process.  Calls on one stream run in order and share that
- * stream's scratch; calls on different streams use different scratch.  The
- * scratch is found by the stream's handle, so a stream must outlive the
- * ranking calls queued on it.
+ * with more sets than resident CTAs, each CTA takes whole sets in turn).  Any
+ * n_sets >= 0 that fits in memory is accepted.
+ * Memory: the call's device scratch is kept per (device, stream) and grown
+ * when a call needs more.  A set of more than 16,384 records takes about 1.8 MB
+ * and, for its CTAs' candidate regions, the larger of 1.6 MB and 25 KB a CTA of
+ * its group: 3.4 MB beside many others, 13 MB for a lone set of 2^24 records
+ * (456 CTAs); a smaller set takes less.  The per-call descriptors that are
+ * uploaded go from a small pinned host ring.  Both are held for the life of the
+ * process.  Calls on one stream run in order and share that stream's scratch;
+ * calls on different streams use different scratch.  The scratch is found by
+ * the stream's handle, so a stream must outlive the ranking calls queued on it.
  * Capture: a call on a stream that is being captured becomes part of the
  * graph, which may then run at any time, on any stream and any number of
  * times, beside other calls; two executables of one graph must not run at the

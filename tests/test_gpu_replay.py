@@ -127,15 +127,12 @@ def test_sweep_iid_gaps_subset(B):
         assert_same(res[i], oracle.replay(trs[ti], to_oracle(p)), i)
 
 
-def test_hbm_tier_past_register_capacity(B):
-    """SPEAR+TIDE replays around the 160 entries (five a lane) the lean launch
-    holds its HBM tier in: with a fast tier of at most 32 entries every replay
-    of the call takes the register tiers.  On seed 0 the oracle counts at most
-    210 and 192 unpinned HBM sessions for the first two configurations, so
-    those replays stop at the 161st entry and run again from their start with
-    the tier in shared memory; 126 for the third; and 142 on the trace with
-    independent gaps (its fifth slot in use).  Every counter and the decision
-    hash against the oracle."""
+def test_hbm_tiers_past_one_pass_of_words(B):
+    """SPEAR+TIDE replays whose HBM tiers hold more and fewer sessions than one
+    pass over the words takes (128): on seed 0 the oracle counts at most 210 and
+    192 unpinned HBM sessions for the first two configurations, 126 for the
+    third, and 142 on the trace with independent gaps.  Every counter and the
+    decision hash against the oracle."""
     trs = [synth.paper_scale_trace(s, "coding") for s in (0, 1)] + [synth.paper_scale_trace(0, "coding", gap_persist=0.0)]
     cfgs = [(28_672, 1 * GIB, 64 * GIB), (131_072, 1 * GIB, 256 * GIB), (28_672, 512 * MIB, 32 * GIB)]
     reps = [(ti, base("spear_tide", cs, ch, kvb)) for ti in range(2) for kvb, cs, ch in cfgs]
@@ -156,9 +153,8 @@ def test_large_pool_replay(B, seed):
 
 def test_large_pool_16_replays_one_call(B):
     """The large-pool launch as the benchmark table runs it: many replays, each
-    on its own 65,536-session trace, in one call (the tier map without pin
-    slots, two CTAs per SM); every replay checked against the oracle in a
-    spawn pool."""
+    on its own 65,536-session trace, in one call (the slot form's deep passes);
+    every replay checked against the oracle in a spawn pool."""
     import multiprocessing as mp
     import os
     from cases import oracle_large_pool_job
@@ -173,6 +169,7 @@ def test_large_pool_16_replays_one_call(B):
 
 
 POLS = ["lru", "timeout", "spear", "spear_tide", "belady", "lru_tide"]
+ONLINE_POLS = ("spear", "spear_tide")
 
 
 @pytest.mark.parametrize("caps", [(1 << 60, 1 << 60), (0, 0), (0, 16 * GIB), (2 * GIB, 0), (300 * MIB, 2 * GIB)])
@@ -281,8 +278,8 @@ def test_global_list_path(B):
 
 
 def test_global_list_path_spear_tide_only(B):
-    """A global-memory launch whose replays are all SPEAR+TIDE runs the
-    kernel specialised for that policy."""
+    """Lists in global memory whose replays are all SPEAR+TIDE: one launch, of
+    the kernel that holds only that policy's body."""
     tr = synth.make_trace(3, np.full(6000, 4), 0.01, synth.GAP_MIX_CODING)
     reps = [(0, base("spear_tide", cs, ch, 1024)) for cs, ch in ((1 << 60, 1 << 60), (400 * MIB, 4 * GIB))]
     res, _, _ = run_gpu(B, [tr], reps)
@@ -391,16 +388,70 @@ def test_mixed_calls_from_two_host_threads(B):
 
 @pytest.mark.parametrize("n_sessions", [20000, 40000, 240000])
 def test_many_sessions_paths(B, n_sessions):
-    """20,000 sessions: tier map and pin slots in shared memory.  40,000: the
-    tier map alone (completions scan the pinned list).  240,000: no map fits
-    beside the lists, so residents are found by a warp-wide search of both
-    tiers."""
+    """20,000 and 40,000 sessions over about 560 slots: the slot form, whose
+    passes are deep from four sessions a slot on.  240,000: no session map fits
+    in shared memory, so the replays run on sorted lists and find residents by a
+    warp-wide search of both tiers."""
     tr = synth.make_trace(4, np.full(n_sessions, 3 if n_sessions < 100000 else 2), 0.005, synth.GAP_MIX_GENERAL)
     pols = ("spear_tide", "belady", "timeout") if n_sessions < 100000 else ("spear_tide", "lru")
     reps = [(0, base(pol, 2 * GIB, 16 * GIB, 16384)) for pol in pols]
     res, _, _ = run_gpu(B, [tr], reps)
     for i, (_, p) in enumerate(reps):
         assert_same(res[i], oracle.replay(tr, to_oracle(p)), p["policy"])
+
+
+@pytest.mark.parametrize("n_sessions", [20000, 40000])
+def test_sorted_lists_with_tier_maps(B, n_sessions):
+    """About 2,360 slots, more than the slot form takes, so the replays run on
+    sorted lists in shared memory.  20,000 sessions: tier map and pin slots beside
+    them.  40,000: the tier map alone (completions scan the pinned list)."""
+    tr = synth.make_trace(39, np.full(n_sessions, 2), 0.005, synth.GAP_MIX_GENERAL)
+    one = int(tr.out_tok.min()) * 16384
+    reps = [(0, base(pol, 60 * one, 2300 * one, 16384))
+            for pol in (POLS if n_sessions == 20000 else ("spear_tide", "belady", "lru"))]
+    res, _, _ = run_gpu(B, [tr], reps)
+    for i, (_, p) in enumerate(reps):
+        o = oracle.replay(tr, to_oracle(p))
+        assert o["evict"] + o["expire"] > n_sessions // 4
+        assert_same(res[i], o, p["policy"])
+
+
+@pytest.mark.parametrize("n_sessions", [2100, 3000])
+def test_sorted_list_variants(B, n_sessions):
+    """The online hazard table and stale snapshots with more residents than the
+    slot form takes, on sorted lists: re-sorts of both tiers under a rebuilt
+    table, syncs that move the few sessions changed and syncs that re-sort, slot
+    limits, SPEAR without TIDE, full logs."""
+    tr = synth.make_trace(40, np.full(n_sessions, 3), 0.01, synth.GAP_MIX_CODING)
+    one = int(tr.out_tok.min()) * 28672
+    kws = [dict(online=True), dict(online=True, bucket=60), dict(online=True, max_sessions=900), dict(stale="event"),
+           dict(stale="arrivals", stale_m=100), dict(stale="arrivals", stale_m=7), dict(stale="gap_start", max_sessions=900)]
+    reps = [(0, base(pol, (30, 200)[(i + j) % 2] * one, 2080 * one, 28672, **kw))
+            for j, pol in enumerate(ONLINE_POLS) for i, kw in enumerate(kws)]
+    cap = 8 * tr.n_events
+    res, log, _ = run_gpu(B, [tr], reps, log_capacity=cap)
+    for i, (_, p) in enumerate(reps):
+        o = oracle.replay(tr, to_oracle(p), log=True, log_capacity=cap)
+        assert_same(res[i], o, (p["policy"], p["cap_s"], p["stale"], p["online"]))
+        assert_same_log(B, log[i], res[i], o, (p["policy"], p["stale"], p["online"]))
+
+
+@pytest.mark.parametrize("load", [1, 4, 7])
+@pytest.mark.parametrize("factor", [0, 1, 2, 64, 1 << 20])
+def test_prefill_times_past_63_bits(B, factor, load):
+    """Prefill costs at the line where the queue's times may pass 2^63 ns (from
+    there one thread walks the recurrence, which wraps) and up to far above it,
+    beside the ordinary cost; with load factors that divide 1,000 and not.  TTFT
+    sums and medians wrap as the oracle's do."""
+    tr, _ = tiny_case()
+    # the largest cost a token, in ns, below the line for this trace, and the first above it
+    span = int(tr.completion_us.max()) - int(tr.arrival_us.min())
+    line = ((1 << 63) - 1 - 1000 * span) // int(tr.in_tok.astype(np.uint64).sum())
+    t_p = (line + (0, 1)[factor > 0]) * max(factor, 1) * 1000
+    reps = [(0, base(pol, 512 * MIB, 8 * GIB, 28672, t_p=min(t_p, (1 << 64) - 1), load=load)) for pol in POLS]
+    res, _, _ = run_gpu(B, [tr], reps + [(0, dict(reps[0][1], t_p=20_000_000))])
+    for i, (_, p) in enumerate(reps):
+        assert_same(res[i], oracle.replay(tr, to_oracle(p)), (p["policy"], t_p))
 
 
 @pytest.mark.parametrize("n_sessions", [127, 128, 129, 256, 2047, 2048])
@@ -569,8 +620,6 @@ def test_hazard_lut_kernel(B):
 
 
 # ---- online hazard table (Sec. V-F) ------------------------------------------
-
-ONLINE_POLS = ("spear", "spear_tide")
 
 
 def test_online_hazard_tiny_full_logs(B):

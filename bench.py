@@ -923,19 +923,20 @@ def main():
                    "share_of_step": avg_rep_ms * args.steps / ms if ms else None,
                    "key_stream_avg_ms": ks_ms / max(ks_n, 1), "ttft_median_avg_ms": md_ms / max(md_n, 1)}
     if replay_roof is not None:
-        # The launch ends with its slowest replay: its cycles per event, against
-        # the chain an event needs with its residents in shared-memory slots
-        # (about 12 dependent steps of about 30 cycles each, the mean of an
-        # arrival and a completion: the event's record, the session's slot, its
-        # payload, the test of room, one pass over the words (load, reduction,
-        # the winner's payload) for a demotion or for TIDE's first choice, a
-        # second pass, the word's store).
+        # The launch ends with its slowest replay: its cycles per event, beside
+        # a yardstick, not a bound: the chain that an event of the slot form
+        # would take at about 12 dependent steps (the mean of an arrival and a
+        # completion: the event's record, the session's slot, its payload, the
+        # test of room, one pass over the words (load, reduction, the winner's
+        # payload) for a demotion or for TIDE's first choice, a second pass, the
+        # word's store) of about 30 cycles.  Both numbers are counted from the
+        # code and from a shared-memory load's latency, not measured.
         mhz = (clocks or {}).get("sm_mhz") or 2070.0
         replay_roof["cycles_per_event_slowest_replay"] = avg_rep_ms * 1e3 * mhz / (events_per_step / n_rep)
         replay_roof["floor_cycles_per_event"] = 12 * 30
-        replay_roof["floor_basis"] = ("12 dependent steps per event x ~30 cycles: shared-memory loads (event, session's "
-                                      "slot, payload), the test of room, two passes over the slot words (load, "
-                                      "reduction, payload) and a store")
+        replay_roof["floor_basis"] = ("a yardstick, not measured: 12 dependent steps per event x ~30 cycles: "
+                                      "shared-memory loads (event, session's slot, payload), the test of room, two "
+                                      "passes over the slot words (load, reduction, payload) and a store")
     avg_rk = rk_ms / max(rk_n, 1) if rk_n else float("nan")
     achieved = rank_bytes / (avg_rk / 1e3) / 1e9 if rk_n else float("nan")
     n_rec = len(r_params) * RANK_N

@@ -12,10 +12,10 @@
 // One cooperative, persistent kernel does a whole call.  Each set owns a
 // group of CTAs (in proportion to its records; with more sets than CTAs,
 // each CTA takes whole sets in turn).  Per set, inside the group:
-//   sample   up to 63 CTAs gather a jittered stratified sample, count it in
-//            shared memory and add it to a 4,096-bin histogram per list (bins
-//            monotone in the list value).  Once every sampling CTA's counts
-//            are in, each CTA of the group cuts the histograms at the lists'
+//   sample   up to 63 CTAs gather a jittered stratified sample and add it to a
+//            4,096-bin histogram per list in global memory (bins monotone in
+//            the list value).  Once every sampling CTA's counts are in, each
+//            CTA of the group cuts the histograms at the lists'
 //            sample ranks itself: per-list thresholds and per-turn thresholds
 //            on the gap average (the score is monotone in the gap for a fixed
 //            turn, so the streaming test needs no division).  Meanwhile every
@@ -37,7 +37,7 @@
 //            items at a time, and writes the outputs.
 // The work words and sample histograms lie in one of two blocks: calls on a
 // stream alternate between them, and each call zeroes what the one before it
-// used.
+// used.  (A captured call has memory of its own, cleared by a node before it.)
 // Every wait on another CTA or on a copy is bounded: a wait that gives up
 // records UNISON_ERR_TIMEOUT in the set's status word and the CTA carries on
 // to the end of the kernel.  A cooperative launch keeps every CTA of the grid
@@ -560,14 +560,7 @@ __device__ void hist_cut3(const uint16_t *hist, const uint32_t (&need)[kLists], 
   for (int L = 0; L < kLists; L++) cut[L] = scut[L];
 }
 
-// Sort, descending, of the distinct values a[0..n) by bucket: the 8 bits
-// below the values' common prefix name 256 buckets, a counting pass places
-// each value in its bucket's range (buckets in descending order, in tmp),
-// and each value's place within its bucket is the count of the bucket's
-// values above it.  pay[] (when given) moves along, through tmp_pay.  Costs
-// the sum over buckets of size^2 comparisons; declines (false, a and pay
-// unchanged) when that sum is large, i.e. the values crowd into few buckets.
-static_assert(kConsumers == 256, "one bucket per consumer thread");
+static_assert(kConsumers == 256, "one bucket per consumer thread");  // the narrowing and the sorts below
 
 // Values beyond the M wanted ones that a selection leaves to the sort: another
 // step of narrow() costs about what sorting twice as many does.
@@ -645,6 +638,13 @@ __device__ uint32_t narrow(Each each, uint64_t &t, int &sh, uint32_t &need, Sele
   return n;
 }
 
+// Sort, descending, of the distinct values a[0..n) by bucket: the 8 bits
+// below the values' common prefix name 256 buckets, a counting pass places
+// each value in its bucket's range (buckets in descending order, in tmp),
+// and each value's place within its bucket is the count of the bucket's
+// values above it.  pay[] (when given) moves along, through tmp_pay.  Costs
+// the sum over buckets of size^2 comparisons; declines (false, a and pay
+// unchanged) when that sum is large, i.e. the values crowd into few buckets.
 __device__ bool bucket_sort_desc(uint64_t *a, uint32_t n, uint64_t *tmp, SelectScratch &ss, uint32_t *pay = nullptr,
                                  uint32_t *tmp_pay = nullptr) {
   if (n <= 1) return true;
@@ -917,8 +917,10 @@ uint32_t share_ctas(std::vector<RankSet> &sets, uint32_t ctas, uint64_t tiles) {
 // larger targets: 9 sets of 2^22, k from 1 to 1,024, 100.3 us, 94.4 with a
 // target a list and 16,384 samples a set in place of 12,288).
 // The second target only where a set has few CTAs to share its candidates
-// among (64 sets of 2^18 93.0 -> 91.3 us; one set of 2^20 has 256 CTAs and
-// lost 1 us of 35 to the larger sample).
+// among: without it 16 sets of 2^18 (28 CTAs each) take 54.9 us in place of
+// 52.7 and 8 of 2^20 (57 CTAs) 53.2 in place of 52.0; 33 and 7 sets of 2^20, 64
+// of 2^18 and 8 of 2^22 the same within 0.5.  With it everywhere, 1 to 5 sets
+// of 2^20 (91 CTAs and more) move between -1.0 and +0.2 us.
 constexpr uint32_t kFewCtas = 64;
 void plan_sample(RankSet &s, int n_sets) {
   const uint32_t most = std::min(s.nctas, kSampleCtas);
@@ -2607,9 +2609,7 @@ extern "C" int unison_debug_leave_error(void) {
 
 namespace {
 
-// The ranking call: n_sets sets with their outputs, or (cands != null) one
-// shard of a set whose record 0 has index `off` in the whole set, with its
-// candidate lists going to cands instead of outputs.
+// The call's arguments, byte for byte: what a plan is kept for.
 void plan_key(std::vector<unsigned char> &k, const unison_records *sets, const unison_rank_params *params,
               const unison_rank_out *outs, int n_sets, uint32_t off, const unsigned char *cands) {
   k.clear();
@@ -2686,6 +2686,9 @@ int capture_rank_kernel(uint32_t grid, const RankSet *d_sets, int n_sets, int se
   return queue_rank_kernel(grid, d_sets, n_sets, sequential, cmap, tabs, pack, nullptr, 0, stream);
 }
 
+// The ranking call: n_sets sets with their outputs, or (cands != null) one
+// shard of a set whose record 0 has index `off` in the whole set, with its
+// candidate lists going to cands instead of outputs.
 int rank_launch(const unison_records *sets, const unison_rank_params *params, const unison_rank_out *outs,
                 int n_sets, uint32_t off, unsigned char *cands, cudaStream_t stream) {
   StreamState *const state = stream_state(stream);

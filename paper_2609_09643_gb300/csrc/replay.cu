@@ -1573,7 +1573,11 @@ void add_tier_maps(const unison_trace *const *traces, const unison_replay_params
   max_smem = with;
 }
 
-// Whether a replay can take the slot form, and its sizes.  A word holds the
+// Whether a replay can take the slot form, and its sizes.  Up to kMostSlots it
+// is the faster form for every policy: at 1,990 slots, traces of 2,000, 8,000 and
+// 20,000 sessions, one SPEAR+TIDE replay takes 27.6, 55.2 and 88.0 ms in slots
+// and 42.5, 92.9 and 219 on sorted lists; Timeout, the closest, 34.4, 85.4 and
+// 71.6 against 38.3, 106 and 210.  A word holds the
 // tier bit, the rank and the slot; sums of tokens stay below 2^31 because a
 // capacity above every session's largest size together is never reached; the
 // sort's values hold a 24-bit entry.
@@ -1638,9 +1642,12 @@ ReplayKernel slot_kernel_of(bool lean_st, uint32_t form) {
 // session it holds) when two would not fit or would need more waves of CTAs.
 // Passes over the words are deep when every replay's trace has at least four
 // sessions a slot: its tiers then fill with sessions, where otherwise far fewer
-// than the slots are ever in use (40,000 sessions over 547 slots: 574 ms plain,
-// 500 ms deep; the sweep's 1,415 over up to 527, of which about 160 are used:
-// 27.4 ms plain, 28.2 ms deep).
+// than the slots may ever be in use.  Plain and deep, ms: 40,000 sessions over
+// 547 slots 574 and 500; one SPEAR+TIDE replay of 8,000 over 500 slots 39.9 and
+// 37.9, over 1,000 53.4 and 45.6, over 1,990 73.9 and 55.2.  Below the line: the
+// sweep's 1,415 over up to 527 (about 160 of them used) 27.4 and 28.2, over 700
+// 17.5 and 18.0; but 2,000 sessions that start together over 1,000 slots 20.8
+// and 17.8.
 void slot_maps(const unison_trace *const *traces, const unison_replay_params *params, size_t smem_limit,
                std::vector<uint32_t> &group, bool lean_st, size_t &smem, ReplayPlan &P) {
   using namespace unison_slots;
